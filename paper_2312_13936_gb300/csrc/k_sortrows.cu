@@ -101,11 +101,35 @@ __global__ void k_gather_entries(const int32_t *ord, int64_t M, const int32_t *i
 
 }  // namespace
 
-size_t sort_rows_tmp_bytes(int64_t cap) {
-    const int64_t M = std::min<int64_t>(cap, kSortChunk) + 1;
-    // keys x2, ord x2, digit, perm, the entries' copy (4 + 8), partition scratch
-    return (size_t)M * (8 + 8 + 4 + 4 + 4 + 4 + 4 + 8) + partition_tmp_bytes(M, 1 << kSortDigitBits) + 256;
-}
+// The scratch of a chunk of M1 - 1 slots: byte offsets of its buffers, each
+// starting at a multiple of 256, and the total. Both the size asked for and
+// the pointers taken come from here.
+namespace {
+struct SortLayout {
+    size_t key, key2, ord, ord2, digit, perm, idx_copy, w_copy, key_off, part, total;
+    explicit SortLayout(int64_t M1) {
+        size_t at = 0;
+        auto take = [&](size_t bytes) {
+            const size_t here = at;
+            at += (bytes + 255) & ~(size_t)255;
+            return here;
+        };
+        key = take(8 * (size_t)M1);
+        key2 = take(8 * (size_t)M1);
+        ord = take(4 * (size_t)M1);
+        ord2 = take(4 * (size_t)M1);
+        digit = take(4 * (size_t)M1);
+        perm = take(4 * (size_t)M1);
+        idx_copy = take(4 * (size_t)M1);
+        w_copy = take(8 * (size_t)M1);
+        key_off = take(8 * ((1 << kSortDigitBits) + 2));
+        part = take(partition_tmp_bytes(M1, 1 << kSortDigitBits));
+        total = at;
+    }
+};
+}  // namespace
+
+size_t sort_rows_tmp_bytes(int64_t cap) { return SortLayout(std::min<int64_t>(cap, kSortChunk) + 1).total; }
 
 cudaError_t launch_sort_rows(int64_t n, const int64_t *off, const int32_t *deg, int32_t *idx, WInt *w, int64_t cap,
                              void *tmp, cudaStream_t s) {
@@ -136,22 +160,17 @@ cudaError_t launch_sort_rows(int64_t n, const int64_t *off, const int32_t *deg, 
     for (size_t k = 0; k + 1 < cut.size(); ++k) chunk_max = std::max(chunk_max, at(cut[k + 1]) - at(cut[k]));
     if (chunk_max > kSortChunk) return cudaErrorInvalidValue;  // one row beyond 2^30 slots
     char *p = static_cast<char *>(tmp);
-    auto take = [&](size_t bytes) {
-        char *q = p;
-        p += (bytes + 255) & ~(size_t)255;
-        return q;
-    };
-    const int64_t M1 = chunk_max + 1;
-    auto *key = reinterpret_cast<unsigned long long *>(take(8 * M1));
-    auto *key2 = reinterpret_cast<unsigned long long *>(take(8 * M1));
-    auto *ord = reinterpret_cast<int32_t *>(take(4 * M1));
-    auto *ord2 = reinterpret_cast<int32_t *>(take(4 * M1));
-    auto *digit = reinterpret_cast<int32_t *>(take(4 * M1));
-    auto *perm = reinterpret_cast<int32_t *>(take(4 * M1));
-    auto *idx_copy = reinterpret_cast<int32_t *>(take(4 * M1));
-    auto *w_copy = reinterpret_cast<WInt *>(take(8 * M1));
-    int64_t *key_off = reinterpret_cast<int64_t *>(take(8 * ((1 << kSortDigitBits) + 2)));
-    void *part_tmp = take(partition_tmp_bytes(M1, 1 << kSortDigitBits));
+    const SortLayout at_byte(chunk_max + 1);
+    auto *key = reinterpret_cast<unsigned long long *>(p + at_byte.key);
+    auto *key2 = reinterpret_cast<unsigned long long *>(p + at_byte.key2);
+    auto *ord = reinterpret_cast<int32_t *>(p + at_byte.ord);
+    auto *ord2 = reinterpret_cast<int32_t *>(p + at_byte.ord2);
+    auto *digit = reinterpret_cast<int32_t *>(p + at_byte.digit);
+    auto *perm = reinterpret_cast<int32_t *>(p + at_byte.perm);
+    auto *idx_copy = reinterpret_cast<int32_t *>(p + at_byte.idx_copy);
+    auto *w_copy = reinterpret_cast<WInt *>(p + at_byte.w_copy);
+    int64_t *key_off = reinterpret_cast<int64_t *>(p + at_byte.key_off);
+    void *part_tmp = p + at_byte.part;
     int tbits = 1;  // targets are row ids of the same graph: below n <= 2^tbits - 1, the gap marker
     while ((1LL << tbits) - 1 < n) ++tbits;
     for (size_t k = 0; k + 1 < cut.size(); ++k) {
