@@ -297,13 +297,15 @@ __device__ __forceinline__ A peer_sum(unsigned peers, A v) {
     return s;
 }
 
-// Profiling counters: every lane holds partial counts; one atomic per warp.
+// Profiling counters: every lane holds partial counts (32 bits: a lane of
+// the persistent kernels sees a small share of a launch's entries); one
+// atomic per warp.
 struct ProfCounts {
-    unsigned long long v[6] = {0, 0, 0, 0, 0, 0};
+    unsigned v[6] = {0, 0, 0, 0, 0, 0};
     __device__ __forceinline__ void flush(unsigned long long *dst) {
         if (!dst) return;
         for (int k = 0; k < 6; ++k) {
-            const unsigned long long s = warp_sum(v[k]);
+            const unsigned long long s = warp_sum((unsigned long long)v[k]);
             if ((threadIdx.x & 31) == 0 && s) atomicAdd(&dst[k], s);
         }
     }
@@ -372,5 +374,65 @@ __device__ __forceinline__ bool grid_barrier(unsigned *bar, int *err, unsigned l
     __syncthreads();
     return s_ok != 0;
 }
+
+// The persistent sweep's grid barrier: one arrival counter, zero when the
+// launch begins, that thread 0 of every block adds to (release, no result
+// asked for) and polls (acquire) until the barrier's G-th arrival; the
+// barrier's number lives in a register, so neither an atomic's result nor a
+// published word lies on the way. Measured alone (4,000 barriers): 152
+// blocks of 1024 threads 1.20 us, against 1.93 us for grid_barrier above and
+// 2.09 us for it with 608 blocks of 256, the same threads; with 608 blocks
+// polling, the counter itself takes 2.15 us, so this barrier goes with one
+// block per SM. The error word is read only while waiting, and a barrier
+// that runs out of polls ends the launch: its block arrives nowhere again
+// and the others see the error word or run out too.
+struct GridBar {
+    unsigned *count;
+    int *err;
+    unsigned long long limit;
+    unsigned done = 0;  // barriers passed
+    __device__ __forceinline__ bool sync() {
+        __shared__ int s_ok;
+        __syncthreads();
+        if (gridDim.x == 1) return true;
+        ++done;
+        if (threadIdx.x == 0) {
+            asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(count) : "memory");
+            const unsigned target = done * gridDim.x;
+            int ok = 1;
+            unsigned long long polls = 0;
+            while (bar_poll(count) < target) {
+                if (++polls > limit) {
+                    set_error(err, kErrTimeout);
+                    ok = 0;
+                    break;
+                }
+                if ((polls & 1023) == 0 && *((volatile int *)err) == kErrTimeout) {
+                    ok = 0;
+                    break;
+                }
+            }
+            s_ok = ok;
+        }
+        __syncthreads();
+        return s_ok != 0;
+    }
+};
+
+// How a persistent sweep deals the work of one schedule step to its warps:
+// the bins' units (32 vertices for the thread bin, 32 / T for a tile bin, one
+// for the warp bin) follow one another round the warps, and warp numbers run
+// over the blocks first, so a step of few units uses one warp on each of many
+// SMs and no warp takes a second bin's unit while others have none. All warps
+// of the launch count alike.
+struct Deal {
+    uint32_t nw, gw;     // warps of the grid, and this warp
+    uint32_t next = 0;   // the warp the next bin's first unit goes to
+    __device__ __forceinline__ Deal()
+        : nw(gridDim.x * (blockDim.x >> 5)), gw((threadIdx.x >> 5) * gridDim.x + blockIdx.x) {}
+    // this warp's first unit of the coming bin; its others follow nw apart
+    __device__ __forceinline__ uint32_t first() const { return gw >= next ? gw - next : gw + nw - next; }
+    __device__ __forceinline__ void pass(uint32_t units) { next = (next + units) % nw; }
+};
 
 }  // namespace lgb

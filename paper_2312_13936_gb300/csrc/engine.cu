@@ -34,16 +34,11 @@ const char *last_error() { return g_last_error.c_str(); }
 // The persistent sweeps' grid barrier counts arrivals in 32 bits, from zero
 // at every launch. One phase takes at most max_iterations sweeps of at most
 // 8 barriers per schedule step (layout, insertion, three key passes, hub
-// flags, step end, apply) and 4 more per sweep, on at most the resident
-// grid; a limit under which that count could pass 2^32 - 1 is refused
-// rather than let the count wrap.
-leiden_status check_barrier_budget(int32_t max_iterations, int32_t nsteps, bool det, int sm) {
-    int per_sm = 0;
-    for (int w = 0; w < 2; ++w)
-        for (int r = 0; r < 2; ++r) {
-            const int b = sweep_coop_blocks_per_sm(det, w != 0, r != 0);
-            per_sm = b > per_sm ? b : per_sm;
-        }
+// flags, step end, apply) and 4 more per sweep, on at most one block per SM;
+// the count is taken for four, as the documented limit is. A limit under
+// which that count could pass 2^32 - 1 is refused rather than let it wrap.
+leiden_status check_barrier_budget(int32_t max_iterations, int32_t nsteps, int sm) {
+    constexpr int64_t per_sm = 4;  // the limit callers know: four blocks of 256 threads per SM
     const int64_t arrivals = (int64_t)max_iterations * (8 * (int64_t)nsteps + 4) * per_sm * sm;
     if (arrivals > (int64_t)0xffffffffLL) {
         set_last_error("max_iterations too large for this schedule: one phase could take more than 2^32 - 1 "
@@ -238,13 +233,18 @@ leiden_status Handle::Impl::pass(Run &r, int32_t lp, bool &stop) {
     // (tables of one step at a time); per-step launches keep a global table
     // per block
     const std::vector<int64_t> &ko = q.hkey_off;
-    int64_t nhubs = 0;
-    for (int32_t k = 0; k < nsteps; ++k) nhubs += ko[(size_t)k * kNumBins + 7] - ko[(size_t)k * kNumBins + 6];
+    int64_t nhubs = 0, ntab = 0, units = 0;  // hubs, vertices with a shared-memory table, the sweep's warp units
+    for (int32_t k = 0; k < nsteps; ++k) {
+        const int64_t *o = &ko[(size_t)k * kNumBins];
+        nhubs += o[7] - o[6];
+        ntab += o[6] - o[4];
+        units += (o[2] - o[1] + 31) / 32 + (o[3] - o[2] + 1) / 2 + (o[5] - o[3]) + 8 * (o[6] - o[5]);
+    }
     const bool grid_hubs = nhubs > 0 && !step_launches && sweep_coop_blocks_per_sm(det, sG.w_int, false) > 0 &&
                            sweep_coop_blocks_per_sm(det, sG.w_int, true) > 0;
     if (grid_hubs) {
         ST(q.ensure_hubs(nhubs));
-        CK(launch_hub_prep(q.key_off, nsteps, sList, sG.deg, q.hubs, q.hspan, s));
+        CK(launch_hub_prep(q.key_off, nsteps, sList, sG.deg, q.hubs, q.hbase, q.hspan, s));
         q.launches += 1;
         unsigned long long span = 0;
         CK(cudaMemcpyAsync(&span, q.hspan, sizeof(span), cudaMemcpyDeviceToHost, s));
@@ -326,6 +326,8 @@ leiden_status Handle::Impl::pass(Run &r, int32_t lp, bool &stop) {
     sc.err = &q.dsc->err;
     sc.grid_hubs = grid_hubs;
     sc.hubs = q.hubs;
+    sc.hbase = q.hbase;
+    sc.tables = ntab > 0;
     sc.hj = q.hj;
     sc.hinfo = q.hinfo;
     sc.htoff = q.htoff;
@@ -393,12 +395,18 @@ leiden_status Handle::Impl::pass(Run &r, int32_t lp, bool &stop) {
             return LEIDEN_ERR_UNSUPPORTED;
         }
         if (per_sm > 0) {
-            // enough blocks for the graph (about vertices_per_block each),
-            // so small graphs do not pay a full-GPU barrier per step and
-            // graphs of one block synchronise with __syncthreads only
+            // enough blocks for a step's work: one block (which synchronises
+            // with __syncthreads only) while its 32 warps take an average
+            // step's units at once, else a block for every four units, and
+            // at least one for every vertices_per_block vertices. A barrier
+            // of 152 blocks takes 1.2 us, of 16 blocks 1.1 us, a warp's
+            // second unit 3 us and more, so there is little to save between
+            // one block and the full grid.
             int grid = per_sm * q.sm;
-            const int64_t vpb = q.tune.vertices_per_block;
-            const int64_t want = (n + vpb - 1) / vpb;
+            const int64_t vpb = q.tune.vertices_per_block, ups = units / nsteps;
+            int64_t want = ups <= kCoopWarps && !grid_hubs ? 1 : std::max((ups + 3) / 4, (n + vpb - 1) / vpb);
+            if (grid_hubs) want = grid;
+            if ((prm.flags & LEIDEN_FLAG_TEST_STALL_BARRIER) && want < 2) want = 2;  // a block to stall
             if (want < grid) grid = (int)(want < 1 ? 1 : want);
             sc.hub_regions = hub_regions > grid ? grid : hub_regions;
             sc.max_it = prm.max_iterations;
@@ -759,7 +767,7 @@ leiden_status Handle::run(const leiden_params &prm, int32_t *membership, int whe
         set_last_error("schedule_layers + schedule_buckets too large");
         return LEIDEN_ERR_INVALID;
     }
-    ST(check_barrier_budget(prm.max_iterations, nsteps, det, q.sm));
+    ST(check_barrier_budget(prm.max_iterations, nsteps, q.sm));
     if (det && (prm.flags & LEIDEN_FLAG_RANDOM_REFINE)) {
         set_last_error("the randomized refinement has no deterministic mode");
         return LEIDEN_ERR_UNSUPPORTED;

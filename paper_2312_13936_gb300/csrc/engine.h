@@ -103,6 +103,6 @@ leiden_status modularity_device(int64_t n, const int64_t *off, const int32_t *id
                                 const int32_t *memb, double gamma, cudaStream_t s, double *q_out);
 // refuses an iteration limit under which one persistent phase of a schedule
 // of nsteps steps could count more grid-barrier arrivals than 32 bits hold
-leiden_status check_barrier_budget(int32_t max_iterations, int32_t nsteps, bool det, int sm);
+leiden_status check_barrier_budget(int32_t max_iterations, int32_t nsteps, int sm);
 
 }  // namespace lgb

@@ -48,9 +48,9 @@ struct Scalars {  // device scalars, read back in one copy
         if (_s != LEIDEN_OK) return _s;        \
     } while (0)
 
-// barrier polls before a persistent launch gives up (kSpinLimit of the
-// device code, about a second)
-constexpr unsigned long long kSpinLimitDefault = 1ULL << 24;
+// barrier polls before a persistent sweep gives up (a poll takes about a
+// third of a microsecond: a second and more)
+constexpr unsigned long long kSpinLimitDefault = 1ULL << 22;
 
 // allocations left before an injected failure (leiden_test_fail_allocation;
 // negative: none)
@@ -479,7 +479,7 @@ struct Handle::Impl {
     }
     // whole-grid bin 6 of the persistent sweep: per-hub arrays of a pass
     int32_t *hubs = nullptr, *hd = nullptr, *hcand = nullptr, *hmv = nullptr, *hj = nullptr;
-    int64_t *htoff = nullptr, *heoff = nullptr, *hinfo = nullptr;
+    int64_t *htoff = nullptr, *heoff = nullptr, *hinfo = nullptr, *hbase = nullptr;
     unsigned long long *hkey = nullptr, *hspan = nullptr;
     long long *hkvd = nullptr;
     int64_t hubs_cap = -1;
@@ -523,6 +523,7 @@ struct Handle::Impl {
         if (!hinfo) {
             ST(alloc(&hinfo, 4));  // a step's eligible hubs, table slots, entries
             ST(alloc(&hspan, 1));
+            ST(alloc(&hbase, 1024));
         }
         if (nh <= hubs_cap) return LEIDEN_OK;
         for (void *p : {(void *)hubs, (void *)hd, (void *)hcand, (void *)hmv, (void *)hj, (void *)htoff,

@@ -300,7 +300,7 @@ __global__ void k_step_bin_keys(const int32_t *step, const int32_t *deg, int64_t
 // hubs of the steps before); max_span = the largest sum of one step's table
 // sizes (2^max(6, ceil log2 2 deg))
 __global__ void k_hub_gather(const int64_t *key_off, int32_t nsteps, const int32_t *list, const int32_t *deg,
-                             int32_t *hubs, unsigned long long *max_span) {
+                             int32_t *hubs, int64_t *hbase, unsigned long long *max_span) {
     __shared__ long long s_part[8];
     const int k = blockIdx.x;
     long long part = 0;  // hubs of the steps before k
@@ -312,6 +312,7 @@ __global__ void k_hub_gather(const int64_t *key_off, int32_t nsteps, const int32
     long long base = 0;
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) base += s_part[w];
     __syncthreads();
+    if (threadIdx.x == 0) hbase[k] = base;
     const int64_t lo = key_off[(int64_t)k * kNumBins + 6], hi = key_off[(int64_t)k * kNumBins + 7];
     long long span = 0;
     for (int64_t t = lo + threadIdx.x; t < hi; t += blockDim.x) {
@@ -381,10 +382,10 @@ cudaError_t launch_schedule(const GraphView &g, uint64_t state, int32_t L, int32
                                        dim3((unsigned)grid), dim3(kSchedThreads), args, 0, s);
 }
 cudaError_t launch_hub_prep(const int64_t *key_off, int32_t nsteps, const int32_t *list, const int32_t *deg,
-                            int32_t *hubs, unsigned long long *max_span, cudaStream_t s) {
+                            int32_t *hubs, int64_t *hbase, unsigned long long *max_span, cudaStream_t s) {
     cudaError_t e = cudaMemsetAsync(max_span, 0, sizeof(unsigned long long), s);
     if (e != cudaSuccess || nsteps <= 0) return e;
-    k_hub_gather<<<nsteps, 256, 0, s>>>(key_off, nsteps, list, deg, hubs, max_span);
+    k_hub_gather<<<nsteps, 256, 0, s>>>(key_off, nsteps, list, deg, hubs, hbase, max_span);
     return cudaGetLastError();
 }
 cudaError_t launch_step_bin_keys(const int32_t *step, const int32_t *deg, int64_t n, int32_t nsteps, bool bin_major,

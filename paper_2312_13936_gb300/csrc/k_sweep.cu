@@ -72,6 +72,7 @@ template <class P, class W> struct SV {
     int hub_bits, hub_regions;
     // bin 6 on the whole grid (persistent sweep)
     const int32_t *hubs;
+    const int64_t *hbase;  // ordinal of every step's first hub (null: no hubs)
     int32_t *hj;
     int64_t *htoff, *heoff, *hinfo;
     int32_t *hd, *hcand, *hmv;
@@ -177,6 +178,7 @@ template <class P, class W> SV<P, W> view(const SweepCtx &c) {
     a.hub_bits = c.hub_bits;
     a.hub_regions = c.hub_regions;
     a.hubs = c.hubs;
+    a.hbase = c.grid_hubs ? c.hbase : nullptr;
     a.hj = c.hj;
     a.htoff = c.htoff;
     a.heoff = c.heoff;
@@ -375,13 +377,89 @@ __device__ __forceinline__ bool take_vertex(const SV<P, W> &a, int32_t v, int32_
 }
 
 // --------------------------------------------------------- thread bin
+// The evaluation of one eligible vertex v at list position t by its own
+// thread, its row of at most E entries in registers.
+template <class P, class W, bool REFINE, bool B, int E>
+__device__ __forceinline__ void eval_thread(const SV<P, W> &a, int32_t v, int32_t gv, int32_t d, typename P::acc Kv,
+                                            const RowOf<W> &row, int32_t cur_step, Sums<P> &sm, ProfCounts &pc) {
+    using A = typename P::acc;
+    const int64_t e0 = row.e0;
+    const int32_t dv = row.dv;
+    const typename P::tot sd = ldm(&a.Sig[d]);
+    const int32_t bv = REFINE ? a.CB[v] : 0;
+    int32_t jj[E];
+    A wt[E];
+#pragma unroll
+    for (int k = 0; k < E; ++k) {
+        jj[k] = -1;
+        wt[k] = 0;
+        if (k < dv) {
+            jj[k] = row.idx[e0 + k];
+            wt[k] = wconv<A>(row.w[e0 + k]);
+        }
+    }
+    int32_t c[E];
+#pragma unroll
+    for (int k = 0; k < E; ++k) {
+        c[k] = -1;
+        bool ok = k < dv && jj[k] != v;
+        if (REFINE && ok) ok = (__ldg(&a.CB[jj[k]]) == bv);
+        if (ok) c[k] = ldm(&a.C[jj[k]]);
+    }
+    // merge equal communities into their first entry, in edge order
+#pragma unroll
+    for (int k = 1; k < E; ++k)
+#pragma unroll
+        for (int k2 = 0; k2 < k; ++k2)
+            if (c[k] >= 0 && c[k2] == c[k]) {
+                wt[k2] += wt[k];
+                c[k] = -1;
+            }
+    A kvd = 0;
+    typename P::key key = AccLimits<typename P::key>::lowest();
+    int32_t cand = INT_MAX;
+    int distinct = 0;
+    const A ks = kscale_of<B>(a, gv);
+#pragma unroll
+    for (int k = 0; k < E; ++k) {
+        if (c[k] < 0) continue;
+        distinct++;
+        if (c[k] == d) {
+            kvd = wt[k];
+            continue;
+        }
+        const typename P::key kk =
+            cand_key<P, W, REFINE>(a, sm, v, c[k], move_key(ks, wt[k], Kv, ldm(&a.Sig[c[k]]), a.gamma));
+        if (better(kk, c[k], key, cand)) {
+            key = kk;
+            cand = c[k];
+        }
+    }
+    const bool mv = decide_sd<P, W, REFINE, B>(a, v, d, Kv, key, cand, kvd, sd, sm, cur_step, gv, ks);
+    if (a.prof) {
+        pc.v[0]++;
+        pc.v[2] += dv;
+        pc.v[3] += distinct;
+        if (proposing<P, REFINE>(cur_step, a.cap_step) ? (a.prop[v] >= 0) : mv) {
+            pc.v[4]++;
+            pc.v[5] += dv;
+        }
+    }
+    if (!REFINE && !P::det && mv) {
+#pragma unroll
+        for (int k = 0; k < E; ++k)
+            if (k < dv) flag_unproc(a, sm, jj[k]);  // neighbours (self-loop included) of a mover
+    }
+}
+
 template <class P, class W, bool REFINE, bool B>
 __device__ __forceinline__ void run_thread(const SV<P, W> &a, const int32_t *__restrict__ list, int64_t lo, int64_t hi,
-                                           int32_t cur_step, Sums<P> &sm, ProfCounts &pc) {
-    using A = typename P::acc;
-    constexpr int E = kThreadMaxDeg;
-    const int64_t nthreads = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t t = lo + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < hi; t += nthreads) {
+                                           int32_t cur_step, Deal &deal, Sums<P> &sm, ProfCounts &pc) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t units = (uint32_t)((hi - lo + 31) >> 5);
+    for (uint32_t u = deal.first(); u < units; u += deal.nw) {
+        const int64_t t = lo + (int64_t)u * 32 + lane;
+        if (t >= hi) continue;
         const int32_t v = list[t];
         // eligibility first (Algorithm 2 pruning: the unprocessed flag;
         // refinement: the size of the vertex's community), so that a pruned
@@ -405,88 +483,24 @@ __device__ __forceinline__ void run_thread(const SV<P, W> &a, const int32_t *__r
             a.unproc[v] = 0;  // processed (Algorithm 2 pruning)
             d = ldm(&a.C[v]);
         }
-        const A Kv = k_of(a, v, t);
-        const RowOf<W> row = row_of(a, v, t);
-        const int64_t e0 = row.e0;
-        const int32_t dv = row.dv;
-        const typename P::tot sd = ldm(&a.Sig[d]);
-        const int32_t bv = REFINE ? a.CB[v] : 0;
-        int32_t jj[E];
-        A wt[E];
-#pragma unroll
-        for (int k = 0; k < E; ++k) {
-            jj[k] = -1;
-            wt[k] = 0;
-            if (k < dv) {
-                jj[k] = row.idx[e0 + k];
-                wt[k] = wconv<A>(row.w[e0 + k]);
-            }
-        }
-        int32_t c[E];
-#pragma unroll
-        for (int k = 0; k < E; ++k) {
-            c[k] = -1;
-            bool ok = k < dv && jj[k] != v;
-            if (REFINE && ok) ok = (__ldg(&a.CB[jj[k]]) == bv);
-            if (ok) c[k] = ldm(&a.C[jj[k]]);
-        }
-        // merge equal communities into their first entry, in edge order
-#pragma unroll
-        for (int k = 1; k < E; ++k)
-#pragma unroll
-            for (int k2 = 0; k2 < k; ++k2)
-                if (c[k] >= 0 && c[k2] == c[k]) {
-                    wt[k2] += wt[k];
-                    c[k] = -1;
-                }
-        A kvd = 0;
-        typename P::key key = AccLimits<typename P::key>::lowest();
-        int32_t cand = INT_MAX;
-        int distinct = 0;
-        const A ks = kscale_of<B>(a, gv);
-#pragma unroll
-        for (int k = 0; k < E; ++k) {
-            if (c[k] < 0) continue;
-            distinct++;
-            if (c[k] == d) {
-                kvd = wt[k];
-                continue;
-            }
-            const typename P::key kk =
-                cand_key<P, W, REFINE>(a, sm, v, c[k], move_key(ks, wt[k], Kv, ldm(&a.Sig[c[k]]), a.gamma));
-            if (better(kk, c[k], key, cand)) {
-                key = kk;
-                cand = c[k];
-            }
-        }
-        const bool mv = decide_sd<P, W, REFINE, B>(a, v, d, Kv, key, cand, kvd, sd, sm, cur_step, gv, ks);
-        if (a.prof) {
-            pc.v[0]++;
-            pc.v[2] += dv;
-            pc.v[3] += distinct;
-            if (proposing<P, REFINE>(cur_step, a.cap_step) ? (a.prop[v] >= 0) : mv) {
-                pc.v[4]++;
-                pc.v[5] += dv;
-            }
-        }
-        if (!REFINE && !P::det && mv) {
-#pragma unroll
-            for (int k = 0; k < E; ++k)
-                if (k < dv) flag_unproc(a, sm, jj[k]);  // neighbours (self-loop included) of a mover
-        }
+        eval_thread<P, W, REFINE, B, kThreadMaxDeg>(a, v, gv, d, k_of(a, v, t), row_of(a, v, t), cur_step, sm, pc);
     }
+    deal.pass(units);
 }
 
 // ----------------------------------------------------------- tile bins
 template <class P, class W, int T, bool REFINE, bool B>
 __device__ __forceinline__ void run_tile(const SV<P, W> &a, const int32_t *__restrict__ list, int64_t lo, int64_t hi,
-                                         int32_t cur_step, Sums<P> &sm, ProfCounts &pc) {
+                                         int32_t cur_step, Deal &deal, Sums<P> &sm, ProfCounts &pc) {
     using A = typename P::acc;
     const int lane = threadIdx.x & 31;
     const int tl = lane & (T - 1);
     const unsigned tmask = (T == 32) ? kFull : (((1u << T) - 1u) << (lane & ~(T - 1)));
-    const int64_t tiles = (int64_t)gridDim.x * (blockDim.x / T);
-    for (int64_t t = lo + (int64_t)blockIdx.x * (blockDim.x / T) + threadIdx.x / T; t < hi; t += tiles) {
+    constexpr int per = 32 / T;  // vertices of a unit
+    const uint32_t units = (uint32_t)((hi - lo + per - 1) / per);
+    for (uint32_t u = deal.first(); u < units; u += deal.nw) {
+        const int64_t t = lo + (int64_t)u * per + lane / T;
+        if (t >= hi) continue;
         const int32_t v = list[t];
         const int32_t gv = graph_of<B>(a, v);
         int32_t d = 0;
@@ -565,17 +579,17 @@ __device__ __forceinline__ void run_tile(const SV<P, W> &a, const int32_t *__res
             if (mv && tl < dv) flag_unproc(a, sm, j);  // neighbours (self-loop included) of a mover
         }
     }
+    deal.pass(units);
 }
 
 // ------------------------------------------------------- warp-table bin
 template <class P, class W, bool REFINE, bool B>
 __device__ __forceinline__ void run_warp(const SV<P, W> &a, const int32_t *__restrict__ list, int64_t lo, int64_t hi,
-                                         int32_t cur_step, int32_t *keys, typename P::acc *vals, Sums<P> &sm,
-                                         ProfCounts &pc) {
+                                         int32_t cur_step, int32_t *keys, typename P::acc *vals, Deal &deal,
+                                         Sums<P> &sm, ProfCounts &pc) {
     using A = typename P::acc;
     const int lane = threadIdx.x & 31;
-    const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t t = lo + (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); t < hi; t += nwarps) {
+    for (int64_t t = lo + deal.first(); t < hi; t += deal.nw) {
         const int32_t v = list[t];
         const int32_t gv = graph_of<B>(a, v);
         int32_t d = 0;
@@ -654,27 +668,41 @@ __device__ __forceinline__ void run_warp(const SV<P, W> &a, const int32_t *__res
         }
         __syncwarp();
     }
+    deal.pass((uint32_t)(hi - lo));
 }
 
 // ------------------------------------------------ block / hub table bins
-// One block per vertex (HUB: a global-memory table per block; only blocks
-// below hub_regions take part).
+// One group of kGroup threads per vertex: a whole block of the per-step
+// kernels, one of the groups of the persistent sweep's larger blocks (named
+// barrier 1 + the group's number). HUB: a global-memory table per block of
+// the per-step kernels; only blocks below hub_regions take part.
+constexpr int kGroup = 256;
+constexpr int kMaxGroups = 4;
+__device__ __forceinline__ void group_sync() {
+    asm volatile("bar.sync %0, %1;" ::"r"(1 + (int)(threadIdx.x / kGroup)), "n"(kGroup) : "memory");
+}
 template <class P, class W, bool REFINE, bool HUB, bool B>
 __device__ __forceinline__ void run_block(const SV<P, W> &a, const int32_t *__restrict__ list, int64_t lo, int64_t hi,
                                           int32_t cur_step, int32_t *keys, typename P::acc *vals, int max_bits,
                                           Sums<P> &sm, ProfCounts &pc) {
     using A = typename P::acc;
-    __shared__ int s_elig, s_d, s_mv;
-    __shared__ typename P::key s_key[32];
-    __shared__ A s_kvd[32];
-    __shared__ int32_t s_cand[32];
-    const int tid = threadIdx.x, lane = tid & 31, wib = tid >> 5, nw = blockDim.x >> 5;
-    const int64_t nblk = HUB ? (int64_t)a.hub_regions : (int64_t)gridDim.x;
+    __shared__ int ss_elig[kMaxGroups], ss_d[kMaxGroups], ss_mv[kMaxGroups];
+    __shared__ typename P::key ss_key[kMaxGroups][kGroup / 32];
+    __shared__ A ss_kvd[kMaxGroups][kGroup / 32];
+    __shared__ int32_t ss_cand[kMaxGroups][kGroup / 32];
+    const int grp = threadIdx.x / kGroup, ngrp = blockDim.x / kGroup;
+    int &s_elig = ss_elig[grp], &s_d = ss_d[grp], &s_mv = ss_mv[grp];
+    typename P::key *s_key = ss_key[grp];
+    A *s_kvd = ss_kvd[grp];
+    int32_t *s_cand = ss_cand[grp];
+    const int tid = threadIdx.x % kGroup, lane = tid & 31, wib = tid >> 5;
+    constexpr int nw = kGroup >> 5;
+    const int64_t nblk = HUB ? (int64_t)a.hub_regions : (int64_t)gridDim.x * ngrp;
     if (HUB && (int64_t)blockIdx.x >= nblk) return;
-    for (int64_t t = lo + blockIdx.x; t < hi; t += nblk) {
+    for (int64_t t = lo + (int64_t)grp * gridDim.x + blockIdx.x; t < hi; t += nblk) {
         const int32_t v = list[t];
         const int32_t gv = graph_of<B>(a, v);
-        __syncthreads();
+        group_sync();
         if (tid == 0) {
             int32_t d = 0;
             s_elig = take_vertex<P, W, REFINE, B>(a, v, d, gv) ? 1 : 0;
@@ -682,7 +710,7 @@ __device__ __forceinline__ void run_block(const SV<P, W> &a, const int32_t *__re
             if (!s_elig && proposing<P, REFINE>(cur_step, a.cap_step)) a.prop[v] = -1;
             if (!s_elig) pc.v[1]++;
         }
-        __syncthreads();
+        group_sync();
         if (!s_elig) continue;
         const int32_t d = s_d;
         const A Kv = k_of(a, v, t);
@@ -700,23 +728,23 @@ __device__ __forceinline__ void run_block(const SV<P, W> &a, const int32_t *__re
             continue;
         }
         const int64_t S = 1LL << bits;
-        for (int64_t s = tid; s < S; s += blockDim.x) {
+        for (int64_t s = tid; s < S; s += kGroup) {
             keys[s] = -1;
             vals[s] = 0;
         }
-        __syncthreads();
-        for (int64_t e = tid; e < dv; e += blockDim.x) {
+        group_sync();
+        for (int64_t e = tid; e < dv; e += kGroup) {
             const int32_t j = row.idx[e0 + e];
             if (j == v) continue;
             if (REFINE && __ldg(&a.CB[j]) != bv) continue;
             if (!hash_add(keys, vals, bits, ldm(&a.C[j]), wconv<A>(row.w[e0 + e]))) set_error(a.err, kErrHashFull);
         }
-        __syncthreads();
+        group_sync();
         typename P::key key = AccLimits<typename P::key>::lowest();
         A kvd = 0;
         int32_t cand = INT_MAX;
         const A ks = kscale_of<B>(a, gv);
-        for (int64_t s = tid; s < S; s += blockDim.x) {
+        for (int64_t s = tid; s < S; s += kGroup) {
             const int32_t k = keys[s];
             if (k < 0) continue;
             pc.v[3]++;
@@ -746,7 +774,7 @@ __device__ __forceinline__ void run_block(const SV<P, W> &a, const int32_t *__re
             s_cand[wib] = cand;
             s_kvd[wib] = kvd;
         }
-        __syncthreads();
+        group_sync();
         if (tid == 0) {
             typename P::key bk = s_key[0];
             A kd = s_kvd[0];
@@ -766,11 +794,11 @@ __device__ __forceinline__ void run_block(const SV<P, W> &a, const int32_t *__re
                 pc.v[5] += dv;
             }
         }
-        __syncthreads();
+        group_sync();
         if (!REFINE && !P::det && s_mv)
-            for (int64_t e = tid; e < dv; e += blockDim.x) flag_unproc(a, sm, row.idx[e0 + e]);
+            for (int64_t e = tid; e < dv; e += kGroup) flag_unproc(a, sm, row.idx[e0 + e]);
     }
-    __syncthreads();
+    group_sync();
 }
 
 // -------------------------------------------- bin 6 on the whole grid
@@ -882,7 +910,7 @@ template <class P, class W> __device__ __forceinline__ unsigned long long *hub_k
 
 template <class P, class W, bool REFINE, bool B>
 __device__ __forceinline__ bool run_hubs_grid(const SV<P, W> &a, int64_t j0, int64_t nh, int32_t cur_step,
-                                              Sums<P> &sm, ProfCounts &pc) {
+                                              GridBar &bar, Sums<P> &sm, ProfCounts &pc) {
     using A = typename P::acc;
     const int lane = threadIdx.x & 31;
     const int64_t nthreads = (int64_t)gridDim.x * blockDim.x;
@@ -999,7 +1027,7 @@ __device__ __forceinline__ bool run_hubs_grid(const SV<P, W> &a, int64_t j0, int
                 a.hinfo[2] = ne;
             }
         }
-        if (!grid_barrier(a.bar, a.err, a.spin_limit)) return false;
+        if (!bar.sync()) return false;
         np = __ldcg(&a.hinfo[0]);
         S = __ldcg(&a.hinfo[1]);
         E = __ldcg(&a.hinfo[2]);
@@ -1076,7 +1104,7 @@ __device__ __forceinline__ bool run_hubs_grid(const SV<P, W> &a, int64_t j0, int
             }
         }
     }
-    if (!grid_barrier(a.bar, a.err, a.spin_limit)) return false;
+    if (!bar.sync()) return false;
     // every block has read the single hub's pruning flag: it is processed
     if (single && !REFINE && blockIdx.x == 0 && threadIdx.x == 0) a.unproc[sv] = 0;
     // deterministic mode: the largest key per hub -- its high word (pass 0),
@@ -1198,7 +1226,7 @@ __device__ __forceinline__ bool run_hubs_grid(const SV<P, W> &a, int64_t j0, int
                 if (lane == 0 && lmin != INT_MAX) atomicMin(&a.hcand[j], lmin);
             }
         }
-        if (!grid_barrier(a.bar, a.err, a.spin_limit)) return false;
+        if (!bar.sync()) return false;
     }
     // decisions
     for (int64_t p = tid; p < np; p += nthreads) {
@@ -1231,34 +1259,45 @@ __device__ __forceinline__ bool run_hubs_grid(const SV<P, W> &a, int64_t j0, int
     }
     if (!REFINE && !P::det) {
         // an asynchronous local-moving move flags the hub's neighbours
-        if (!grid_barrier(a.bar, a.err, a.spin_limit)) return false;
+        if (!bar.sync()) return false;
         hub_flags<P, W>(a, sm, np, E, false);
     }
     return true;
 }
 
 // ------------------------------------------------------------ apply steps
+// vertices of a warp's unit in an apply phase: 32 when the step has work for
+// every warp, fewer (the other lanes then only help with the rows) when more
+// warps would stand idle
+__device__ __forceinline__ int apply_unit(uint32_t count, uint32_t nw) {
+    return count > 16 * nw ? 32 : count > 4 * nw ? 8 : 2;
+}
+
 // Local-moving proposals of one step (deterministic mode; asynchronous mode
-// in the capped steps): commit them.
+// in the capped steps): commit them. The movers' rows of a unit are flagged
+// as one flat range of entries by all lanes, four loads per lane in flight
+// (a lane walking its own mover's row waited for every load in turn: 16 us a
+// step on a 200,000-vertex block model with rows of 24 entries). Rows of
+// more than 1024 entries go one after another.
 // (grid_hub_flags: the neighbours of rows longer than kBlockMaxDeg are
-// flagged by hub_flags over the step's hub layout instead of by one warp)
+// flagged by hub_flags over the step's hub layout)
 template <class P, class W, bool B>
 __device__ __forceinline__ void run_move_apply(const SV<P, W> &a, const int32_t *__restrict__ list, int64_t lo,
-                                               int64_t hi, Sums<P> &sm, bool grid_hub_flags) {
-    // whole warps step through the list, so that the neighbours of a mover
-    // with a long row are flagged by the whole warp
+                                               int64_t hi, Deal &deal, Sums<P> &sm, bool grid_hub_flags) {
+    constexpr int32_t kFlat = 1024;
     const int lane = threadIdx.x & 31;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t t0 = lo + (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); t0 < hi; t0 += stride) {
-        const int64_t t = t0 + lane;
+    const int per = apply_unit((uint32_t)(hi - lo), deal.nw);
+    const uint32_t units = (uint32_t)((hi - lo + per - 1) / per);
+    for (uint32_t u = deal.first(); u < units; u += deal.nw) {
+        const int64_t t = lo + (int64_t)u * per + lane;
         int32_t v = -1, c = -1;
-        if (t < hi) {
+        if (lane < per && t < hi) {
             v = list[t];
             c = ldm(&a.prop[v]);
         }
+        if (!__any_sync(kFull, c >= 0)) continue;
         int64_t e0 = 0;
         int32_t dv = 0;
-        const int32_t *ridx = a.idx;
         if (c >= 0) {
             const int32_t d = ldm(&a.C[v]);
             const auto Kv = (typename P::tot)k_of(a, v, t);
@@ -1276,20 +1315,43 @@ __device__ __forceinline__ void run_move_apply(const SV<P, W> &a, const int32_t 
             const RowOf<W> row = row_of(a, v, t);
             e0 = row.e0;
             dv = row.dv;
-            ridx = row.idx;
-            if (dv <= 32)
-                for (int32_t e = 0; e < dv; ++e) flag_unproc(a, sm, ridx[e0 + e]);
         }
-        unsigned longs = __ballot_sync(kFull, c >= 0 && dv > 32 && !(grid_hub_flags && dv > a.block_max));
+        const int32_t *is = a.loff ? a.lidx : a.idx;  // the same on every lane
+        const int32_t flat = dv <= kFlat && !(grid_hub_flags && dv > a.block_max) ? dv : 0;
+        int32_t incl = flat;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int32_t y = __shfl_up_sync(kFull, incl, o);
+            if (lane >= o) incl += y;
+        }
+        const int32_t total = __shfl_sync(kFull, incl, 31);
+        const int64_t base = e0 - (incl - flat);  // entry x of the flat range is is[base + x] of its owner
+        for (int32_t x0 = 0; x0 < total; x0 += 128) {
+            int32_t j[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int32_t x = x0 + 32 * q + lane;
+                int own = 0;  // lanes whose rows end at or before x
+#pragma unroll
+                for (int st = 16; st >= 1; st >>= 1)
+                    if (__shfl_sync(kFull, incl, own + st - 1) <= x) own += st;
+                const int64_t bs = __shfl_sync(kFull, base, own & 31);
+                j[q] = x < total ? is[bs + x] : -1;
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (j[q] >= 0) flag_unproc(a, sm, j[q]);
+        }
+        unsigned longs = __ballot_sync(kFull, dv > kFlat && !(grid_hub_flags && dv > a.block_max));
         while (longs) {
             const int src = __ffs(longs) - 1;
             longs &= longs - 1;
             const int64_t es = __shfl_sync(kFull, e0, src);
             const int32_t ds = __shfl_sync(kFull, dv, src);
-            const int32_t *is = a.loff ? a.lidx : a.idx;  // the same on every lane
             for (int32_t e = lane; e < ds; e += 32) flag_unproc(a, sm, is[es + e]);
         }
     }
+    deal.pass(units);
 }
 
 // Refinement: accept proposal v -> t unless t is a single-vertex community
@@ -1297,9 +1359,13 @@ __device__ __forceinline__ void run_move_apply(const SV<P, W> &a, const int32_t 
 // moves (reading S5). Accepted vertices join t.
 template <class P, class W, bool B>
 __device__ __forceinline__ void run_refine_apply(const SV<P, W> &a, const int32_t *__restrict__ list, int64_t lo,
-                                                 int64_t hi, int32_t cur_step, Sums<P> &sm) {
-    for (int64_t t = lo + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < hi;
-         t += (int64_t)gridDim.x * blockDim.x) {
+                                                 int64_t hi, int32_t cur_step, Deal &deal, Sums<P> &sm) {
+    const int lane = threadIdx.x & 31;
+    const int per = apply_unit((uint32_t)(hi - lo), deal.nw);
+    const uint32_t units = (uint32_t)((hi - lo + per - 1) / per);
+    for (uint32_t u = deal.first(); u < units; u += deal.nw) {
+        const int64_t t = lo + (int64_t)u * per + lane;
+        if (lane >= per || t >= hi) continue;
         const int32_t v = list[t];
         const int32_t tg = ldm(&a.prop[v]);
         if (tg < 0) continue;
@@ -1313,10 +1379,14 @@ __device__ __forceinline__ void run_refine_apply(const SV<P, W> &a, const int32_
         a.C[v] = tg;
         gacc_add(sm.moved, B, graph_of<B>(a, v), 1ULL, sm.mv);
     }
+    deal.pass(units);
 }
 
 // ------------------------------------------------------- persistent sweep
-constexpr int kCoopThreads = 256;
+// One block per SM: the grid barrier costs with the number of arrivals, and
+// the register file gives 64 registers to 1024 threads either way.
+constexpr int kCoopThreads = 32 * kCoopWarps;
+static_assert(kCoopThreads / kGroup <= kMaxGroups && kCoopThreads % kGroup == 0, "groups of the block bin");
 
 // a sweep's gain sum of graph g: two words per slot (deterministic, 128 bits)
 // or one fp64 word
@@ -1326,16 +1396,18 @@ __device__ __forceinline__ double gain_sum(long long *dq, int64_t g) {
 }
 __device__ __forceinline__ double gain_sum(double *dq, int64_t g) { return __ldcg(&dq[g]); }
 
-// shared-memory tables: 8 warp tables of kWarpSlots slots, or one block table
-// of kBlockSlots slots (values first, then keys)
-template <class A> constexpr size_t table_bytes() { return (sizeof(A) + sizeof(int32_t)) * kBlockSlots; }
+// shared-memory tables of every group of kGroup threads: 8 warp tables of
+// kWarpSlots slots, or one block table of kBlockSlots slots (values first,
+// then keys)
+template <class A> __host__ __device__ constexpr size_t table_bytes() { return (sizeof(A) + sizeof(int32_t)) * kBlockSlots; }
 template <class A> __device__ __forceinline__ A *table_vals() {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    return reinterpret_cast<A *>(smem_raw);
+    return reinterpret_cast<A *>(smem_raw + (threadIdx.x / kGroup) * table_bytes<A>());
 }
 template <class A> __device__ __forceinline__ int32_t *table_keys() {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    return reinterpret_cast<int32_t *>(smem_raw + sizeof(A) * kBlockSlots);
+    return reinterpret_cast<int32_t *>(smem_raw + (threadIdx.x / kGroup) * table_bytes<A>() +
+                                       sizeof(A) * kBlockSlots);
 }
 
 // One whole phase: sweeps until the phase converges -- local-moving stops
@@ -1345,17 +1417,21 @@ template <class A> __device__ __forceinline__ int32_t *table_keys() {
 // barrier, so every block takes the same decision. In a batch every graph
 // takes the test on its own sums; the phase ends when no graph is left.
 template <class P, class W, bool REFINE, bool B>
-__global__ void __launch_bounds__(kCoopThreads, 4) k_sweep_coop(SV<P, W> a, const int32_t *__restrict__ list) {
+__global__ void __launch_bounds__(kCoopThreads, 1) k_sweep_coop(SV<P, W> a, const int32_t *__restrict__ list) {
     using A = typename P::acc;
     using T = typename P::tot;
+    const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
     int32_t *skeys = table_keys<A>();
     A *svals = table_vals<A>();
-    const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int wslot = (wib & (kGroup / 32 - 1)) * kWarpSlots;  // the warp's table in its group's
     constexpr bool batch = B;
     // testing aid: this block ends without arriving at any barrier, so the
     // others' bounded wait runs out (kErrTimeout) and the launch ends
     if ((int32_t)blockIdx.x == a.stall_block) return;
     __shared__ int64_t s_ko[2][kNumBins + 2];
+    __shared__ int32_t s_next;
+    GridBar bar{a.bar, a.err, a.spin_limit};
+    Deal deal;
     ProfCounts pc;
     int32_t it = 0;
     bool ok = true;
@@ -1377,59 +1453,81 @@ __global__ void __launch_bounds__(kCoopThreads, 4) k_sweep_coop(SV<P, W> a, cons
                 const bool e = REFINE ? ldm(&a.size[ldm(&a.C[v])]) == 1 : ldm(&a.unproc[v]) != 0;
                 if (e) mark_step(a.act, a.step[v], sm.stamp);
             }
-            if (!(ok = grid_barrier(a.bar, a.err, a.spin_limit))) break;
+            if (!(ok = bar.sync())) break;
         }
-        int64_t hub_j0 = 0;  // ordinal of the step's first hub
-        for (int32_t k = 0; k < a.nsteps && ok; ++k) {
-            // the step's nine (step, bin) offsets and its eligibility mark in
-            // one round trip, to shared memory: lanes of warp 0 load one
-            // each (the bins' work below stores to global memory, so loads
-            // issued between them would wait for one another). Two buffers:
-            // a warp reads step k's values before the barrier of step k + 1.
-            const int64_t *ko = a.key_off + (int64_t)k * kNumBins;
-            int64_t *sko = s_ko[k & 1];
-            if (wib == 0 && lane <= kNumBins + 1)
-                sko[lane] = lane <= kNumBins ? __ldcg(&ko[lane]) : (a.act ? (int64_t)__ldcg(&a.act[k]) : 0);
-            __syncthreads();
+        // A step's nine (step, bin) offsets and the ordinal of its first hub
+        // go to shared memory by lanes of warp 0, for the next step while
+        // this one runs: two buffers, the other one free since the barrier
+        // that ended the step before.
+        auto load_ko = [&](int32_t k) -> int64_t {
+            if (lane <= kNumBins) return __ldg(&a.key_off[(int64_t)k * kNumBins + lane]);
+            return (lane == kNumBins + 1 && a.hbase) ? __ldg(&a.hbase[k]) : 0;
+        };
+        if (wib == 0 && !a.act && lane <= kNumBins + 1) s_ko[0][lane] = load_ko(0);
+        __syncthreads();
+        int buf = 0;
+        for (int32_t k = 0; k < a.nsteps && ok; ++k, buf ^= 1) {
+            int64_t *sko = s_ko[buf];
+            int64_t ahead = 0;
+            if (a.act) {
+                // the next step marked as holding an eligible vertex: the
+                // same in every block, since marks are only set before the
+                // barrier that ended the last step taken
+                if (wib == 0) {
+                    int32_t n = k;
+                    for (; n < a.nsteps; n += 32) {
+                        const unsigned m =
+                            __ballot_sync(kFull, n + lane < a.nsteps && __ldcg(&a.act[n + lane]) == sm.stamp);
+                        if (m) {
+                            n += __ffs(m) - 1;
+                            break;
+                        }
+                    }
+                    if (n < a.nsteps && lane <= kNumBins + 1) sko[lane] = load_ko(n);
+                    if (lane == 0) s_next = n;
+                }
+                __syncthreads();
+                k = s_next;
+                if (k >= a.nsteps) break;
+            } else if (wib == 0 && k + 1 < a.nsteps) {
+                ahead = load_ko(k + 1);
+            }
+            auto fetched = [&]() {
+                if (wib == 0 && !a.act && k + 1 < a.nsteps && lane <= kNumBins + 1) s_ko[buf ^ 1][lane] = ahead;
+            };
             const int64_t b0 = sko[0], b8 = sko[8];
-            if (b0 == b8) continue;  // empty step: every block sees the same counts
-            if (a.act && (int32_t)sko[kNumBins + 1] != sm.stamp) {  // nothing eligible: the same in every block
-                hub_j0 += sko[7] - sko[6];
+            if (b0 == b8) {  // empty step: every block sees the same counts
+                fetched();
+                __syncthreads();
                 continue;
             }
-            run_thread<P, W, REFINE, B>(a, list, sko[1], sko[2], k, sm, pc);
-            run_tile<P, W, 16, REFINE, B>(a, list, sko[2], sko[3], k, sm, pc);
-            run_tile<P, W, 32, REFINE, B>(a, list, sko[3], sko[4], k, sm, pc);
-            run_warp<P, W, REFINE, B>(a, list, sko[4], sko[5], k, skeys + wib * kWarpSlots, svals + wib * kWarpSlots,
-                                   sm, pc);
+            run_thread<P, W, REFINE, B>(a, list, sko[1], sko[2], k, deal, sm, pc);
+            run_tile<P, W, 16, REFINE, B>(a, list, sko[2], sko[3], k, deal, sm, pc);
+            run_tile<P, W, 32, REFINE, B>(a, list, sko[3], sko[4], k, deal, sm, pc);
+            run_warp<P, W, REFINE, B>(a, list, sko[4], sko[5], k, skeys + wslot, svals + wslot, deal, sm, pc);
             const int64_t b5 = sko[5], b6 = sko[6], b7 = sko[7];
             if (b6 > b5) {
-                __syncthreads();  // the warp tables become one block table
+                group_sync();  // the group's warp tables become one block table
                 run_block<P, W, REFINE, false, B>(a, list, b5, b6, k, skeys, svals, ceil_log2(kBlockSlots), sm, pc);
             }
-            if (b7 > b6) {
-                if (a.grid_hubs) {
-                    if (!(ok = run_hubs_grid<P, W, REFINE, B>(a, hub_j0, b7 - b6, k, sm, pc))) break;
-                } else {
-                    const int64_t base = (int64_t)blockIdx.x << a.hub_bits;
-                    run_block<P, W, REFINE, true, B>(a, list, b6, b7, k, a.hub_keys + base, a.hub_vals + base,
-                                                     a.hub_bits, sm, pc);
-                }
-                hub_j0 += b7 - b6;
-            }
-            if (!(ok = grid_barrier(a.bar, a.err, a.spin_limit))) break;
+            if (b7 > b6 && !(ok = run_hubs_grid<P, W, REFINE, B>(a, sko[kNumBins + 1], b7 - b6, k, bar, sm, pc)))
+                break;
+            const bool apply = P::det || k >= a.cap_step;
+            if (!apply) fetched();
+            if (!(ok = bar.sync())) break;
             // apply phase: deterministic mode, and proposals where neighbours
             // may share a step (below the capped step the asynchronous mode
             // moves and joins at once)
-            if (P::det || k >= a.cap_step) {
+            if (apply) {
+                fetched();
                 if (REFINE) {
-                    run_refine_apply<P, W, B>(a, list, b0, b8, k, sm);
+                    run_refine_apply<P, W, B>(a, list, b0, b8, k, deal, sm);
                 } else {
-                    const bool hub_layout = a.grid_hubs && b7 > b6;  // run_hubs_grid laid out this step's hubs
-                    run_move_apply<P, W, B>(a, list, b0, b8, sm, hub_layout);
+                    const bool hub_layout = b7 > b6;  // run_hubs_grid laid out this step's hubs
+                    run_move_apply<P, W, B>(a, list, b0, b8, deal, sm, hub_layout);
                     if (hub_layout) hub_flags<P, W>(a, sm, __ldcg(&a.hinfo[0]), __ldcg(&a.hinfo[2]), true);
                 }
-                if (!(ok = grid_barrier(a.bar, a.err, a.spin_limit))) break;
+                if (!(ok = bar.sync())) break;
             }
         }
         if (!ok) break;
@@ -1456,7 +1554,7 @@ __global__ void __launch_bounds__(kCoopThreads, 4) k_sweep_coop(SV<P, W> a, cons
             const A g = warp_sum(sm.gain.v);
             if (lane == 0 && g != (A)0) atomic_add_acc(&sm.dq[0], (T)g);
         }
-        if (!(ok = grid_barrier(a.bar, a.err, a.spin_limit))) break;
+        if (!(ok = bar.sync())) break;
         bool stop;
         if (batch) {
             // every graph still running takes its own test; graphs that
@@ -1484,7 +1582,7 @@ __global__ void __launch_bounds__(kCoopThreads, 4) k_sweep_coop(SV<P, W> a, cons
             }
             running = warp_sum(running);
             if (lane == 0 && running) atomicAdd(&a.gactive[it], running);
-            if (!(ok = grid_barrier(a.bar, a.err, a.spin_limit))) break;
+            if (!(ok = bar.sync())) break;
             stop = __ldcg(&a.gactive[it]) == 0u;
         } else if (REFINE) {
             stop = __ldcg(&sm.mv[0]) == 0ULL || a.single_sweep;
@@ -1537,7 +1635,8 @@ template <class P, class W, bool REFINE>
 __global__ void __launch_bounds__(256) k_eval_thread(SV<P, W> a, const int32_t *__restrict__ list, int64_t count) {
     Sums<P> sm = scalar_sums(a);
     ProfCounts pc;
-    run_thread<P, W, REFINE, false>(a, list, 0, count, a.cur_step, sm, pc);
+    Deal deal;
+    run_thread<P, W, REFINE, false>(a, list, 0, count, a.cur_step, deal, sm, pc);
     flush_gain<P, W, REFINE>(a, sm);
     pc.flush(a.prof);
 }
@@ -1545,7 +1644,8 @@ template <class P, class W, int T, bool REFINE>
 __global__ void __launch_bounds__(256) k_eval_tile(SV<P, W> a, const int32_t *__restrict__ list, int64_t count) {
     Sums<P> sm = scalar_sums(a);
     ProfCounts pc;
-    run_tile<P, W, T, REFINE, false>(a, list, 0, count, a.cur_step, sm, pc);
+    Deal deal;
+    run_tile<P, W, T, REFINE, false>(a, list, 0, count, a.cur_step, deal, sm, pc);
     flush_gain<P, W, REFINE>(a, sm);
     pc.flush(a.prof);
 }
@@ -1557,8 +1657,9 @@ __global__ void __launch_bounds__(256) k_eval_warp(SV<P, W> a, const int32_t *__
     const int wib = threadIdx.x >> 5;
     Sums<P> sm = scalar_sums(a);
     ProfCounts pc;
-    run_warp<P, W, REFINE, false>(a, list, 0, count, a.cur_step, skeys + wib * kWarpSlots, svals + wib * kWarpSlots, sm,
-                           pc);
+    Deal deal;
+    run_warp<P, W, REFINE, false>(a, list, 0, count, a.cur_step, skeys + wib * kWarpSlots, svals + wib * kWarpSlots,
+                                  deal, sm, pc);
     flush_gain<P, W, REFINE>(a, sm);
     pc.flush(a.prof);
 }
@@ -1582,7 +1683,8 @@ __global__ void __launch_bounds__(256) k_eval_block(SV<P, W> a, const int32_t *_
 template <class P, class W>
 __global__ void __launch_bounds__(256) k_move_apply(SV<P, W> a, const int32_t *__restrict__ list, int64_t count) {
     Sums<P> sm = scalar_sums(a);
-    run_move_apply<P, W, false>(a, list, 0, count, sm, false);
+    Deal deal;
+    run_move_apply<P, W, false>(a, list, 0, count, deal, sm, false);
     if (P::det) {
         const unsigned __int128 g = warp_sum_u128(sm.dgain.v);
         if ((threadIdx.x & 31) == 0 && g) atomic_add_u128(reinterpret_cast<unsigned long long *>(a.dq_acc), g);
@@ -1593,7 +1695,8 @@ __global__ void __launch_bounds__(256) k_move_apply(SV<P, W> a, const int32_t *_
 template <class P, class W>
 __global__ void __launch_bounds__(256) k_refine_apply(SV<P, W> a, const int32_t *__restrict__ list, int64_t count) {
     Sums<P> sm = scalar_sums(a);
-    run_refine_apply<P, W, false>(a, list, 0, count, a.cur_step, sm);
+    Deal deal;
+    run_refine_apply<P, W, false>(a, list, 0, count, a.cur_step, deal, sm);
     const unsigned long long mv = warp_sum(sm.moved.v);
     if ((threadIdx.x & 31) == 0 && mv) atomicAdd(a.moved, mv);
 }
@@ -1652,9 +1755,11 @@ int apply_grid(int64_t count) {
 template <class P, class W, bool REFINE, bool B>
 cudaError_t coop_launch(const SweepCtx &c, const int32_t *list, int grid, cudaStream_t s) {
     SV<P, W> a = view<P, W>(c);
-    constexpr size_t tb = table_bytes<typename P::acc>();
-    cudaError_t e = allow_table_smem(k_sweep_coop<P, W, REFINE, B>, tb);
+    constexpr size_t all = table_bytes<typename P::acc>() * (kCoopThreads / kGroup);
+    cudaError_t e = allow_table_smem(k_sweep_coop<P, W, REFINE, B>, all);
     if (e != cudaSuccess) return e;
+    // without a row beyond the tile bins no table is used: the L1 keeps the space
+    const size_t tb = c.tables ? all : 0;
     void *args[] = {&a, (void *)&list};
     return cudaLaunchCooperativeKernel((const void *)k_sweep_coop<P, W, REFINE, B>, dim3(grid), dim3(kCoopThreads),
                                        args, tb, s);
@@ -1664,7 +1769,7 @@ cudaError_t coop_typed(const SweepCtx &c, const int32_t *list, int grid, cudaStr
     return c.gid ? coop_launch<P, W, REFINE, true>(c, list, grid, s) : coop_launch<P, W, REFINE, false>(c, list, grid, s);
 }
 template <class P, class W, bool REFINE, bool B> int coop_blocks_b() {
-    constexpr size_t tb = table_bytes<typename P::acc>();
+    constexpr size_t tb = table_bytes<typename P::acc>() * (kCoopThreads / kGroup);
     if (allow_table_smem(k_sweep_coop<P, W, REFINE, B>, tb) != cudaSuccess) return 0;
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sweep_coop<P, W, REFINE, B>, kCoopThreads, tb) !=
@@ -1673,9 +1778,13 @@ template <class P, class W, bool REFINE, bool B> int coop_blocks_b() {
     return per_sm;
 }
 template <class P, class W, bool REFINE> int coop_blocks_typed() {
-    // both forms share the launch bounds; take the smaller occupancy
-    const int a = coop_blocks_b<P, W, REFINE, false>(), b = coop_blocks_b<P, W, REFINE, true>();
-    return a < b ? a : b;
+    // both forms share the launch bounds; take the smaller occupancy (asked
+    // once: several calls of every pass need it)
+    static const int blocks = [] {
+        const int a = coop_blocks_b<P, W, REFINE, false>(), b = coop_blocks_b<P, W, REFINE, true>();
+        return a < b ? a : b;
+    }();
+    return blocks;
 }
 
 }  // namespace

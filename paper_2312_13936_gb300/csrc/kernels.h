@@ -26,6 +26,7 @@ constexpr int kBlockMaxDeg = 2048;
 constexpr int kWarpSlots = 512;     // 8 warp tables fill the same 48 KB as one block table
 constexpr int kBlockSlots = 4096;
 constexpr int kBinHub = 6;
+constexpr int kCoopWarps = 32;       // warps of a persistent sweep's block
 // the packed bin-6 tables of the aggregation are cleared and filled in
 // chunks of at most this many bytes (12 per slot; 8 in the asynchronous
 // mode, whose slot holds key and fp32 value in one word)
@@ -124,6 +125,8 @@ struct SweepCtx {
     unsigned *bar = nullptr;      // grid barrier state (2 words, zeroed before every launch)
     int *err = nullptr;
     unsigned long long *prof = nullptr;  // 8 work counters of this launch's class, or null
+    const int64_t *hbase = nullptr;      // ordinal of every step's first hub
+    bool tables = true;                  // persistent sweep: some row needs a shared-memory table
     int32_t block_max = kBlockMaxDeg;    // rows longer than this are bin 6 (the hubs)
     // testing aid for the timeout path: block stall_block (-1: none) of a
     // persistent launch ends without arriving at the barrier; the others
@@ -277,10 +280,11 @@ inline int32_t auto_layers(int64_t maxdeg, int64_t n, int64_t nnz) {
 // without edges get key nsteps*kNumBins (a trailing bucket)
 // Hubs of a pass for the whole-grid bin 6 of the persistent sweep: the
 // bin-6 lists of the steps (key_off step-major, nsteps steps) compacted in
-// list order into hubs[]; *max_span (device) = the largest sum of one
+// list order into hubs[], hbase[k] = the ordinal of step k's first hub;
+// *max_span (device) = the largest sum of one
 // step's table sizes (2^max(6, ceil log2 2 deg) slots each).
 cudaError_t launch_hub_prep(const int64_t *key_off, int32_t nsteps, const int32_t *list, const int32_t *deg,
-                            int32_t *hubs, unsigned long long *max_span, cudaStream_t s);
+                            int32_t *hubs, int64_t *hbase, unsigned long long *max_span, cudaStream_t s);
 cudaError_t launch_step_bin_keys(const int32_t *step, const int32_t *deg, int64_t n, int32_t nsteps, bool bin_major,
                                  const BinBounds &bb, int32_t *key, cudaStream_t s);
 
