@@ -368,11 +368,9 @@ __device__ __forceinline__ bool take_vertex(const SV<P, W> &a, int32_t v, int32_
         d = ldm(&a.C[v]);
         return ldm(&a.size[d]) == 1 && !(B && ldm(&a.gdone[gv]));
     }
+    d = ldm(&a.C[v]);  // in flight together with the flag
     const bool e = ldm(&a.unproc[v]) != 0 && !(B && ldm(&a.gdone[gv]));
-    if (e) {
-        a.unproc[v] = 0;
-        d = ldm(&a.C[v]);
-    }
+    if (e) a.unproc[v] = 0;
     return e;
 }
 
@@ -489,6 +487,11 @@ __device__ __forceinline__ void run_thread(const SV<P, W> &a, const int32_t *__r
 }
 
 // ----------------------------------------------------------- tile bins
+// Equal communities of a tile find one another with one match instruction and
+// sum in shared memory at their first lane's place (T rounds of two or three
+// shuffles each, for every lane to see every other, kept the SM's one shuffle
+// pipe busy: about 140 of its cycles per vertex). The vertex's header loads do
+// not wait for its eligibility.
 template <class P, class W, int T, bool REFINE, bool B>
 __device__ __forceinline__ void run_tile(const SV<P, W> &a, const int32_t *__restrict__ list, int64_t lo, int64_t hi,
                                          int32_t cur_step, Deal &deal, Sums<P> &sm, ProfCounts &pc) {
@@ -496,6 +499,8 @@ __device__ __forceinline__ void run_tile(const SV<P, W> &a, const int32_t *__res
     const int lane = threadIdx.x & 31;
     const int tl = lane & (T - 1);
     const unsigned tmask = (T == 32) ? kFull : (((1u << T) - 1u) << (lane & ~(T - 1)));
+    __shared__ A s_sum[kCoopWarps][32];
+    A *wsum = s_sum[threadIdx.x >> 5];
     constexpr int per = 32 / T;  // vertices of a unit
     const uint32_t units = (uint32_t)((hi - lo + per - 1) / per);
     for (uint32_t u = deal.first(); u < units; u += deal.nw) {
@@ -503,6 +508,8 @@ __device__ __forceinline__ void run_tile(const SV<P, W> &a, const int32_t *__res
         if (t >= hi) continue;
         const int32_t v = list[t];
         const int32_t gv = graph_of<B>(a, v);
+        const A Kv = k_of(a, v, t);
+        const RowOf<W> row = row_of(a, v, t);
         int32_t d = 0;
         int elig = 0;
         if (tl == 0) elig = take_vertex<P, W, REFINE, B>(a, v, d, gv) ? 1 : 0;
@@ -513,8 +520,6 @@ __device__ __forceinline__ void run_tile(const SV<P, W> &a, const int32_t *__res
             if (tl == 0) pc.v[1]++;
             continue;
         }
-        const A Kv = k_of(a, v, t);
-        const RowOf<W> row = row_of(a, v, t);
         const int64_t e0 = row.e0;
         const int32_t dv = row.dv;
         const int32_t bv = REFINE ? a.CB[v] : 0;
@@ -527,19 +532,16 @@ __device__ __forceinline__ void run_tile(const SV<P, W> &a, const int32_t *__res
             if (REFINE && ok) ok = (__ldg(&a.CB[j]) == bv);
             if (ok) c = ldm(&a.C[j]);
         }
-        // merge equal communities: each lane sums the lanes of its community
-        // in lane order; the first lane of each community leads
-        A sum = 0;
-        bool lead = (c >= 0);
-#pragma unroll
-        for (int k = 0; k < T; ++k) {
-            const int32_t ck = __shfl_sync(tmask, c, k, T);
-            const A wk = __shfl_sync(tmask, wv, k, T);
-            if (c >= 0 && ck == c) {
-                sum += wk;
-                if (k < tl) lead = false;
-            }
-        }
+        // merge equal communities into their first lane's sum
+        const unsigned peers = __match_any_sync(tmask, c);
+        const int first = __ffs(peers) - 1;
+        const bool lead = c >= 0 && first == lane;
+        wsum[lane] = wv;
+        __syncwarp(tmask);
+        if (c >= 0 && !lead) atomic_add_acc(&wsum[first], wv);
+        __syncwarp(tmask);
+        const A sum = wsum[lane];
+        __syncwarp(tmask);
         const unsigned dball = __ballot_sync(tmask, lead && c == d) & tmask;
         const int dsrc = dball ? ((__ffs(dball) - 1) & (T - 1)) : 0;
         const A kvd_b = __shfl_sync(tmask, sum, dsrc, T);
@@ -582,6 +584,74 @@ __device__ __forceinline__ void run_tile(const SV<P, W> &a, const int32_t *__res
     deal.pass(units);
 }
 
+// Entries of a row into a table by the threads first, first + stride, ...:
+// four entries of a thread in flight, each load of the chain (target, its
+// bound, its community) for all four before the next.
+template <class P, class W, bool REFINE>
+__device__ __forceinline__ void table_insert(const SV<P, W> &a, const RowOf<W> &row, int32_t v, int32_t bv, int first,
+                                             int stride, int32_t *keys, typename P::acc *vals, int bits) {
+    using A = typename P::acc;
+    for (int32_t x = first; x < row.dv; x += 4 * stride) {
+        int32_t j[4], c[4];
+        A w[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int32_t e = x + q * stride;
+            j[q] = -1;
+            w[q] = 0;
+            if (e < row.dv) {
+                j[q] = row.idx[row.e0 + e];
+                w[q] = wconv<A>(row.w[row.e0 + e]);
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            bool ok = j[q] >= 0 && j[q] != v;
+            if (REFINE && ok) ok = __ldg(&a.CB[j[q]]) == bv;
+            c[q] = ok ? ldm(&a.C[j[q]]) : -1;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (c[q] >= 0 && !hash_add(keys, vals, bits, c[q], w[q])) set_error(a.err, kErrHashFull);
+    }
+}
+// The best candidate of a filled table over the slots first, first + stride,
+// ...: four slots of a thread at a time, so that their community totals are
+// in flight together; the sum of v's own community goes to kvd.
+template <class P, class W, bool REFINE>
+__device__ __forceinline__ void table_best(const SV<P, W> &a, const Sums<P> &sm, int32_t v, int32_t d,
+                                           typename P::acc Kv, typename P::acc ks, int first, int stride, int S,
+                                           const int32_t *keys, const typename P::acc *vals, typename P::key &key,
+                                           int32_t &cand, typename P::acc &kvd, ProfCounts &pc) {
+    for (int s0 = first; s0 < S; s0 += 4 * stride) {
+        int32_t k[4];
+        typename P::tot sc[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int s = s0 + q * stride;
+            k[q] = s < S ? keys[s] : -1;
+            sc[q] = 0;
+            if (k[q] >= 0 && k[q] != d) sc[q] = ldm(&a.Sig[k[q]]);
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            if (k[q] < 0) continue;
+            pc.v[3]++;
+            const typename P::acc sum = vals[s0 + q * stride];
+            if (k[q] == d) {
+                kvd = sum;
+                continue;
+            }
+            const typename P::key kk =
+                cand_key<P, W, REFINE>(a, sm, v, k[q], move_key(ks, sum, Kv, sc[q], a.gamma));
+            if (better(kk, k[q], key, cand)) {
+                key = kk;
+                cand = k[q];
+            }
+        }
+    }
+}
+
 // ------------------------------------------------------- warp-table bin
 template <class P, class W, bool REFINE, bool B>
 __device__ __forceinline__ void run_warp(const SV<P, W> &a, const int32_t *__restrict__ list, int64_t lo, int64_t hi,
@@ -592,6 +662,9 @@ __device__ __forceinline__ void run_warp(const SV<P, W> &a, const int32_t *__res
     for (int64_t t = lo + deal.first(); t < hi; t += deal.nw) {
         const int32_t v = list[t];
         const int32_t gv = graph_of<B>(a, v);
+        const A Kv = k_of(a, v, t);
+        const RowOf<W> row = row_of(a, v, t);
+        const int32_t dv = row.dv;
         int32_t d = 0;
         int elig = 0;
         if (lane == 0) elig = take_vertex<P, W, REFINE, B>(a, v, d, gv) ? 1 : 0;
@@ -602,10 +675,6 @@ __device__ __forceinline__ void run_warp(const SV<P, W> &a, const int32_t *__res
             if (lane == 0) pc.v[1]++;
             continue;
         }
-        const A Kv = k_of(a, v, t);
-        const RowOf<W> row = row_of(a, v, t);
-        const int64_t e0 = row.e0;
-        const int32_t dv = row.dv;
         const int32_t bv = REFINE ? a.CB[v] : 0;
         int bits = ceil_log2(2 * (int64_t)dv);
         if (bits < 6) bits = 6;
@@ -615,33 +684,13 @@ __device__ __forceinline__ void run_warp(const SV<P, W> &a, const int32_t *__res
             vals[s] = 0;
         }
         __syncwarp();
-        for (int32_t e = lane; e < dv; e += 32) {
-            const int32_t j = row.idx[e0 + e];
-            if (j == v) continue;
-            if (REFINE && __ldg(&a.CB[j]) != bv) continue;
-            if (!hash_add(keys, vals, bits, ldm(&a.C[j]), wconv<A>(row.w[e0 + e]))) set_error(a.err, kErrHashFull);
-        }
+        table_insert<P, W, REFINE>(a, row, v, bv, lane, 32, keys, vals, bits);
         __syncwarp();
         typename P::key key = AccLimits<typename P::key>::lowest();
         A kvd = 0;
         int32_t cand = INT_MAX;
         const A ks = kscale_of<B>(a, gv);
-        for (int s = lane; s < S; s += 32) {
-            const int32_t k = keys[s];
-            if (k < 0) continue;
-            pc.v[3]++;
-            const A sum = vals[s];
-            if (k == d) {
-                kvd = sum;
-                continue;
-            }
-            const typename P::key kk =
-                cand_key<P, W, REFINE>(a, sm, v, k, move_key(ks, sum, Kv, ldm(&a.Sig[k]), a.gamma));
-            if (better(kk, k, key, cand)) {
-                key = kk;
-                cand = k;
-            }
-        }
+        table_best<P, W, REFINE>(a, sm, v, d, Kv, ks, lane, 32, S, keys, vals, key, cand, kvd, pc);
         for (int o = 16; o > 0; o >>= 1) {
             const typename P::key ok = kshfl_xor(kFull, key, o);
             const int32_t oc = __shfl_xor_sync(kFull, cand, o);
@@ -664,7 +713,7 @@ __device__ __forceinline__ void run_warp(const SV<P, W> &a, const int32_t *__res
         if (!REFINE && !P::det) {
             mv = __shfl_sync(kFull, mv, 0);
             if (mv)
-                for (int32_t e = lane; e < dv; e += 32) flag_unproc(a, sm, row.idx[e0 + e]);
+                for (int32_t e = lane; e < dv; e += 32) flag_unproc(a, sm, row.idx[row.e0 + e]);
         }
         __syncwarp();
     }
@@ -733,33 +782,13 @@ __device__ __forceinline__ void run_block(const SV<P, W> &a, const int32_t *__re
             vals[s] = 0;
         }
         group_sync();
-        for (int64_t e = tid; e < dv; e += kGroup) {
-            const int32_t j = row.idx[e0 + e];
-            if (j == v) continue;
-            if (REFINE && __ldg(&a.CB[j]) != bv) continue;
-            if (!hash_add(keys, vals, bits, ldm(&a.C[j]), wconv<A>(row.w[e0 + e]))) set_error(a.err, kErrHashFull);
-        }
+        table_insert<P, W, REFINE>(a, row, v, bv, tid, kGroup, keys, vals, bits);
         group_sync();
         typename P::key key = AccLimits<typename P::key>::lowest();
         A kvd = 0;
         int32_t cand = INT_MAX;
         const A ks = kscale_of<B>(a, gv);
-        for (int64_t s = tid; s < S; s += kGroup) {
-            const int32_t k = keys[s];
-            if (k < 0) continue;
-            pc.v[3]++;
-            const A sum = vals[s];
-            if (k == d) {
-                kvd = sum;
-                continue;
-            }
-            const typename P::key kk =
-                cand_key<P, W, REFINE>(a, sm, v, k, move_key(ks, sum, Kv, ldm(&a.Sig[k]), a.gamma));
-            if (better(kk, k, key, cand)) {
-                key = kk;
-                cand = k;
-            }
-        }
+        table_best<P, W, REFINE>(a, sm, v, d, Kv, ks, tid, kGroup, (int)S, keys, vals, key, cand, kvd, pc);
         for (int o = 16; o > 0; o >>= 1) {
             const typename P::key ok = kshfl_xor(kFull, key, o);
             const int32_t oc = __shfl_xor_sync(kFull, cand, o);
