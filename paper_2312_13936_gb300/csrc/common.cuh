@@ -8,28 +8,44 @@ namespace lgb {
 constexpr int kWarp = 32;
 constexpr unsigned kFull = 0xffffffffu;
 
-// Arithmetic policies. acc is the type of per-edge sums (K_{i->c}) and
-// vertex weights K_i; key the type of move keys and their gains; tot the
+// Arithmetic policies. acc is the type of vertex weights K_i; sum that of
+// per-edge sums K_{i->c}; key the type of move keys and their gains; tot the
 // type of community totals Sigma_c and of the asynchronous sweep's
 // delta-modularity sums. The deterministic mode decides moves in exact
 // integer arithmetic on integer weights: sums, K and Sigma in int64, keys
 // (products of two such sums) in 128 bits, and a sweep's gain sum in 128
-// bits (two 64-bit words, lo then hi). The asynchronous mode keeps Sigma
-// and 2m in fp64 and everything per edge in fp32: on this GPU the fp64 pipe
-// is a small fraction of the fp32 rate, and the move key
+// bits (two 64-bit words, lo then hi). Det64 is the same arithmetic for
+// graphs of 2m < 2^31, where it is exact in narrower words: every sum of
+// entries is at most 2m and fits in 32 bits, every product is below 2^62 and
+// every key and gain fits in 64; the decisions are the same bit for bit. (A
+// 128-bit key took twice the registers of a 64-bit one and spilled at 64
+// registers a thread, and shared memory has no 64-bit add: every insertion
+// was a compare-and-swap loop.) The asynchronous mode keeps Sigma and 2m in
+// fp64 and everything per edge in fp32: on this GPU the fp64 pipe is a small
+// fraction of the fp32 rate, and the move key
 // K_{i->c} - gamma K_i Sigma_c / 2m has terms of the order of K_i, so fp32
-// keeps its relative precision.
+// keeps its relative precision. packed: a global table's slot is one 8-byte
+// word of a key and a 32-bit sum.
 struct Det {
     using acc = long long;
+    using sum = long long;
     using tot = long long;
     using key = __int128;
-    static constexpr bool det = true;
+    static constexpr bool det = true, packed = false;
+};
+struct Det64 {
+    using acc = long long;
+    using sum = int32_t;
+    using tot = long long;
+    using key = long long;
+    static constexpr bool det = true, packed = true;
 };
 struct Async {
     using acc = float;
+    using sum = float;
     using tot = double;
     using key = float;
-    static constexpr bool det = false;
+    static constexpr bool det = false, packed = true;
 };
 
 template <class A> struct AccLimits;
@@ -50,20 +66,14 @@ template <> struct AccLimits<__int128> {
 __device__ __forceinline__ float kshfl_xor(unsigned mask, float x, int o, int w = 32) {
     return __shfl_xor_sync(mask, x, o, w);
 }
+__device__ __forceinline__ long long kshfl_xor(unsigned mask, long long x, int o, int w = 32) {
+    return __shfl_xor_sync(mask, x, o, w);
+}
 __device__ __forceinline__ __int128 kshfl_xor(unsigned mask, __int128 x, int o, int w = 32) {
     const unsigned long long lo = __shfl_xor_sync(mask, (unsigned long long)x, o, w);
     const long long hi = __shfl_xor_sync(mask, (long long)(x >> 64), o, w);
     return (__int128)(((unsigned __int128)(unsigned long long)hi << 64) | lo);
 }
-__device__ __forceinline__ float kshfl(unsigned mask, float x, int src, int w = 32) {
-    return __shfl_sync(mask, x, src, w);
-}
-__device__ __forceinline__ __int128 kshfl(unsigned mask, __int128 x, int src, int w = 32) {
-    const unsigned long long lo = __shfl_sync(mask, (unsigned long long)x, src, w);
-    const long long hi = __shfl_sync(mask, (long long)(x >> 64), src, w);
-    return (__int128)(((unsigned __int128)(unsigned long long)hi << 64) | lo);
-}
-
 // A 128-bit unsigned sum held as two words (lo, hi) in global memory:
 // atomically add x, carrying into hi when lo wraps. Every addition that
 // wraps lo adds exactly one carry, so the pair is the exact sum mod 2^128
@@ -87,6 +97,7 @@ __device__ __forceinline__ void atomic_add_acc(long long *p, long long v) {
 __device__ __forceinline__ void atomic_add_acc(double *p, double v) { atomicAdd(p, v); }
 __device__ __forceinline__ void atomic_add_acc(float *p, float v) { atomicAdd(p, v); }
 __device__ __forceinline__ void atomic_add_acc(unsigned long long *p, unsigned long long v) { atomicAdd(p, v); }
+__device__ __forceinline__ void atomic_add_acc(int32_t *p, int32_t v) { atomicAdd(p, v); }
 
 // Running per-graph sum of one thread (sweep gains, move counts). In a batch
 // of graphs the sum of the previous graph goes to its slot base[g] when the
@@ -139,7 +150,7 @@ __device__ __forceinline__ unsigned __int128 warp_sum_u128(unsigned __int128 v) 
 template <class A> __device__ __forceinline__ A load_cg(const A *p) { return __ldcg(p); }
 
 // Move keys (Eq. 2). Deterministic mode, Eq. 2 times 2m^2 (kscale = 2m), in
-// 128 bits (each product is below (2m)^2):
+// 128 bits (each product is below (2m)^2; Det64: 64 bits):
 //   key(c) = 2m K_{i->c} - K_i Sigma_c,  stay = 2m K_{i->d} - K_i (Sigma_d - K_i).
 // Asynchronous mode, Eq. 2 times m (kscale = 1/2m):
 //   key(c) = K_{i->c} - gamma K_i Sigma_c / 2m,  stay = K_{i->d} - gamma K_i (Sigma_d - K_i) / 2m.
@@ -148,11 +159,17 @@ template <class A> __device__ __forceinline__ A load_cg(const A *p) { return __l
 __device__ __forceinline__ __int128 move_key(long long two_m, long long kic, long long ki, long long sc, double) {
     return (__int128)two_m * kic - (__int128)ki * sc;
 }
+__device__ __forceinline__ long long move_key(long long two_m, int32_t kic, long long ki, long long sc, double) {
+    return two_m * kic - ki * sc;  // Det64
+}
 __device__ __forceinline__ float move_key(float inv2m, float kic, float ki, double sc, double gamma) {
     return kic - (float)gamma * ki * ((float)sc * inv2m);
 }
 __device__ __forceinline__ __int128 stay_key(long long two_m, long long kid, long long ki, long long sd, double) {
     return (__int128)two_m * kid - (__int128)ki * (sd - ki);
+}
+__device__ __forceinline__ long long stay_key(long long two_m, int32_t kid, long long ki, long long sd, double) {
+    return two_m * kid - ki * (sd - ki);  // Det64
 }
 __device__ __forceinline__ float stay_key(float inv2m, float kid, float ki, double sd, double gamma) {
     return kid - (float)gamma * ki * (((float)sd - ki) * inv2m);
@@ -198,23 +215,27 @@ __device__ __forceinline__ bool hash_add(int32_t *keys, A *vals, int bits, int32
 }
 
 // Open-addressing table whose slot is one 8-byte word: the key in the low
-// half (-1: empty), an fp32 value in the high half, so that an insertion
-// touches one memory sector (the asynchronous mode's global tables). A new
-// key goes in with its value by one 64-bit compare-and-swap against the
-// empty word; a failed swap returns the slot's word, and if its key is ours
-// the value is added to the high half. A slot's key never changes once set,
-// so the key half of a returned word is exact even while other threads add
-// to its value half.
-constexpr unsigned long long kEmptyKV = 0x00000000ffffffffULL;  // key -1, value 0.0f
-__device__ __forceinline__ bool hash_add_kv(unsigned long long *kv, int bits, int32_t k, float v) {
+// half (-1: empty), a 32-bit sum (fp32, or an integer of Det64) in the high
+// half, so that an insertion touches one memory sector. A new key goes in
+// with its value by one 64-bit compare-and-swap against the empty word; a
+// failed swap returns the slot's word, and if its key is ours the value is
+// added to the high half. A slot's key never changes once set, so the key
+// half of a returned word is exact even while other threads add to its value
+// half.
+constexpr unsigned long long kEmptyKV = 0x00000000ffffffffULL;  // key -1, value 0 (0.0f)
+__device__ __forceinline__ unsigned kv_bits(float v) { return __float_as_uint(v); }
+__device__ __forceinline__ unsigned kv_bits(int32_t v) { return (unsigned)v; }
+__device__ __forceinline__ void kv_value(unsigned long long w, float &v) { v = __uint_as_float((uint32_t)(w >> 32)); }
+__device__ __forceinline__ void kv_value(unsigned long long w, int32_t &v) { v = (int32_t)(uint32_t)(w >> 32); }
+template <class V> __device__ __forceinline__ bool hash_add_kv(unsigned long long *kv, int bits, int32_t k, V v) {
     const uint32_t mask = (1u << bits) - 1u;
-    const unsigned long long mine = ((unsigned long long)__float_as_uint(v) << 32) | (uint32_t)k;
+    const unsigned long long mine = ((unsigned long long)kv_bits(v) << 32) | (uint32_t)k;
     uint32_t s = hslot(k, bits);
     for (uint32_t probe = 0; probe <= mask; ++probe) {
         const unsigned long long cur = atomicCAS(&kv[s], kEmptyKV, mine);
         if (cur == kEmptyKV) return true;
         if ((int32_t)(uint32_t)cur == k) {
-            atomicAdd(reinterpret_cast<float *>(&kv[s]) + 1, v);
+            atomicAdd(reinterpret_cast<V *>(&kv[s]) + 1, v);
             return true;
         }
         s = (s + 1u) & mask;
@@ -286,6 +307,10 @@ __device__ __forceinline__ void warp_add_by_key(double *arr, int64_t key, double
         todo &= ~same;
     }
 }
+
+// Sum over a full warp, in one instruction for 32-bit integers.
+template <class T> __device__ __forceinline__ T full_sum(T v) { return warp_sum(v); }
+__device__ __forceinline__ int32_t full_sum(int32_t v) { return __reduce_add_sync(kFull, v); }
 
 // Sum of v over the lanes of peers (every lane of peers calls it, with the
 // same peers).
@@ -382,8 +407,8 @@ __device__ __forceinline__ bool grid_barrier(unsigned *bar, int *err, unsigned l
 // published word lies on the way. Measured alone (4,000 barriers): 152
 // blocks of 1024 threads 1.20 us, against 1.93 us for grid_barrier above and
 // 2.09 us for it with 608 blocks of 256, the same threads; with 608 blocks
-// polling, the counter itself takes 2.15 us, so this barrier goes with one
-// block per SM. The error word is read only while waiting, and a barrier
+// polling, the counter itself takes 2.15 us, so this barrier goes with few
+// blocks per SM. The error word is read only while waiting, and a barrier
 // that runs out of polls ends the launch: its block arrives nowhere again
 // and the others see the error word or run out too.
 struct GridBar {
@@ -432,7 +457,10 @@ struct Deal {
         : nw(gridDim.x * (blockDim.x >> 5)), gw((threadIdx.x >> 5) * gridDim.x + blockIdx.x) {}
     // this warp's first unit of the coming bin; its others follow nw apart
     __device__ __forceinline__ uint32_t first() const { return gw >= next ? gw - next : gw + nw - next; }
-    __device__ __forceinline__ void pass(uint32_t units) { next = (next + units) % nw; }
+    __device__ __forceinline__ void pass(uint32_t units) {
+        next += units;
+        if (next >= nw) next %= nw;
+    }
 };
 
 }  // namespace lgb

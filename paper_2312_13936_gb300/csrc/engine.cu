@@ -34,7 +34,7 @@ const char *last_error() { return g_last_error.c_str(); }
 // The persistent sweeps' grid barrier counts arrivals in 32 bits, from zero
 // at every launch. One phase takes at most max_iterations sweeps of at most
 // 8 barriers per schedule step (layout, insertion, three key passes, hub
-// flags, step end, apply) and 4 more per sweep, on at most one block per SM;
+// flags, step end, apply) and 4 more per sweep, on at most two blocks per SM;
 // the count is taken for four, as the documented limit is. A limit under
 // which that count could pass 2^32 - 1 is refused rather than let it wrap.
 leiden_status check_barrier_budget(int32_t max_iterations, int32_t nsteps, int sm) {
@@ -229,19 +229,24 @@ leiden_status Handle::Impl::pass(Run &r, int32_t lp, bool &stop) {
     CK(launch_community_totals(sC, sK, det, n, q.Sig, q.size, s));
     q.launches += 1;
     const bool step_launches = (prm.flags & LEIDEN_FLAG_STEP_LAUNCHES) != 0;
-    // bin 6: in the persistent sweep the whole grid takes each step's hubs
+    // bin 7: in the persistent sweep the whole grid takes each step's hubs
     // (tables of one step at a time); per-step launches keep a global table
     // per block
     const std::vector<int64_t> &ko = q.hkey_off;
     int64_t nhubs = 0, ntab = 0, units = 0;  // hubs, vertices with a shared-memory table, the sweep's warp units
     for (int32_t k = 0; k < nsteps; ++k) {
         const int64_t *o = &ko[(size_t)k * kNumBins];
-        nhubs += o[7] - o[6];
-        ntab += o[6] - o[4];
-        units += (o[2] - o[1] + 31) / 32 + (o[3] - o[2] + 1) / 2 + (o[5] - o[3]) + 8 * (o[6] - o[5]);
+        nhubs += o[kBinGrid + 1] - o[kBinGrid];
+        ntab += o[kBinGrid] - o[4];
+        units += (o[2] - o[1] + 31) / 32 + (o[3] - o[2] + 1) / 2 + (o[5] - o[3]) + 8 * (o[6] - o[5]) +
+                 kCoopWarps * (o[7] - o[6]);
     }
-    const bool grid_hubs = nhubs > 0 && !step_launches && sweep_coop_blocks_per_sm(det, sG.w_int, false) > 0 &&
-                           sweep_coop_blocks_per_sm(det, sG.w_int, true) > 0;
+    // exact in 64-bit keys and 32-bit sums (two_m_i is the sum over all graphs
+    // of a batch, so each one's is below it)
+    const bool narrow = det && two_m_i < ((long long)1 << 31);
+    const bool coop = !step_launches && sweep_coop_blocks_per_sm(det, narrow, sG.w_int, false) > 0 &&
+                      sweep_coop_blocks_per_sm(det, narrow, sG.w_int, true) > 0;
+    const bool grid_hubs = nhubs > 0 && coop;
     if (grid_hubs) {
         ST(q.ensure_hubs(nhubs));
         CK(launch_hub_prep(q.key_off, nsteps, sList, sG.deg, q.hubs, q.hbase, q.hspan, s));
@@ -254,10 +259,10 @@ leiden_status Handle::Impl::pass(Run &r, int32_t lp, bool &stop) {
             return LEIDEN_ERR_OOM;
         }
         ST(q.ensure_hub(0, (int)span, det));
-        // clean tables; every step's last scan leaves them clean again. The
-        // asynchronous mode keeps key and fp32 value in one 8-byte word per
-        // slot (key -1 and value 0 when empty), in the value buffer.
-        if (det) {
+        // clean tables; every step's last scan leaves them clean again. Packed
+        // tables keep key and 32-bit sum in one 8-byte word per slot (key -1
+        // and value 0 when empty), in the value buffer.
+        if (det && !narrow) {
             CK(cudaMemsetAsync(q.hub_keys, 0xff, sizeof(int32_t) * span, s));
             CK(cudaMemsetAsync(q.hub_vals, 0, 8 * span, s));
         } else {
@@ -266,9 +271,10 @@ leiden_status Handle::Impl::pass(Run &r, int32_t lp, bool &stop) {
             q.launches += 1;
         }
     }
-    // global tables for bin 6 (one per block)
+    // per-step launches: global tables for the rows beyond the block bin (one
+    // per block)
     int hub_bits = 0, hub_regions = 0;
-    if (!grid_hubs) {
+    if (!coop) {
         const int maxdeg = q.hsc->maxdeg;
         if (maxdeg > q.tune.block_max_deg) {
             hub_bits = ceil_log2_h(2 * (int64_t)maxdeg);
@@ -305,6 +311,7 @@ leiden_status Handle::Impl::pass(Run &r, int32_t lp, bool &stop) {
         sc.lK = q.lo_K;
     }
     sc.det = det;
+    sc.narrow = narrow;
     sc.C = sC;
     sc.CB = sCB;
     sc.K = sK;
@@ -336,6 +343,7 @@ leiden_status Handle::Impl::pass(Run &r, int32_t lp, bool &stop) {
     sc.hcand = q.hcand;
     sc.hmv = q.hmv;
     sc.hkey = q.hkey;
+    sc.hslot = q.hslot;
     sc.hkvd = q.hkvd;
     sc.nsteps = nsteps;
     sc.key_off = q.key_off;
@@ -359,9 +367,10 @@ leiden_status Handle::Impl::pass(Run &r, int32_t lp, bool &stop) {
             for (int b = 1; b < kNumBins; ++b) {
                 const int64_t lo = ko[k * kNumBins + b], hi = ko[k * kNumBins + b + 1];
                 if (hi == lo) continue;
-                const int mb = b <= 4 ? tile_blocks : (b == 5 ? big_blocks : hub_regions);
-                sc.prof = prof_begin((refine ? 8 : 0) + b);
-                CK(launch_sweep_eval(sc, b, sList + lo, hi - lo, mb, s));
+                const int kb = b == kBinGrid ? kBinHub : b;  // one launch shape for both here
+                const int mb = kb <= 4 ? tile_blocks : (kb == 5 ? big_blocks : hub_regions);
+                sc.prof = prof_begin((refine ? 8 : 0) + kb);
+                CK(launch_sweep_eval(sc, kb, sList + lo, hi - lo, mb, s));
                 prof_end();
                 q.launches++;
             }
@@ -385,7 +394,7 @@ leiden_status Handle::Impl::pass(Run &r, int32_t lp, bool &stop) {
         sc.rand_refine = refine && (prm.flags & LEIDEN_FLAG_RANDOM_REFINE) != 0;
         sc.rseed = prm.seed + 0xD1B54A32D192ED03ULL * (uint64_t)(64 * (r.gpass ? 0 : lp));
         const bool single = refine && (prm.flags & LEIDEN_FLAG_REFINE_SINGLE_SWEEP);
-        int per_sm = step_launches ? 0 : sweep_coop_blocks_per_sm(det, sG.w_int, refine);
+        int per_sm = coop ? sweep_coop_blocks_per_sm(det, narrow, sG.w_int, refine) : 0;
         if (per_sm > 0 && q.tune.coop_blocks_per_sm > 0 && q.tune.coop_blocks_per_sm < per_sm)
             per_sm = q.tune.coop_blocks_per_sm;  // the handle's launch shape
         CK(launch_phase_init(q.gstate, NG, q.gdone, giters, s));
@@ -396,14 +405,15 @@ leiden_status Handle::Impl::pass(Run &r, int32_t lp, bool &stop) {
         }
         if (per_sm > 0) {
             // enough blocks for a step's work: one block (which synchronises
-            // with __syncthreads only) while its 32 warps take an average
+            // with __syncthreads only) while its warps take an average
             // step's units at once, else a block for every four units, and
             // at least one for every vertices_per_block vertices. A barrier
             // of 152 blocks takes 1.2 us, of 16 blocks 1.1 us, a warp's
             // second unit 3 us and more, so there is little to save between
             // one block and the full grid.
-            int grid = per_sm * q.sm;
             const int64_t vpb = q.tune.vertices_per_block, ups = units / nsteps;
+            if (ups < 4 * (int64_t)kCoopWarps * q.sm) per_sm = 1;  // (kCoopThreads)
+            int grid = per_sm * q.sm;
             int64_t want = ups <= kCoopWarps && !grid_hubs ? 1 : std::max((ups + 3) / 4, (n + vpb - 1) / vpb);
             if (grid_hubs) want = grid;
             if ((prm.flags & LEIDEN_FLAG_TEST_STALL_BARRIER) && want < 2) want = 2;  // a block to stall

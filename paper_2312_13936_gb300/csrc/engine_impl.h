@@ -480,7 +480,7 @@ struct Handle::Impl {
     // whole-grid bin 6 of the persistent sweep: per-hub arrays of a pass
     int32_t *hubs = nullptr, *hd = nullptr, *hcand = nullptr, *hmv = nullptr, *hj = nullptr;
     int64_t *htoff = nullptr, *heoff = nullptr, *hinfo = nullptr, *hbase = nullptr;
-    unsigned long long *hkey = nullptr, *hspan = nullptr;
+    unsigned long long *hkey = nullptr, *hspan = nullptr, *hslot = nullptr;
     long long *hkvd = nullptr;
     int64_t hubs_cap = -1;
     // the rows and vertex weights of a pass's graph in list order
@@ -524,6 +524,7 @@ struct Handle::Impl {
             ST(alloc(&hinfo, 4));  // a step's eligible hubs, table slots, entries
             ST(alloc(&hspan, 1));
             ST(alloc(&hbase, 1024));
+            ST(alloc(&hslot, 8 * (int64_t)sm));  // a persistent sweep has at most two blocks per SM
         }
         if (nh <= hubs_cap) return LEIDEN_OK;
         for (void *p : {(void *)hubs, (void *)hd, (void *)hcand, (void *)hmv, (void *)hj, (void *)htoff,

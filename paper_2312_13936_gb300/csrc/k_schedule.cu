@@ -290,7 +290,7 @@ template <bool LONG> int sched_blocks_per_sm() {
 __global__ void k_step_bin_keys(const int32_t *step, const int32_t *deg, int64_t n, int32_t nsteps, bool bin_major,
                                 BinBounds bb, int32_t *key) {
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
-        const int b = degree_bin(deg[v], bb);
+        const int b = sweep_bin(deg[v], bb);
         // vertices without edges go to a trailing bucket (never swept)
         key[v] = b == 0 ? nsteps * kNumBins : (bin_major ? b * nsteps + step[v] : step[v] * kNumBins + b);
     }
@@ -305,7 +305,7 @@ __global__ void k_hub_gather(const int64_t *key_off, int32_t nsteps, const int32
     const int k = blockIdx.x;
     long long part = 0;  // hubs of the steps before k
     for (int q = threadIdx.x; q < k; q += blockDim.x)
-        part += key_off[(int64_t)q * kNumBins + 7] - key_off[(int64_t)q * kNumBins + 6];
+        part += key_off[(int64_t)q * kNumBins + kBinGrid + 1] - key_off[(int64_t)q * kNumBins + kBinGrid];
     part = warp_sum(part);
     if ((threadIdx.x & 31) == 0) s_part[threadIdx.x >> 5] = part;
     __syncthreads();
@@ -313,7 +313,7 @@ __global__ void k_hub_gather(const int64_t *key_off, int32_t nsteps, const int32
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) base += s_part[w];
     __syncthreads();
     if (threadIdx.x == 0) hbase[k] = base;
-    const int64_t lo = key_off[(int64_t)k * kNumBins + 6], hi = key_off[(int64_t)k * kNumBins + 7];
+    const int64_t lo = key_off[(int64_t)k * kNumBins + kBinGrid], hi = key_off[(int64_t)k * kNumBins + kBinGrid + 1];
     long long span = 0;
     for (int64_t t = lo + threadIdx.x; t < hi; t += blockDim.x) {
         const int32_t v = list[t];

@@ -26,7 +26,15 @@ constexpr int kBlockMaxDeg = 2048;
 constexpr int kWarpSlots = 512;     // 8 warp tables fill the same 48 KB as one block table
 constexpr int kBlockSlots = 4096;
 constexpr int kBinHub = 6;
-constexpr int kCoopWarps = 32;       // warps of a persistent sweep's block
+constexpr int kCoopWarps = 16;       // warps of a persistent sweep's block
+constexpr int kGroup = 256;          // threads of a block-bin group
+// The persistent sweep's own split of the rows beyond the block bin: up to
+// kCtaMaxDeg entries a block's shared memory holds the table (bin 6), and the
+// row needs no grid barrier; longer rows take the whole grid and a global
+// table (bin 7), two barriers and the same chain of loads.
+constexpr int kCtaSlots = 8192;
+constexpr int32_t kCtaMaxDeg = kCtaSlots / 2;
+constexpr int kBinGrid = 7;
 // the packed bin-6 tables of the aggregation are cleared and filled in
 // chunks of at most this many bytes (12 per slot; 8 in the asynchronous
 // mode, whose slot holds key and fp32 value in one word)
@@ -43,6 +51,11 @@ struct BinBounds {
 };
 __host__ __device__ inline int degree_bin(int64_t d, const BinBounds &b) {
     return d <= 0 ? 0 : d <= b.thread_max ? 1 : d <= 16 ? 2 : d <= 32 ? 3 : d <= b.warp_max ? 4 : d <= b.block_max ? 5 : 6;
+}
+// bin of a row in the persistent sweep: degree_bin's, bin 6 split
+__host__ __device__ inline int sweep_bin(int64_t d, const BinBounds &b) {
+    const int k = degree_bin(d, b);
+    return k == kBinHub && d > kCtaMaxDeg ? kBinGrid : k;
 }
 
 // Weights of aggregated graphs in the deterministic mode: exact integers
@@ -107,7 +120,7 @@ struct SweepCtx {
     int32_t *hub_keys = nullptr;  // global tables for bin 6 (one region per block)
     void *hub_vals = nullptr;
     int hub_bits = 0, hub_regions = 0;
-    // persistent sweep: bin 6 evaluated by the whole grid (launch_hub_prep
+    // persistent sweep: bin 7 evaluated by the whole grid (launch_hub_prep
     // fills hubs; hub_keys/hub_vals then hold one step's tables); per hub:
     // hd, hcand, hmv, hkey, hkvd (8 bytes); per eligible hub of a step: hj,
     // htoff, heoff (+1); hinfo: 3 words
@@ -125,7 +138,9 @@ struct SweepCtx {
     unsigned *bar = nullptr;      // grid barrier state (2 words, zeroed before every launch)
     int *err = nullptr;
     unsigned long long *prof = nullptr;  // 8 work counters of this launch's class, or null
+    bool narrow = false;                 // deterministic, 2m < 2^31: Det64 (its hub tables are packed words)
     const int64_t *hbase = nullptr;      // ordinal of every step's first hub
+    unsigned long long *hslot = nullptr; // 4 words per block: its best candidate of a single hub
     bool tables = true;                  // persistent sweep: some row needs a shared-memory table
     int32_t block_max = kBlockMaxDeg;    // rows longer than this are bin 6 (the hubs)
     // testing aid for the timeout path: block stall_block (-1: none) of a
@@ -161,7 +176,7 @@ cudaError_t launch_refine_apply(const SweepCtx &c, const int32_t *list, int64_t 
 // one whole phase (sweeps of every step, grid barriers between steps, the
 // convergence test on the device) in one cooperative launch
 cudaError_t launch_sweep_coop(const SweepCtx &c, const int32_t *list, int grid, cudaStream_t s);
-int sweep_coop_blocks_per_sm(bool det, bool w_int, bool refine);
+int sweep_coop_blocks_per_sm(bool det, bool narrow, bool w_int, bool refine);
 
 // Aggregation (Algorithm 4) of G' by dense labels Cd into the holey CSR G''.
 struct AggCtx {

@@ -1,7 +1,7 @@
 """GPU tests of the persistent sweep's work division: graphs at the edges of
 its rules (one block or many, units of 2, 8 or 32 vertices in the apply phase,
-rows at the flat walk's bound, the bins' bounds) against the oracle's SYNC
-mode, bit for bit."""
+rows at the flat walk's bound, the bins' bounds, the weight sum up to which
+keys are 64 bits wide) against the oracle's SYNC mode, bit for bit."""
 import numpy as np
 import pytest
 
@@ -41,7 +41,31 @@ def test_sizes_around_one_block(n):
     _equal(gen.sbm(n, max(1, n // 100), 0.1 if n < 2000 else 200.0 / n, 1.0 / n, seed=n))
 
 
-@pytest.mark.parametrize("d", [8, 9, 16, 17, 32, 33, 256, 257, 1023, 1024, 1025, 2048, 2049, 5000])
+@pytest.mark.parametrize("d", [8, 9, 16, 17, 32, 33, 256, 257, 1023, 1024, 1025, 2048, 2049, 4096, 4097, 9000])
 @pytest.mark.parametrize("hubs", [1, 5])
 def test_row_lengths(d, hubs):
     _equal(_star(d, hubs))
+
+
+@pytest.mark.parametrize("over", [-2, 0, 2])
+def test_weight_sums_around_the_narrow_arithmetic(over):
+    """2m two below, at and two above 2^31 (each weight exact in fp32)."""
+    g = gen.sbm(600, 6, 0.1, 0.01, seed=5)
+    row = np.repeat(np.arange(g.n), np.diff(g.offsets))
+    w = np.full(g.nnz, float((1 << 31) // g.nnz & ~63), np.float32)
+    gap = (1 << 31) + over - int(w.astype(np.int64).sum())  # even, spread over pairs of entries
+    for v in range(g.n):
+        if gap == 0:
+            break
+        for e in range(g.offsets[v], g.offsets[v + 1]):
+            u = g.indices[e]
+            if u <= v or gap == 0:
+                continue
+            add = min(gap // 2, 1 << 20)
+            back = g.offsets[u] + int(np.searchsorted(g.indices[g.offsets[u]:g.offsets[u + 1]], v))
+            assert g.indices[back] == v and row[back] == u
+            w[e] += add
+            w[back] += add
+            gap -= 2 * add
+    assert gap == 0 and int(w.astype(np.int64).sum()) == (1 << 31) + over
+    _equal(gen.CSR(g.n, g.offsets, g.indices, w))
