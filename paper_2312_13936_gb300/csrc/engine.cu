@@ -259,6 +259,7 @@ leiden_status Handle::Impl::pass(Run &r, int32_t lp, bool &stop) {
             return LEIDEN_ERR_OOM;
         }
         ST(q.ensure_hub(0, (int)span, det));
+        CK(cudaMemsetAsync(q.sigtot, 0, sizeof(double) * n, s));  // a single hub's sums
         // clean tables; every step's last scan leaves them clean again. Packed
         // tables keep key and 32-bit sum in one 8-byte word per slot (key -1
         // and value 0 when empty), in the value buffer.
@@ -344,6 +345,7 @@ leiden_status Handle::Impl::pass(Run &r, int32_t lp, bool &stop) {
     sc.hmv = q.hmv;
     sc.hkey = q.hkey;
     sc.hslot = q.hslot;
+    sc.hacc = q.sigtot;  // free until the result is scored
     sc.hkvd = q.hkvd;
     sc.nsteps = nsteps;
     sc.key_off = q.key_off;

@@ -80,6 +80,7 @@ template <class P, class W> struct SV {
     int64_t *htoff, *heoff, *hinfo;
     int32_t *hd, *hcand, *hmv;
     unsigned long long *hkey;
+    S *hacc;                    // sums of a step's single hub by community (zero between steps)
     unsigned long long *hslot;  // every block's best candidate of a step's single hub (4 words each)
     S *hkvd;
     bool grid_hubs;
@@ -192,6 +193,7 @@ template <class P, class W> SV<P, W> view(const SweepCtx &c) {
     a.hmv = c.hmv;
     a.hkey = c.hkey;
     a.hslot = c.hslot;
+    a.hacc = static_cast<typename P::sum *>(c.hacc);
     a.hkvd = static_cast<typename P::sum *>(c.hkvd);
     a.grid_hubs = c.grid_hubs;
     a.bar = c.bar;
@@ -1248,19 +1250,24 @@ __device__ __forceinline__ bool run_hubs_grid(const SV<P, W> &a, int64_t j0, int
 
 // A layered step (below cap_step: no two of its vertices are adjacent) with
 // one such hub, as most steps of a heavy-tailed schedule have: two grid
-// barriers here and the step's own end. Every block reads the hub's
-// eligibility itself -- no vertex of the step can change it (a flag is set,
-// or a community joined, only by a neighbour), and the barriers of the
-// previous step made its last writes visible. Chunks of 32 entries, then of
-// 128 slots, go round the warps after the step's smaller units. Each block
-// reduces its slots' best candidate and leaves it in its own word; after the
-// second barrier every block reduces those words and knows the decision (the
-// hub's own total is read between the barriers, where nothing writes it), so
-// the neighbours' flags need no barrier of their own. Block 0 commits: in the
-// deterministic mode too, since every evaluation of the step is over by then,
-// and the other proposals' apply phase follows without a barrier between
-// (the layout, three key passes and an apply phase of their own took seven
-// barriers a step, four in the asynchronous mode).
+// barriers here and the step's own end. One thread of every block reads the
+// hub's eligibility -- no vertex of the step can change it (a flag is set, or
+// a community joined, only by a neighbour), and the barriers of the previous
+// step made its last writes visible. Chunks of 32 entries go round the warps
+// after the step's smaller units. The sums K_{v->c} are added, without asking
+// for a result, into a vector addressed by community (hacc, zero between
+// steps); after the first barrier the same chunks read the sum and the
+// community's total of their entries, so the row is its own list of
+// candidates: no table is probed (a chain of up to a dozen L2 atomics at half
+// load) and no empty slots are scanned, and C of a hub's neighbours does not
+// change within the step. Each block reduces its best candidate and leaves it
+// in its own word; after the second barrier every block reduces those words
+// and knows the decision (the hub's own sum and total are read between the
+// barriers, where nothing writes them), so the neighbours' flags need no
+// barrier of their own, and the chunks clear the sums. Block 0 commits: in
+// the deterministic mode too, since every evaluation of the step is over by
+// then, and the other proposals' apply phase follows without a barrier
+// between.
 // Returns 0 when a barrier ran out, 1 when the hub is not eligible (no
 // barrier passed), 2 when it was evaluated.
 template <class P, class W, bool REFINE, bool B>
@@ -1284,93 +1291,61 @@ __device__ __forceinline__ int run_hub_single(const SV<P, W> &a, int64_t j0, int
         if (B && x) x = !ldm(&a.gdone[gv]);
         s_e = x ? 1 : 0;
     }
+    const int64_t e0 = a.off[v];
+    const int32_t dv = a.deg[v];
+    const int32_t bv = REFINE ? __ldg(&a.CB[v]) : 0;
     __syncthreads();
     const int32_t d = s_d;
-    const bool e = s_e != 0;
-    if (!e) {  // the same in every block
+    if (!s_e) {  // the same in every block
         if (first_thread) {
             if (proposing<P, REFINE>(cur_step, a.cap_step)) a.prop[v] = -1;
             pc.v[1]++;
         }
         return 1;
     }
-    if (first_thread) a.hkvd[j0] = 0;
-    const int64_t e0 = a.off[v];
-    const int32_t dv = a.deg[v];
-    const int bits = ceil_log2(2 * (int64_t)dv);
-    const int32_t bv = REFINE ? __ldg(&a.CB[v]) : 0;
-    const uint32_t chunks = ((uint32_t)dv + 31) / 32;
-    for (uint32_t i = deal.first(); i < chunks; i += deal.nw) {
+    // the entry of chunk i in this lane: its vertex (-1: none) and community
+    // (-1: not a candidate)
+    auto entry = [&](uint32_t i, int32_t &u, int32_t &c) {
         const int64_t x = (int64_t)i * 32 + lane;
-        int32_t key = -1;
-        S val = 0;
-        if (x < dv) {
-            const int32_t u = a.idx[e0 + x];
-            if (u != v && (!REFINE || __ldg(&a.CB[u]) == bv)) {
-                key = ldm(&a.C[u]);
-                val = wconv<S>(a.w[e0 + x]);
-            }
+        u = x < dv ? a.idx[e0 + x] : -1;
+        c = u >= 0 && u != v && (!REFINE || __ldg(&a.CB[u]) == bv) ? ldm(&a.C[u]) : -1;
+    };
+    const uint32_t chunks = ((uint32_t)dv + 31) / 32, i0 = deal.first();
+    int32_t u0 = -1, c0 = -1;  // the warp's first chunk stays in registers
+    for (uint32_t i = i0; i < chunks; i += deal.nw) {
+        int32_t u, c;
+        entry(i, u, c);
+        if (i == i0) {
+            u0 = u;
+            c0 = c;
         }
-        const unsigned peers = __match_any_sync(kFull, key);
+        S val = c >= 0 ? wconv<S>(a.w[e0 + (int64_t)i * 32 + lane]) : (S)0;
+        const unsigned peers = __match_any_sync(kFull, c);
         val = peer_sum(peers, val);
-        if (key >= 0 && lane == __ffs(peers) - 1) {
-            bool ok;
-            if constexpr (!P::packed) ok = hash_add(a.hub_keys, a.hub_vals, bits, key, val);
-            else ok = hash_add_kv(hub_kv<P>(a), bits, key, val);
-            if (!ok) set_error(a.err, kErrHashFull);
+        if (c >= 0 && lane == __ffs(peers) - 1) {
+            atomic_add_acc(&a.hacc[c], val);
+            pc.v[3]++;
         }
     }
     deal.pass(chunks);
     if (!bar.sync()) return 0;
     if (!REFINE && first_thread) a.unproc[v] = 0;  // every block has read the flag
     const T sd = ldm(&a.Sig[d]);
+    const S kd = __ldcg(&a.hacc[d]);
     const A kv = a.K[v], ks = kscale_of<B>(a, gv);
     K key = AccLimits<K>::lowest();
     int32_t cand = INT_MAX;
-    constexpr int Q = 4;
-    const uint32_t schunks = (uint32_t)((1u << bits) / (32 * Q));
-    for (uint32_t i = deal.first(); i < schunks; i += deal.nw) {
-        const int64_t s0 = (int64_t)i * (32 * Q) + lane;
-        int32_t kq[Q];
-        S vq[Q];
-        T sq[Q];
-        if constexpr (!P::packed) {
-#pragma unroll
-            for (int q = 0; q < Q; ++q) kq[q] = __ldcg(&a.hub_keys[s0 + 32 * q]);
-#pragma unroll
-            for (int q = 0; q < Q; ++q) vq[q] = kq[q] >= 0 ? __ldcg(&a.hub_vals[s0 + 32 * q]) : (S)0;
-        } else {
-#pragma unroll
-            for (int q = 0; q < Q; ++q) {
-                const unsigned long long w = __ldcg(&hub_kv<P>(a)[s0 + 32 * q]);
-                kq[q] = (int32_t)(uint32_t)w;
-                kv_value(w, vq[q]);
-            }
-        }
-#pragma unroll
-        for (int q = 0; q < Q; ++q) sq[q] = kq[q] >= 0 && kq[q] != d ? ldm(&a.Sig[kq[q]]) : (T)0;
-#pragma unroll
-        for (int q = 0; q < Q; ++q) {
-            if (kq[q] < 0) continue;
-            if constexpr (!P::packed) {  // the table is left clean
-                a.hub_keys[s0 + 32 * q] = -1;
-                a.hub_vals[s0 + 32 * q] = 0;
-            } else {
-                hub_kv<P>(a)[s0 + 32 * q] = kEmptyKV;
-            }
-            pc.v[3]++;
-            if (kq[q] == d) {
-                a.hkvd[j0] = vq[q];
-                continue;
-            }
-            const K kk = cand_key<P, W, REFINE>(a, sm, v, kq[q], move_key(ks, vq[q], kv, sq[q], a.gamma));
-            if (better(kk, kq[q], key, cand)) {
-                key = kk;
-                cand = kq[q];
-            }
+    for (uint32_t i = i0; i < chunks; i += deal.nw) {
+        int32_t u = u0, c = c0;
+        if (i != i0) entry(i, u, c);
+        if (c < 0 || c == d) continue;
+        const S sum = __ldcg(&a.hacc[c]);
+        const K kk = cand_key<P, W, REFINE>(a, sm, v, c, move_key(ks, sum, kv, ldm(&a.Sig[c]), a.gamma));
+        if (better(kk, c, key, cand)) {
+            key = kk;
+            cand = c;
         }
     }
-    deal.pass(schunks);
     warp_best(key, cand);
     if (lane == 0) {
         key_order(key, s_hi[wib], s_lo[wib]);
@@ -1407,7 +1382,6 @@ __device__ __forceinline__ int run_hub_single(const SV<P, W> &a, int64_t j0, int
         }
         warp_best(key, cand);
         if (lane == 0) {
-            const S kd = __ldcg(&a.hkvd[j0]);
             bool mv = cand != INT_MAX && key > stay_key(ks, kd, kv, sd, a.gamma);
             s_moves = mv ? 1 : 0;
             if (blockIdx.x == 0) {
@@ -1440,14 +1414,13 @@ __device__ __forceinline__ int run_hub_single(const SV<P, W> &a, int64_t j0, int
             }
         }
     }
-    if (!REFINE) {
-        __syncthreads();
-        if (s_moves)
-            for (uint32_t i = deal.first(); i < chunks; i += deal.nw) {
-                const int64_t x = (int64_t)i * 32 + lane;
-                if (x < dv) flag_unproc(a, sm, a.idx[e0 + x]);
-            }
-        deal.pass(chunks);
+    if (!REFINE) __syncthreads();
+    const bool flag = !REFINE && s_moves;
+    for (uint32_t i = i0; i < chunks; i += deal.nw) {
+        int32_t u = u0, c = c0;
+        if (i != i0) entry(i, u, c);
+        if (c >= 0) a.hacc[c] = 0;
+        if (flag && u >= 0) flag_unproc(a, sm, u);
     }
     return 2;
 }

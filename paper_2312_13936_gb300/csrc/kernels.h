@@ -140,6 +140,7 @@ struct SweepCtx {
     unsigned long long *prof = nullptr;  // 8 work counters of this launch's class, or null
     bool narrow = false;                 // deterministic, 2m < 2^31: Det64 (its hub tables are packed words)
     const int64_t *hbase = nullptr;      // ordinal of every step's first hub
+    void *hacc = nullptr;                // n words of 8 bytes, zero: sums of a single hub by community
     unsigned long long *hslot = nullptr; // 4 words per block: its best candidate of a single hub
     bool tables = true;                  // persistent sweep: some row needs a shared-memory table
     int32_t block_max = kBlockMaxDeg;    // rows longer than this are bin 6 (the hubs)
