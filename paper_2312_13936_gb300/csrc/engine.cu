@@ -317,6 +317,10 @@ leiden_status Handle::Impl::pass(Run &r, int32_t lp, bool &stop) {
     sc.CB = sCB;
     sc.K = sK;
     sc.Sig = q.Sig;
+    if (det && coop) {  // free during the sweeps
+        sc.Sig2 = q.Kagg;
+        sc.old = q.bnd;
+    }
     sc.size = q.size;
     sc.unproc = q.unproc;
     sc.prop = q.prop;
@@ -431,6 +435,7 @@ leiden_status Handle::Impl::pass(Run &r, int32_t lp, bool &stop) {
             CK(cudaMemsetAsync(q.phase_moved, 0, sizeof(unsigned long long) * prm.max_iterations * NG, s));
             CK(cudaMemsetAsync(q.gactive, 0, sizeof(unsigned) * prm.max_iterations, s));
             CK(cudaMemsetAsync(q.bar, 0, 2 * sizeof(unsigned), s));  // barrier state starts clean
+            if (det) CK(cudaMemcpyAsync(q.Kagg, q.Sig, accsz * n, cudaMemcpyDeviceToDevice, s));
             sc.prof = prof_begin(refine ? 8 : 0);
             // steps without an eligible vertex are skipped where there are
             // many steps (heavy-tailed schedules): in the refinement, and in

@@ -49,6 +49,8 @@ template <class P, class W> struct SV {
     const int32_t *CB;
     const A *K;
     T *Sig;
+    T *Sig2;       // the second copy (persistent deterministic sweep)
+    int32_t *old;  // the community a vertex moved from in its step (null: no moves at once in the deterministic mode)
     int32_t *size;
     uint8_t *unproc;
     int32_t *prop;
@@ -140,6 +142,9 @@ template <class P> struct Sums {
     typename P::tot *dq;
     unsigned long long *mv;
     int32_t stamp = 0;  // this sweep's mark in act (persistent sweep)
+    // Sigma as the step reads it and as its moves leave it: two copies in the
+    // persistent deterministic sweep (see catch_up), else the same array
+    typename P::tot *sr, *sw;
 };
 
 template <class P, class W> SV<P, W> view(const SweepCtx &c) {
@@ -154,6 +159,8 @@ template <class P, class W> SV<P, W> view(const SweepCtx &c) {
     a.CB = c.CB;
     a.K = static_cast<const A *>(c.K);
     a.Sig = static_cast<T *>(c.Sig);
+    a.Sig2 = P::det ? static_cast<T *>(c.Sig2) : a.Sig;
+    a.old = P::det ? c.old : nullptr;
     a.size = c.size;
     a.unproc = c.unproc;
     a.prop = c.prop;
@@ -265,9 +272,9 @@ template <class K> __device__ __forceinline__ unsigned __int128 load_gain128(con
 }
 
 // Decision for vertex v (one thread, graph gv, key scale kscale) with best
-// candidate (key, cand), K_{v->d} = kvd and Sigma_d = sd. Returns true if
-// an asynchronous local-moving move was applied (its neighbours must then be
-// marked unprocessed).
+// candidate (key, cand), K_{v->d} = kvd and Sigma_d = sd. Returns true if a
+// local-moving move was made at once (its neighbours must then be marked
+// unprocessed).
 template <class P, class W, bool REFINE, bool B>
 __device__ __forceinline__ bool decide_sd(const SV<P, W> &a, int32_t v, int32_t d, typename P::acc Kv,
                                           typename P::key key, int32_t cand, typename P::sum kvd,
@@ -289,9 +296,24 @@ __device__ __forceinline__ bool decide_sd(const SV<P, W> &a, int32_t v, int32_t 
         g = key - ks;
     }
     if constexpr (P::det) {
-        // the deterministic mode always proposes (an apply phase commits)
         a.prop[v] = mv ? cand : -1;
-        if (!REFINE && mv) store_gain(a.gain, v, g);
+        if (a.old && cur_step < a.cap_step) {
+            // Below the capped step of a persistent sweep the move is made at
+            // once: no vertex of the step reads C, the size or the flags it
+            // changes (they concern v's neighbours and v), and Sigma's change
+            // goes to the copy the step does not read.
+            if (!mv) return false;
+            a.old[v] = d;
+            atomic_add_acc(&sm.sw[d], -(T)Kv);
+            atomic_add_acc(&sm.sw[cand], (T)Kv);
+            atomicSub(&a.size[d], 1);
+            atomicAdd(&a.size[cand], 1);
+            a.C[v] = cand;
+            if (REFINE) gacc_add(sm.moved, B, gv, 1ULL, sm.mv);
+            else gacc_add(sm.dgain, B, gv, (unsigned __int128)g, reinterpret_cast<unsigned long long *>(sm.dq));
+            return !REFINE;
+        }
+        if (!REFINE && mv) store_gain(a.gain, v, g);  // proposed: an apply phase commits
         return false;
     } else {
         if (REFINE && cur_step < a.cap_step) {
@@ -300,8 +322,8 @@ __device__ __forceinline__ bool decide_sd(const SV<P, W> &a, int32_t v, int32_t 
             // cand stays in cand and nobody joins v while it leaves: the join
             // is applied at once (the gain sum counts joins in this phase).
             if (mv) {
-                atomic_add_acc(&a.Sig[d], -(T)Kv);
-                atomic_add_acc(&a.Sig[cand], (T)Kv);
+                atomic_add_acc(&sm.sw[d], -(T)Kv);
+                atomic_add_acc(&sm.sw[cand], (T)Kv);
                 atomicSub(&a.size[d], 1);
                 atomicAdd(&a.size[cand], 1);
                 a.C[v] = cand;
@@ -315,8 +337,8 @@ __device__ __forceinline__ bool decide_sd(const SV<P, W> &a, int32_t v, int32_t 
             return false;
         }
         if (mv) {
-            atomic_add_acc(&a.Sig[d], -(T)Kv);
-            atomic_add_acc(&a.Sig[cand], (T)Kv);
+            atomic_add_acc(&sm.sw[d], -(T)Kv);
+            atomic_add_acc(&sm.sw[cand], (T)Kv);
             atomicSub(&a.size[d], 1);
             atomicAdd(&a.size[cand], 1);
             a.C[v] = cand;
@@ -329,7 +351,7 @@ template <class P, class W, bool REFINE, bool B>
 __device__ __forceinline__ bool decide(const SV<P, W> &a, int32_t v, int32_t d, typename P::acc Kv,
                                        typename P::key key, int32_t cand, typename P::sum kvd, Sums<P> &sm,
                                        int32_t cur_step, int32_t gv, typename P::acc kscale) {
-    return decide_sd<P, W, REFINE, B>(a, v, d, Kv, key, cand, kvd, ldm(&a.Sig[d]), sm, cur_step, gv, kscale);
+    return decide_sd<P, W, REFINE, B>(a, v, d, Kv, key, cand, kvd, ldm(&sm.sr[d]), sm, cur_step, gv, kscale);
 }
 
 // Key of candidate community c for vertex v. The randomized refinement
@@ -393,7 +415,7 @@ __device__ __forceinline__ void eval_thread(const SV<P, W> &a, int32_t v, int32_
     using S = typename P::sum;
     const int64_t e0 = row.e0;
     const int32_t dv = row.dv;
-    const typename P::tot sd = ldm(&a.Sig[d]);
+    const typename P::tot sd = ldm(&sm.sr[d]);
     const int32_t bv = REFINE ? a.CB[v] : 0;
     int32_t jj[E];
     S wt[E];
@@ -437,7 +459,7 @@ __device__ __forceinline__ void eval_thread(const SV<P, W> &a, int32_t v, int32_
             continue;
         }
         const typename P::key kk =
-            cand_key<P, W, REFINE>(a, sm, v, c[k], move_key(ks, wt[k], Kv, ldm(&a.Sig[c[k]]), a.gamma));
+            cand_key<P, W, REFINE>(a, sm, v, c[k], move_key(ks, wt[k], Kv, ldm(&sm.sr[c[k]]), a.gamma));
         if (better(kk, c[k], key, cand)) {
             key = kk;
             cand = c[k];
@@ -453,7 +475,7 @@ __device__ __forceinline__ void eval_thread(const SV<P, W> &a, int32_t v, int32_
             pc.v[5] += dv;
         }
     }
-    if (!REFINE && !P::det && mv) {
+    if (!REFINE && mv) {
 #pragma unroll
         for (int k = 0; k < E; ++k)
             if (k < dv) flag_unproc(a, sm, jj[k]);  // neighbours (self-loop included) of a mover
@@ -564,7 +586,7 @@ __device__ __forceinline__ void run_tile(const SV<P, W> &a, const int32_t *__res
         int32_t cand = INT_MAX;
         const A ks = kscale_of<B>(a, gv);
         if (lead && c != d) {
-            key = cand_key<P, W, REFINE>(a, sm, v, c, move_key(ks, sum, Kv, ldm(&a.Sig[c]), a.gamma));
+            key = cand_key<P, W, REFINE>(a, sm, v, c, move_key(ks, sum, Kv, ldm(&sm.sr[c]), a.gamma));
             cand = c;
         }
 #pragma unroll
@@ -590,7 +612,7 @@ __device__ __forceinline__ void run_tile(const SV<P, W> &a, const int32_t *__res
                 }
             }
         }
-        if (!REFINE && !P::det) {
+        if (!REFINE) {
             mv = __shfl_sync(tmask, mv, 0, T);
             if (mv && tl < dv) flag_unproc(a, sm, j);  // neighbours (self-loop included) of a mover
         }
@@ -669,7 +691,7 @@ __device__ __forceinline__ void table_best(const SV<P, W> &a, const Sums<P> &sm,
             const int s = s0 + q * stride;
             k[q] = s < S ? keys[s] : -1;
             sc[q] = 0;
-            if (k[q] >= 0) sc[q] = ldm(&a.Sig[k[q]]);
+            if (k[q] >= 0) sc[q] = ldm(&sm.sr[k[q]]);
         }
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -748,7 +770,7 @@ __device__ __forceinline__ void run_warp(const SV<P, W> &a, const int32_t *__res
                 pc.v[5] += dv;
             }
         }
-        if (!REFINE && !P::det) {
+        if (!REFINE) {
             mv = __shfl_sync(kFull, mv, 0);
             if (mv)
                 for (int32_t e = lane; e < dv; e += 32) flag_unproc(a, sm, row.idx[row.e0 + e]);
@@ -850,7 +872,7 @@ __device__ __forceinline__ void run_block(const SV<P, W> &a, const int32_t *__re
                 }
             }
         }
-        if (!REFINE && !P::det) {
+        if (!REFINE) {
             group_sync<GS>();
             if (s_mv)
                 for (int64_t e = tid; e < dv; e += GS) flag_unproc(a, sm, row.idx[row.e0 + e]);
@@ -1155,7 +1177,7 @@ __device__ __forceinline__ bool run_hubs_grid(const SV<P, W> &a, int64_t j0, int
 #pragma unroll
             for (int q = 0; q < Q; ++q) {
                 sq[q] = 0;
-                if (kq[q] >= 0 && kq[q] != d) sq[q] = ldm(&a.Sig[kq[q]]);
+                if (kq[q] >= 0 && kq[q] != d) sq[q] = ldm(&sm.sr[kq[q]]);
             }
             unsigned long long lmax = 0ULL;
             int32_t lmin = INT_MAX;
@@ -1238,10 +1260,10 @@ __device__ __forceinline__ bool run_hubs_grid(const SV<P, W> &a, int64_t j0, int
             pc.v[4]++;
             pc.v[5] += dv;
         }
-        if (!REFINE && !P::det && mv) a.hmv[j] = 1;
+        if (!REFINE && mv) a.hmv[j] = 1;
     }
-    if (!REFINE && !P::det) {
-        // an asynchronous local-moving move flags the hub's neighbours
+    if (!REFINE && cur_step < a.cap_step) {
+        // a local-moving move made at once flags the hub's neighbours
         if (!bar.sync()) return false;
         hub_flags<P, W>(a, sm, np, E, false);
     }
@@ -1264,14 +1286,11 @@ __device__ __forceinline__ bool run_hubs_grid(const SV<P, W> &a, int64_t j0, int
 // in its own word; after the second barrier every block reduces those words
 // and knows the decision (the hub's own sum and total are read between the
 // barriers, where nothing writes them), so the neighbours' flags need no
-// barrier of their own, and the chunks clear the sums. Block 0 commits: in
-// the deterministic mode too, since every evaluation of the step is over by
-// then, and the other proposals' apply phase follows without a barrier
-// between.
-// Returns 0 when a barrier ran out, 1 when the hub is not eligible (no
-// barrier passed), 2 when it was evaluated.
+// barrier of their own, and the chunks clear the sums. Block 0 makes the
+// move.
+// False when a barrier ran out.
 template <class P, class W, bool REFINE, bool B>
-__device__ __forceinline__ int run_hub_single(const SV<P, W> &a, int64_t j0, int32_t cur_step, GridBar &bar,
+__device__ __forceinline__ bool run_hub_single(const SV<P, W> &a, int64_t j0, int32_t cur_step, GridBar &bar,
                                               Deal &deal, Sums<P> &sm, ProfCounts &pc) {
     using A = typename P::acc;
     using S = typename P::sum;
@@ -1301,7 +1320,7 @@ __device__ __forceinline__ int run_hub_single(const SV<P, W> &a, int64_t j0, int
             if (proposing<P, REFINE>(cur_step, a.cap_step)) a.prop[v] = -1;
             pc.v[1]++;
         }
-        return 1;
+        return true;
     }
     // the entry of chunk i in this lane: its vertex (-1: none) and community
     // (-1: not a candidate)
@@ -1328,9 +1347,9 @@ __device__ __forceinline__ int run_hub_single(const SV<P, W> &a, int64_t j0, int
         }
     }
     deal.pass(chunks);
-    if (!bar.sync()) return 0;
+    if (!bar.sync()) return false;
     if (!REFINE && first_thread) a.unproc[v] = 0;  // every block has read the flag
-    const T sd = ldm(&a.Sig[d]);
+    const T sd = ldm(&sm.sr[d]);
     const S kd = __ldcg(&a.hacc[d]);
     const A kv = a.K[v], ks = kscale_of<B>(a, gv);
     K key = AccLimits<K>::lowest();
@@ -1340,7 +1359,7 @@ __device__ __forceinline__ int run_hub_single(const SV<P, W> &a, int64_t j0, int
         if (i != i0) entry(i, u, c);
         if (c < 0 || c == d) continue;
         const S sum = __ldcg(&a.hacc[c]);
-        const K kk = cand_key<P, W, REFINE>(a, sm, v, c, move_key(ks, sum, kv, ldm(&a.Sig[c]), a.gamma));
+        const K kk = cand_key<P, W, REFINE>(a, sm, v, c, move_key(ks, sum, kv, ldm(&sm.sr[c]), a.gamma));
         if (better(kk, c, key, cand)) {
             key = kk;
             cand = c;
@@ -1366,7 +1385,7 @@ __device__ __forceinline__ int run_hub_single(const SV<P, W> &a, int64_t j0, int
             slot[2] = (unsigned long long)(uint32_t)cand;
         }
     }
-    if (!bar.sync()) return 0;
+    if (!bar.sync()) return false;
     if (wib == 0) {
         key = AccLimits<K>::lowest();
         cand = INT_MAX;
@@ -1382,31 +1401,12 @@ __device__ __forceinline__ int run_hub_single(const SV<P, W> &a, int64_t j0, int
         }
         warp_best(key, cand);
         if (lane == 0) {
-            bool mv = cand != INT_MAX && key > stay_key(ks, kd, kv, sd, a.gamma);
+            const bool mv = cand != INT_MAX && key > stay_key(ks, kd, kv, sd, a.gamma);
             s_moves = mv ? 1 : 0;
             if (blockIdx.x == 0) {
                 decide_sd<P, W, REFINE, B>(a, v, d, kv, key, cand, kd, sd, sm, cur_step, gv, ks);
                 pc.v[0]++;
                 pc.v[2] += dv;
-                if constexpr (P::det) {  // commit (S5 on a refinement proposal, as in run_refine_apply)
-                    if (REFINE && mv) {
-                        const int32_t pt = __ldg(&a.step[cand]) == cur_step ? ldm(&a.prop[cand]) : -1;
-                        mv = pt < 0 || (pt == v && v > cand);
-                    }
-                    if (mv) {
-                        atomic_add_acc(&a.Sig[d], -(T)kv);
-                        atomic_add_acc(&a.Sig[cand], (T)kv);
-                        atomicSub(&a.size[d], 1);
-                        atomicAdd(&a.size[cand], 1);
-                        a.C[v] = cand;
-                        if (REFINE)
-                            gacc_add(sm.moved, B, gv, 1ULL, sm.mv);
-                        else
-                            gacc_add(sm.dgain, B, gv,
-                                     (unsigned __int128)(key - stay_key(ks, kd, kv, sd, a.gamma)),
-                                     reinterpret_cast<unsigned long long *>(sm.dq));
-                    }
-                }
                 if (mv) {
                     pc.v[4]++;
                     pc.v[5] += dv;
@@ -1422,7 +1422,7 @@ __device__ __forceinline__ int run_hub_single(const SV<P, W> &a, int64_t j0, int
         if (c >= 0) a.hacc[c] = 0;
         if (flag && u >= 0) flag_unproc(a, sm, u);
     }
-    return 2;
+    return true;
 }
 
 // ------------------------------------------------------------ apply steps
@@ -1433,8 +1433,36 @@ __device__ __forceinline__ int apply_unit(uint32_t count, uint32_t nw) {
     return count > 16 * nw ? 32 : count > 4 * nw ? 8 : 2;
 }
 
-// Local-moving proposals of one step (deterministic mode; asynchronous mode
-// in the capped steps): commit them. The movers' rows of a unit are flagged
+// The persistent deterministic sweep keeps two copies of Sigma, so that a
+// layered step needs one grid barrier: the step reads one copy (sr) while its
+// moves change the other (sw), and the copies change places at its end. What
+// a step's moves wrote is missing from the copy it read; the next step, which
+// does not read that copy, adds it there (the vertices of [lo, hi) that moved
+// in their step: prop, from old). The sums are integers, so the order in
+// which the two steps' changes arrive does not matter. (With proposals that
+// an apply phase committed, every layered step took two barriers and walked
+// its movers' rows a second time for their flags.)
+template <class P, class W>
+__device__ __forceinline__ void catch_up(const SV<P, W> &a, const int32_t *__restrict__ list, int64_t lo, int64_t hi,
+                                         Deal &deal, const Sums<P> &sm) {
+    const int lane = threadIdx.x & 31;
+    const int per = apply_unit((uint32_t)(hi - lo), deal.nw);
+    const uint32_t units = (uint32_t)((hi - lo + per - 1) / per);
+    for (uint32_t u = deal.first(); u < units; u += deal.nw) {
+        const int64_t t = lo + (int64_t)u * per + lane;
+        if (lane >= per || t >= hi) continue;
+        const int32_t v = list[t];
+        const int32_t c = ldm(&a.prop[v]), d = ldm(&a.old[v]);
+        if (c < 0) continue;
+        const auto Kv = (typename P::tot)k_of(a, v, t);
+        atomic_add_acc(&sm.sw[d], -Kv);
+        atomic_add_acc(&sm.sw[c], Kv);
+    }
+    deal.pass(units);
+}
+
+// Local-moving proposals of one capped step (of any step in the per-step
+// launches of the deterministic mode): commit them. The movers' rows of a unit are flagged
 // as one flat range of entries by all lanes, four loads per lane in flight
 // (a lane walking its own mover's row waited for every load in turn: 16 us a
 // step on a 200,000-vertex block model with rows of 24 entries). Rows of
@@ -1461,8 +1489,12 @@ __device__ __forceinline__ void run_move_apply(const SV<P, W> &a, const int32_t 
         if (c >= 0) {
             const int32_t d = ldm(&a.C[v]);
             const auto Kv = (typename P::tot)k_of(a, v, t);
-            atomic_add_acc(&a.Sig[d], -Kv);
-            atomic_add_acc(&a.Sig[c], Kv);
+            atomic_add_acc(&sm.sr[d], -Kv);
+            atomic_add_acc(&sm.sr[c], Kv);
+            if (P::det && sm.sw != sm.sr) {
+                atomic_add_acc(&sm.sw[d], -Kv);
+                atomic_add_acc(&sm.sw[c], Kv);
+            }
             atomicSub(&a.size[d], 1);
             atomicAdd(&a.size[c], 1);
             a.C[v] = c;
@@ -1532,8 +1564,12 @@ __device__ __forceinline__ void run_refine_apply(const SV<P, W> &a, const int32_
         const int32_t pt = (__ldg(&a.step[tg]) == cur_step) ? ldm(&a.prop[tg]) : -1;
         if (!(pt < 0 || (pt == v && v > tg))) continue;
         const auto Kv = (typename P::tot)k_of(a, v, t);
-        atomic_add_acc(&a.Sig[v], -Kv);
-        atomic_add_acc(&a.Sig[tg], Kv);
+        atomic_add_acc(&sm.sr[v], -Kv);
+        atomic_add_acc(&sm.sr[tg], Kv);
+        if (P::det && sm.sw != sm.sr) {
+            atomic_add_acc(&sm.sw[v], -Kv);
+            atomic_add_acc(&sm.sw[tg], Kv);
+        }
         atomicSub(&a.size[v], 1);
         atomicAdd(&a.size[tg], 1);
         a.C[v] = tg;
@@ -1615,6 +1651,9 @@ __global__ void __launch_bounds__(kCoopThreads, 2) k_sweep_coop(SV<P, W> a, cons
         sm.dq = a.dq_arr + (size_t)it * a.G * (P::det ? 2 : 1);  // deterministic: two words per slot
         sm.mv = a.moved_arr + (size_t)it * a.G;
         sm.stamp = it + 1;
+        sm.sr = a.Sig;
+        sm.sw = a.Sig2;
+        int64_t late0 = 0, late1 = 0;  // the step whose moves sw lacks (catch_up)
         if (a.act) {
             // steps holding an eligible vertex at the start of the sweep
             // (unprocessed, or isolated in the refinement); moves mark the
@@ -1702,35 +1741,40 @@ __global__ void __launch_bounds__(kCoopThreads, 2) k_sweep_coop(SV<P, W> a, cons
                 }
                 deal.pass((uint32_t)((b7 - b5) % gridDim.x));
             }
-            const bool apply = P::det || k >= a.cap_step;
-            int hubs = 1;  // 2: a single hub took its barriers, and in the deterministic mode its commit
+            if (P::det && late1 > late0) catch_up<P, W>(a, list, late0, late1, deal, sm);
+            bool hub_layout = false;  // run_hubs_grid laid out this step's hubs
             if (b8 > b7) {
                 if (b8 - b7 == 1 && k < a.cap_step) {
-                    hubs = run_hub_single<P, W, REFINE, B>(a, sko[kNumBins + 1], k, bar, deal, sm, pc);
-                    ok = hubs != 0;
+                    ok = run_hub_single<P, W, REFINE, B>(a, sko[kNumBins + 1], k, bar, deal, sm, pc);
                 } else {
                     ok = run_hubs_grid<P, W, REFINE, B>(a, sko[kNumBins + 1], b8 - b7, k, bar, sm, pc);
-                    hubs = 3;  // laid out for hub_flags
+                    hub_layout = true;
                 }
                 if (!ok) break;
             }
             fetched();
-            if (!(apply && hubs == 2) && !(ok = bar.sync())) break;
-            // apply phase: deterministic mode, and proposals where neighbours
-            // may share a step (below the capped step the asynchronous mode
-            // moves and joins at once)
-            if (apply) {
-                const int64_t end = hubs == 2 ? b7 : b8;
+            if (!(ok = bar.sync())) break;
+            // a layered step's moves are made; an apply phase commits the
+            // proposals where neighbours may share a step
+            late0 = late1 = 0;
+            if (k >= a.cap_step) {
                 if (REFINE) {
-                    run_refine_apply<P, W, B>(a, list, b0, end, k, deal, sm);
+                    run_refine_apply<P, W, B>(a, list, b0, b8, k, deal, sm);
                 } else {
-                    run_move_apply<P, W, B>(a, list, b0, end, deal, sm, hubs == 3);
-                    if (hubs == 3) hub_flags<P, W>(a, sm, __ldcg(&a.hinfo[0]), __ldcg(&a.hinfo[2]), true);
+                    run_move_apply<P, W, B>(a, list, b0, b8, deal, sm, hub_layout);
+                    if (hub_layout) hub_flags<P, W>(a, sm, __ldcg(&a.hinfo[0]), __ldcg(&a.hinfo[2]), true);
                 }
                 if (!(ok = bar.sync())) break;
+            } else if (P::det) {
+                late0 = b0;
+                late1 = b8;
+                typename P::tot *const sr = sm.sr;
+                sm.sr = sm.sw;
+                sm.sw = sr;
             }
         }
         if (!ok) break;
+        if (P::det && late1 > late0) catch_up<P, W>(a, list, late0, late1, deal, sm);  // both copies are whole
         // this sweep's sums: one graph reduces per warp, a batch flushes
         // every thread's running sum into its graph's slot
         if (batch) {
@@ -1816,6 +1860,7 @@ template <class P, class W> __device__ __forceinline__ Sums<P> scalar_sums(const
     sm.dq = a.dq_acc;
     sm.mv = a.moved;
     sm.stamp = a.sweep + 1;
+    sm.sr = sm.sw = a.Sig;
     return sm;
 }
 template <class P, class W, bool REFINE>

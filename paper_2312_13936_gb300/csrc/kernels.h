@@ -91,6 +91,10 @@ struct SweepCtx {
     const int32_t *CB = nullptr;  // C'_B, community bound (refinement)
     const void *K = nullptr;  // K' (acc type)
     void *Sig = nullptr;      // Sigma' (acc type)
+    // persistent deterministic sweep: a second copy of Sigma', equal to it, and
+    // n words for its moves (null in per-step launches)
+    void *Sig2 = nullptr;
+    int32_t *old = nullptr;
     int32_t *size = nullptr;  // members per community
     uint8_t *unproc = nullptr;    // Algorithm 2 pruning flags (1 = unprocessed)
     int32_t *prop = nullptr;      // proposed target (-1 none)
