@@ -343,74 +343,25 @@ __device__ __forceinline__ void set_error(int *err, int code) {
     if (err) atomicCAS(err, 0, code);
 }
 
-// Grid-wide barrier of a cooperative launch. bar[0] counts the arrivals of
-// the launch and bar[1] the barriers completed; both are zero when the launch
-// begins (the launcher clears them). Thread 0 of each block arrives with a
-// release add on bar[0]: an arrival that returns old learns its barrier
-// r = old / G + 1 (no block arrives at barrier r + 1 before all G blocks
-// arrived at barrier r), and the G-th arrival publishes r in bar[1] with a
-// release store, which the others poll with acquire loads. Compared with
-// resetting a counter and advancing a generation (three dependent atomics
-// on the last arrival) this took a barrier of 608 blocks from 3.1 to 2.2
-// microseconds on this GPU. Spins are bounded: after spin_limit polls (2^24,
-// about a second, by default) without progress the kernel records
-// kErrTimeout and every later barrier returns at once, so the launch always
-// ends. A grid of one block needs only __syncthreads.
-constexpr unsigned long long kSpinLimit = 1ULL << 24;
-__device__ __forceinline__ unsigned bar_arrive(unsigned *p) {
-    unsigned r;
-    asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(r) : "l"(p) : "memory");
-    return r;
-}
 __device__ __forceinline__ unsigned bar_poll(const unsigned *p) {
     unsigned r;
     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(r) : "l"(p) : "memory");
     return r;
 }
-__device__ __forceinline__ void bar_publish(unsigned *p, unsigned v) {
-    asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
-__device__ __forceinline__ bool grid_barrier(unsigned *bar, int *err, unsigned long long spin_limit = kSpinLimit) {
-    __shared__ int s_ok;
-    __syncthreads();
-    if (gridDim.x == 1) return true;
-    if (threadIdx.x == 0) {
-        int ok = *((volatile int *)err) == 0;
-        if (ok) {
-            const unsigned G = gridDim.x;
-            const unsigned old = bar_arrive(&bar[0]);
-            const unsigned r = old / G + 1;
-            if (old == r * G - 1) {
-                bar_publish(&bar[1], r);
-            } else {
-                unsigned long long spins = 0;
-                while (bar_poll(&bar[1]) < r) {
-                    if (++spins > spin_limit) {
-                        set_error(err, kErrTimeout);
-                        ok = 0;
-                        break;
-                    }
-                    __nanosleep(32);
-                }
-            }
-        }
-        s_ok = ok;
-    }
-    __syncthreads();
-    return s_ok != 0;
-}
-
-// The persistent sweep's grid barrier: one arrival counter, zero when the
-// launch begins, that thread 0 of every block adds to (release, no result
-// asked for) and polls (acquire) until the barrier's G-th arrival; the
-// barrier's number lives in a register, so neither an atomic's result nor a
-// published word lies on the way. Measured alone (4,000 barriers): 152
-// blocks of 1024 threads 1.20 us, against 1.93 us for grid_barrier above and
-// 2.09 us for it with 608 blocks of 256, the same threads; with 608 blocks
-// polling, the counter itself takes 2.15 us, so this barrier goes with few
-// blocks per SM. The error word is read only while waiting, and a barrier
-// that runs out of polls ends the launch: its block arrives nowhere again
-// and the others see the error word or run out too.
+// Grid-wide barrier of a cooperative launch: one arrival counter, zero when
+// the launch begins (the launcher clears it), that thread 0 of every block
+// adds to (release, no result asked for) and polls (acquire) until the
+// barrier's G-th arrival; the barrier's number lives in a register, so
+// neither an atomic's result nor a published word lies on the way. Measured
+// alone (4,000 barriers): 152 blocks of 1024 threads 1.20 us, against 1.93 us
+// for an arrival that learns its barrier from the count and a last one that
+// publishes its number, and 2.09 us for that with 608 blocks of 256, the same
+// threads; with 608 blocks polling, the counter itself takes 2.15 us, so this
+// barrier goes with few blocks per SM. The wait is bounded: the error word is
+// read only while waiting, and a barrier that runs out of polls records
+// kErrTimeout and ends the launch, since its block arrives nowhere again and
+// the others see the error word or run out too. A grid of one block needs
+// only __syncthreads.
 struct GridBar {
     unsigned *count;
     int *err;

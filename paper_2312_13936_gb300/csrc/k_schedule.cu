@@ -21,7 +21,8 @@
 namespace lgb {
 namespace {
 
-constexpr int kSchedThreads = 256;
+constexpr int kSchedThreads = 512;
+constexpr unsigned long long kSchedSpinLimit = 1ULL << 22;  // a second and more of polls
 
 // first vertex of v's graph (0 for a single graph)
 __device__ __forceinline__ int64_t graph_base(const int32_t *gid, const int64_t *vseg, int64_t v) {
@@ -103,29 +104,24 @@ __device__ __forceinline__ void share_long_rows(int64_t R, int64_t warps, int64_
     }
 }
 
-// preceding neighbours of v among row entries [from, to) taken with stride step
+// preceding neighbours of v among row entries [from, to) taken with stride
+// step, four entries in flight
 __device__ __forceinline__ int32_t count_preceding(const SA &a, int64_t e0, int64_t from, int64_t to, int64_t step,
                                                    uint64_t state, int64_t base, int64_t v, uint64_t pv) {
     int32_t c = 0;
-    for (int64_t e = from; e < to; e += step) {
-        const int32_t u = a.idx[e0 + e];
-        if (u != (int32_t)v && precedes(vprio(state, u - base, __ldg(&a.deg[u])), u, pv, (int32_t)v)) c++;
+    for (int64_t e = from; e < to; e += 4 * step) {
+        int32_t u[4], d[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) u[q] = e + q * step < to ? a.idx[e0 + e + q * step] : (int32_t)v;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) d[q] = u[q] != (int32_t)v ? __ldg(&a.deg[u[q]]) : 0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (u[q] != (int32_t)v && precedes(vprio(state, u[q] - base, d[q]), u[q], pv, (int32_t)v)) c++;
     }
     return c;
 }
 
-// entry e of v's row: true when its vertex u is released by v (v precedes
-// u) and v was the last of u's preceding neighbours; u then joins layer r+1
-// (Lv: the layer cap of v's graph; layers stop at Lv-2, vertices past it
-// stay unplaced)
-__device__ __forceinline__ bool release(const SA &a, int64_t e, uint64_t state, int64_t base, int64_t v, uint64_t pv,
-                                        int32_t r, int32_t Lv, int32_t &u) {
-    u = a.idx[e];
-    if (u == (int32_t)v || !precedes(pv, (int32_t)v, vprio(state, u - base, __ldg(&a.deg[u])), u)) return false;
-    if (atomicSub(&a.cnt[u], 1) != 1 || r + 2 > Lv - 1) return false;
-    a.layer[u] = r + 1;
-    return true;
-}
 __device__ __forceinline__ int32_t layer_cap(const SA &a, int64_t v) {
     return a.gL ? __ldg(&a.gL[__ldg(&a.gid[v])]) : a.L;
 }
@@ -146,6 +142,44 @@ __device__ __forceinline__ VHead vhead(const SA &a, int64_t v) {
     return h;
 }
 
+// Four entries of v's row (e + q stride < end; the lane has none: end = 0):
+// releases the vertices that v precedes. Bit q of the result: entry q's
+// vertex u[q] lost its last preceding neighbour here and joins layer r + 1
+// (h.Lv: the layer cap of v's graph; layers stop at Lv - 2, vertices past it
+// stay unplaced). The targets, their degrees and the counters' atomics of the
+// four are each in flight together.
+__device__ __forceinline__ unsigned release4(const SA &a, const VHead &h, int32_t v, int64_t e, int64_t stride,
+                                             int64_t end, int32_t r, int32_t u[4]) {
+    int32_t d[4], left[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) u[q] = e + q * stride < end ? a.idx[h.e0 + e + q * stride] : v;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) d[q] = u[q] != v ? __ldg(&a.deg[u[q]]) : 0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+        left[q] = u[q] != v && precedes(h.pv, v, vprio(h.state, u[q] - h.base, d[q]), u[q])
+                      ? atomicSub(&a.cnt[u[q]], 1)
+                      : 0;
+    unsigned take = 0;
+    if (r + 2 > h.Lv - 1) return 0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+        if (left[q] == 1) {
+            a.layer[u[q]] = r + 1;
+            take |= 1u << q;
+        }
+    return take;
+}
+
+// lanes that share a row of a layer of cnt vertices: as many as leave every
+// thread of the grid work, up to the row's usual length (a layer of a few
+// hundred vertices used to give each row to one lane, which waited for every
+// entry's target, degree and atomic in turn: 16 us a round on 10,007 vertices
+// of 32 entries)
+__device__ __forceinline__ int row_lanes(int64_t cnt, int64_t threads) {
+    return cnt * 8 <= threads ? 8 : cnt * 2 <= threads ? 2 : 1;
+}
+
 template <bool LONG>
 __global__ void __launch_bounds__(kSchedThreads) k_sched_coop(SA a) {
     __shared__ int32_t s_stage[kSchedThreads / 32][kStage];
@@ -153,30 +187,37 @@ __global__ void __launch_bounds__(kSchedThreads) k_sched_coop(SA a) {
     const int lane = threadIdx.x & 31;
     Stage st{s_stage[threadIdx.x >> 5], 0};
     Stage lst{s_lstage[LONG ? (threadIdx.x >> 5) : 0], 0};
+    GridBar bar{a.bar, a.err, kSchedSpinLimit};
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    const int64_t gw = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    // warp numbers run over the blocks first: a layer of few rows uses many SMs
+    const int64_t gw = (int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+    const int64_t threads = warps * 32;
     // cnt[v] = number of v's preceding neighbours; short rows are counted
     // here (layer 0 if none), long rows are listed (in step[], free until
     // the end) and counted by the whole grid next
-    for (int64_t v0 = gw * 32; v0 < a.n; v0 += warps * 32) {
-        const int64_t v = v0 + lane;
-        const bool in = v < a.n;
-        VHead h{};
-        if (in) h = vhead(a, v);
-        const bool lng = LONG && in && h.dv > kLongRow;
-        const int32_t c = (in && !lng) ? count_preceding(a, h.e0, 0, h.dv, 1, h.state, h.base, v, h.pv) : 0;
-        if (in) {
-            a.cnt[v] = c;
-            a.layer[v] = (!lng && c == 0) ? 0 : -1;
+    {
+        const int T = row_lanes(a.n, threads), per = 32 / T, tl = lane & (T - 1);
+        for (int64_t v0 = gw * per; v0 < a.n; v0 += warps * per) {
+            const int64_t v = v0 + lane / T;
+            const bool in = v < a.n, lead = in && tl == 0;
+            VHead h{};
+            if (in) h = vhead(a, v);
+            const bool lng = LONG && in && h.dv > kLongRow;
+            int32_t c = (in && !lng) ? count_preceding(a, h.e0, tl, h.dv, T, h.state, h.base, v, h.pv) : 0;
+            for (int o = T >> 1; o > 0; o >>= 1) c += __shfl_xor_sync(kFull, c, o);
+            if (lead) {
+                a.cnt[v] = c;
+                a.layer[v] = (!lng && c == 0) ? 0 : -1;
+            }
+            st.push(lead && !lng && c == 0, (int32_t)v, a.ord, &a.size[0]);
+            if (LONG) lst.push(lead && lng, (int32_t)v, a.step, &a.size[6]);
         }
-        st.push(in && !lng && c == 0, (int32_t)v, a.ord, &a.size[0]);
-        if (LONG) lst.push(lng, (int32_t)v, a.step, &a.size[6]);
     }
     st.flush(a.ord, &a.size[0]);
     bool ok = true;
     if (LONG) {
         lst.flush(a.step, &a.size[6]);
-        ok = grid_barrier(a.bar, a.err);
+        ok = bar.sync();
         const int64_t nl = ok ? (int64_t)__ldcg(&a.size[6]) : 0;
         share_long_rows(nl, warps, gw, [&](int64_t i, int64_t from, int64_t stride) {
             const int32_t v = __ldcg(&a.step[i]);
@@ -184,7 +225,7 @@ __global__ void __launch_bounds__(kSchedThreads) k_sched_coop(SA a) {
             const int32_t c = warp_sum(count_preceding(a, h.e0, from, h.dv, stride, h.state, h.base, v, h.pv));
             if (lane == 0 && c) atomicAdd(&a.cnt[v], c);
         });
-        ok = ok && grid_barrier(a.bar, a.err);
+        ok = ok && bar.sync();
         for (int64_t i0 = gw * 32; i0 < nl; i0 += warps * 32) {
             const int64_t i = i0 + lane;
             int32_t v = 0;
@@ -200,7 +241,7 @@ __global__ void __launch_bounds__(kSchedThreads) k_sched_coop(SA a) {
         st.flush(a.ord, &a.size[0]);
         lst.flush(a.lord, &a.size[3]);
     }
-    ok = ok && grid_barrier(a.bar, a.err);
+    ok = ok && bar.sync();
     // round r: layer r is ord[lo, hi) (its long rows also lord[llo, lhi));
     // it appends layer r+1 (up to L-2) from ord[hi] and lord[lhi]
     int64_t lo = 0, hi = ok ? (int64_t)__ldcg(&a.size[0]) : 0;
@@ -213,27 +254,31 @@ __global__ void __launch_bounds__(kSchedThreads) k_sched_coop(SA a) {
             a.size[(r + 2) % 3] = 0u;
             a.size[3 + (r + 2) % 3] = 0u;
         }
-        auto placed = [&](bool take, int32_t u) {
-            st.push(take, u, nord, nsz);
-            if (LONG) lst.push(take && __ldg(&a.deg[u]) > kLongRow, u, nlord, nlsz);
+        auto placed = [&](unsigned take, const int32_t u[4]) {
+            if (!__any_sync(kFull, take != 0)) return;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const bool t = take >> q & 1u;
+                st.push(t, u[q], nord, nsz);
+                if (LONG) lst.push(t && __ldg(&a.deg[u[q]]) > kLongRow, u[q], nlord, nlsz);
+            }
         };
-        // short rows: one lane each, stepping together to the warp's
-        // longest short row so that every lane reaches the append
-        for (int64_t i0 = lo + gw * 32; i0 < hi; i0 += warps * 32) {
-            const int64_t i = i0 + lane;
-            int64_t v = 0;
+        // short rows: T lanes each, stepping together to the warp's longest
+        // short row so that every lane reaches the append
+        const int T = row_lanes(hi - lo, threads), per = 32 / T, tl = lane & (T - 1);
+        for (int64_t i0 = lo + gw * per; i0 < hi; i0 += warps * per) {
+            const int64_t i = i0 + lane / T;
+            int32_t v = -1;
             VHead h{};
             if (i < hi) {
                 v = __ldcg(&a.ord[i]);
                 h = vhead(a, v);
             }
             const int32_t ds = (i < hi && (!LONG || h.dv <= kLongRow)) ? h.dv : 0;
-            int32_t dmax = ds;
-            for (int o = 16; o > 0; o >>= 1) dmax = max(dmax, __shfl_xor_sync(kFull, dmax, o));
-            for (int32_t j = 0; j < dmax; ++j) {
-                int32_t u = 0;
-                const bool take = j < ds && release(a, h.e0 + j, h.state, h.base, v, h.pv, r, h.Lv, u);
-                placed(take, u);
+            const int32_t dmax = (int32_t)__reduce_max_sync(kFull, (unsigned)ds);
+            for (int32_t j = 0; j < dmax; j += 4 * T) {
+                int32_t u[4];
+                placed(release4(a, h, v, j + tl, T, ds, r, u), u);
             }
         }
         // long rows: shared by the whole grid
@@ -241,16 +286,14 @@ __global__ void __launch_bounds__(kSchedThreads) k_sched_coop(SA a) {
             share_long_rows(lhi - llo, warps, gw, [&](int64_t i, int64_t from, int64_t stride) {
                 const int32_t v = __ldcg(&a.lord[llo + i]);
                 const VHead h = vhead(a, v);
-                for (int64_t j0 = from - lane; j0 < h.dv; j0 += stride) {
-                    int32_t u = 0;
-                    const int64_t j = j0 + lane;
-                    const bool take = j < h.dv && release(a, h.e0 + j, h.state, h.base, v, h.pv, r, h.Lv, u);
-                    placed(take, u);
+                for (int64_t j0 = from - lane; j0 < h.dv; j0 += 4 * stride) {
+                    int32_t u[4];
+                    placed(release4(a, h, v, j0 + lane, stride, h.dv, r, u), u);
                 }
             });
         st.flush(nord, nsz);
         if (LONG) lst.flush(nlord, nlsz);
-        ok = grid_barrier(a.bar, a.err);
+        ok = bar.sync();
         lo = hi;
         hi = ok ? hi + (int64_t)__ldcg(nsz) : lo;
         llo = lhi;
@@ -353,8 +396,14 @@ cudaError_t launch_schedule(const GraphView &g, uint64_t state, int32_t L, int32
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
     const int per_sm = long_rows ? sched_blocks_per_sm<true>() : sched_blocks_per_sm<false>();
     if (per_sm <= 0) return cudaErrorLaunchOutOfResources;
-    int64_t grid = (g.n + 4 * kSchedThreads - 1) / (4 * kSchedThreads);  // a few vertices per thread
-    if (grid > (int64_t)per_sm * sms) grid = (int64_t)per_sm * sms;
+    // one block (no grid barrier) for a graph whose layers it holds at eight
+    // lanes a vertex, then a block for every 64 vertices up to one per SM;
+    // more where the vertices alone give each thread several
+    int64_t grid = g.n <= 2 * kSchedThreads ? 1 : (g.n + 63) / 64;
+    const int64_t one = sms, all = (int64_t)per_sm * sms;
+    if (grid > one) grid = one;
+    const int64_t many = (g.n + 4 * kSchedThreads - 1) / (4 * kSchedThreads);
+    if (many > grid) grid = many < all ? many : all;
     if (grid < 1) grid = 1;
     SA a;
     a.n = g.n;
