@@ -667,20 +667,16 @@ leiden_status Handle::Impl::pass(Run &r, int32_t lp, bool &stop) {
             }
         }
     }
-    // deterministic mode: rows in ascending target order (reading R10)
-    if (det && cap > 1) {
-        void *stmp = nullptr;
-        const size_t sb = sort_rows_tmp_bytes(cap);
-        if (cudaMallocAsync(&stmp, sb, s) != cudaSuccess) {
-            set_last_error("device allocation of " + std::to_string(sb) + " bytes for the row sort failed");
-            return LEIDEN_ERR_OOM;
+    // deterministic mode: rows in ascending target order (reading R10; those of
+    // the tile bins were written so)
+    if (det)
+        for (int b = 4; b <= kBinHub; ++b) {
+            const int64_t lo = ako[b], hi = ako[b + 1];
+            if (hi == lo) continue;
+            CK(launch_sort_rows(b, q.list + lo, hi - lo, ncomm, q.agg[dst].off, q.agg[dst].deg, q.agg[dst].idx,
+                                static_cast<WInt *>(q.agg[dst].w), r.deg_bound, q.sm, s));
+            q.launches++;
         }
-        const cudaError_t e = launch_sort_rows(ncomm, q.agg[dst].off, q.agg[dst].deg, q.agg[dst].idx,
-                                               static_cast<WInt *>(q.agg[dst].w), cap, stmp, s);
-        cudaFreeAsync(stmp, s);
-        CK(e);
-        q.launches += 1;
-    }
     // move-based labels of the super-vertices (reading R3), or each alone
     // (refine-based labels)
     if (prm.flags & LEIDEN_FLAG_REFINE_LABELS) {

@@ -6,8 +6,9 @@
 // degree like the sweep kernels: a tile of lanes (<= 32 member edges), one
 // warp with a shared-memory table (<= 256), one block with a shared-memory
 // table (<= 4096), one block with a global-memory table (larger).
-// Row order inside G'' is unspecified; deterministic mode writes exact
-// integer sums, so the rows are equal as sets.
+// Row order inside G'' is unspecified in the asynchronous mode; the
+// deterministic mode writes exact integer sums, the tiles in ascending target
+// order, and k_sortrows.cu sorts the longer rows.
 #include <climits>
 
 #include "common.cuh"
@@ -80,6 +81,8 @@ __global__ void __launch_bounds__(256) k_agg_tile(AV<P, Wi, Wo> a, const int32_t
     const int base_lane = lane & ~(T - 1);
     const unsigned tmask = (T == 32) ? kFull : (((1u << T) - 1u) << base_lane);
     const int64_t tiles = (int64_t)gridDim.x * (blockDim.x / T);
+    __shared__ A s_sum[8][32];
+    A *wsum = s_sum[threadIdx.x >> 5];
     ProfCounts pc;
     for (int64_t t = (int64_t)blockIdx.x * (blockDim.x / T) + threadIdx.x / T; t < count; t += tiles) {
         const int32_t c = list[t];
@@ -101,14 +104,12 @@ __global__ void __launch_bounds__(256) k_agg_tile(AV<P, Wi, Wo> a, const int32_t
         }
         const int32_t excl = incl - du;
         const int32_t total = __shfl_sync(tmask, incl, T - 1, T);
-        // the lane whose member owns edge slot tl
+        // the lane whose member owns edge slot tl: the members before it end
+        // at or before tl
         int owner = 0;
 #pragma unroll
-        for (int k = 0; k < T; ++k) {
-            const int32_t ek = __shfl_sync(tmask, excl, k, T);
-            const int32_t ik = __shfl_sync(tmask, incl, k, T);
-            if (tl >= ek && tl < ik) owner = k;
-        }
+        for (int st = T / 2; st >= 1; st >>= 1)
+            if (__shfl_sync(tmask, incl, owner + st - 1, T) <= tl) owner += st;
         const int64_t s_own = __shfl_sync(tmask, su, owner, T);
         const int32_t e_own = __shfl_sync(tmask, excl, owner, T);
         int32_t key = -1;
@@ -118,19 +119,26 @@ __global__ void __launch_bounds__(256) k_agg_tile(AV<P, Wi, Wo> a, const int32_t
             key = a.Cd[a.idx[e]];
             wv = wconv<A>(a.w[e]);
         }
-        A sum = 0;
-        bool lead = (key >= 0);
-#pragma unroll
-        for (int k = 0; k < T; ++k) {
-            const int32_t kk = __shfl_sync(tmask, key, k, T);
-            const A wk = __shfl_sync(tmask, wv, k, T);
-            if (key >= 0 && kk == key) {
-                sum += wk;
-                if (k < tl) lead = false;
-            }
-        }
+        // equal targets find one another with one match and sum in shared
+        // memory at their first lane's place
+        const unsigned peers = __match_any_sync(tmask, key);
+        const int first = __ffs(peers) - 1;
+        const bool lead = key >= 0 && first == lane;
+        wsum[lane] = wv;
+        __syncwarp(tmask);
+        if (key >= 0 && !lead) atomic_add_acc(&wsum[first], wv);
+        __syncwarp(tmask);
+        const A sum = wsum[lane];
+        __syncwarp(tmask);
         const unsigned ball = (__ballot_sync(tmask, lead) & tmask) >> base_lane;
-        const int pos = __popc(ball & ((1u << tl) - 1u));
+        int pos = 0;
+        if (P::det) {  // the row's targets ascend (reading R10)
+            const int32_t mine = lead ? key : INT_MAX;
+#pragma unroll
+            for (int k = 0; k < T; ++k) pos += __shfl_sync(tmask, mine, k, T) < mine ? 1 : 0;
+        } else {
+            pos = __popc(ball & ((1u << tl) - 1u));
+        }
         const int64_t o0 = a.out_off[c];
         A kpart = 0;
         if (lead) {

@@ -1,17 +1,17 @@
 // Rows of a holey CSR sorted by target: the deterministic mode writes every
 // aggregated row in ascending target order (reading R10), so the stored
 // super-vertex graph is the same bit for bit whatever order the hash tables
-// held. Every entry gets the key (row << tb) | target, and the unused slots
-// after a row's fill the key (row << tb) | (2^tb - 1), with tb the fewest
-// bits that hold every target below the marker, so a stable LSD radix sort
-// of the key's tb + row bits (8-bit digits, the counting sort of k_util.cu)
-// leaves every row in place with its entries ascending and its unused slots
-// last.
-// The sort carries a permutation; targets and weights are gathered by it.
-// Rows go in chunks of at most 2^30 entries (the counting sort's positions
-// are int32).
+// held. The targets of a row differ from one another, so an entry's place is
+// the number of smaller targets in its row, and each row is sorted by itself
+// where it lies: communities of up to 32 member entries when the tile kernels
+// of the aggregation write them; rows of up to 256 entries by a warp that
+// counts smaller targets; of up to kRowSmem entries by a block in shared
+// memory; longer ones through a bitmap of their targets, whose running
+// population count is every target's place. (Sorting all slots, unused ones
+// included, as one sequence of (row, target) keys by 8-bit digits read and
+// wrote some 50 bytes a slot and digit, four to seven digits: 45 of the 103 ms
+// of a deterministic run of road 5000 x 5000.)
 #include <algorithm>
-#include <vector>
 
 #include "common.cuh"
 #include "kernels.h"
@@ -19,194 +19,232 @@
 namespace lgb {
 namespace {
 
-constexpr int kSortDigitBits = 8;
-constexpr int64_t kSortChunk = (int64_t)1 << 30;
+constexpr int kRowWarp = 256;    // longest row of a warp: eight entries a lane
+constexpr int kRowSmem = 8192;   // longest row of a block: 16 bytes an entry of shared memory
+constexpr int kBigSplit = 32;    // blocks that share a longer row
+constexpr int64_t kBitmapBytes = (int64_t)1 << 30;  // bitmaps and their counts, for the rows taken at once
 
-inline int sgrid(int64_t n) {
-    int64_t b = (n + 255) / 256;
-    if (b < 1) b = 1;
-    return (int)(b > 152 * 16 ? 152 * 16 : b);
-}
-#define SGRID_STRIDE(i, n) \
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < (n); i += (int64_t)gridDim.x * blockDim.x)
-
-// keys of the slots [e0, e0 + M) of rows [r0, r1): (row - r0) << tb |
-// target, and (row - r0) << tb | (2^tb - 1) for a row's unused slots (the
-// targets are below 2^tb - 1); ord = iota. Rows and slots take positions of
-// one merged sequence (row rr = r - r0 at rr + off[r] - e0, its slot e at
-// rr + 1 + e - e0) and warp k of W takes an equal range of it: a binary
-// search over the rows finds where its range starts, then it walks its rows
-// 32 at a time and writes the keys of their slots in the range with all
-// lanes. No per-slot search, and no warp walks more than its share of rows.
-__global__ void k_row_keys(const int64_t *off, const int32_t *deg, const int32_t *idx, int64_t r0, int64_t r1,
-                           int64_t e0, int64_t M, int tb, unsigned long long *key, int32_t *ord) {
+// A warp per row of up to kRowWarp entries: its targets in shared memory, each
+// lane counting the smaller ones of its up to eight, four targets a read.
+__global__ void __launch_bounds__(256) k_sort_warp(const int32_t *__restrict__ list, int64_t count,
+                                                   const int64_t *__restrict__ off, const int32_t *__restrict__ deg,
+                                                   int32_t *idx, WInt *w) {
+    __shared__ __align__(16) int32_t s_key[8][kRowWarp];
     const int lane = threadIdx.x & 31;
-    const int64_t R = r1 - r0, Tn = R + M;
-    const int64_t W = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t P0 = (int64_t)((__int128)Tn * wid / W), P1 = (int64_t)((__int128)Tn * (wid + 1) / W);
-    if (P0 >= P1) return;
-    const unsigned long long gap = (1ULL << tb) - 1ULL;
-    int64_t lo = 0, hi = R;  // the last row rr with rr + off[r0 + rr] - e0 <= P0
-    while (hi - lo > 1) {
-        const int64_t mid = lo + (hi - lo) / 2;
-        if (mid + off[r0 + mid] - e0 <= P0) lo = mid;
-        else hi = mid;
-    }
-    for (int64_t rb = lo; rb < R; rb += 32) {
-        const int64_t rr = rb + lane;
-        const bool valid = rr < R;
-        const int64_t a = valid ? off[r0 + rr] - e0 : M;
-        const int64_t b = valid ? (rr + 1 < R ? off[r0 + rr + 1] - e0 : M) : M;
-        const int32_t d = valid ? deg[r0 + rr] : 0;
-        const int64_t s0 = a > P0 - rr - 1 ? a : P0 - rr - 1;  // its slots in the range
-        const int64_t t0 = b < P1 - rr - 1 ? b : P1 - rr - 1;
-        unsigned todo = __ballot_sync(0xffffffffu, valid && s0 < t0);
-        while (todo) {
-            const int src = __ffs(todo) - 1;
-            todo &= todo - 1;
-            const int64_t xs = __shfl_sync(0xffffffffu, s0, src), xt = __shfl_sync(0xffffffffu, t0, src);
-            const int64_t as = __shfl_sync(0xffffffffu, a, src);
-            const int32_t ds = __shfl_sync(0xffffffffu, d, src);
-            const unsigned long long hk = (unsigned long long)(rb + src) << tb;
-            for (int64_t x = xs + lane; x < xt; x += 32) {
-                key[x] = hk | (x < as + ds ? (unsigned long long)(uint32_t)idx[e0 + x] : gap);
-                ord[x] = (int32_t)x;
+    int32_t *key = s_key[threadIdx.x >> 5];
+    const int64_t warps = (int64_t)gridDim.x * 8;
+    for (int64_t t = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); t < count; t += warps) {
+        const int32_t c = list[t];
+        const int32_t d = deg[c];
+        if (d <= 1 || d > kRowWarp) continue;  // bins bound d: longer rows never come here
+        const int64_t o = off[c];
+        const int pad = (d + 3) & ~3;
+        int32_t k[8], rank[8];
+        WInt x[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const int e = q * 32 + lane;
+            k[q] = INT32_MAX;
+            x[q] = 0;
+            rank[q] = 0;
+            if (e < d) {
+                k[q] = idx[o + e];
+                x[q] = w[o + e];
             }
+            if (e < pad) key[e] = k[q];
         }
-        const int64_t next = rr + 1 < R ? rr + 1 + off[r0 + rr + 1] - e0 : Tn;  // the next row's position
-        if (__ballot_sync(0xffffffffu, !valid || next >= P1)) break;
+        __syncwarp();
+        const int n = (d + 31) / 32;  // entries of a lane
+        for (int e = 0; e < pad; e += 4) {
+            const int4 y = *reinterpret_cast<const int4 *>(&key[e]);
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+                if (q < n) rank[q] += (y.x < k[q]) + (y.y < k[q]) + (y.z < k[q]) + (y.w < k[q]);
+        }
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+            if (q * 32 + lane < d) {
+                idx[o + rank[q]] = k[q];
+                w[o + rank[q]] = x[q];
+            }
+        __syncwarp();
     }
 }
-__global__ void k_key_digit(const unsigned long long *key, int64_t M, int shift, int32_t *digit) {
-    SGRID_STRIDE(i, M) digit[i] = (int32_t)((key[i] >> shift) & ((1u << kSortDigitBits) - 1));
-}
-__global__ void k_gather_key_ord(const unsigned long long *key, const int32_t *ord, const int32_t *perm, int64_t M,
-                                 unsigned long long *key2, int32_t *ord2) {
-    SGRID_STRIDE(i, M) {
-        const int32_t p = perm[i];
-        key2[i] = key[p];
-        ord2[i] = ord[p];
+
+// A block per row of up to kRowSmem entries: (target, place) words sorted by
+// a bitonic network in shared memory, then the weights follow their places.
+__global__ void k_sort_block(const int32_t *__restrict__ list, int64_t count, const int64_t *__restrict__ off,
+                             const int32_t *__restrict__ deg, int32_t *idx, WInt *w, int cap) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    unsigned long long *key = reinterpret_cast<unsigned long long *>(smem);
+    WInt *x = reinterpret_cast<WInt *>(smem) + cap;
+    for (int64_t t = blockIdx.x; t < count; t += gridDim.x) {
+        const int32_t c = list[t];
+        const int32_t d = deg[c];
+        if (d <= 1 || d > cap) continue;  // the same in every thread
+        const int64_t o = off[c];
+        int P = 32;
+        while (P < d) P <<= 1;
+        for (int e = threadIdx.x; e < P; e += blockDim.x) {
+            key[e] = e < d ? ((unsigned long long)(uint32_t)idx[o + e] << 32) | (uint32_t)e : ~0ULL;
+            if (e < d) x[e] = w[o + e];
+        }
+        __syncthreads();
+        for (int size = 2; size <= P; size <<= 1)
+            for (int st = size >> 1; st > 0; st >>= 1) {
+                for (int i = threadIdx.x; i < P / 2; i += blockDim.x) {
+                    const int lo = 2 * i - (i & (st - 1));
+                    const unsigned long long p = key[lo], q = key[lo + st];
+                    if ((p > q) == ((lo & size) == 0)) {
+                        key[lo] = q;
+                        key[lo + st] = p;
+                    }
+                }
+                __syncthreads();
+            }
+        for (int e = threadIdx.x; e < d; e += blockDim.x) {
+            const unsigned long long k = key[e];
+            idx[o + e] = (int32_t)(k >> 32);
+            w[o + e] = x[(uint32_t)k];
+        }
+        __syncthreads();
     }
 }
-template <class W>
-__global__ void k_gather_entries(const int32_t *ord, int64_t M, const int32_t *idx_in, const W *w_in, int32_t *idx_out,
-                                 W *w_out) {
-    SGRID_STRIDE(i, M) {
-        const int32_t p = ord[i];
-        idx_out[i] = idx_in[p];
-        w_out[i] = w_in[p];
+
+// ---- rows of more than kRowSmem entries
+__global__ void k_big_rows(const int32_t *list, int64_t count, const int32_t *deg, int32_t *big, int32_t *bdeg,
+                           unsigned *nbig) {
+    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < count; t += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t c = list[t];
+        if (deg[c] <= kRowSmem) continue;
+        const unsigned p = atomicAdd(nbig, 1u);
+        big[p] = c;
+        bdeg[p] = deg[c];
     }
 }
+// row blockIdx.x of the rows taken at once: its entries to the scratch, its
+// targets into its bitmap
+__global__ void k_big_set(const int32_t *big, const int64_t *boff, int64_t p0, const int64_t *off, const int32_t *idx,
+                          const WInt *w, int32_t *cidx, WInt *cw, unsigned *bits, int64_t nwords) {
+    const int64_t p = p0 + blockIdx.x, o = off[big[p]], b = boff[p], d = boff[p + 1] - b;
+    unsigned *m = bits + (int64_t)blockIdx.x * nwords;
+    for (int64_t e = (int64_t)blockIdx.y * blockDim.x + threadIdx.x; e < d; e += (int64_t)gridDim.y * blockDim.x) {
+        const int32_t k = idx[o + e];
+        cidx[b + e] = k;
+        cw[b + e] = w[o + e];
+        atomicOr(&m[k >> 5], 1u << (k & 31));
+    }
+}
+// targets of row blockIdx.x before each word of its bitmap
+__global__ void __launch_bounds__(1024) k_big_count(const unsigned *bits, unsigned *before, int64_t nwords) {
+    __shared__ unsigned s_w[32];
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    const unsigned *m = bits + (int64_t)blockIdx.x * nwords;
+    unsigned *out = before + (int64_t)blockIdx.x * nwords;
+    unsigned carry = 0;
+    for (int64_t i0 = 0; i0 < nwords; i0 += blockDim.x) {
+        const int64_t i = i0 + threadIdx.x;
+        const unsigned own = i < nwords ? __popc(m[i]) : 0;
+        unsigned inc = own;
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned y = __shfl_up_sync(kFull, inc, o);
+            if (lane >= o) inc += y;
+        }
+        if (lane == 31) s_w[wib] = inc;
+        __syncthreads();
+        unsigned mine = carry, all = 0;
+        for (int k = 0; k < 32; ++k) {
+            if (k < wib) mine += s_w[k];
+            all += s_w[k];
+        }
+        if (i < nwords) out[i] = mine + inc - own;
+        carry += all;
+        __syncthreads();
+    }
+}
+__global__ void k_big_place(const int32_t *big, const int64_t *boff, int64_t p0, const int64_t *off,
+                            const int32_t *cidx, const WInt *cw, const unsigned *bits, const unsigned *before,
+                            int64_t nwords, int32_t *idx, WInt *w) {
+    const int64_t p = p0 + blockIdx.x, o = off[big[p]], b = boff[p], d = boff[p + 1] - b;
+    const unsigned *m = bits + (int64_t)blockIdx.x * nwords, *f = before + (int64_t)blockIdx.x * nwords;
+    for (int64_t e = (int64_t)blockIdx.y * blockDim.x + threadIdx.x; e < d; e += (int64_t)gridDim.y * blockDim.x) {
+        const int32_t k = cidx[b + e];
+        const int64_t at = o + f[k >> 5] + __popc(m[k >> 5] & ((1u << (k & 31)) - 1u));
+        idx[at] = k;
+        w[at] = cw[b + e];
+    }
+}
+
+inline int blocks_for(int64_t items, int64_t most) { return (int)std::max<int64_t>(1, std::min(items, most)); }
 
 }  // namespace
 
-// The scratch of a chunk of M1 - 1 slots: byte offsets of its buffers, each
-// starting at a multiple of 256, and the total. Both the size asked for and
-// the pointers taken come from here.
-namespace {
-struct SortLayout {
-    size_t key, key2, ord, ord2, digit, perm, idx_copy, w_copy, key_off, part, total;
-    explicit SortLayout(int64_t M1) {
-        size_t at = 0;
-        auto take = [&](size_t bytes) {
-            const size_t here = at;
-            at += (bytes + 255) & ~(size_t)255;
-            return here;
-        };
-        key = take(8 * (size_t)M1);
-        key2 = take(8 * (size_t)M1);
-        ord = take(4 * (size_t)M1);
-        ord2 = take(4 * (size_t)M1);
-        digit = take(4 * (size_t)M1);
-        perm = take(4 * (size_t)M1);
-        idx_copy = take(4 * (size_t)M1);
-        w_copy = take(8 * (size_t)M1);
-        key_off = take(8 * ((1 << kSortDigitBits) + 2));
-        part = take(partition_tmp_bytes(M1, 1 << kSortDigitBits));
-        total = at;
-    }
-};
-}  // namespace
-
-size_t sort_rows_tmp_bytes(int64_t cap) { return SortLayout(std::min<int64_t>(cap, kSortChunk) + 1).total; }
-
-cudaError_t launch_sort_rows(int64_t n, const int64_t *off, const int32_t *deg, int32_t *idx, WInt *w, int64_t cap,
-                             void *tmp, cudaStream_t s) {
-    if (n <= 0 || cap <= 1) return cudaSuccess;
+cudaError_t launch_sort_rows(int bin, const int32_t *list, int64_t count, int64_t n, const int64_t *off,
+                             const int32_t *deg, int32_t *idx, WInt *w, int64_t max_row, int sms, cudaStream_t s) {
+    if (count <= 0) return cudaSuccess;
     cudaError_t e;
-    // row chunks of at most kSortChunk slots (the offsets come to the host
-    // only when the graph needs more than one chunk)
-    std::vector<int64_t> cut = {0, n}, hoff;
-    if (cap > kSortChunk) {
-        hoff.resize((size_t)n + 1);
-        if ((e = cudaMemcpyAsync(hoff.data(), off, 8 * (size_t)(n + 1), cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
-            (e = cudaStreamSynchronize(s)) != cudaSuccess)
-            return e;
-        cut = {0};
-        for (int64_t r = 0; r < n;) {
-            int64_t lo = r + 1, hi = n;
-            while (lo < hi) {
-                const int64_t mid = (lo + hi + 1) / 2;
-                if (hoff[(size_t)mid] - hoff[(size_t)r] <= kSortChunk) lo = mid;
-                else hi = mid - 1;
-            }
-            r = lo;
-            cut.push_back(r);
-        }
+    if (bin <= 4) {
+        k_sort_warp<<<blocks_for((count + 7) / 8, (int64_t)sms * 8), 256, 0, s>>>(list, count, off, deg, idx, w);
+        return cudaGetLastError();
     }
-    auto at = [&](int64_t r) { return hoff.empty() ? (r == 0 ? (int64_t)0 : cap) : hoff[(size_t)r]; };
-    int64_t chunk_max = 0;
-    for (size_t k = 0; k + 1 < cut.size(); ++k) chunk_max = std::max(chunk_max, at(cut[k + 1]) - at(cut[k]));
-    if (chunk_max > kSortChunk) return cudaErrorInvalidValue;  // one row beyond 2^30 slots
-    char *p = static_cast<char *>(tmp);
-    const SortLayout at_byte(chunk_max + 1);
-    auto *key = reinterpret_cast<unsigned long long *>(p + at_byte.key);
-    auto *key2 = reinterpret_cast<unsigned long long *>(p + at_byte.key2);
-    auto *ord = reinterpret_cast<int32_t *>(p + at_byte.ord);
-    auto *ord2 = reinterpret_cast<int32_t *>(p + at_byte.ord2);
-    auto *digit = reinterpret_cast<int32_t *>(p + at_byte.digit);
-    auto *perm = reinterpret_cast<int32_t *>(p + at_byte.perm);
-    auto *idx_copy = reinterpret_cast<int32_t *>(p + at_byte.idx_copy);
-    auto *w_copy = reinterpret_cast<WInt *>(p + at_byte.w_copy);
-    int64_t *key_off = reinterpret_cast<int64_t *>(p + at_byte.key_off);
-    void *part_tmp = p + at_byte.part;
-    int tbits = 1;  // targets are row ids of the same graph: below n <= 2^tbits - 1, the gap marker
-    while ((1LL << tbits) - 1 < n) ++tbits;
-    for (size_t k = 0; k + 1 < cut.size(); ++k) {
-        const int64_t r0 = cut[k], r1 = cut[k + 1];
-        const int64_t e0 = at(r0), M = at(r1) - e0;
-        if (M <= 1) continue;
-        int rbits = 0;
-        while ((1LL << rbits) < r1 - r0) ++rbits;
-        if (rbits + tbits > 64) return cudaErrorInvalidValue;
-        // warps of about 4096 merged positions each, at most one resident wave's worth of blocks per pass
-        const int64_t kb = ((r1 - r0) + M + 8 * 4096 - 1) / (8 * 4096);
-        k_row_keys<<<(int)(kb < 1 ? 1 : (kb > 152 * 64 ? 152 * 64 : kb)), 256, 0, s>>>(off, deg, idx, r0, r1, e0, M,
-                                                                                      tbits, key, ord);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        // the key's bits: targets and the gap marker, then the row
-        std::vector<int> shifts;
-        for (int sh = 0; sh < tbits + rbits; sh += kSortDigitBits) shifts.push_back(sh);
-        unsigned long long *ck = key, *ck2 = key2;
-        int32_t *co = ord, *co2 = ord2;
-        for (int sh : shifts) {
-            k_key_digit<<<sgrid(M), 256, 0, s>>>(ck, M, sh, digit);
-            if ((e = cudaGetLastError()) != cudaSuccess) return e;
-            if ((e = launch_partition(digit, M, 1 << kSortDigitBits, key_off, perm, part_tmp, s)) != cudaSuccess)
-                return e;
-            k_gather_key_ord<<<sgrid(M), 256, 0, s>>>(ck, co, perm, M, ck2, co2);
-            if ((e = cudaGetLastError()) != cudaSuccess) return e;
-            std::swap(ck, ck2);
-            std::swap(co, co2);
-        }
-        if ((e = cudaMemcpyAsync(idx_copy, idx + e0, 4 * (size_t)M, cudaMemcpyDeviceToDevice, s)) != cudaSuccess ||
-            (e = cudaMemcpyAsync(w_copy, w + e0, 8 * (size_t)M, cudaMemcpyDeviceToDevice, s)) != cudaSuccess)
-            return e;
-        k_gather_entries<WInt><<<sgrid(M), 256, 0, s>>>(co, M, idx_copy, w_copy, idx + e0, w + e0);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    // rows of bin 5 have up to kBlockMaxDeg entries; bin 6 takes all the
+    // shared memory a row may need, bounded by the longest row's capacity
+    int cap = kBlockMaxDeg;
+    if (bin > 5)
+        while (cap < max_row && cap < kRowSmem) cap <<= 1;
+    const size_t bytes = (size_t)cap * 16;
+    if ((e = cudaFuncSetAttribute(k_sort_block, cudaFuncAttributeMaxDynamicSharedMemorySize, kRowSmem * 16)) !=
+        cudaSuccess)
+        return e;
+    k_sort_block<<<blocks_for(count, (int64_t)sms * 8), cap > kBlockMaxDeg ? 512 : 256, bytes, s>>>(list, count, off, deg,
+                                                                                               idx, w, cap);
+    if ((e = cudaGetLastError()) != cudaSuccess || bin <= 5 || max_row <= kRowSmem) return e;
+    // longer rows
+    int32_t *big = nullptr, *cidx = nullptr;
+    WInt *cw = nullptr;
+    int64_t *boff = nullptr;
+    unsigned *nbig = nullptr, *bits = nullptr;
+    unsigned nb = 0;
+    void *stmp = nullptr;
+    auto get = [&](auto **p, size_t bytes2) {
+        return cudaMallocAsync(reinterpret_cast<void **>(p), bytes2, s);
+    };
+    auto done = [&](cudaError_t r) {
+        for (void *p : {(void *)big, (void *)cidx, (void *)cw, (void *)boff, (void *)nbig, (void *)bits, stmp})
+            if (p) cudaFreeAsync(p, s);
+        return r;
+    };
+    if ((e = get(&big, 8 * (size_t)count)) != cudaSuccess || (e = get(&nbig, sizeof(unsigned))) != cudaSuccess)
+        return done(e);
+    int32_t *bdeg = big + count;
+    if ((e = cudaMemsetAsync(nbig, 0, sizeof(unsigned), s)) != cudaSuccess) return done(e);
+    k_big_rows<<<blocks_for((count + 255) / 256, (int64_t)sms * 8), 256, 0, s>>>(list, count, deg, big, bdeg, nbig);
+    if ((e = cudaGetLastError()) != cudaSuccess ||
+        (e = cudaMemcpyAsync(&nb, nbig, sizeof(nb), cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
+        (e = cudaStreamSynchronize(s)) != cudaSuccess || nb == 0)
+        return done(e);
+    int64_t entries = 0;
+    if ((e = get(&boff, 8 * ((size_t)nb + 1))) != cudaSuccess || (e = get(&stmp, scan_tmp_bytes(nb))) != cudaSuccess ||
+        (e = launch_exclusive_scan_i32(bdeg, boff, nb, stmp, s)) != cudaSuccess ||
+        (e = cudaMemcpyAsync(&entries, boff + nb, 8, cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
+        (e = cudaStreamSynchronize(s)) != cudaSuccess)
+        return done(e);
+    const int64_t nwords = (n + 31) / 32;
+    const int64_t rows = std::max<int64_t>(1, std::min<int64_t>(nb, kBitmapBytes / (8 * nwords)));
+    if ((e = get(&cidx, 4 * (size_t)entries)) != cudaSuccess || (e = get(&cw, 8 * (size_t)entries)) != cudaSuccess ||
+        (e = get(&bits, 8 * (size_t)(rows * nwords))) != cudaSuccess)
+        return done(e);
+    unsigned *before = bits + rows * nwords;
+    for (int64_t p0 = 0; p0 < (int64_t)nb; p0 += rows) {
+        const int64_t r = std::min<int64_t>(rows, (int64_t)nb - p0);
+        const dim3 grid((unsigned)r, kBigSplit);
+        if ((e = cudaMemsetAsync(bits, 0, 4 * (size_t)(r * nwords), s)) != cudaSuccess) return done(e);
+        k_big_set<<<grid, 256, 0, s>>>(big, boff, p0, off, idx, w, cidx, cw, bits, nwords);
+        k_big_count<<<(unsigned)r, 1024, 0, s>>>(bits, before, nwords);
+        k_big_place<<<grid, 256, 0, s>>>(big, boff, p0, off, cidx, cw, bits, before, nwords, idx, w);
+        if ((e = cudaGetLastError()) != cudaSuccess) return done(e);
     }
-    return cudaSuccess;
+    return done(cudaSuccess);
 }
 
 }  // namespace lgb

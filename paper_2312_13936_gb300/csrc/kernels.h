@@ -234,14 +234,13 @@ cudaError_t launch_table_members(const int32_t *list, int64_t K6, const int64_t 
 // rows, 32 slots per warp
 cudaError_t launch_aggregate_tables(const AggCtx &c, const int32_t *list, int sms, cudaStream_t s);
 
-// Rows of a holey CSR (n rows, cap = offsets[n] slots, weights WInt)
-// sorted by target in place, each row's unused slots kept after its fill
-// (reading R10, the deterministic mode); tmp >= sort_rows_tmp_bytes(cap)
-// bytes of device scratch. Synchronises the stream when cap > 2^30 (the row
-// offsets are then read on the host to cut the rows into chunks).
-size_t sort_rows_tmp_bytes(int64_t cap);
-cudaError_t launch_sort_rows(int64_t n, const int64_t *off, const int32_t *deg, int32_t *idx, WInt *w, int64_t cap,
-                             void *tmp, cudaStream_t s);
+// Rows of the aggregated graph of n vertices sorted by target in place, those
+// of the communities list[0, count) of one bin of the aggregation (4, 5 or 6;
+// reading R10, the deterministic mode: the tile bins' rows are written in
+// order). max_row: the longest row's capacity. Synchronises the stream when
+// rows of bin 6 may exceed what a block's shared memory sorts.
+cudaError_t launch_sort_rows(int bin, const int32_t *list, int64_t count, int64_t n, const int64_t *off,
+                             const int32_t *deg, int32_t *idx, WInt *w, int64_t max_row, int sms, cudaStream_t s);
 
 // ---- utilities (k_util.cu)
 cudaError_t launch_iota(int32_t *a, int64_t n, cudaStream_t s);
