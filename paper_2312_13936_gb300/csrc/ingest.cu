@@ -2,15 +2,18 @@
 // paper's experiments (edges made undirected, reverse edges added, unit
 // weight by default; Section 5.1, Table 2). Every edge (u, v) with u != v
 // gives the entries (u, v) and (v, u); a self-loop gives one entry (reading
-// R11) unless dropped. Entries are first counted per row and scattered into
-// row segments (a counting sort by row, with 64-bit positions, so edge lists
-// of billions of edges fit); then the rows are cut into chunks of at most
-// 2^30 entries, and each chunk is sorted by (row, target) with an LSD radix
-// sort whose passes are the stable counting sort of k_util.cu (8-bit digits,
-// so its per-block histograms stay small), and entries with equal (row,
-// target) are merged (weights summed in fp64 and rounded once, or the
-// largest kept) straight into the output. Row offsets come from a scan of
-// the merged row lengths.
+// R11) unless dropped. Entries are counted per row and scattered into row
+// segments (a counting sort by row, with 64-bit positions, so edge lists of
+// billions of edges fit); then every row is sorted by target by itself and
+// its entries with equal targets are merged (weights summed in fp64 and
+// rounded once, or the largest kept) at the front of its segment: rows of up
+// to 32 entries by a tile of lanes, of up to 256 by a warp, of up to kRowSmem
+// by a block in shared memory. Row offsets come from a scan of the merged row
+// lengths, and the fronts are copied to their places. Longer rows are never
+// sorted: a bitmap of their targets counts them, and its running population
+// count is every target's place. (Sorting all entries by (row, target) with
+// 8-bit digits moved them six times at a million vertices, some 50 bytes an
+// entry and digit: 24 of 28.5 ms for 47M edges.)
 #include <cmath>
 #include <string>
 #include <utility>
@@ -23,9 +26,12 @@
 namespace lgb {
 namespace {
 
-constexpr int kDigitBits = 8;
-// entries sorted at once: the counting sort's positions are int32
-constexpr int64_t kChunkEntries = (int64_t)1 << 30;
+constexpr int kRowWarp = 256;
+constexpr int kRowSmem = 16384;  // 12 bytes an entry of shared memory
+constexpr int64_t kMaxRow = (int64_t)1 << 30;
+constexpr int kBigSplit = 32;    // blocks that share a row of more than kRowSmem entries
+constexpr int64_t kBitmapBytes = (int64_t)1 << 31;  // bitmaps and their counts, for the long rows taken at once
+constexpr int kRowBins = 6;      // 1: up to 8 entries, 2: 32, 3: kRowWarp, 4: 2048, 5: kRowSmem, 6: longer (0 unused)
 
 inline int grid_for(int64_t n, int threads) {
     int64_t b = (n + threads - 1) / threads;
@@ -55,64 +61,293 @@ __global__ void k_count_rows(int64_t n, int64_t m, const int32_t *src, const int
         }
     }
 }
-// scatter every entry into its row segment: key = (row << 32) | target
-// (rows in order, entries of a row in no particular order)
+// scatter every entry into its row segment (the targets of a row in no
+// particular order)
 __global__ void k_scatter_rows(int64_t m, const int32_t *src, const int32_t *dst, const float *w, int drop_self,
-                               const int64_t *rowstart, unsigned long long *cursor, unsigned long long *key,
-                               float *wt) {
+                               const int64_t *rowstart, unsigned long long *cursor, int32_t *tgt, float *wt) {
     GRID_STRIDE(e, m) {
         const int32_t u = src[e], v = dst[e];
-        const float x = w ? w[e] : 1.0f;
         if (u == v && drop_self) continue;
+        const float x = wt ? w[e] : 1.0f;
         const int64_t p = rowstart[u] + (int64_t)atomicAdd(&cursor[u], 1ULL);
-        key[p] = ((unsigned long long)(uint32_t)u << 32) | (uint32_t)v;
+        tgt[p] = v;
         if (wt) wt[p] = x;
         if (u != v) {
             const int64_t q = rowstart[v] + (int64_t)atomicAdd(&cursor[v], 1ULL);
-            key[q] = ((unsigned long long)(uint32_t)v << 32) | (uint32_t)u;
+            tgt[q] = u;
             if (wt) wt[q] = x;
         }
     }
 }
-// sort digit of entry i of a chunk whose rows start at r0: bits
-// [shift, shift + 8) of the relative key ((row - r0) << 32) | target
-__global__ void k_digit(const unsigned long long *key, int64_t M, unsigned long long r0, int shift, int32_t *digit) {
-    GRID_STRIDE(i, M) digit[i] = (int32_t)(((key[i] - (r0 << 32)) >> shift) & ((1u << kDigitBits) - 1));
-}
-__global__ void k_gather_kw(const unsigned long long *key, const float *wt, const int32_t *perm, int64_t M,
-                            unsigned long long *key2, float *wt2) {
-    GRID_STRIDE(i, M) {
-        const int32_t p = perm[i];
-        key2[i] = key[p];
-        if (wt) wt2[i] = wt[p];
+__global__ void k_row_bins(const int64_t *rowstart, int64_t n, int32_t *bin) {
+    GRID_STRIDE(r, n) {
+        const int64_t d = rowstart[r + 1] - rowstart[r];
+        bin[r] = d <= 0 ? -1 : d <= 8 ? 1 : d <= 32 ? 2 : d <= kRowWarp ? 3 : d <= 2048 ? 4 : d <= kRowSmem ? 5 : 6;
     }
 }
-// first[i] = 1 when sorted entry i starts a run of equal keys
-__global__ void k_run_starts(const unsigned long long *key, int64_t M, int32_t *first) {
-    GRID_STRIDE(i, M) first[i] = (i == 0 || key[i] != key[i - 1]) ? 1 : 0;
+
+__device__ __forceinline__ double combined(double s, double x, int combine) { return combine ? fmax(s, x) : s + x; }
+
+// T lanes per row of up to T entries: equal targets find one another with one
+// match, the first lane of each keeps the merged weight, and its place is the
+// number of first lanes with smaller targets.
+template <int T>
+__global__ void __launch_bounds__(256) k_row_tile(const int32_t *__restrict__ list, int64_t count,
+                                                  const int64_t *__restrict__ rowstart, int32_t *tgt, float *wt,
+                                                  float *mw, int combine, int64_t *rowlen) {
+    const int lane = threadIdx.x & 31, tl = lane & (T - 1), base = lane & ~(T - 1);
+    const unsigned tmask = T == 32 ? kFull : ((1u << T) - 1u) << base;
+    const int64_t tiles = (int64_t)gridDim.x * (blockDim.x / T);
+    for (int64_t t = (int64_t)blockIdx.x * (blockDim.x / T) + threadIdx.x / T; t < count; t += tiles) {
+        const int32_t r = list[t];
+        const int64_t o = rowstart[r];
+        const int d = (int)(rowstart[r + 1] - o);
+        const int32_t k = tl < d ? tgt[o + tl] : -1;
+        const float x = (wt && tl < d) ? wt[o + tl] : 1.0f;
+        const unsigned peers = __match_any_sync(tmask, k);
+        const bool head = k >= 0 && __ffs(peers) - 1 == lane;
+        const int32_t mine = head ? k : INT32_MAX;
+        int pos = 0;
+#pragma unroll
+        for (int j = 0; j < T; ++j) pos += __shfl_sync(tmask, mine, j, T) < mine ? 1 : 0;
+        double s = wt ? (double)x : (combine ? 1.0 : (double)__popc(peers));
+        if (wt && __any_sync(tmask, k >= 0 && !head)) {
+            for (int j = 0; j < T; ++j) {
+                const float y = __shfl_sync(tmask, x, j, T);
+                if (head && base + j != lane && (peers >> (base + j) & 1u)) s = combined(s, (double)y, combine);
+            }
+        }
+        const unsigned heads = __ballot_sync(tmask, head) & tmask;
+        if (head) {
+            tgt[o + pos] = k;
+            mw[o + pos] = (float)s;
+        }
+        if (tl == 0) rowlen[r] = __popc(heads);
+    }
 }
-// run r of the chunk (starting at sorted entry i, pos[i] = r) writes its
-// target and merged weight (fp64 sum rounded once, or the largest; unit
-// weights when wt is null) to out + base + r, while it fits in cap; the
-// run's row gains one entry
-__global__ void k_merge_runs(const unsigned long long *key, const float *wt, const int32_t *first, const int64_t *pos,
-                             int64_t M, int combine, int64_t base, int64_t cap, int32_t *idx, float *wout,
-                             unsigned long long *rowlen) {
-    GRID_STRIDE(i, M) {
-        if (!first[i]) continue;
-        const unsigned long long k = key[i];
-        double s = wt ? (double)wt[i] : 1.0;
-        int64_t j = i + 1;
-        for (; j < M && key[j] == k; ++j) {
-            const double x = wt ? (double)wt[j] : 1.0;
-            s = combine ? fmax(s, x) : s + x;
+
+// A warp per row of up to kRowWarp entries: the lanes count each target's
+// smaller ones (equal ones by place) for its place in order, and the sorted
+// targets, in shared memory, are merged by neighbour.
+__global__ void __launch_bounds__(256) k_row_warp(const int32_t *__restrict__ list, int64_t count,
+                                                  const int64_t *__restrict__ rowstart, int32_t *tgt, float *wt,
+                                                  float *mw, int combine, int64_t *rowlen) {
+    __shared__ __align__(16) int32_t s_key[8][kRowWarp];
+    __shared__ float s_w[8][kRowWarp];
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    int32_t *key = s_key[wib];
+    float *sw = s_w[wib];
+    const int64_t warps = (int64_t)gridDim.x * 8;
+    for (int64_t t = (int64_t)blockIdx.x * 8 + wib; t < count; t += warps) {
+        const int32_t r = list[t];
+        const int64_t o = rowstart[r];
+        const int d = (int)(rowstart[r + 1] - o), pad = (d + 3) & ~3, n = (d + 31) / 32;
+        int32_t k[8], rank[8];
+        float x[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const int e = q * 32 + lane;
+            k[q] = INT32_MAX;
+            x[q] = 1.0f;
+            rank[q] = 0;
+            if (e < d) {
+                k[q] = tgt[o + e];
+                if (wt) x[q] = wt[o + e];
+            }
+            if (e < pad) key[e] = k[q];
         }
-        const int64_t r = base + pos[i];
-        if (r < cap) {
-            idx[r] = (int32_t)(uint32_t)k;
-            wout[r] = (float)s;
+        __syncwarp();
+        for (int e = 0; e < pad; e += 4) {
+            const int4 y = *reinterpret_cast<const int4 *>(&key[e]);
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+                if (q < n) {
+                    const int p = q * 32 + lane;  // an equal target before this one counts as smaller
+                    rank[q] += (y.x < k[q] + (e < p)) + (y.y < k[q] + (e + 1 < p)) + (y.z < k[q] + (e + 2 < p)) +
+                               (y.w < k[q] + (e + 3 < p));
+                }
         }
-        atomicAdd(&rowlen[k >> 32], 1ULL);
+        __syncwarp();
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+            if (q * 32 + lane < d) {
+                key[rank[q]] = k[q];
+                sw[rank[q]] = x[q];
+            }
+        __syncwarp();
+        int done = 0;
+        for (int e0 = 0; e0 < d; e0 += 32) {
+            const int e = e0 + lane;
+            const bool head = e < d && (e == 0 || key[e] != key[e - 1]);
+            const unsigned heads = __ballot_sync(kFull, head);
+            if (head) {
+                double s = (double)sw[e];
+                for (int j = e + 1; j < d && key[j] == key[e]; ++j) s = combined(s, (double)sw[j], combine);
+                const int64_t at = o + done + __popc(heads & ((1u << lane) - 1u));
+                tgt[at] = key[e];
+                mw[at] = (float)s;
+            }
+            done += __popc(heads);
+        }
+        if (lane == 0) rowlen[r] = done;
+        __syncwarp();
+    }
+}
+
+// A block per row of up to cap entries: (target, place) words sorted by a
+// bitonic network in shared memory, then merged by neighbour, every thread a
+// run of consecutive ones.
+__global__ void __launch_bounds__(512) k_row_block(const int32_t *__restrict__ list, int64_t count,
+                                                   const int64_t *__restrict__ rowstart, int32_t *tgt, float *wt,
+                                                   float *mw, int combine, int64_t *rowlen, int cap) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ int s_part[16];
+    unsigned long long *key = reinterpret_cast<unsigned long long *>(smem);
+    float *x = reinterpret_cast<float *>(key + cap);
+    const int tid = threadIdx.x, lane = tid & 31, wib = tid >> 5, nw = blockDim.x >> 5;
+    for (int64_t t = blockIdx.x; t < count; t += gridDim.x) {
+        const int32_t r = list[t];
+        const int64_t o = rowstart[r];
+        const int d = (int)(rowstart[r + 1] - o);
+        int P = 32;
+        while (P < d) P <<= 1;
+        for (int e = tid; e < P; e += blockDim.x) {
+            key[e] = e < d ? ((unsigned long long)(uint32_t)tgt[o + e] << 32) | (uint32_t)e : ~0ULL;
+            if (e < d) x[e] = wt ? wt[o + e] : 1.0f;
+        }
+        __syncthreads();
+        for (int size = 2; size <= P; size <<= 1)
+            for (int st = size >> 1; st > 0; st >>= 1) {
+                for (int i = tid; i < P / 2; i += blockDim.x) {
+                    const int lo = 2 * i - (i & (st - 1));
+                    const unsigned long long p = key[lo], q = key[lo + st];
+                    if ((p > q) == ((lo & size) == 0)) {
+                        key[lo] = q;
+                        key[lo + st] = p;
+                    }
+                }
+                __syncthreads();
+            }
+        const int per = (d + blockDim.x - 1) / blockDim.x, e0 = min(d, tid * per), e1 = min(d, e0 + per);
+        int heads = 0;
+        for (int e = e0; e < e1; ++e) heads += e == 0 || key[e] >> 32 != key[e - 1] >> 32;
+        int inc = heads;
+        for (int q = 1; q < 32; q <<= 1) {
+            const int y = __shfl_up_sync(kFull, inc, q);
+            if (lane >= q) inc += y;
+        }
+        if (lane == 31) s_part[wib] = inc;
+        __syncthreads();
+        int at = inc - heads, all = 0;
+        for (int q = 0; q < nw; ++q) {
+            if (q < wib) at += s_part[q];
+            all += s_part[q];
+        }
+        for (int e = e0; e < e1; ++e) {
+            const uint32_t k = (uint32_t)(key[e] >> 32);
+            if (e > 0 && k == (uint32_t)(key[e - 1] >> 32)) continue;
+            double s = (double)x[(uint32_t)key[e]];
+            for (int j = e + 1; j < d && (uint32_t)(key[j] >> 32) == k; ++j)
+                s = combined(s, (double)x[(uint32_t)key[j]], combine);
+            tgt[o + at] = (int32_t)k;
+            mw[o + at] = (float)s;
+            ++at;
+        }
+        if (tid == 0) rowlen[r] = all;
+        __syncthreads();
+    }
+}
+
+// ---- rows of more than kRowSmem entries: rows [p0, p0 + gridDim.x) of list
+__global__ void k_long_set(const int32_t *list, int64_t p0, const int64_t *rowstart, const int32_t *tgt,
+                           unsigned *bits, int64_t nwords) {
+    const int32_t r = list[p0 + blockIdx.x];
+    const int64_t o = rowstart[r], d = rowstart[r + 1] - o;
+    unsigned *m = bits + (int64_t)blockIdx.x * nwords;
+    for (int64_t e = (int64_t)blockIdx.y * blockDim.x + threadIdx.x; e < d; e += (int64_t)gridDim.y * blockDim.x) {
+        const int32_t k = tgt[o + e];
+        atomicOr(&m[k >> 5], 1u << (k & 31));
+    }
+}
+// targets before each word of a row's bitmap, and the row's merged length
+__global__ void __launch_bounds__(1024) k_long_count(const int32_t *list, int64_t p0, const unsigned *bits,
+                                                     unsigned *before, int64_t nwords, int64_t *rowlen) {
+    __shared__ unsigned s_w[32];
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    const unsigned *m = bits + (int64_t)blockIdx.x * nwords;
+    unsigned *out = before + (int64_t)blockIdx.x * nwords;
+    unsigned carry = 0;
+    for (int64_t i0 = 0; i0 < nwords; i0 += blockDim.x) {
+        const int64_t i = i0 + threadIdx.x;
+        const unsigned own = i < nwords ? __popc(m[i]) : 0;
+        unsigned inc = own;
+        for (int q = 1; q < 32; q <<= 1) {
+            const unsigned y = __shfl_up_sync(kFull, inc, q);
+            if (lane >= q) inc += y;
+        }
+        if (lane == 31) s_w[wib] = inc;
+        __syncthreads();
+        unsigned mine = carry, all = 0;
+        for (int q = 0; q < 32; ++q) {
+            if (q < wib) mine += s_w[q];
+            all += s_w[q];
+        }
+        if (i < nwords) out[i] = mine + inc - own;
+        carry += all;
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) rowlen[list[p0 + blockIdx.x]] = carry;
+}
+// every entry to its target's place: the target to the output, its weight
+// into the place's fp64 sum (or maximum) acc, which holds the places of the
+// rows taken at once (row p at abase[p - p0])
+__global__ void k_long_place(const int32_t *list, int64_t p0, const int64_t *rowstart, const int32_t *tgt,
+                             const float *wt, int combine, const unsigned *bits, const unsigned *before,
+                             int64_t nwords, const int64_t *off, int32_t *idx, double *acc, const int64_t *abase) {
+    const int32_t r = list[p0 + blockIdx.x];
+    const int64_t o = rowstart[r], d = rowstart[r + 1] - o, out = off[r];
+    const unsigned *m = bits + (int64_t)blockIdx.x * nwords, *f = before + (int64_t)blockIdx.x * nwords;
+    double *s = acc + abase[blockIdx.x];
+    for (int64_t e = (int64_t)blockIdx.y * blockDim.x + threadIdx.x; e < d; e += (int64_t)gridDim.y * blockDim.x) {
+        const int32_t k = tgt[o + e];
+        const int64_t at = f[k >> 5] + __popc(m[k >> 5] & ((1u << (k & 31)) - 1u));
+        idx[out + at] = k;
+        const double x = wt ? (double)wt[o + e] + 0.0 : 1.0;  // (no -0.0)
+        if (combine)  // weights are not negative: their bits are ordered as they are
+            atomicMax(reinterpret_cast<unsigned long long *>(&s[at]), (unsigned long long)__double_as_longlong(x));
+        else
+            atomicAdd(&s[at], x);
+    }
+}
+__global__ void k_long_weights(const int32_t *list, int64_t p0, const int64_t *off, const double *acc,
+                               const int64_t *abase, float *w) {
+    const int32_t r = list[p0 + blockIdx.x];
+    const int64_t o = off[r], d = off[r + 1] - o;
+    const double *s = acc + abase[blockIdx.x];
+    for (int64_t e = (int64_t)blockIdx.y * blockDim.x + threadIdx.x; e < d; e += (int64_t)gridDim.y * blockDim.x)
+        w[o + e] = (float)s[e];
+}
+
+__global__ void k_long_lens(const int32_t *list, int64_t p0, int64_t c, const int64_t *rowlen, int64_t *lens) {
+    GRID_STRIDE(k, c) lens[k] = rowlen[list[p0 + k]];
+}
+
+// the merged front of every row of the list to its place in the output: T
+// lanes a row
+template <int T>
+__global__ void __launch_bounds__(256) k_row_copy(const int32_t *__restrict__ list, int64_t count,
+                                                  const int64_t *__restrict__ rowstart,
+                                                  const int64_t *__restrict__ off, const int32_t *tgt,
+                                                  const float *mw, int32_t *idx, float *w) {
+    const int tl = threadIdx.x & (T - 1);
+    const int64_t tiles = (int64_t)gridDim.x * (blockDim.x / T);
+    for (int64_t t = (int64_t)blockIdx.x * (blockDim.x / T) + threadIdx.x / T; t < count; t += tiles) {
+        const int32_t r = list[t];
+        const int64_t s = rowstart[r], o = off[r], d = off[r + 1] - o;
+        for (int64_t e = tl; e < d; e += T) {
+            idx[o + e] = tgt[s + e];
+            w[o + e] = mw[s + e];
+        }
     }
 }
 
@@ -152,8 +387,8 @@ leiden_status csr_from_edges(int64_t n, int64_t m, const int32_t *src, const int
     const cudaMemcpyKind out_kind = where == LEIDEN_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
     const int32_t *dsrc = src, *ddst = dst;
     const float *dw = w;
-    unsigned long long *cnt = nullptr, *rowlen = nullptr;
-    int64_t *rowstart = nullptr, *doff = nullptr;
+    unsigned long long *cnt = nullptr;
+    int64_t *rowstart = nullptr, *doff = nullptr, *rowlen = nullptr;
     int *err = nullptr;
     void *scan_tmp = nullptr;
     if (!get((void **)&cnt, 8 * (size_t)(n + 1)) || !get((void **)&rowstart, 8 * (size_t)(n + 1)) ||
@@ -172,7 +407,9 @@ leiden_status csr_from_edges(int64_t n, int64_t m, const int32_t *src, const int
         ddst = b;
         dw = c;
     }
-    // ---- entries per row, row starts
+    // ---- entries per row, row starts, the longest row
+    unsigned long long *longest = nullptr;
+    if (!get((void **)&longest, 8)) return fail(LEIDEN_ERR_OOM, "leiden_csr_from_edges: device allocation failed");
     IK(cudaMemsetAsync(err, 0, sizeof(int), s));
     IK(cudaMemsetAsync(cnt, 0, 8 * (size_t)(n + 1), s));
     IK(cudaMemsetAsync(rowlen, 0, 8 * (size_t)(n + 1), s));
@@ -181,104 +418,126 @@ leiden_status csr_from_edges(int64_t n, int64_t m, const int32_t *src, const int
         IK(cudaGetLastError());
     }
     IK(launch_exclusive_scan(reinterpret_cast<const int64_t *>(cnt), rowstart, n, scan_tmp, s));
-    std::vector<int64_t> hstart((size_t)n + 1, 0);
+    IK(launch_max_i64(reinterpret_cast<const int64_t *>(cnt), n, longest, s));
     int herr = 0;
-    IK(cudaMemcpyAsync(hstart.data(), rowstart, 8 * (size_t)(n + 1), cudaMemcpyDeviceToHost, s));
+    int64_t M = 0;  // entries before merging
+    unsigned long long hlongest = 0;
     IK(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, s));
+    IK(cudaMemcpyAsync(&M, rowstart + n, 8, cudaMemcpyDeviceToHost, s));
+    IK(cudaMemcpyAsync(&hlongest, longest, 8, cudaMemcpyDeviceToHost, s));
     IK(cudaStreamSynchronize(s));
     if (herr) return fail(LEIDEN_ERR_INVALID, "leiden_csr_from_edges: endpoint outside [0, n) or bad weight");
-    const int64_t M = hstart[(size_t)n];  // entries before merging
-    // ---- rows into chunks of at most kChunkEntries entries
-    std::vector<int64_t> cut = {0};
-    for (int64_t r = 0; r < n;) {
-        int64_t r1 = r + 1;
-        if (hstart[(size_t)r1] - hstart[(size_t)r] > kChunkEntries)
-            return fail(LEIDEN_ERR_INVALID, "leiden_csr_from_edges: a row of more than 2^30 entries before merging");
-        // the furthest row end within the chunk budget (binary search)
-        int64_t lo = r1, hi = n;
-        while (lo < hi) {
-            const int64_t mid = (lo + hi + 1) / 2;
-            if (hstart[(size_t)mid] - hstart[(size_t)r] <= kChunkEntries) lo = mid;
-            else hi = mid - 1;
-        }
-        r = lo;
-        cut.push_back(r);
-    }
-    int64_t chunk_max = 0;
-    for (size_t k = 0; k + 1 < cut.size(); ++k)
-        chunk_max = std::max(chunk_max, hstart[(size_t)cut[k + 1]] - hstart[(size_t)cut[k]]);
-    // ---- scatter into row segments
-    unsigned long long *key = nullptr, *key2 = nullptr;
-    float *wt = nullptr, *wt2 = nullptr, *stw = nullptr;
-    int32_t *digit = nullptr, *perm = nullptr, *first = nullptr, *sti = nullptr;
-    int64_t *pos = nullptr, *key_off = nullptr;
-    void *part_tmp = nullptr, *cscan_tmp = nullptr;
+    if ((int64_t)hlongest > kMaxRow)
+        return fail(LEIDEN_ERR_INVALID, "leiden_csr_from_edges: a row of more than 2^30 entries before merging");
+    int64_t nnz = 0;
+    int32_t *tgt = nullptr, *bin = nullptr, *list = nullptr, *sti = indices;
+    float *wt = nullptr, *mw = nullptr, *stw = weights;
+    unsigned *bits = nullptr, *before = nullptr;
+    int64_t *bin_off = nullptr, *abase = nullptr;
+    void *part_tmp = nullptr;
+    int64_t hb[kRowBins + 2] = {0};
+    const int64_t nwords = (n + 31) / 32;
+    int64_t nlong = 0, at_once = 0;
+    const int32_t *llong = nullptr;
     if (M > 0) {
-        if (!get((void **)&key, 8 * (size_t)M) || (dw && !get((void **)&wt, 4 * (size_t)M)) ||
-            !get((void **)&key2, 8 * (size_t)chunk_max) || (dw && !get((void **)&wt2, 4 * (size_t)chunk_max)) ||
-            !get((void **)&digit, 4 * (size_t)chunk_max) || !get((void **)&perm, 4 * (size_t)chunk_max) ||
-            !get((void **)&first, 4 * (size_t)chunk_max) || !get((void **)&pos, 8 * (size_t)(chunk_max + 1)) ||
-            !get((void **)&key_off, 8 * ((1 << kDigitBits) + 2)) ||
-            !get(&part_tmp, partition_tmp_bytes(chunk_max, 1 << kDigitBits)) ||
-            !get(&cscan_tmp, scan_tmp_bytes(chunk_max + 1)))
-            return fail(LEIDEN_ERR_OOM, "leiden_csr_from_edges: device allocation failed");
-        if (where == LEIDEN_HOST &&
-            (!get((void **)&sti, 4 * (size_t)chunk_max) || !get((void **)&stw, 4 * (size_t)chunk_max)))
+        // ---- scatter into row segments; rows by length
+        if (!get((void **)&tgt, 4 * (size_t)M) || !get((void **)&mw, 4 * (size_t)M) ||
+            (dw && !get((void **)&wt, 4 * (size_t)M)) || !get((void **)&bin, 4 * (size_t)n) ||
+            !get((void **)&list, 4 * (size_t)n) || !get((void **)&bin_off, 8 * (kRowBins + 2)) ||
+            !get(&part_tmp, partition_tmp_bytes(n, kRowBins + 1)))
             return fail(LEIDEN_ERR_OOM, "leiden_csr_from_edges: device allocation failed");
         IK(cudaMemsetAsync(cnt, 0, 8 * (size_t)(n + 1), s));  // the cursors
-        k_scatter_rows<<<grid_for(m, 256), 256, 0, s>>>(m, dsrc, ddst, dw, drop_self, rowstart, cnt, key, wt);
+        k_scatter_rows<<<grid_for(m, 256), 256, 0, s>>>(m, dsrc, ddst, dw, drop_self, rowstart, cnt, tgt, wt);
         IK(cudaGetLastError());
-    }
-    int tbits = 1;  // bits of a target
-    while ((1LL << tbits) < n) ++tbits;
-    // ---- per chunk: sort by (row, target), merge runs into the output
-    int64_t nnz = 0;
-    for (size_t k = 0; k + 1 < cut.size(); ++k) {
-        const int64_t r0 = cut[k], r1 = cut[k + 1];
-        const int64_t a = hstart[(size_t)r0], Mc = hstart[(size_t)r1] - a;
-        if (Mc == 0) continue;
-        int rbits = 0;  // bits of a row relative to r0
-        while ((1LL << rbits) < r1 - r0) ++rbits;
-        unsigned long long *ck = key + a, *ck2 = key2;
-        float *cw = wt ? wt + a : nullptr, *cw2 = wt2;
-        std::vector<int> shifts;
-        for (int sh = 0; sh < tbits; sh += kDigitBits) shifts.push_back(sh);
-        for (int sh = 0; sh < rbits; sh += kDigitBits) shifts.push_back(32 + sh);
-        for (int sh : shifts) {
-            k_digit<<<grid_for(Mc, 256), 256, 0, s>>>(ck, Mc, (unsigned long long)r0, sh, digit);
-            IK(cudaGetLastError());
-            IK(launch_partition(digit, Mc, 1 << kDigitBits, key_off, perm, part_tmp, s));
-            k_gather_kw<<<grid_for(Mc, 256), 256, 0, s>>>(ck, cw, perm, Mc, ck2, cw2);
-            IK(cudaGetLastError());
-            std::swap(ck, ck2);
-            std::swap(cw, cw2);
-        }
-        k_run_starts<<<grid_for(Mc, 256), 256, 0, s>>>(ck, Mc, first);
+        k_row_bins<<<grid_for(n, 256), 256, 0, s>>>(rowstart, n, bin);
         IK(cudaGetLastError());
-        IK(launch_exclusive_scan_i32(first, pos, Mc, cscan_tmp, s));
-        int64_t runs = 0;
-        IK(cudaMemcpyAsync(&runs, pos + Mc, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+        IK(launch_partition(bin, n, kRowBins + 1, bin_off, list, part_tmp, s));
+        IK(cudaMemcpyAsync(hb, bin_off, 8 * (kRowBins + 2), cudaMemcpyDeviceToHost, s));
         IK(cudaStreamSynchronize(s));
-        const bool fits = nnz + runs <= cap && (runs == 0 || (indices && weights));
-        if (where == LEIDEN_DEVICE || !fits) {
-            k_merge_runs<<<grid_for(Mc, 256), 256, 0, s>>>(ck, cw, first, pos, Mc, combine, nnz, fits ? cap : 0,
-                                                           indices, weights, rowlen);
-            IK(cudaGetLastError());
-        } else {  // staged on the device, then to the host buffers
-            k_merge_runs<<<grid_for(Mc, 256), 256, 0, s>>>(ck, cw, first, pos, Mc, combine, 0, runs, sti, stw,
-                                                           rowlen);
-            IK(cudaGetLastError());
-            IK(cudaMemcpyAsync(indices + nnz, sti, 4 * (size_t)runs, out_kind, s));
-            IK(cudaMemcpyAsync(weights + nnz, stw, 4 * (size_t)runs, out_kind, s));
-            IK(cudaStreamSynchronize(s));
+        // ---- every row sorted and merged at the front of its segment
+        auto rows = [&](int b, const int32_t *&l) {
+            l = list + hb[b];
+            return hb[b + 1] - hb[b];
+        };
+        const int32_t *l = nullptr;
+        if (const int64_t c = rows(1, l))
+            k_row_tile<8><<<grid_for(c, 32), 256, 0, s>>>(l, c, rowstart, tgt, wt, mw, combine, rowlen);
+        if (const int64_t c = rows(2, l))
+            k_row_tile<32><<<grid_for(c, 8), 256, 0, s>>>(l, c, rowstart, tgt, wt, mw, combine, rowlen);
+        if (const int64_t c = rows(3, l))
+            k_row_warp<<<grid_for(c, 8), 256, 0, s>>>(l, c, rowstart, tgt, wt, mw, combine, rowlen);
+        IK(cudaGetLastError());
+        IK(cudaFuncSetAttribute(k_row_block, cudaFuncAttributeMaxDynamicSharedMemorySize, kRowSmem * 12));
+        if (const int64_t c = rows(4, l))
+            k_row_block<<<grid_for(c, 1), 256, 2048 * 12, s>>>(l, c, rowstart, tgt, wt, mw, combine, rowlen, 2048);
+        if (const int64_t c = rows(5, l)) {
+            int cap = 4096;
+            while (cap < (int64_t)hlongest && cap < kRowSmem) cap <<= 1;
+            k_row_block<<<grid_for(c, 1), 512, (size_t)cap * 12, s>>>(l, c, rowstart, tgt, wt, mw, combine, rowlen,
+                                                                      cap);
         }
-        nnz += runs;
+        IK(cudaGetLastError());
+        // the long rows' merged lengths, from their bitmaps (kept for the
+        // output when they all fit at once)
+        nlong = rows(6, llong);
+        if (nlong > 0) {
+            at_once = std::max<int64_t>(1, std::min<int64_t>(nlong, kBitmapBytes / (8 * nwords)));
+            if (!get((void **)&bits, 8 * (size_t)(at_once * nwords)) || !get((void **)&abase, 8 * (size_t)(at_once + 1)))
+                return fail(LEIDEN_ERR_OOM, "leiden_csr_from_edges: device allocation failed");
+            before = bits + at_once * nwords;
+        }
     }
+    auto map_long = [&](int64_t p0, int64_t c) -> cudaError_t {
+        cudaError_t x = cudaMemsetAsync(bits, 0, 4 * (size_t)(c * nwords), s);
+        if (x != cudaSuccess) return x;
+        k_long_set<<<dim3((unsigned)c, kBigSplit), 256, 0, s>>>(llong, p0, rowstart, tgt, bits, nwords);
+        k_long_count<<<(unsigned)c, 1024, 0, s>>>(llong, p0, bits, before, nwords, rowlen);
+        return cudaGetLastError();
+    };
+    for (int64_t p0 = 0; p0 < nlong; p0 += at_once) IK(map_long(p0, std::min<int64_t>(at_once, nlong - p0)));
+    // ---- offsets: scan of the merged row lengths
+    IK(launch_exclusive_scan(rowlen, doff, n, scan_tmp, s));
+    IK(cudaMemcpyAsync(&nnz, doff + n, 8, cudaMemcpyDeviceToHost, s));
+    IK(cudaStreamSynchronize(s));
     *nnz_io = nnz;
     if (nnz > cap || (nnz > 0 && (!indices || !weights)))
         return fail(LEIDEN_ERR_INVALID, "leiden_csr_from_edges: output capacity below the entry count");
-    // ---- offsets: scan of the merged row lengths
-    IK(launch_exclusive_scan(reinterpret_cast<const int64_t *>(rowlen), doff, n, scan_tmp, s));
+    if (nnz > 0) {
+        if (where == LEIDEN_HOST && (!get((void **)&sti, 4 * (size_t)nnz) || !get((void **)&stw, 4 * (size_t)nnz)))
+            return fail(LEIDEN_ERR_OOM, "leiden_csr_from_edges: device allocation failed");
+        const int64_t c1 = hb[2] - hb[1], c2 = hb[6] - hb[2];
+        if (c1 > 0)
+            k_row_copy<8><<<grid_for(c1, 32), 256, 0, s>>>(list + hb[1], c1, rowstart, doff, tgt, mw, sti, stw);
+        if (c2 > 0)
+            k_row_copy<32><<<grid_for(c2, 8), 256, 0, s>>>(list + hb[2], c2, rowstart, doff, tgt, mw, sti, stw);
+        IK(cudaGetLastError());
+        for (int64_t p0 = 0; p0 < nlong; p0 += at_once) {
+            const int64_t c = std::min<int64_t>(at_once, nlong - p0);
+            if (nlong > at_once) IK(map_long(p0, c));
+            // where each row's sums start
+            int64_t *lens = reinterpret_cast<int64_t *>(cnt), sums = 0;  // (the cursors' space)
+            k_long_lens<<<grid_for(c, 256), 256, 0, s>>>(llong, p0, c, rowlen, lens);
+            IK(cudaGetLastError());
+            IK(launch_exclusive_scan(lens, abase, c, scan_tmp, s));
+            IK(cudaMemcpyAsync(&sums, abase + c, 8, cudaMemcpyDeviceToHost, s));
+            IK(cudaStreamSynchronize(s));
+            double *acc = nullptr;
+            if (cudaMallocAsync((void **)&acc, 8 * (size_t)(sums > 0 ? sums : 1), s) != cudaSuccess)
+                return fail(LEIDEN_ERR_OOM, "leiden_csr_from_edges: device allocation failed");
+            cudaMemsetAsync(acc, 0, 8 * (size_t)sums, s);
+            const dim3 grid((unsigned)c, kBigSplit);
+            k_long_place<<<grid, 256, 0, s>>>(llong, p0, rowstart, tgt, wt, combine, bits, before, nwords, doff, sti,
+                                              acc, abase);
+            k_long_weights<<<grid, 256, 0, s>>>(llong, p0, doff, acc, abase, stw);
+            e = cudaGetLastError();
+            cudaFreeAsync(acc, s);
+            IK(e);
+        }
+        if (where == LEIDEN_HOST) {
+            IK(cudaMemcpyAsync(indices, sti, 4 * (size_t)nnz, out_kind, s));
+            IK(cudaMemcpyAsync(weights, stw, 4 * (size_t)nnz, out_kind, s));
+        }
+    }
     IK(cudaMemcpyAsync(offsets, doff, 8 * (size_t)(n + 1), out_kind, s));
     IK(cudaStreamSynchronize(s));
 #undef IK
