@@ -437,12 +437,13 @@ leiden_status Handle::Impl::pass(Run &r, int32_t lp, bool &stop) {
             CK(cudaMemsetAsync(q.bar, 0, 2 * sizeof(unsigned), s));  // barrier state starts clean
             if (det) CK(cudaMemcpyAsync(q.Kagg, q.Sig, accsz * n, cudaMemcpyDeviceToDevice, s));
             sc.prof = prof_begin(refine ? 8 : 0);
-            // steps without an eligible vertex are skipped where there are
-            // many steps (heavy-tailed schedules): in the refinement, and in
-            // the local-moving of a union of graphs, whose converged graphs
-            // leave whole steps idle (for one graph the marks of flagged
-            // neighbours cost about what they save)
-            sc.act = (nsteps > 64 && (refine || batch)) ? q.act : nullptr;
+            // steps without an eligible vertex are skipped in the refinement,
+            // and in the local-moving of a union of graphs with many steps
+            // (heavy-tailed schedules), whose converged graphs leave whole
+            // steps idle (for one graph the marks of flagged neighbours cost
+            // about what they save)
+            sc.act = (refine || (nsteps > 64 && batch)) ? q.act : nullptr;
+            if (sc.act) CK(cudaMemsetAsync(q.act, 0, sizeof(int32_t) * nsteps, s));
             const bool stall = (prm.flags & LEIDEN_FLAG_TEST_STALL_BARRIER) != 0;
             sc.stall_block = (stall && grid > 1) ? 1 : -1;
             sc.spin_limit = stall ? (1ULL << 14) : kSpinLimitDefault;

@@ -93,7 +93,8 @@ template <class P, class W> struct SV {
     int32_t stall_block;            // testing aid: this block never arrives at a barrier
     unsigned long long spin_limit;  // barrier polls before giving up
     // persistent sweep: act[k] == it + 1 marks step k as holding an eligible
-    // vertex in sweep it (steps without one are skipped); null elsewhere
+    // vertex in sweep it (steps without one are skipped; the refinement from
+    // its second sweep on, the local-moving of batches); null elsewhere
     int32_t *act;
     // randomized refinement (asynchronous mode): draws from SplitMix64 with
     // state rseed + 0xD1B54A32D192ED03 * (sweep + 1); sweep: the sweep of a
@@ -145,6 +146,9 @@ template <class P> struct Sums {
     // Sigma as the step reads it and as its moves leave it: two copies in the
     // persistent deterministic sweep (see catch_up), else the same array
     typename P::tot *sr, *sw;
+    // refinement: set (in shared memory) when a vertex of the step may be
+    // eligible again in the next sweep (null in per-step launches)
+    int *keep = nullptr;
 };
 
 template <class P, class W> SV<P, W> view(const SweepCtx &c) {
@@ -295,6 +299,7 @@ __device__ __forceinline__ bool decide_sd(const SV<P, W> &a, int32_t v, int32_t 
         }
         g = key - ks;
     }
+    if (REFINE && sm.keep && (!mv || cur_step >= a.cap_step)) *sm.keep = 1;
     if constexpr (P::det) {
         a.prop[v] = mv ? cand : -1;
         if (a.old && cur_step < a.cap_step) {
@@ -546,6 +551,7 @@ __device__ __forceinline__ void run_tile(const SV<P, W> &a, const int32_t *__res
         const int32_t gv = graph_of<B>(a, v);
         const A Kv = k_of(a, v, t);
         const RowOf<W> row = row_of(a, v, t);
+        const int32_t bv = REFINE ? a.CB[v] : 0;
         int32_t d = 0;
         int elig = 0;
         if (tl == 0) elig = take_vertex<P, W, REFINE, B>(a, v, d, gv) ? 1 : 0;
@@ -558,15 +564,14 @@ __device__ __forceinline__ void run_tile(const SV<P, W> &a, const int32_t *__res
         }
         const int64_t e0 = row.e0;
         const int32_t dv = row.dv;
-        const int32_t bv = REFINE ? a.CB[v] : 0;
+        const typename P::tot sd = ldm(&sm.sr[d]);
         int32_t j = -1, c = -1;
         S wv = 0;
         if (tl < dv) {
             j = row.idx[e0 + tl];
             wv = wconv<S>(row.w[e0 + tl]);
-            bool ok = (j != v);
-            if (REFINE && ok) ok = (__ldg(&a.CB[j]) == bv);
-            if (ok) c = ldm(&a.C[j]);
+            c = ldm(&a.C[j]);  // beside its bound
+            if (j == v || (REFINE && __ldg(&a.CB[j]) != bv)) c = -1;
         }
         // merge equal communities into their first lane's sum
         const unsigned peers = __match_any_sync(tmask, c);
@@ -599,7 +604,7 @@ __device__ __forceinline__ void run_tile(const SV<P, W> &a, const int32_t *__res
             }
         }
         int mv = 0;
-        if (tl == 0) mv = decide<P, W, REFINE, B>(a, v, d, Kv, key, cand, kvd, sm, cur_step, gv, ks) ? 1 : 0;
+        if (tl == 0) mv = decide_sd<P, W, REFINE, B>(a, v, d, Kv, key, cand, kvd, sd, sm, cur_step, gv, ks) ? 1 : 0;
         if (a.prof) {
             const unsigned lb = __ballot_sync(tmask, lead) & tmask;
             if (tl == 0) {
@@ -648,9 +653,9 @@ __device__ __forceinline__ void table_insert(const SV<P, W> &a, const RowOf<W> &
         }
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            bool ok = j[q] >= 0 && j[q] != v;
-            if (REFINE && ok) ok = __ldg(&a.CB[j[q]]) == bv;
-            c[q] = ok ? ldm(&a.C[j[q]]) : -1;
+            const bool ok = j[q] >= 0 && j[q] != v;
+            c[q] = ok ? ldm(&a.C[j[q]]) : -1;  // beside its bound
+            if (REFINE && ok && __ldg(&a.CB[j[q]]) != bv) c[q] = -1;
         }
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -731,6 +736,7 @@ __device__ __forceinline__ void run_warp(const SV<P, W> &a, const int32_t *__res
         const A Kv = k_of(a, v, t);
         const RowOf<W> row = row_of(a, v, t);
         const int32_t dv = row.dv;
+        const int32_t bv = REFINE ? a.CB[v] : 0;
         int32_t d = 0;
         int elig = 0;
         if (lane == 0) elig = take_vertex<P, W, REFINE, B>(a, v, d, gv) ? 1 : 0;
@@ -741,7 +747,6 @@ __device__ __forceinline__ void run_warp(const SV<P, W> &a, const int32_t *__res
             if (lane == 0) pc.v[1]++;
             continue;
         }
-        const int32_t bv = REFINE ? a.CB[v] : 0;
         int bits = ceil_log2(2 * (int64_t)dv);
         if (bits < 6) bits = 6;
         const int S = 1 << bits;
@@ -750,6 +755,7 @@ __device__ __forceinline__ void run_warp(const SV<P, W> &a, const int32_t *__res
             vals[s] = 0;
         }
         __syncwarp();
+        const typename P::tot sd = ldm(&sm.sr[d]);
         typename P::sum kvd = 0;
         table_insert<P, W, REFINE>(a, row, v, d, bv, lane, 32, keys, vals, bits, kvd);
         __syncwarp();
@@ -761,7 +767,7 @@ __device__ __forceinline__ void run_warp(const SV<P, W> &a, const int32_t *__res
         kvd = full_sum(kvd);
         int mv = 0;
         if (lane == 0) {
-            mv = decide<P, W, REFINE, B>(a, v, d, Kv, key, cand, kvd, sm, cur_step, gv, ks) ? 1 : 0;
+            mv = decide_sd<P, W, REFINE, B>(a, v, d, Kv, key, cand, kvd, sd, sm, cur_step, gv, ks) ? 1 : 0;
             pc.v[0]++;
             pc.v[2] += dv;
             if (kvd != 0) pc.v[3]++;
@@ -814,6 +820,7 @@ __device__ __forceinline__ void run_block(const SV<P, W> &a, const int32_t *__re
         const A Kv = k_of(a, v, t);
         const RowOf<W> row = row_of(a, v, t);
         const int32_t dv = row.dv;
+        const int32_t bv = REFINE ? a.CB[v] : 0;
         int bits = ceil_log2(2 * (int64_t)dv);
         if (bits < 6) bits = 6;
         const bool fits = bits <= max_bits;
@@ -840,7 +847,7 @@ __device__ __forceinline__ void run_block(const SV<P, W> &a, const int32_t *__re
             group_sync<GS>();
             continue;
         }
-        const int32_t bv = REFINE ? a.CB[v] : 0;
+        const typename P::tot sd = ldm(&sm.sr[d]);
         S kvd = 0;
         table_insert<P, W, REFINE>(a, row, v, d, bv, tid, GS, keys, vals, bits, kvd);
         group_sync<GS>();
@@ -862,7 +869,8 @@ __device__ __forceinline__ void run_block(const SV<P, W> &a, const int32_t *__re
             kvd = full_sum(lane < nw ? s_kvd[lane] : (S)0);
             warp_best(key, cand);
             if (lane == 0) {
-                s_mv = decide<P, W, REFINE, B>(a, v, d, Kv, key, cand, kvd, sm, cur_step, gv, ks) ? 1 : 0;
+                s_mv =
+                    decide_sd<P, W, REFINE, B>(a, v, d, Kv, key, cand, kvd, sd, sm, cur_step, gv, ks) ? 1 : 0;
                 pc.v[0]++;
                 pc.v[2] += dv;
                 if (kvd != 0) pc.v[3]++;
@@ -1641,6 +1649,8 @@ __global__ void __launch_bounds__(kCoopThreads, 2) k_sweep_coop(SV<P, W> a, cons
     if ((int32_t)blockIdx.x == a.stall_block) return;
     __shared__ int64_t s_ko[2][kNumBins + 2];
     __shared__ int32_t s_next;
+    __shared__ int s_keep;
+    if (threadIdx.x == 0) s_keep = 0;
     GridBar bar{a.bar, a.err, a.spin_limit};
     Deal deal;
     ProfCounts pc;
@@ -1654,18 +1664,24 @@ __global__ void __launch_bounds__(kCoopThreads, 2) k_sweep_coop(SV<P, W> a, cons
         sm.sr = a.Sig;
         sm.sw = a.Sig2;
         int64_t late0 = 0, late1 = 0;  // the step whose moves sw lacks (catch_up)
-        if (a.act) {
-            // steps holding an eligible vertex at the start of the sweep
-            // (unprocessed, or isolated in the refinement); moves mark the
-            // steps of the neighbours they flag as the sweep goes on, and
-            // nothing makes a vertex isolated during the refinement
+        if (REFINE && a.act) sm.keep = &s_keep;
+        // Steps without an eligible vertex are passed over where a.act says
+        // so (act[k] == the sweep's stamp: step k holds one). In the
+        // refinement a vertex stays eligible only by staying isolated, so a
+        // step's own evaluation in one sweep marks it for the next (all steps
+        // run in the first); without the marks the sweeps after the first, in
+        // which few vertices or none are left, took every step's barrier.
+        const bool pick = a.act && (!REFINE || it > 0);
+        if (!REFINE && a.act) {
+            // local-moving of a batch: steps holding an unprocessed vertex at
+            // the start of the sweep; moves mark the steps of the neighbours
+            // they flag as the sweep goes on
             const int64_t nl = __ldcg(&a.key_off[(int64_t)a.nsteps * kNumBins]);
             for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < nl;
                  t += (int64_t)gridDim.x * blockDim.x) {
                 const int32_t v = list[t];
                 if (B && ldm(&a.gdone[graph_of<B>(a, v)])) continue;
-                const bool e = REFINE ? ldm(&a.size[ldm(&a.C[v])]) == 1 : ldm(&a.unproc[v]) != 0;
-                if (e) mark_step(a.act, a.step[v], sm.stamp);
+                if (ldm(&a.unproc[v]) != 0) mark_step(a.act, a.step[v], sm.stamp);
             }
             if (!(ok = bar.sync())) break;
         }
@@ -1677,13 +1693,13 @@ __global__ void __launch_bounds__(kCoopThreads, 2) k_sweep_coop(SV<P, W> a, cons
             if (lane <= kNumBins) return __ldg(&a.key_off[(int64_t)k * kNumBins + lane]);
             return (lane == kNumBins + 1 && a.hbase) ? __ldg(&a.hbase[k]) : 0;
         };
-        if (wib == 0 && !a.act && lane <= kNumBins + 1) s_ko[0][lane] = load_ko(0);
+        if (wib == 0 && !pick && lane <= kNumBins + 1) s_ko[0][lane] = load_ko(0);
         __syncthreads();
         int buf = 0;
         for (int32_t k = 0; k < a.nsteps && ok; ++k, buf ^= 1) {
             int64_t *sko = s_ko[buf];
             int64_t ahead = 0;
-            if (a.act) {
+            if (pick) {
                 // the next step marked as holding an eligible vertex: the
                 // same in every block, since marks are only set before the
                 // barrier that ended the last step taken
@@ -1707,7 +1723,7 @@ __global__ void __launch_bounds__(kCoopThreads, 2) k_sweep_coop(SV<P, W> a, cons
                 ahead = load_ko(k + 1);
             }
             auto fetched = [&]() {
-                if (wib == 0 && !a.act && k + 1 < a.nsteps && lane <= kNumBins + 1) s_ko[buf ^ 1][lane] = ahead;
+                if (wib == 0 && !pick && k + 1 < a.nsteps && lane <= kNumBins + 1) s_ko[buf ^ 1][lane] = ahead;
             };
             const int64_t b0 = sko[0], b8 = sko[8];
             if (b0 == b8) {  // empty step: every block sees the same counts
@@ -1753,6 +1769,14 @@ __global__ void __launch_bounds__(kCoopThreads, 2) k_sweep_coop(SV<P, W> a, cons
                 if (!ok) break;
             }
             fetched();
+            if (REFINE && a.act) {
+                // one store a block marks the step for the next sweep
+                __syncthreads();
+                if (threadIdx.x == 0 && s_keep) {
+                    a.act[k] = sm.stamp + 1;
+                    s_keep = 0;
+                }
+            }
             if (!(ok = bar.sync())) break;
             // a layered step's moves are made; an apply phase commits the
             // proposals where neighbours may share a step
