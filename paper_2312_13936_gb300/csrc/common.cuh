@@ -317,6 +317,9 @@ __device__ __forceinline__ int32_t full_sum(int32_t v) { return __reduce_add_syn
 template <class A>
 __device__ __forceinline__ A peer_sum(unsigned peers, A v) {
     if (peers == kFull) return warp_sum(v);
+    // alone: no shuffle (lanes of different peers run one group after another,
+    // so 32 groups of one took 32 turns)
+    if ((peers & (peers - 1u)) == 0u) return v;
     A s = 0;
     for (unsigned m = peers; m; m &= m - 1) s += __shfl_sync(peers, v, __ffs(m) - 1);
     return s;

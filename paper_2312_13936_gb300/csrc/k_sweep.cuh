@@ -1321,6 +1321,21 @@ __device__ __forceinline__ bool run_hub_single(const SV<P, W> &a, int64_t j0, in
     const int64_t e0 = a.off[v];
     const int32_t dv = a.deg[v];
     const int32_t bv = REFINE ? __ldg(&a.CB[v]) : 0;
+    // the entry of chunk i in this lane: its vertex (-1: none) and community
+    // (-1: not a candidate)
+    auto entry = [&](uint32_t i, int32_t &u, int32_t &c) {
+        const int64_t x = (int64_t)i * 32 + lane;
+        u = x < dv ? a.idx[e0 + x] : -1;
+        c = u >= 0 ? ldm(&a.C[u]) : -1;
+        if (u == v || (REFINE && u >= 0 && __ldg(&a.CB[u]) != bv)) c = -1;
+    };
+    const uint32_t chunks = ((uint32_t)dv + 31) / 32, i0 = deal.first();
+    int32_t u0 = -1, c0 = -1;  // the warp's first chunk stays in registers; it loads beside the eligibility
+    S w0 = 0;
+    if (i0 < chunks) {
+        entry(i0, u0, c0);
+        if (u0 >= 0) w0 = wconv<S>(a.w[e0 + (int64_t)i0 * 32 + lane]);
+    }
     __syncthreads();
     const int32_t d = s_d;
     if (!s_e) {  // the same in every block
@@ -1330,23 +1345,14 @@ __device__ __forceinline__ bool run_hub_single(const SV<P, W> &a, int64_t j0, in
         }
         return true;
     }
-    // the entry of chunk i in this lane: its vertex (-1: none) and community
-    // (-1: not a candidate)
-    auto entry = [&](uint32_t i, int32_t &u, int32_t &c) {
-        const int64_t x = (int64_t)i * 32 + lane;
-        u = x < dv ? a.idx[e0 + x] : -1;
-        c = u >= 0 && u != v && (!REFINE || __ldg(&a.CB[u]) == bv) ? ldm(&a.C[u]) : -1;
-    };
-    const uint32_t chunks = ((uint32_t)dv + 31) / 32, i0 = deal.first();
-    int32_t u0 = -1, c0 = -1;  // the warp's first chunk stays in registers
     for (uint32_t i = i0; i < chunks; i += deal.nw) {
-        int32_t u, c;
-        entry(i, u, c);
-        if (i == i0) {
-            u0 = u;
-            c0 = c;
+        int32_t u = u0, c = c0;
+        S val = w0;
+        if (i != i0) {
+            entry(i, u, c);
+            val = u >= 0 ? wconv<S>(a.w[e0 + (int64_t)i * 32 + lane]) : (S)0;
         }
-        S val = c >= 0 ? wconv<S>(a.w[e0 + (int64_t)i * 32 + lane]) : (S)0;
+        if (c < 0) val = 0;
         const unsigned peers = __match_any_sync(kFull, c);
         val = peer_sum(peers, val);
         if (c >= 0 && lane == __ffs(peers) - 1) {
@@ -1469,55 +1475,66 @@ __device__ __forceinline__ void catch_up(const SV<P, W> &a, const int32_t *__res
     deal.pass(units);
 }
 
-// Local-moving proposals of one capped step (of any step in the per-step
-// launches of the deterministic mode): commit them. The movers' rows of a unit are flagged
-// as one flat range of entries by all lanes, four loads per lane in flight
-// (a lane walking its own mover's row waited for every load in turn: 16 us a
-// step on a 200,000-vertex block model with rows of 24 entries). Rows of
-// more than 1024 entries go one after another.
-// (grid_hub_flags: the neighbours of rows longer than kCtaMaxDeg are
-// flagged by hub_flags over the step's hub layout)
+// Commits the proposal of list position t (v = -1: none) and returns v's row
+// (empty when v stays).
+template <class P, class W, bool B>
+__device__ __forceinline__ RowOf<W> commit_move(const SV<P, W> &a, int32_t v, int64_t t, Sums<P> &sm) {
+    const int32_t c = v >= 0 ? ldm(&a.prop[v]) : -1;
+    if (c < 0) return {0, 0, nullptr, nullptr};
+    const int32_t d = ldm(&a.C[v]);
+    const auto Kv = (typename P::tot)k_of(a, v, t);
+    atomic_add_acc(&sm.sr[d], -Kv);
+    atomic_add_acc(&sm.sr[c], Kv);
+    if (P::det && sm.sw != sm.sr) {
+        atomic_add_acc(&sm.sw[d], -Kv);
+        atomic_add_acc(&sm.sw[c], Kv);
+    }
+    atomicSub(&a.size[d], 1);
+    atomicAdd(&a.size[c], 1);
+    a.C[v] = c;
+    if (P::det)
+        gacc_add(sm.dgain, B, graph_of<B>(a, v), load_gain128<typename P::key>(a.gain, v),
+                 reinterpret_cast<unsigned long long *>(sm.dq));
+    else
+        gacc_add(sm.gain, B, graph_of<B>(a, v),
+                 (typename P::acc)__ldcg(reinterpret_cast<const float *>(a.gain) + v), sm.dq);
+    return row_of(a, v, t);
+}
+
+// Proposals of one capped step (of any step in the per-step launches of the
+// deterministic mode): commit them and flag the movers' neighbours.
+// [lo, mid): rows of up to kFlat entries (longer ones among them go to a warp
+// each): the movers' rows of a unit are flagged as one flat range of entries
+// by all lanes, four loads per lane in flight (a lane walking its own mover's
+// row waited for every load in turn: 16 us a step on a 200,000-vertex block
+// model with rows of 24 entries). [mid, flags): a vertex a warp (32 rows of
+// thousands of entries in one warp's unit kept the grid waiting for 260 us a
+// step on R-MAT 1M). [flags, hi): the commit alone (their neighbours are
+// flagged by hub_flags over the step's hub layout).
 template <class P, class W, bool B>
 __device__ __forceinline__ void run_move_apply(const SV<P, W> &a, const int32_t *__restrict__ list, int64_t lo,
-                                               int64_t hi, Deal &deal, Sums<P> &sm, bool grid_hub_flags) {
+                                               int64_t mid, int64_t flags, int64_t hi, Deal &deal, Sums<P> &sm) {
     constexpr int32_t kFlat = 1024;
     const int lane = threadIdx.x & 31;
-    const int per = apply_unit((uint32_t)(hi - lo), deal.nw);
-    const uint32_t units = (uint32_t)((hi - lo + per - 1) / per);
+    const int32_t *is = a.loff ? a.lidx : a.idx;
+    // row entries [e0, e0 + dv) by the whole warp
+    auto flag_row = [&](int64_t e0, int32_t dv) {
+        for (int32_t x = 0; x < dv; x += 128) {
+            int32_t j[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) j[q] = x + 32 * q + lane < dv ? is[e0 + x + 32 * q + lane] : -1;
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (j[q] >= 0) flag_unproc(a, sm, j[q]);
+        }
+    };
+    const int per = apply_unit((uint32_t)(mid - lo), deal.nw);
+    const uint32_t units = (uint32_t)((mid - lo + per - 1) / per);
     for (uint32_t u = deal.first(); u < units; u += deal.nw) {
         const int64_t t = lo + (int64_t)u * per + lane;
-        int32_t v = -1, c = -1;
-        if (lane < per && t < hi) {
-            v = list[t];
-            c = ldm(&a.prop[v]);
-        }
-        if (!__any_sync(kFull, c >= 0)) continue;
-        int64_t e0 = 0;
-        int32_t dv = 0;
-        if (c >= 0) {
-            const int32_t d = ldm(&a.C[v]);
-            const auto Kv = (typename P::tot)k_of(a, v, t);
-            atomic_add_acc(&sm.sr[d], -Kv);
-            atomic_add_acc(&sm.sr[c], Kv);
-            if (P::det && sm.sw != sm.sr) {
-                atomic_add_acc(&sm.sw[d], -Kv);
-                atomic_add_acc(&sm.sw[c], Kv);
-            }
-            atomicSub(&a.size[d], 1);
-            atomicAdd(&a.size[c], 1);
-            a.C[v] = c;
-            if (P::det)
-                gacc_add(sm.dgain, B, graph_of<B>(a, v), load_gain128<typename P::key>(a.gain, v),
-                         reinterpret_cast<unsigned long long *>(sm.dq));
-            else
-                gacc_add(sm.gain, B, graph_of<B>(a, v),
-                         (typename P::acc)__ldcg(reinterpret_cast<const float *>(a.gain) + v), sm.dq);
-            const RowOf<W> row = row_of(a, v, t);
-            e0 = row.e0;
-            dv = row.dv;
-        }
-        const int32_t *is = a.loff ? a.lidx : a.idx;  // the same on every lane
-        const int32_t flat = dv <= kFlat && !(grid_hub_flags && dv > kCtaMaxDeg) ? dv : 0;
+        const RowOf<W> row = commit_move<P, W, B>(a, lane < per && t < mid ? list[t] : -1, t, sm);
+        if (!__any_sync(kFull, row.dv > 0)) continue;
+        const int32_t flat = row.dv <= kFlat ? row.dv : 0;
         int32_t incl = flat;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -1525,7 +1542,7 @@ __device__ __forceinline__ void run_move_apply(const SV<P, W> &a, const int32_t 
             if (lane >= o) incl += y;
         }
         const int32_t total = __shfl_sync(kFull, incl, 31);
-        const int64_t base = e0 - (incl - flat);  // entry x of the flat range is is[base + x] of its owner
+        const int64_t base = row.e0 - (incl - flat);  // entry x of the flat range is is[base + x] of its owner
         for (int32_t x0 = 0; x0 < total; x0 += 128) {
             int32_t j[4];
 #pragma unroll
@@ -1542,16 +1559,20 @@ __device__ __forceinline__ void run_move_apply(const SV<P, W> &a, const int32_t 
             for (int q = 0; q < 4; ++q)
                 if (j[q] >= 0) flag_unproc(a, sm, j[q]);
         }
-        unsigned longs = __ballot_sync(kFull, dv > kFlat && !(grid_hub_flags && dv > kCtaMaxDeg));
+        unsigned longs = __ballot_sync(kFull, row.dv > kFlat);
         while (longs) {
             const int src = __ffs(longs) - 1;
             longs &= longs - 1;
-            const int64_t es = __shfl_sync(kFull, e0, src);
-            const int32_t ds = __shfl_sync(kFull, dv, src);
-            for (int32_t e = lane; e < ds; e += 32) flag_unproc(a, sm, is[es + e]);
+            flag_row(__shfl_sync(kFull, row.e0, src), __shfl_sync(kFull, row.dv, src));
         }
     }
     deal.pass(units);
+    for (int64_t t = mid + deal.first(); t < hi; t += deal.nw) {
+        RowOf<W> row{0, 0, nullptr, nullptr};
+        if (lane == 0) row = commit_move<P, W, B>(a, list[t], t, sm);
+        if (t < flags) flag_row(__shfl_sync(kFull, row.e0, 0), __shfl_sync(kFull, row.dv, 0));
+    }
+    deal.pass((uint32_t)(hi - mid));
 }
 
 // Refinement: accept proposal v -> t unless t is a single-vertex community
@@ -1785,7 +1806,7 @@ __global__ void __launch_bounds__(kCoopThreads, 2) k_sweep_coop(SV<P, W> a, cons
                 if (REFINE) {
                     run_refine_apply<P, W, B>(a, list, b0, b8, k, deal, sm);
                 } else {
-                    run_move_apply<P, W, B>(a, list, b0, b8, deal, sm, hub_layout);
+                    run_move_apply<P, W, B>(a, list, b0, b5, hub_layout ? b7 : b8, b8, deal, sm);
                     if (hub_layout) hub_flags<P, W>(a, sm, __ldcg(&a.hinfo[0]), __ldcg(&a.hinfo[2]), true);
                 }
                 if (!(ok = bar.sync())) break;
@@ -1957,7 +1978,7 @@ template <class P, class W>
 __global__ void __launch_bounds__(256) k_move_apply(SV<P, W> a, const int32_t *__restrict__ list, int64_t count) {
     Sums<P> sm = scalar_sums(a);
     Deal deal;
-    run_move_apply<P, W, false>(a, list, 0, count, deal, sm, false);
+    run_move_apply<P, W, false>(a, list, 0, count, count, count, deal, sm);
     if (P::det) {
         const unsigned __int128 g = warp_sum_u128(sm.dgain.v);
         if ((threadIdx.x & 31) == 0 && g) atomic_add_u128(reinterpret_cast<unsigned long long *>(a.dq_acc), g);
