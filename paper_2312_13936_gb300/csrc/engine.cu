@@ -443,7 +443,7 @@ leiden_status Handle::Impl::pass(Run &r, int32_t lp, bool &stop) {
             // steps idle (for one graph the marks of flagged neighbours cost
             // about what they save)
             sc.act = (refine || (nsteps > 64 && batch)) ? q.act : nullptr;
-            if (sc.act) CK(cudaMemsetAsync(q.act, 0, sizeof(int32_t) * nsteps, s));
+            if (sc.act) CK(cudaMemsetAsync(q.act, 0, sizeof(int32_t) * 2 * kActSteps, s));
             const bool stall = (prm.flags & LEIDEN_FLAG_TEST_STALL_BARRIER) != 0;
             sc.stall_block = (stall && grid > 1) ? 1 : -1;
             sc.spin_limit = stall ? (1ULL << 14) : kSpinLimitDefault;

@@ -319,8 +319,8 @@ struct Handle::Impl {
         ST(alloc(&key_cnt, key_cap));
         ST(alloc(&key_off, key_cap + 1));
         ST(alloc(&sfcount, 4096 + 1));
-        ST(alloc(&act, 1024));
-        CK(cudaMemsetAsync(act, 0, sizeof(int32_t) * 1024, s));
+        ST(alloc(&act, 2 * kActSteps));
+        CK(cudaMemsetAsync(act, 0, sizeof(int32_t) * 2 * kActSteps, s));
         for (int64_t **a : {&vseg0, &vseg, &vseg2}) ST(alloc(a, ng + 1));
         for (int32_t **a : {&gstate, &gdone, &gli, &glj, &gpasses, &gfresh}) ST(alloc(a, ng));
         for (int64_t **a : {&gkeep, &gcomm}) ST(alloc(a, ng));

@@ -143,6 +143,7 @@ template <class P> struct Sums {
     typename P::tot *dq;
     unsigned long long *mv;
     int32_t stamp = 0;  // this sweep's mark in act (persistent sweep)
+    int32_t cur = -1;   // the step being run (persistent sweep)
     // Sigma as the step reads it and as its moves leave it: two copies in the
     // persistent deterministic sweep (see catch_up), else the same array
     typename P::tot *sr, *sw;
@@ -387,11 +388,16 @@ __device__ __forceinline__ void mark_step(int32_t *act, int32_t k, int32_t stamp
     if (__ldcg(&act[k]) != stamp) act[k] = stamp;
 }
 // A neighbour u of a mover becomes unprocessed (Algorithm 2 pruning); its
-// step is marked active for the rest of this sweep.
+// step, if it is still to come in this sweep, is marked active. (A step
+// before the one being run is not marked: a block that is still choosing its
+// next step would take it, and meet the others at no barrier.)
 template <class P, class W>
 __device__ __forceinline__ void flag_unproc(const SV<P, W> &a, const Sums<P> &sm, int32_t u) {
     a.unproc[u] = 1;
-    if (a.act) mark_step(a.act, a.step[u], sm.stamp);
+    if (a.act) {
+        const int32_t k = a.step[u];
+        if (k > sm.cur) mark_step(a.act, k, sm.stamp);
+    }
 }
 
 // Eligibility: local-moving takes unprocessed vertices and marks them
@@ -1693,6 +1699,10 @@ __global__ void __launch_bounds__(kCoopThreads, 2) k_sweep_coop(SV<P, W> a, cons
         // run in the first); without the marks the sweeps after the first, in
         // which few vertices or none are left, took every step's barrier.
         const bool pick = a.act && (!REFINE || it > 0);
+        // (two sets of marks by sweep in the refinement: a block may mark a
+        // step for the next sweep while another still looks for it in this one)
+        const int32_t *act_now = REFINE ? a.act + (it & 1) * kActSteps : a.act;
+        int32_t *act_next = REFINE ? a.act + ((it + 1) & 1) * kActSteps : nullptr;
         if (!REFINE && a.act) {
             // local-moving of a batch: steps holding an unprocessed vertex at
             // the start of the sweep; moves mark the steps of the neighbours
@@ -1728,7 +1738,7 @@ __global__ void __launch_bounds__(kCoopThreads, 2) k_sweep_coop(SV<P, W> a, cons
                     int32_t n = k;
                     for (; n < a.nsteps; n += 32) {
                         const unsigned m =
-                            __ballot_sync(kFull, n + lane < a.nsteps && __ldcg(&a.act[n + lane]) == sm.stamp);
+                            __ballot_sync(kFull, n + lane < a.nsteps && __ldcg(&act_now[n + lane]) == sm.stamp);
                         if (m) {
                             n += __ffs(m) - 1;
                             break;
@@ -1752,6 +1762,7 @@ __global__ void __launch_bounds__(kCoopThreads, 2) k_sweep_coop(SV<P, W> a, cons
                 __syncthreads();
                 continue;
             }
+            sm.cur = k;
             const int64_t b2 = sko[2], b3 = sko[3], b4 = sko[4], b5 = sko[5], b6 = sko[6], b7 = sko[7];
             if (b2 > b0) run_thread<P, W, REFINE, B>(a, list, b0, b2, k, deal, sm, pc);
             if (b3 > b2) run_tile<P, W, 16, REFINE, B>(a, list, b2, b3, k, deal, sm, pc);
@@ -1794,7 +1805,7 @@ __global__ void __launch_bounds__(kCoopThreads, 2) k_sweep_coop(SV<P, W> a, cons
                 // one store a block marks the step for the next sweep
                 __syncthreads();
                 if (threadIdx.x == 0 && s_keep) {
-                    a.act[k] = sm.stamp + 1;
+                    act_next[k] = sm.stamp + 1;
                     s_keep = 0;
                 }
             }

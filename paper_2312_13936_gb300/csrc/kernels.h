@@ -28,6 +28,7 @@ constexpr int kBlockSlots = 4096;
 constexpr int kBinHub = 6;
 constexpr int kCoopWarps = 16;       // warps of a persistent sweep's block
 constexpr int kGroup = 256;          // threads of a block-bin group
+constexpr int kActSteps = 1024;      // step marks of a sweep (two sets: act holds 2 kActSteps words)
 // The persistent sweep's own split of the rows beyond the block bin: up to
 // kCtaMaxDeg entries a block's shared memory holds the table (bin 6), and the
 // row needs no grid barrier; longer rows take the whole grid and a global
