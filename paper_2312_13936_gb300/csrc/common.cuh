@@ -255,13 +255,28 @@ template <class T> __device__ __forceinline__ T warp_sum(T v) {
 }
 
 // Row i of a CSR against labels C: K_i (sum of weights) and the weight to
-// vertices labelled ci, over entries [from, to) of the row with stride step.
-__device__ __forceinline__ void row_part(const int32_t *idx, const float *w, const int32_t *C, int64_t e0,
-                                         int64_t from, int64_t to, int step, int32_t ci, double &k, double &in) {
-    for (int64_t e = e0 + from; e < e0 + to; e += step) {
-        const double x = w ? (double)w[e] : 1.0;
-        k += x;
-        if (C[idx[e]] == ci) in += x;
+// vertices labelled ci, over entries [from, to) of the row with stride step,
+// four entries in flight.
+__device__ __forceinline__ void row_part(const int32_t *__restrict__ idx, const float *__restrict__ w,
+                                         const int32_t *__restrict__ C, int64_t e0, int64_t from, int64_t to, int step,
+                                         int32_t ci, double &k, double &in) {
+    for (int64_t e = e0 + from; e < e0 + to; e += 4 * (int64_t)step) {
+        int32_t j[4], c[4];
+        float x[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const bool has = e + q * step < e0 + to;
+            j[q] = has ? idx[e + q * step] : -1;
+            x[q] = !has ? 0.0f : w ? w[e + q * step] : 1.0f;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) c[q] = j[q] >= 0 ? C[j[q]] : -1;
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (j[q] >= 0) {
+                k += (double)x[q];
+                if (c[q] == ci) in += (double)x[q];
+            }
     }
 }
 // the same for every lane's row of a full warp: short rows by their lane,

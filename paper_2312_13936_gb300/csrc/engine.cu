@@ -1022,42 +1022,18 @@ leiden_status disconnected_device(int64_t n, const int64_t *off, const int32_t *
         set_last_error("scratch allocation failed");
         return LEIDEN_ERR_OOM;
     }
-    int32_t *parent = buf, *roots = buf + n;
-    int *changed = reinterpret_cast<int *>(flags);
-    unsigned long long *cnt = flags + 1;
     unsigned long long h[2] = {0, 0};
     leiden_status st = LEIDEN_OK;
-    // labels out of range are an error
     cudaError_t e = cudaMemsetAsync(flags, 0, sizeof(unsigned long long) * 2, s);
-    if (e == cudaSuccess) e = launch_cc_labels(n, memb, changed, s);
+    if (e == cudaSuccess)
+        e = launch_disconnected(n, off, idx, memb, buf, buf + n, reinterpret_cast<int *>(flags), flags + 1, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(h, flags, sizeof(h), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e == cudaSuccess && (h[0] & 0xffffffffULL)) {
         set_last_error("leiden_disconnected: membership labels must lie in [0, n)");
         st = LEIDEN_ERR_INVALID;
     }
-    if (e == cudaSuccess && st == LEIDEN_OK) {
-        e = launch_cc_init(n, parent, roots, s);
-        // a pass that finds an edge between two trees lowers some parent,
-        // and on the graphs here components settle within a few passes; 64
-        // is a safety bound, reported as a timeout
-        int pass = 0;
-        for (; e == cudaSuccess && pass < 64; ++pass) {
-            e = cudaMemsetAsync(flags, 0, sizeof(unsigned long long) * 2, s);
-            if (e == cudaSuccess) e = launch_cc_pass(n, off, idx, memb, parent, changed, s);
-            if (e == cudaSuccess) e = cudaMemcpyAsync(h, flags, sizeof(h), cudaMemcpyDeviceToHost, s);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-            if (e != cudaSuccess || !(h[0] & 0xffffffffULL)) break;
-        }
-        if (e == cudaSuccess && pass == 64) {
-            set_last_error("leiden_disconnected: components did not settle");
-            st = LEIDEN_ERR_TIMEOUT;
-        }
-        if (e == cudaSuccess && st == LEIDEN_OK) e = launch_cc_count(n, memb, parent, roots, cnt, s);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(h, flags, sizeof(h), cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-        if (e == cudaSuccess && st == LEIDEN_OK) *count = (int64_t)h[1];
-    }
+    if (e == cudaSuccess && st == LEIDEN_OK) *count = (int64_t)h[1];
     cudaFreeAsync(buf, s);
     cudaFreeAsync(flags, s);
     if (e != cudaSuccess) {
@@ -1085,7 +1061,7 @@ leiden_status modularity_device(int64_t n, const int64_t *off, const int32_t *id
         set_last_error("scratch allocation failed");
         return LEIDEN_ERR_OOM;
     }
-    e = cudaMallocAsync(&sums, sizeof(double) * 4, s);
+    e = cudaMallocAsync(&sums, sizeof(double) * 5, s);  // four sums and the word for long rows
     if (e != cudaSuccess) {
         cudaFreeAsync(sig, s);
         set_last_error("scratch allocation failed");
@@ -1093,8 +1069,8 @@ leiden_status modularity_device(int64_t n, const int64_t *off, const int32_t *id
     }
     double h[4] = {0, 0, 0, 0};
     cudaMemsetAsync(sig, 0, sizeof(double) * n, s);
-    cudaMemsetAsync(sums, 0, sizeof(double) * 4, s);
-    launch_modularity_parts(n, off, idx, w, memb, sig, sums, s);
+    cudaMemsetAsync(sums, 0, sizeof(double) * 5, s);
+    launch_modularity_parts(n, off, idx, w, memb, sig, sums, s, true, reinterpret_cast<unsigned *>(sums + 4));
     launch_sum_squares(sig, n, &sums[2], s);
     cudaMemcpyAsync(h, sums, sizeof(h), cudaMemcpyDeviceToHost, s);
     cudaFreeAsync(sig, s);

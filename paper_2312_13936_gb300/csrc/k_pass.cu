@@ -98,8 +98,9 @@ __global__ void k_canonical(const int32_t *C0, const int32_t *minv, const int64_
 // (LONG): by k_modularity_long below, so that no warp walks a hub alone.
 template <bool LONG>
 __global__ void k_modularity_parts(int64_t n, const int64_t *off, const int32_t *idx, const float *w,
-                                   const int32_t *C, double *sigtot, double *sums) {
+                                   const int32_t *C, double *sigtot, double *sums, unsigned *longs) {
     double intra = 0, tot = 0;
+    bool any_long = false;
     for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x; i0 < n; i0 += (int64_t)gridDim.x * blockDim.x) {
         const int64_t i = i0 + threadIdx.x;
         int32_t ci = -1;
@@ -113,6 +114,7 @@ __global__ void k_modularity_parts(int64_t n, const int64_t *off, const int32_t 
             if (ci >= 0) {
                 const int64_t e0 = off[i], d = off[i + 1] - e0;
                 if (!LONG || d <= kLongRow) row_part(idx, w, C, e0, 0, d, 1, ci, k, in);
+                else any_long = true;
             }
         }
         warp_add_by_key(sigtot, k != 0.0 ? ci : -1, k);
@@ -125,9 +127,10 @@ __global__ void k_modularity_parts(int64_t n, const int64_t *off, const int32_t 
         atomicAdd(&sums[0], intra);
         atomicAdd(&sums[1], tot);
     }
+    if (LONG && longs && __any_sync(kFull, any_long) && (threadIdx.x & 31) == 0) *longs = 1u;
 }
 
-// Rows longer than kLongRow, balanced over rows and entries together: row r
+// Rows longer than kLongRow (*longs, when given, says whether there are any), balanced over rows and entries together: row r
 // and its entry e take positions r + off[r] and r + 1 + e of one merged
 // sequence of n + m items; warp k of W takes positions [T k / W,
 // T (k+1) / W) (W at most T / 4096), finds the row at its first position by
@@ -138,7 +141,8 @@ __global__ void k_modularity_parts(int64_t n, const int64_t *off, const int32_t 
 constexpr int kModUnroll = 4;
 constexpr int64_t kModMinRange = 4096;
 __global__ void k_modularity_long(int64_t n, const int64_t *off, const int32_t *idx, const float *w,
-                                  const int32_t *C, double *sigtot, double *sums) {
+                                  const int32_t *C, double *sigtot, double *sums, const unsigned *longs) {
+    if (longs && *longs == 0u) return;
     const int lane = threadIdx.x & 31;
     const int64_t m = off[n], Tn = n + m;
     const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -310,12 +314,12 @@ cudaError_t launch_canonical(const int32_t *C0, const int32_t *minv, const int64
 }
 cudaError_t launch_modularity_parts(int64_t n, const int64_t *off, const int32_t *idx, const float *w,
                                     const int32_t *C, double *sigtot, double *sums, cudaStream_t s,
-                                    bool long_rows) {
+                                    bool long_rows, unsigned *longs) {
     if (n <= 0) return cudaSuccess;
     auto kern = long_rows ? k_modularity_parts<true> : k_modularity_parts<false>;
-    kern<<<grid_for(n, 256), 256, 0, s>>>(n, off, idx, w, C, sigtot, sums);
+    kern<<<grid_for(n, 256), 256, 0, s>>>(n, off, idx, w, C, sigtot, sums, longs);
     if (!long_rows) return cudaGetLastError();
-    k_modularity_long<<<152 * 8, 256, 0, s>>>(n, off, idx, w, C, sigtot, sums);
+    k_modularity_long<<<152 * 8, 256, 0, s>>>(n, off, idx, w, C, sigtot, sums, longs);
     return cudaGetLastError();
 }
 cudaError_t launch_max_i64(const int64_t *a, int64_t n, unsigned long long *out, cudaStream_t s) {

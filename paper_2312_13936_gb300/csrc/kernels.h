@@ -386,16 +386,12 @@ cudaError_t launch_modularity_batch(int64_t n0, const int64_t *off, const int32_
                                     cudaStream_t s, bool long_rows = true);
 
 // ---- disconnected communities (k_check.cu, Algorithm 5): components of the
-// intra-community subgraph by hooking and pointer jumping
-// *bad = 1 if a label lies outside [0, n)
-cudaError_t launch_cc_labels(int64_t n, const int32_t *C, int *bad, cudaStream_t s);
-cudaError_t launch_cc_init(int64_t n, int32_t *parent, int32_t *roots, cudaStream_t s);
-// one hooking pass and one jump; *changed = 1 if anything was hooked
-cudaError_t launch_cc_pass(int64_t n, const int64_t *off, const int32_t *idx, const int32_t *C, int32_t *parent,
-                           int *changed, cudaStream_t s);
-// *count += communities with more than one component (labels C in [0, n))
-cudaError_t launch_cc_count(int64_t n, const int32_t *C, const int32_t *parent, int32_t *roots,
-                            unsigned long long *count, cudaStream_t s);
+// intra-community subgraph by a concurrent union-find; *count += communities
+// with more than one, *bad = 1 if a label lies outside [0, n) (the count then
+// means nothing). parent, roots: n words of scratch.
+cudaError_t launch_disconnected(int64_t n, const int64_t *off, const int32_t *idx, const int32_t *C,
+                                int32_t *parent, int32_t *roots, int *bad, unsigned long long *count,
+                                cudaStream_t s);
 
 // ---- pass bookkeeping (k_pass.cu)
 // Sigma[c] += K[i], size[c] += 1 over C (acc type)
@@ -432,7 +428,7 @@ cudaError_t launch_canonical(const int32_t *C0, const int32_t *minv, const int64
 // then sums[2] += sum_c sigtot[c]^2
 cudaError_t launch_modularity_parts(int64_t n, const int64_t *off, const int32_t *idx, const float *w,
                                     const int32_t *C, double *sigtot, double *sums, cudaStream_t s,
-                                    bool long_rows = true);
+                                    bool long_rows = true, unsigned *longs = nullptr);
 cudaError_t launch_sum_squares(const double *x, int64_t n, double *out, cudaStream_t s);
 cudaError_t launch_max_i64(const int64_t *a, int64_t n, unsigned long long *out, cudaStream_t s);
 // nonint = 1 if some weight is not an integer; sum += sum of weights (fp64)
