@@ -111,7 +111,11 @@ __global__ void k_vertex_weights_long(int64_t n, const int64_t *off, const int32
     if (lane == 0 && local != (T)0) atomic_add_acc(two_m, local);
 }
 
-// ---- exclusive scan: tile reduce, scan of tile sums, tile rescan
+// ---- exclusive scan: one launch for a tile; tile sums and a rescan whose
+// blocks add up the sums before theirs for up to kScanSumTiles tiles; else
+// tile reduce, scan of tile sums, tile rescan. (A pass of a small graph takes
+// nine scans; at three launches of 2-3 us each they were a tenth of its time.)
+constexpr int64_t kScanSumTiles = 2048;
 constexpr int kScanThreads = 512;
 constexpr int kScanItems = 8;
 constexpr int kScanTile = kScanThreads * kScanItems;
@@ -165,7 +169,7 @@ __global__ void __launch_bounds__(1024) k_scan_parts(int64_t *part, int64_t nb) 
         carry += total;
     }
 }
-template <class T>
+template <class T, bool SUMS>
 __global__ void __launch_bounds__(kScanThreads) k_scan_down(const T *in, int64_t *out, int64_t n, const int64_t *part,
                                                             int64_t nb) {
     __shared__ int64_t s_warp[32];
@@ -177,23 +181,40 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_down(const T *in, int64_t
         v[k] = i < n ? (int64_t)in[i] : 0;
         s += v[k];
     }
-    int64_t total;
-    int64_t run = block_excl_scan(s, s_warp, &total) + part[blockIdx.x];
+    // what lies before the tile: its scanned sum, the sums of the tiles before
+    // it (SUMS), or nothing (one tile)
+    int64_t before = 0, total;
+    if (SUMS) {
+        int64_t mine = 0;
+        for (int64_t b = threadIdx.x; b < (int64_t)blockIdx.x; b += kScanThreads) mine += part[b];
+        block_excl_scan(mine, s_warp, &before);
+    } else if (part) {
+        before = part[blockIdx.x];
+    }
+    int64_t run = block_excl_scan(s, s_warp, &total) + before;
     for (int k = 0; k < kScanItems; ++k) {
         const int64_t i = base + k;
         if (i < n) out[i] = run;
         run += v[k];
     }
-    if (blockIdx.x == nb - 1 && threadIdx.x == 0) out[n] = part[blockIdx.x] + total;
+    if (blockIdx.x == nb - 1 && threadIdx.x == 0) out[n] = before + total;
 }
 
 template <class T> cudaError_t scan_impl(const T *in, int64_t *out, int64_t n, void *tmp, cudaStream_t s) {
     if (n <= 0) return cudaMemsetAsync(out, 0, sizeof(int64_t), s);
     const int64_t nb = (n + kScanTile - 1) / kScanTile;
     int64_t *part = static_cast<int64_t *>(tmp);
+    if (nb == 1) {
+        k_scan_down<T, false><<<1, kScanThreads, 0, s>>>(in, out, n, nullptr, nb);
+        return cudaGetLastError();
+    }
     k_scan_reduce<T><<<(unsigned)nb, kScanThreads, 0, s>>>(in, n, part);
-    k_scan_parts<<<1, 1024, 0, s>>>(part, nb);
-    k_scan_down<T><<<(unsigned)nb, kScanThreads, 0, s>>>(in, out, n, part, nb);
+    if (nb <= kScanSumTiles) {
+        k_scan_down<T, true><<<(unsigned)nb, kScanThreads, 0, s>>>(in, out, n, part, nb);
+    } else {
+        k_scan_parts<<<1, 1024, 0, s>>>(part, nb);
+        k_scan_down<T, false><<<(unsigned)nb, kScanThreads, 0, s>>>(in, out, n, part, nb);
+    }
     return cudaGetLastError();
 }
 
@@ -224,6 +245,53 @@ __global__ void __launch_bounds__(kPartThreads) k_spart_count(const int32_t *key
 __global__ void k_spart_key_off(const int64_t *pos, int32_t nkeys, int64_t nblocks, int64_t *key_off) {
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k <= nkeys; k += (int64_t)gridDim.x * blockDim.x)
         key_off[k] = pos[k * nblocks];
+}
+
+// Scatter of a tile, up to kPartWarpKeys keys: every warp owns a run of
+// consecutive items, counts their keys in its own row of shared memory, and
+// the rows are scanned over the warps, so each warp places its items by
+// itself in order.
+constexpr int kPartWarpKeys = 512;
+__global__ void __launch_bounds__(kPartThreads) k_spart_scatter_warps(const int32_t *key, int64_t n, int32_t nkeys,
+                                                                      int64_t nblocks, const int64_t *pos,
+                                                                      int32_t *list) {
+    extern __shared__ int32_t s_cnt[];  // [warps][nkeys]
+    constexpr int nw = kPartThreads / 32, run = kPartTile / nw;
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    for (int k = threadIdx.x; k < nw * nkeys; k += kPartThreads) s_cnt[k] = 0;
+    __syncthreads();
+    int32_t *mine = s_cnt + wib * nkeys;
+    const int64_t base = (int64_t)blockIdx.x * kPartTile + (int64_t)wib * run;
+    int32_t kk[run / 32];
+#pragma unroll
+    for (int r = 0; r < run / 32; ++r) {
+        const int64_t i = base + r * 32 + lane;
+        kk[r] = i < n ? key[i] : -1;
+        if (kk[r] >= 0) atomicAdd(&mine[kk[r]], 1);
+    }
+    __syncthreads();
+    for (int k = threadIdx.x; k < nkeys; k += kPartThreads) {
+        int32_t before = 0;
+        for (int w = 0; w < nw; ++w) {
+            const int32_t c = s_cnt[w * nkeys + k];
+            s_cnt[w * nkeys + k] = before;
+            before += c;
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < run / 32; ++r) {
+        const int32_t k = kk[r];
+        const unsigned peers = __match_any_sync(kFull, k);
+        const int rank = __popc(peers & ((1u << lane) - 1u));
+        const int32_t at = k >= 0 ? mine[k] : 0;
+        __syncwarp();
+        if (k >= 0) {
+            list[pos[(int64_t)k * nblocks + blockIdx.x] + at + rank] = (int32_t)(base + r * 32 + lane);
+            if (rank == 0) mine[k] = at + __popc(peers);
+        }
+        __syncwarp();
+    }
 }
 
 // within a tile, warps take the items of a round in lane order; per key, a
@@ -445,7 +513,10 @@ cudaError_t launch_partition(const int32_t *key, int64_t n, int32_t nkeys, int64
     }
     if ((e = scan_impl<int64_t>(counts, pos, cells, stmp, s)) != cudaSuccess) return e;
     k_spart_key_off<<<grid_for(nkeys + 1, 256), 256, 0, s>>>(pos, nkeys, nblocks, key_off);
-    if (n > 0)
+    if (n > 0 && nkeys <= kPartWarpKeys)
+        k_spart_scatter_warps<<<(unsigned)nblocks, kPartThreads, sizeof(int32_t) * nkeys * (kPartThreads / 32), s>>>(
+            key, n, nkeys, nblocks, pos, list);
+    else if (n > 0)
         k_spart_scatter<<<(unsigned)nblocks, kPartThreads, sizeof(int32_t) * nkeys, s>>>(key, n, nkeys, nblocks, pos,
                                                                                        list);
     return cudaGetLastError();

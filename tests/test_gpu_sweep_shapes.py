@@ -36,7 +36,7 @@ def _equal(g, **kw):
         h.close()
 
 
-@pytest.mark.parametrize("n", [1, 2, 31, 33, 500, 1023, 1025, 1537, 4999, 40001])
+@pytest.mark.parametrize("n", [1, 2, 31, 33, 500, 1023, 1025, 1537, 4095, 4097, 4999, 40001])
 def test_sizes_around_one_block(n):
     _equal(gen.sbm(n, max(1, n // 100), 0.1 if n < 2000 else 200.0 / n, 1.0 / n, seed=n))
 
