@@ -192,26 +192,29 @@ __device__ __forceinline__ bool precedes(uint64_t pu, int32_t u, uint64_t pv, in
 __device__ __forceinline__ uint32_t hslot(int32_t key, int bits) {
     return ((uint32_t)key * 0x9E3779B1u) >> (32 - bits);
 }
-template <class A>
-__device__ __forceinline__ bool hash_add(int32_t *keys, A *vals, int bits, int32_t k, A v) {
+// the slot of key k, taken for it if it has none yet (fresh); -1: no room
+__device__ __forceinline__ int hash_slot(int32_t *keys, int bits, int32_t k, bool &fresh) {
     const uint32_t mask = (1u << bits) - 1u;
     uint32_t s = hslot(k, bits);
     for (uint32_t probe = 0; probe <= mask; ++probe) {
         int32_t cur = *((volatile int32_t *)&keys[s]);
-        if (cur == k) {
-            atomic_add_acc(&vals[s], v);
-            return true;
-        }
         if (cur == -1) {
-            int32_t prev = atomicCAS(&keys[s], -1, k);
-            if (prev == -1 || prev == k) {
-                atomic_add_acc(&vals[s], v);
-                return true;
-            }
+            cur = atomicCAS(&keys[s], -1, k);
+            fresh = cur == -1;
+            if (fresh) return (int)s;
         }
+        if (cur == k) return (int)s;
         s = (s + 1u) & mask;
     }
-    return false;
+    return -1;
+}
+template <class A>
+__device__ __forceinline__ bool hash_add(int32_t *keys, A *vals, int bits, int32_t k, A v) {
+    bool fresh;
+    const int s = hash_slot(keys, bits, k, fresh);
+    if (s < 0) return false;
+    atomic_add_acc(&vals[s], v);
+    return true;
 }
 
 // Open-addressing table whose slot is one 8-byte word: the key in the low

@@ -424,6 +424,7 @@ leiden_status Handle::Impl::pass(Run &r, int32_t lp, bool &stop) {
             if (grid_hubs) want = grid;
             if ((prm.flags & LEIDEN_FLAG_TEST_STALL_BARRIER) && want < 2) want = 2;  // a block to stall
             if (want < grid) grid = (int)(want < 1 ? 1 : want);
+            sc.two = grid > q.sm;
             sc.hub_regions = hub_regions > grid ? grid : hub_regions;
             sc.max_it = prm.max_iterations;
             sc.single_sweep = single ? 1 : 0;

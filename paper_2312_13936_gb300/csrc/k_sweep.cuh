@@ -717,6 +717,94 @@ __device__ __forceinline__ void table_best(const SV<P, W> &a, const Sums<P> &sm,
         }
     }
 }
+
+// The best candidate of a row by the threads ti of stride (keys, vals: a
+// clear table of 2^bits slots; sync: their barrier). Up to four entries a
+// thread, which is nearly every row, the entries stay in registers from their
+// loads to their keys: a community's total is on its way while the sums are
+// added, and each thread then takes the sums of its own entries' slots
+// instead of scanning the table's two to four slots an entry. What a step of
+// few units costs is the instructions that one warp runs one after another
+// (about 11 cycles each, with 16 warps an SM of which few have work): a row
+// of 37 entries spent 3,100 cycles inserting and 2,100 scanning 128 slots.
+template <class P, class W, bool REFINE, class F>
+__device__ __forceinline__ void table_row(const SV<P, W> &a, const Sums<P> &sm, const RowOf<W> &row, int32_t v,
+                                          int32_t d, int32_t bv, typename P::acc Kv, typename P::acc ks, int ti,
+                                          int stride, int32_t *keys, typename P::sum *vals, int bits,
+                                          typename P::key &key, int32_t &cand, typename P::sum &kvd, ProfCounts &pc,
+                                          F &&sync) {
+    using S = typename P::sum;
+    if (row.dv > 4 * stride) {
+        table_insert<P, W, REFINE>(a, row, v, d, bv, ti, stride, keys, vals, bits, kvd);
+        sync();
+        table_best<P, W, REFINE>(a, sm, v, Kv, ks, ti, stride, 1 << bits, keys, vals, key, cand, pc);
+        return;
+    }
+    const int lane = threadIdx.x & 31;
+    int32_t c[4], at[4];
+    S w[4];
+    typename P::tot sc[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int32_t e = ti + q * stride;
+        c[q] = -1;
+        w[q] = 0;
+        at[q] = -1;
+        if (e < row.dv) {
+            c[q] = row.idx[row.e0 + e];
+            w[q] = wconv<S>(row.w[row.e0 + e]);
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int32_t j = c[q];
+        if (j < 0) continue;
+        c[q] = ldm(&a.C[j]);  // beside its bound
+        if (j == v || (REFINE && __ldg(&a.CB[j]) != bv)) c[q] = -1;
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        sc[q] = 0;
+        if (c[q] == d) {
+            kvd += w[q];
+            c[q] = -1;
+        }
+        if (c[q] >= 0) sc[q] = ldm(&sm.sr[c[q]]);
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        if (ti - lane + q * stride >= row.dv) break;  // the same on every lane
+        unsigned left = __ballot_sync(kFull, c[q] >= 0);
+        for (int r = 0; r < 3 && left; ++r) {  // as in table_insert
+            const int lead = __ffs(left) - 1;
+            const bool mine = c[q] == __shfl_sync(kFull, c[q], lead);
+            const unsigned same = __ballot_sync(kFull, mine);
+            if (__popc(same) < 4) break;
+            const S sum = full_sum(mine ? w[q] : (S)0);
+            if (lane == lead) w[q] = sum;
+            else if (mine) c[q] = -1;
+            left &= ~same;
+        }
+        if (c[q] >= 0) {
+            bool fresh = false;
+            at[q] = hash_slot(keys, bits, c[q], fresh);
+            if (fresh) pc.v[3]++;
+            if (at[q] < 0) set_error(a.err, kErrHashFull);
+            else atomic_add_acc(&vals[at[q]], w[q]);
+        }
+    }
+    sync();
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        if (at[q] < 0) continue;
+        const typename P::key kk =
+            cand_key<P, W, REFINE>(a, sm, v, c[q], move_key(ks, vals[at[q]], Kv, sc[q], a.gamma));
+        if (better(kk, c[q], key, cand)) {
+            key = kk;
+            cand = c[q];
+        }
+    }
+}
 // the best of a warp's candidates, in every lane
 template <class K> __device__ __forceinline__ void warp_best(K &key, int32_t &cand) {
     for (int o = 16; o > 0; o >>= 1) {
@@ -763,12 +851,11 @@ __device__ __forceinline__ void run_warp(const SV<P, W> &a, const int32_t *__res
         __syncwarp();
         const typename P::tot sd = ldm(&sm.sr[d]);
         typename P::sum kvd = 0;
-        table_insert<P, W, REFINE>(a, row, v, d, bv, lane, 32, keys, vals, bits, kvd);
-        __syncwarp();
         typename P::key key = AccLimits<typename P::key>::lowest();
         int32_t cand = INT_MAX;
         const A ks = kscale_of<B>(a, gv);
-        table_best<P, W, REFINE>(a, sm, v, Kv, ks, lane, 32, S, keys, vals, key, cand, pc);
+        table_row<P, W, REFINE>(a, sm, row, v, d, bv, Kv, ks, lane, 32, keys, vals, bits, key, cand, kvd, pc,
+                                [] { __syncwarp(); });
         warp_best(key, cand);
         kvd = full_sum(kvd);
         int mv = 0;
@@ -855,12 +942,11 @@ __device__ __forceinline__ void run_block(const SV<P, W> &a, const int32_t *__re
         }
         const typename P::tot sd = ldm(&sm.sr[d]);
         S kvd = 0;
-        table_insert<P, W, REFINE>(a, row, v, d, bv, tid, GS, keys, vals, bits, kvd);
-        group_sync<GS>();
         typename P::key key = AccLimits<typename P::key>::lowest();
         int32_t cand = INT_MAX;
         const A ks = kscale_of<B>(a, gv);
-        table_best<P, W, REFINE>(a, sm, v, Kv, ks, tid, GS, Sz, keys, vals, key, cand, pc);
+        table_row<P, W, REFINE>(a, sm, row, v, d, bv, Kv, ks, tid, GS, keys, vals, bits, key, cand, kvd, pc,
+                                [] { group_sync<GS>(); });
         warp_best(key, cand);
         kvd = full_sum(kvd);
         if (lane == 0) {
@@ -1619,7 +1705,9 @@ __device__ __forceinline__ void run_refine_apply(const SV<P, W> &a, const int32_
 // arrivals at its barrier and with the instructions of warps that have
 // nothing to do, a step of many with the loads in flight. (R-MAT 1M, one block
 // of 1024 threads 242.0 ms, of 512 229.9 ms; road 25M, one block of 512
-// threads with 128 registers each 107.8 ms, two of 512 with 64 101.1 ms.)
+// threads with 128 registers each 107.8 ms, two of 512 with 64 101.1 ms.) Both
+// forms are compiled (MB blocks per SM), so that the one block has 128
+// registers a thread and the table bins nothing to spill.
 constexpr int kCoopThreads = 32 * kCoopWarps;
 static_assert(kCoopThreads / kGroup <= kMaxGroups && kCoopThreads % kGroup == 0, "groups of the block bin");
 static_assert(kCtaSlots <= kBlockSlots * (kCoopThreads / kGroup), "the block's table lies in its groups' tables");
@@ -1661,8 +1749,8 @@ template <class A> __device__ __forceinline__ int32_t *cta_keys() {
 // R6) -- or max_it sweeps ran. The test reads per-sweep sums after a grid
 // barrier, so every block takes the same decision. In a batch every graph
 // takes the test on its own sums; the phase ends when no graph is left.
-template <class P, class W, bool REFINE, bool B>
-__global__ void __launch_bounds__(kCoopThreads, 2) k_sweep_coop(SV<P, W> a, const int32_t *__restrict__ list) {
+template <class P, class W, bool REFINE, bool B, int MB>
+__global__ void __launch_bounds__(kCoopThreads, MB) k_sweep_coop(SV<P, W> a, const int32_t *__restrict__ list) {
     using A = typename P::acc;
     using T = typename P::tot;
     const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -2057,36 +2145,36 @@ int apply_grid(int64_t count) {
     return (int)(b < 1 ? 1 : (b > 4096 ? 4096 : b));
 }
 
-template <class P, class W, bool REFINE, bool B>
+template <class P, class W, bool REFINE, bool B, int MB>
 cudaError_t coop_launch(const SweepCtx &c, const int32_t *list, int grid, cudaStream_t s) {
     SV<P, W> a = view<P, W>(c);
     constexpr size_t all = table_bytes<typename P::sum>() * (kCoopThreads / kGroup);
-    cudaError_t e = allow_table_smem(k_sweep_coop<P, W, REFINE, B>, all);
+    cudaError_t e = allow_table_smem(k_sweep_coop<P, W, REFINE, B, MB>, all);
     if (e != cudaSuccess) return e;
     // without a row beyond the tile bins no table is used: the L1 keeps the space
     const size_t tb = c.tables ? all : 0;
     void *args[] = {&a, (void *)&list};
-    return cudaLaunchCooperativeKernel((const void *)k_sweep_coop<P, W, REFINE, B>, dim3(grid), dim3(kCoopThreads),
+    return cudaLaunchCooperativeKernel((const void *)k_sweep_coop<P, W, REFINE, B, MB>, dim3(grid), dim3(kCoopThreads),
                                        args, tb, s);
 }
-template <class P, class W, bool REFINE>
+template <class P, class W, bool REFINE, int MB>
 cudaError_t coop_typed(const SweepCtx &c, const int32_t *list, int grid, cudaStream_t s) {
-    return c.gid ? coop_launch<P, W, REFINE, true>(c, list, grid, s) : coop_launch<P, W, REFINE, false>(c, list, grid, s);
+    return c.gid ? coop_launch<P, W, REFINE, true, MB>(c, list, grid, s) : coop_launch<P, W, REFINE, false, MB>(c, list, grid, s);
 }
-template <class P, class W, bool REFINE, bool B> int coop_blocks_b() {
+template <class P, class W, bool REFINE, bool B, int MB> int coop_blocks_b() {
     constexpr size_t tb = table_bytes<typename P::sum>() * (kCoopThreads / kGroup);
-    if (allow_table_smem(k_sweep_coop<P, W, REFINE, B>, tb) != cudaSuccess) return 0;
+    if (allow_table_smem(k_sweep_coop<P, W, REFINE, B, MB>, tb) != cudaSuccess) return 0;
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sweep_coop<P, W, REFINE, B>, kCoopThreads, tb) !=
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sweep_coop<P, W, REFINE, B, MB>, kCoopThreads, tb) !=
         cudaSuccess)
         return 0;
     return per_sm;
 }
-template <class P, class W, bool REFINE> int coop_blocks_typed() {
+template <class P, class W, bool REFINE, int MB> int coop_blocks_typed() {
     // both forms share the launch bounds; take the smaller occupancy (asked
     // once: several calls of every pass need it)
     static const int blocks = [] {
-        const int a = coop_blocks_b<P, W, REFINE, false>(), b = coop_blocks_b<P, W, REFINE, true>();
+        const int a = coop_blocks_b<P, W, REFINE, false, MB>(), b = coop_blocks_b<P, W, REFINE, true, MB>();
         return a < b ? a : b;
     }();
     return blocks;
@@ -2094,18 +2182,18 @@ template <class P, class W, bool REFINE> int coop_blocks_typed() {
 
 }  // namespace
 
-template <class P>
-cudaError_t SweepOps<P>::eval(const SweepCtx &c, int bin, const int32_t *list, int64_t count, int max_blocks,
+template <class P, int MB>
+cudaError_t SweepOps<P, MB>::eval(const SweepCtx &c, int bin, const int32_t *list, int64_t count, int max_blocks,
                               cudaStream_t s) {
-    if constexpr (std::is_same_v<P, Det64>) return cudaErrorInvalidValue;  // per-step launches take Det
+    if constexpr (MB == 1 || std::is_same_v<P, Det64>) return cudaErrorInvalidValue;  // per-step launches take <Det, 2>, <Async, 2>
     else if constexpr (P::det)
         return c.g.w_int ? eval_mode<P, WInt>(c, bin, list, count, max_blocks, s)
                          : eval_mode<P, float>(c, bin, list, count, max_blocks, s);
     else return eval_mode<P, float>(c, bin, list, count, max_blocks, s);
 }
-template <class P>
-cudaError_t SweepOps<P>::apply(const SweepCtx &c, bool refine, const int32_t *list, int64_t count, cudaStream_t s) {
-    if constexpr (std::is_same_v<P, Det64>) return cudaErrorInvalidValue;
+template <class P, int MB>
+cudaError_t SweepOps<P, MB>::apply(const SweepCtx &c, bool refine, const int32_t *list, int64_t count, cudaStream_t s) {
+    if constexpr (MB == 1 || std::is_same_v<P, Det64>) return cudaErrorInvalidValue;
     else {
         const int g = apply_grid(count);
         if (P::det && c.g.w_int) {
@@ -2120,17 +2208,17 @@ cudaError_t SweepOps<P>::apply(const SweepCtx &c, bool refine, const int32_t *li
         return cudaGetLastError();
     }
 }
-template <class P> int SweepOps<P>::blocks(bool w_int, bool refine) {
+template <class P, int MB> int SweepOps<P, MB>::blocks(bool w_int, bool refine) {
     if constexpr (P::det)
-        if (w_int) return refine ? coop_blocks_typed<P, WInt, true>() : coop_blocks_typed<P, WInt, false>();
-    return refine ? coop_blocks_typed<P, float, true>() : coop_blocks_typed<P, float, false>();
+        if (w_int) return refine ? coop_blocks_typed<P, WInt, true, MB>() : coop_blocks_typed<P, WInt, false, MB>();
+    return refine ? coop_blocks_typed<P, float, true, MB>() : coop_blocks_typed<P, float, false, MB>();
 }
-template <class P>
-cudaError_t SweepOps<P>::coop(const SweepCtx &c, const int32_t *list, int grid, cudaStream_t s) {
+template <class P, int MB>
+cudaError_t SweepOps<P, MB>::coop(const SweepCtx &c, const int32_t *list, int grid, cudaStream_t s) {
     if constexpr (P::det)
         if (c.g.w_int)
-            return c.refine ? coop_typed<P, WInt, true>(c, list, grid, s) : coop_typed<P, WInt, false>(c, list, grid, s);
-    return c.refine ? coop_typed<P, float, true>(c, list, grid, s) : coop_typed<P, float, false>(c, list, grid, s);
+            return c.refine ? coop_typed<P, WInt, true, MB>(c, list, grid, s) : coop_typed<P, WInt, false, MB>(c, list, grid, s);
+    return c.refine ? coop_typed<P, float, true, MB>(c, list, grid, s) : coop_typed<P, float, false, MB>(c, list, grid, s);
 }
 
 }  // namespace lgb

@@ -1,5 +1,5 @@
 #include "k_sweep.cuh"
 
 namespace lgb {
-template struct SweepOps<Det>;
+template struct SweepOps<Det64, 2>;
 }  // namespace lgb

@@ -1,5 +1,5 @@
 #include "k_sweep.cuh"
 
 namespace lgb {
-template struct SweepOps<Async>;
+template struct SweepOps<Det, 1>;
 }  // namespace lgb

@@ -1,5 +1,5 @@
 #include "k_sweep.cuh"
 
 namespace lgb {
-template struct SweepOps<Det64>;
+template struct SweepOps<Det, 2>;
 }  // namespace lgb

@@ -143,6 +143,7 @@ struct SweepCtx {
     unsigned *bar = nullptr;      // grid barrier state (2 words, zeroed before every launch)
     int *err = nullptr;
     unsigned long long *prof = nullptr;  // 8 work counters of this launch's class, or null
+    bool two = false;                    // persistent sweep: more than one block per SM
     bool narrow = false;                 // deterministic, 2m < 2^31: Det64 (its hub tables are packed words)
     const int64_t *hbase = nullptr;      // ordinal of every step's first hub
     void *hacc = nullptr;                // n words of 8 bytes, zero: sums of a single hub by community
