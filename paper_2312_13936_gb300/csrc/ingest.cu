@@ -200,8 +200,13 @@ __global__ void __launch_bounds__(256) k_row_warp(const int32_t *__restrict__ li
 // of a row's targets -- for its place in order, and equal neighbours are
 // merged, every thread a run of consecutive ones. (A bitonic network of
 // (target, place) words took 66 to 105 rounds of the block: 5.3 of 10 ms for
-// 47M edges.)
+// 47M edges.) A row whose targets crowd into few buckets -- neighbours close
+// by in a graph of many vertices, one edge listed over and over -- would
+// compare every entry with hundreds or thousands, up to the square of the row:
+// beyond kRowCrowd comparisons an entry on average the network is the shorter
+// way, and its work does not depend on the targets.
 constexpr int kRowBuckets = 2048;
+constexpr int kRowCrowd = 256;
 __global__ void __launch_bounds__(512) k_row_block(const int32_t *__restrict__ list, int64_t count,
                                                    const int64_t *__restrict__ rowstart, int32_t *tgt, float *wt,
                                                    float *mw, int combine, int64_t *rowlen, int cap, int shift) {
@@ -245,13 +250,16 @@ __global__ void __launch_bounds__(512) k_row_block(const int32_t *__restrict__ l
             atomicAdd(&end[k >> shift], 1);
         }
         __syncthreads();
+        int crowd = 0;  // comparisons of the row: every bucket's square
         {
             constexpr int own = kRowBuckets / 256;  // of a thread, in 256 threads
-            int c[own], sum = 0;
+            int c[own], sum = 0, sq = 0;
             for (int q = 0; q < own; ++q) {
                 c[q] = tid < 256 ? end[tid * own + q] : 0;
                 sum += c[q];
+                sq += c[q] * c[q];
             }
+            block_scan(sq, &crowd);
             int run = block_scan(sum, &all);
             for (int q = 0; q < own; ++q)
                 if (tid < 256) {
@@ -260,31 +268,66 @@ __global__ void __launch_bounds__(512) k_row_block(const int32_t *__restrict__ l
                 }
         }
         __syncthreads();
-        for (int e = tid; e < d; e += blockDim.x) {
-            const int32_t k = key[e];
-            const int at = atomicAdd(&end[k >> shift], 1);
-            raw[at] = k;
-            x[at] = wt ? wt[o + e] : 1.0f;
-        }
-        __syncthreads();
         float keep[kPer];
         int place[kPer];
-        for (int q = 0, e = tid; q < kPer; ++q, e += blockDim.x) {
-            if (e >= d) break;
-            const int32_t k = raw[e];
-            const int b = k >> shift, lo = b > 0 ? end[b - 1] : 0, hi = end[b];
-            int rank = lo;
-            for (int j = lo; j < hi; ++j) rank += raw[j] < k + (j < e);  // an equal one before counts as smaller
-            keep[q] = x[e];
-            place[q] = rank;
+        if (crowd <= d * kRowCrowd) {
+            for (int e = tid; e < d; e += blockDim.x) {
+                const int32_t k = key[e];
+                const int at = atomicAdd(&end[k >> shift], 1);
+                raw[at] = k;
+                x[at] = wt ? wt[o + e] : 1.0f;
+            }
+            __syncthreads();
+            for (int q = 0, e = tid; q < kPer; ++q, e += blockDim.x) {
+                if (e >= d) break;
+                const int32_t k = raw[e];
+                const int b = k >> shift, lo = b > 0 ? end[b - 1] : 0, hi = end[b];
+                int rank = lo;
+                for (int j = lo; j < hi; ++j) rank += raw[j] < k + (j < e);  // an equal one before counts as smaller
+                keep[q] = x[e];
+                place[q] = rank;
+            }
+            __syncthreads();
+            for (int q = 0, e = tid; q < kPer; ++q, e += blockDim.x) {
+                if (e >= d) break;
+                key[place[q]] = raw[e];
+                x[place[q]] = keep[q];
+            }
+            __syncthreads();
+        } else {
+            unsigned long long *word = reinterpret_cast<unsigned long long *>(smem);  // over raw and key
+            int P = 32;
+            while (P < d) P <<= 1;
+            for (int e = tid; e < P; e += blockDim.x) {
+                word[e] = e < d ? ((unsigned long long)(uint32_t)tgt[o + e] << 32) | (uint32_t)e : ~0ULL;
+                if (e < d) x[e] = wt ? wt[o + e] : 1.0f;
+            }
+            __syncthreads();
+            for (int size = 2; size <= P; size <<= 1)
+                for (int st = size >> 1; st > 0; st >>= 1) {
+                    for (int i = tid; i < P / 2; i += blockDim.x) {
+                        const int lo = 2 * i - (i & (st - 1));
+                        const unsigned long long p = word[lo], q = word[lo + st];
+                        if ((p > q) == ((lo & size) == 0)) {
+                            word[lo] = q;
+                            word[lo + st] = p;
+                        }
+                    }
+                    __syncthreads();
+                }
+            for (int q = 0, e = tid; q < kPer; ++q, e += blockDim.x) {
+                if (e >= d) break;
+                place[q] = (int)(word[e] >> 32);
+                keep[q] = x[(uint32_t)word[e]];
+            }
+            __syncthreads();
+            for (int q = 0, e = tid; q < kPer; ++q, e += blockDim.x) {
+                if (e >= d) break;
+                key[e] = place[q];
+                x[e] = keep[q];
+            }
+            __syncthreads();
         }
-        __syncthreads();
-        for (int q = 0, e = tid; q < kPer; ++q, e += blockDim.x) {
-            if (e >= d) break;
-            key[place[q]] = raw[e];
-            x[place[q]] = keep[q];
-        }
-        __syncthreads();
         const int per = (d + blockDim.x - 1) / blockDim.x, e0 = min(d, tid * per), e1 = min(d, e0 + per);
         int heads = 0;
         for (int e = e0; e < e1; ++e) heads += e == 0 || key[e] != key[e - 1];

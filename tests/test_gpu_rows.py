@@ -56,3 +56,22 @@ def test_edge_rows_of_every_length(d, combine, weighted):
                             None if w is None else torch.from_numpy(w).cuda(), combine=combine)
     for x, y, what in zip(got, ref, ("offsets", "indices", "weights")):
         assert np.array_equal(x.cpu().numpy(), y), what
+
+
+@pytest.mark.parametrize("d", [257, 300, 1025, 2048, 2049, 9001, 16384])
+@pytest.mark.parametrize("span", [1, 40, 2000, 30000])
+def test_edge_rows_of_crowded_targets(d, span):
+    """Vertex 0 listed with d edges into a range of span vertices among two
+    million, so that its row's targets share few of the high-bit buckets."""
+    rng = np.random.default_rng(d * 7 + span)
+    n = 2_000_000
+    u = (1_234_567 + rng.integers(0, span, d)).astype(np.int32)
+    a, b = rng.integers(0, n, 5000).astype(np.int32), rng.integers(0, n, 5000).astype(np.int32)
+    src, dst = np.concatenate([np.zeros(d, np.int32), a]), np.concatenate([u, b])
+    order = rng.permutation(len(src))
+    src, dst = src[order], dst[order]
+    w = rng.integers(1, 9, len(src)).astype(np.float32)  # sums below 2^24: exact in any order
+    ref = oracle.csr_from_edges(n, src, dst, w)
+    got = lg.csr_from_edges(n, torch.from_numpy(src).cuda(), torch.from_numpy(dst).cuda(), torch.from_numpy(w).cuda())
+    for x, y, what in zip(got, ref, ("offsets", "indices", "weights")):
+        assert np.array_equal(x.cpu().numpy(), y), what
