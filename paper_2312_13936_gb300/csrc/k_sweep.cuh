@@ -7,10 +7,14 @@
 //   bin 1     one thread per vertex, up to 8 edges in registers, merged by
 //             pairwise comparison (32 vertices per warp, 8 loads in flight each);
 //   bins 2-3  a tile of 16/32 lanes holds one edge per lane; equal
-//             communities are merged with register shuffles;
+//             communities find one another with one match and sum in shared
+//             memory;
 //   bin 4     one warp per vertex, open-addressing table in shared memory;
-//   bin 5     one block per vertex, shared-memory table;
-//   bin 6     one block per vertex, table in global memory (hubs).
+//   bin 5     a group of 256 threads per vertex, shared-memory table;
+//   bin 6     persistent sweep: one block per vertex of up to kCtaMaxDeg
+//             entries, all the block's shared memory one table; per-step
+//             launches: one block per vertex, table in global memory;
+//   bin 7     persistent sweep: the whole grid (longer hubs).
 //
 // A sweep visits the schedule steps in order (reading S0). The main kernel,
 // k_sweep_coop, is persistent: one cooperative launch runs every step of a
@@ -18,8 +22,10 @@
 // whatever the number of steps. Asynchronous local-moving applies each move
 // at once below the capped step (atomics on Sigma, the paper's asynchronous
 // execution) and records proposals in the capped steps, where neighbours
-// share a step; the deterministic mode records proposals in every step. An
-// apply phase after the step's evaluation commits them; the refinement's
+// share a step; the deterministic mode moves at once into a second copy of
+// Sigma below the capped step (nothing else that a step reads is changed by
+// its own moves) and records proposals from there on. An apply phase after
+// the step's evaluation commits them; the refinement's
 // proposals are accepted by reading S5. The per-(step, bin) kernels
 // below run the same routines one launch at a time; the engine uses them if
 // a cooperative launch is not possible.
