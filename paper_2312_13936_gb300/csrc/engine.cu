@@ -18,6 +18,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <map>
+#include <numeric>
 #include <string>
 #include <utility>
 #include <vector>
@@ -241,9 +242,11 @@ leiden_status Handle::Impl::pass(Run &r, int32_t lp, bool &stop) {
         units += (o[2] - o[1] + 31) / 32 + (o[3] - o[2] + 1) / 2 + (o[5] - o[3]) + 8 * (o[6] - o[5]) +
                  kCoopWarps * (o[7] - o[6]);
     }
-    // exact in 64-bit keys and 32-bit sums (two_m_i is the sum over all graphs
-    // of a batch, so each one's is below it)
-    const bool narrow = det && two_m_i < ((long long)1 << 31);
+    // exact in 64-bit keys and 32-bit sums: two_m_i is the sum over all graphs
+    // of a batch, so each one's is below it -- unless the sum wrapped (the
+    // 2m < 2^53 rule holds for each graph, and a batch has any number of them),
+    // which its fp64 bound tells
+    const bool narrow = det && r.sum_2m < kDetMaxSum && two_m_i < ((long long)1 << 31);
     const bool coop = !step_launches && sweep_coop_blocks_per_sm(det, narrow, sG.w_int, false) > 0 &&
                       sweep_coop_blocks_per_sm(det, narrow, sG.w_int, true) > 0;
     const bool grid_hubs = nhubs > 0 && coop;
@@ -866,6 +869,8 @@ leiden_status Handle::run(const leiden_params &prm, int32_t *membership, int whe
     r.G.idx = q.idx0;
     r.G.w = q.w0;
     r.G.w_int = false;
+    r.sum_2m = q.wsum;
+    if (batch) r.sum_2m = std::accumulate(q.hgw.begin(), q.hgw.end(), 0.0);
     r.tau = prm.tolerance;
     r.cur_agg = 1;  // next pass writes agg[cur_agg ^ 1]
     r.Gcap = q.m0;  // entry capacity of G' (holey after aggregation)

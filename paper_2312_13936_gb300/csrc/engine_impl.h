@@ -59,6 +59,9 @@ extern std::atomic<int64_t> g_fail_alloc_after;
 // the deterministic mode's bound on 2m (reading S1): weight sums are then
 // exact in fp64, and every key and a sweep's sum of gains fit in 128 bits
 constexpr double kDetMaxTwoM = 9007199254740992.0;  // 2^53
+// sums of 2m over the graphs of a batch below this (in fp64, of row sums
+// rounded to fp32: a relative error far below one half) fit in 63 bits
+constexpr double kDetMaxSum = 4611686018427387904.0;  // 2^62
 
 inline int ceil_log2_h(int64_t x) {
     int b = 0;
@@ -84,6 +87,7 @@ struct Run {
     int passes = 0;
     bool no_edges = false;
     int64_t n0 = 0;               // vertices of the dendrogram C0
+    double sum_2m = 0;            // 2m of all graphs together, about (see kDetMaxSum)
     int64_t deg_bound = INT64_MAX;  // bound on the degrees of G' (picks the long-row kernels)
     // graphs at different passes (serving): the first n_cont vertices of G'
     // continue with move-based labels, the others start as singletons;
@@ -120,6 +124,7 @@ struct Request {
     int32_t *memb = nullptr;  // result: canonical labels
     int64_t bytes = 0;        // device bytes held
     int32_t L = 0;            // layer cap of its schedule (reading S0)
+    double wsum = 0;          // 2m
     // in flight
     int32_t pass = 0;
     int32_t fresh = 1;        // its next pass begins from singletons (reading R5')

@@ -135,6 +135,7 @@ static leiden_status upload(Handle::Impl &q, Request &r, const int64_t *off, con
     }
     const int32_t pl = q.srv->prm.schedule_layers;
     r.L = pl > 0 ? pl : auto_layers(q.hsc->maxdeg, n, m);
+    r.wsum = q.hsc->wsum;
     if (q.srv->prm.mode == LEIDEN_DETERMINISTIC) {
         if (q.hsc->nonint) {
             set_last_error("deterministic mode needs integer weights");
@@ -344,6 +345,7 @@ leiden_status Handle::server_step(int32_t *finished_out) {
     r.gpass = v.gpass;
     r.gtau = v.gtau;
     r.graph_max_passes = prm.max_passes;
+    for (int64_t id : v.inflight) r.sum_2m += v.reqs[id].wsum;
     bool stop = false;
     ST(q.pass(r, 0, stop));
     v.steps++;
