@@ -35,10 +35,12 @@ const char *last_error() { return g_last_error.c_str(); }
 // The persistent sweeps' grid barrier counts arrivals in 32 bits, from zero
 // at every launch. One phase takes at most max_iterations sweeps of at most
 // 8 barriers per schedule step (layout, insertion, three key passes, hub
-// flags, step end, apply) and 4 more per sweep, on at most two blocks per SM;
-// the count is taken for four, as the documented limit is. A limit under
-// which that count could pass 2^32 - 1 is refused rather than let it wrap.
+// flags, step end, apply) and 4 more per sweep, on at most kCoopMaxBlocks
+// blocks per SM; the count is taken for four, as the documented limit is. A
+// limit under which that count could pass 2^32 - 1 is refused rather than let
+// it wrap.
 leiden_status check_barrier_budget(int32_t max_iterations, int32_t nsteps, int sm) {
+    static_assert(kCoopMaxBlocks <= 4, "blocks per SM of the documented limit");
     constexpr int64_t per_sm = 4;  // the limit callers know: four blocks of 256 threads per SM
     const int64_t arrivals = (int64_t)max_iterations * (8 * (int64_t)nsteps + 4) * per_sm * sm;
     if (arrivals > (int64_t)0xffffffffLL) {
@@ -403,9 +405,9 @@ leiden_status Handle::Impl::pass(Run &r, int32_t lp, bool &stop) {
         sc.rand_refine = refine && (prm.flags & LEIDEN_FLAG_RANDOM_REFINE) != 0;
         sc.rseed = prm.seed + 0xD1B54A32D192ED03ULL * (uint64_t)(64 * (r.gpass ? 0 : lp));
         const bool single = refine && (prm.flags & LEIDEN_FLAG_REFINE_SINGLE_SWEEP);
-        int per_sm = coop ? sweep_coop_blocks_per_sm(det, narrow, sG.w_int, refine) : 0;
-        if (per_sm > 0 && q.tune.coop_blocks_per_sm > 0 && q.tune.coop_blocks_per_sm < per_sm)
-            per_sm = q.tune.coop_blocks_per_sm;  // the handle's launch shape
+        const int per_sm = coop ? sweep_blocks_per_sm(sweep_coop_blocks_per_sm(det, narrow, sG.w_int, refine),
+                                                      q.tune.coop_blocks_per_sm)
+                                : 0;
         CK(launch_phase_init(q.gstate, NG, q.gdone, giters, s));
         sc.giters = giters;
         if (batch && per_sm <= 0) {
@@ -413,20 +415,8 @@ leiden_status Handle::Impl::pass(Run &r, int32_t lp, bool &stop) {
             return LEIDEN_ERR_UNSUPPORTED;
         }
         if (per_sm > 0) {
-            // enough blocks for a step's work: one block (which synchronises
-            // with __syncthreads only) while its warps take an average
-            // step's units at once, else a block for every four units, and
-            // at least one for every vertices_per_block vertices. A barrier
-            // of 152 blocks takes 1.2 us, of 16 blocks 1.1 us, a warp's
-            // second unit 3 us and more, so there is little to save between
-            // one block and the full grid.
-            const int64_t vpb = q.tune.vertices_per_block, ups = units / nsteps;
-            if (ups < 4 * (int64_t)kCoopWarps * q.sm) per_sm = 1;  // (kCoopThreads)
-            int grid = per_sm * q.sm;
-            int64_t want = ups <= kCoopWarps && !grid_hubs ? 1 : std::max((ups + 3) / 4, (n + vpb - 1) / vpb);
-            if (grid_hubs) want = grid;
-            if ((prm.flags & LEIDEN_FLAG_TEST_STALL_BARRIER) && want < 2) want = 2;  // a block to stall
-            if (want < grid) grid = (int)(want < 1 ? 1 : want);
+            int grid = sweep_grid(per_sm, q.sm, units, nsteps, n, q.tune.vertices_per_block, grid_hubs);
+            if ((prm.flags & LEIDEN_FLAG_TEST_STALL_BARRIER) && grid < 2) grid = 2;  // a block to stall
             sc.two = grid > q.sm;
             sc.hub_regions = hub_regions > grid ? grid : hub_regions;
             sc.max_it = prm.max_iterations;

@@ -529,7 +529,7 @@ struct Handle::Impl {
             ST(alloc(&hinfo, 4));  // a step's eligible hubs, table slots, entries
             ST(alloc(&hspan, 1));
             ST(alloc(&hbase, 1024));
-            ST(alloc(&hslot, 8 * (int64_t)sm));  // a persistent sweep has at most two blocks per SM
+            ST(alloc(&hslot, 4 * (int64_t)kCoopMaxBlocks * sm));  // four words for every block of a persistent sweep
         }
         if (nh <= hubs_cap) return LEIDEN_OK;
         for (void *p : {(void *)hubs, (void *)hd, (void *)hcand, (void *)hmv, (void *)hj, (void *)htoff,

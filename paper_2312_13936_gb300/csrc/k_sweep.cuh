@@ -1757,6 +1757,7 @@ template <class A> __device__ __forceinline__ int32_t *cta_keys() {
 // takes the test on its own sums; the phase ends when no graph is left.
 template <class P, class W, bool REFINE, bool B, int MB>
 __global__ void __launch_bounds__(kCoopThreads, MB) k_sweep_coop(SV<P, W> a, const int32_t *__restrict__ list) {
+    static_assert(MB <= kCoopMaxBlocks, "scratch of the blocks of a launch");
     using A = typename P::acc;
     using T = typename P::tot;
     const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;

@@ -4,6 +4,8 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "sweep_shape.h"
+
 namespace lgb {
 
 // Degree bins of the sweep and aggregation kernels: a vertex (or community)
@@ -26,7 +28,6 @@ constexpr int kBlockMaxDeg = 2048;
 constexpr int kWarpSlots = 512;     // 8 warp tables fill the same 48 KB as one block table
 constexpr int kBlockSlots = 4096;
 constexpr int kBinHub = 6;
-constexpr int kCoopWarps = 16;       // warps of a persistent sweep's block
 constexpr int kGroup = 256;          // threads of a block-bin group
 constexpr int kActSteps = 1024;      // step marks of a sweep (two sets: act holds 2 kActSteps words)
 // The persistent sweep's own split of the rows beyond the block bin: up to
