@@ -13,7 +13,7 @@ INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 BUILD = os.path.join(os.path.dirname(HERE), "_build")
 LIB = os.path.join(HERE, "libleiden_gb300.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-NVCC_FLAGS = ARCH + ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I" + INCLUDE]
+NVCC_FLAGS = ARCH + ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xptxas", "-v", "-I" + INCLUDE]
 
 
 def _nvcc() -> str:
@@ -25,6 +25,12 @@ def _nvcc() -> str:
 
 def sources() -> list[str]:
     return sorted(glob.glob(os.path.join(CSRC, "*.cu")))
+
+
+def resource_log(unit: str) -> str:
+    """The file that a build writes of csrc/<unit>.cu's registers, stack and
+    spills per kernel (ptxas -v)."""
+    return os.path.join(BUILD, unit + ".ptxas")
 
 
 def _stale() -> bool:
@@ -49,6 +55,8 @@ def build(force: bool = False, verbose: bool = False) -> str:
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:
             raise RuntimeError(f"nvcc failed on {src}:\n{r.stderr}")
+        with open(resource_log(os.path.basename(src)[:-3]), "w") as f:
+            f.write(r.stderr)
         if verbose and r.stderr:
             print(r.stderr)
         return obj

@@ -725,22 +725,28 @@ __device__ __forceinline__ void table_best(const SV<P, W> &a, const Sums<P> &sm,
 }
 
 // The best candidate of a row by the threads ti of stride (keys, vals: a
-// clear table of 2^bits slots; sync: their barrier). Up to four entries a
-// thread, which is nearly every row, the entries stay in registers from their
-// loads to their keys: a community's total is on its way while the sums are
-// added, and each thread then takes the sums of its own entries' slots
+// clear table of 2^bits slots; sync: their barrier). KEEP: up to four entries
+// a thread, which is nearly every row, the entries stay in registers from
+// their loads to their keys: a community's total is on its way while the sums
+// are added, and each thread then takes the sums of its own entries' slots
 // instead of scanning the table's two to four slots an entry. What a step of
 // few units costs is the instructions that one warp runs one after another
 // (about 11 cycles each, with 16 warps an SM of which few have work): a row
-// of 37 entries spent 3,100 cycles inserting and 2,100 scanning 128 slots.
-template <class P, class W, bool REFINE, class F>
+// of 37 entries spent 3,100 cycles inserting and 2,100 scanning 128 slots. The
+// forms of the persistent sweep with two blocks per SM, which have 64 registers
+// a thread and many units a step, go without where the four arrays spill:
+// asynchronous ones stored 2.0 to 3.4 KB a thread (R-MAT of 2^25 vertices
+// 2000 ms instead of 1755, a batch of 4,096 block models 1739 instead of
+// 1296). Det64 spills half a KB either way and keeps its rows (the batch, in
+// the deterministic mode: local-moving 818 ms, 837 without).
+template <class P, class W, bool REFINE, bool KEEP, class F>
 __device__ __forceinline__ void table_row(const SV<P, W> &a, const Sums<P> &sm, const RowOf<W> &row, int32_t v,
                                           int32_t d, int32_t bv, typename P::acc Kv, typename P::acc ks, int ti,
                                           int stride, int32_t *keys, typename P::sum *vals, int bits,
                                           typename P::key &key, int32_t &cand, typename P::sum &kvd, ProfCounts &pc,
                                           F &&sync) {
     using S = typename P::sum;
-    if (row.dv > 4 * stride) {
+    if (!KEEP || row.dv > 4 * stride) {
         table_insert<P, W, REFINE>(a, row, v, d, bv, ti, stride, keys, vals, bits, kvd);
         sync();
         table_best<P, W, REFINE>(a, sm, v, Kv, ks, ti, stride, 1 << bits, keys, vals, key, cand, pc);
@@ -824,7 +830,7 @@ template <class K> __device__ __forceinline__ void warp_best(K &key, int32_t &ca
 }
 
 // ------------------------------------------------------- warp-table bin
-template <class P, class W, bool REFINE, bool B>
+template <class P, class W, bool REFINE, bool B, bool KEEP>
 __device__ __forceinline__ void run_warp(const SV<P, W> &a, const int32_t *__restrict__ list, int64_t lo, int64_t hi,
                                          int32_t cur_step, int32_t *keys, typename P::sum *vals, Deal &deal,
                                          Sums<P> &sm, ProfCounts &pc) {
@@ -860,7 +866,7 @@ __device__ __forceinline__ void run_warp(const SV<P, W> &a, const int32_t *__res
         typename P::key key = AccLimits<typename P::key>::lowest();
         int32_t cand = INT_MAX;
         const A ks = kscale_of<B>(a, gv);
-        table_row<P, W, REFINE>(a, sm, row, v, d, bv, Kv, ks, lane, 32, keys, vals, bits, key, cand, kvd, pc,
+        table_row<P, W, REFINE, KEEP>(a, sm, row, v, d, bv, Kv, ks, lane, 32, keys, vals, bits, key, cand, kvd, pc,
                                 [] { __syncwarp(); });
         warp_best(key, cand);
         kvd = full_sum(kvd);
@@ -897,7 +903,7 @@ template <int GS> __device__ __forceinline__ void group_sync() {
     if (GS == kGroup) asm volatile("bar.sync %0, %1;" ::"r"(1 + (int)(threadIdx.x / kGroup)), "n"(kGroup) : "memory");
     else __syncthreads();
 }
-template <class P, class W, bool REFINE, int GS, bool B>
+template <class P, class W, bool REFINE, int GS, bool B, bool KEEP>
 __device__ __forceinline__ void run_block(const SV<P, W> &a, const int32_t *__restrict__ list, int64_t lo, int64_t hi,
                                           int64_t first, int64_t step, int32_t cur_step, int32_t *keys,
                                           typename P::sum *vals, int max_bits, Sums<P> &sm, ProfCounts &pc) {
@@ -951,7 +957,7 @@ __device__ __forceinline__ void run_block(const SV<P, W> &a, const int32_t *__re
         typename P::key key = AccLimits<typename P::key>::lowest();
         int32_t cand = INT_MAX;
         const A ks = kscale_of<B>(a, gv);
-        table_row<P, W, REFINE>(a, sm, row, v, d, bv, Kv, ks, tid, GS, keys, vals, bits, key, cand, kvd, pc,
+        table_row<P, W, REFINE, KEEP>(a, sm, row, v, d, bv, Kv, ks, tid, GS, keys, vals, bits, key, cand, kvd, pc,
                                 [] { group_sync<GS>(); });
         warp_best(key, cand);
         kvd = full_sum(kvd);
@@ -1766,6 +1772,7 @@ __global__ void __launch_bounds__(kCoopThreads, MB) k_sweep_coop(SV<P, W> a, con
     S *svals = table_vals<S>();
     const int wslot = (wib & (kGroup / 32 - 1)) * kWarpSlots;  // the warp's table in its group's
     constexpr bool batch = B;
+    constexpr bool KEEP = MB == 1 || std::is_same_v<P, Det64>;  // table_row
     // testing aid: this block ends without arriving at any barrier, so the
     // others' bounded wait runs out (kErrTimeout) and the launch ends
     if ((int32_t)blockIdx.x == a.stall_block) return;
@@ -1862,7 +1869,7 @@ __global__ void __launch_bounds__(kCoopThreads, MB) k_sweep_coop(SV<P, W> a, con
             if (b2 > b0) run_thread<P, W, REFINE, B>(a, list, b0, b2, k, deal, sm, pc);
             if (b3 > b2) run_tile<P, W, 16, REFINE, B>(a, list, b2, b3, k, deal, sm, pc);
             if (b4 > b3) run_tile<P, W, 32, REFINE, B>(a, list, b3, b4, k, deal, sm, pc);
-            if (b5 > b4) run_warp<P, W, REFINE, B>(a, list, b4, b5, k, skeys + wslot, svals + wslot, deal, sm, pc);
+            if (b5 > b4) run_warp<P, W, REFINE, B, KEEP>(a, list, b4, b5, k, skeys + wslot, svals + wslot, deal, sm, pc);
             if (b7 > b5) {
                 // rows of up to kBlockMaxDeg entries: a group each, or a
                 // whole block each while the step has no more of them than
@@ -1871,14 +1878,14 @@ __global__ void __launch_bounds__(kCoopThreads, MB) k_sweep_coop(SV<P, W> a, con
                 const int64_t turn = (blockIdx.x + gridDim.x - deal.next % gridDim.x) % gridDim.x;
                 if (b6 > b5 && !blocks) {
                     group_sync<kGroup>();  // the group's warp tables become one block table
-                    run_block<P, W, REFINE, kGroup, B>(a, list, b5, b6,
+                    run_block<P, W, REFINE, kGroup, B, KEEP>(a, list, b5, b6,
                                                        (int64_t)(threadIdx.x / kGroup) * gridDim.x + blockIdx.x,
                                                        (int64_t)gridDim.x * (kCoopThreads / kGroup), k, skeys, svals,
                                                        ceil_log2(kBlockSlots), sm, pc);
                 }
                 if (blocks || b7 > b6) {
                     __syncthreads();  // all tables become one
-                    run_block<P, W, REFINE, kCoopThreads, B>(a, list, blocks ? b5 : b6, b7, turn, gridDim.x, k,
+                    run_block<P, W, REFINE, kCoopThreads, B, KEEP>(a, list, blocks ? b5 : b6, b7, turn, gridDim.x, k,
                                                              cta_keys<S>(), cta_vals<S>(), ceil_log2(kCtaSlots), sm,
                                                              pc);
                 }
@@ -2055,7 +2062,7 @@ __global__ void __launch_bounds__(256) k_eval_warp(SV<P, W> a, const int32_t *__
     Sums<P> sm = scalar_sums(a);
     ProfCounts pc;
     Deal deal;
-    run_warp<P, W, REFINE, false>(a, list, 0, count, a.cur_step, skeys + wib * kWarpSlots, svals + wib * kWarpSlots,
+    run_warp<P, W, REFINE, false, true>(a, list, 0, count, a.cur_step, skeys + wib * kWarpSlots, svals + wib * kWarpSlots,
                                   deal, sm, pc);
     flush_gain<P, W, REFINE>(a, sm);
     pc.flush(a.prof);
@@ -2071,10 +2078,10 @@ __global__ void __launch_bounds__(256) k_eval_block(SV<P, W> a, const int32_t *_
     if (HUB) {
         const int64_t base = (int64_t)blockIdx.x << a.hub_bits;
         if ((int64_t)blockIdx.x < (int64_t)a.hub_regions)
-            run_block<P, W, REFINE, kGroup, false>(a, list, 0, count, blockIdx.x, a.hub_regions, a.cur_step,
+            run_block<P, W, REFINE, kGroup, false, true>(a, list, 0, count, blockIdx.x, a.hub_regions, a.cur_step,
                                                    a.hub_keys + base, a.hub_vals + base, a.hub_bits, sm, pc);
     } else {
-        run_block<P, W, REFINE, kGroup, false>(a, list, 0, count, blockIdx.x, gridDim.x, a.cur_step, skeys, svals,
+        run_block<P, W, REFINE, kGroup, false, true>(a, list, 0, count, blockIdx.x, gridDim.x, a.cur_step, skeys, svals,
                                                ceil_log2(kBlockSlots), sm, pc);
     }
     flush_gain<P, W, REFINE>(a, sm);
