@@ -3,8 +3,9 @@
 //
 // Algorithm 5 runs a BFS inside each community. Here the connected
 // components of the subgraph of intra-community edges are found for all
-// communities at once by a concurrent union-find: every intra-community edge
-// (u, v), u < v, of row u unites the trees of its ends -- the larger root
+// communities at once by a concurrent union-find (the method of Jayanti and
+// Tarjan, PODC 2016, with the vertex ids as its order): every intra-community
+// edge (u, v), u < v, of row u unites the trees of its ends -- the larger root
 // goes under the smaller one by a compare-and-swap that is retried from the
 // roots found anew when another edge came first, so a parent is always
 // smaller than its child, no cycle can form, and one pass over the edges
@@ -34,19 +35,19 @@ __global__ void k_cc_init(int64_t n, const int32_t *__restrict__ C, int32_t *par
     }
 }
 
-// the root of x; vertices passed on the way are moved to their grandparents
-// (a parent only ever decreases and stays in the same component, so a plain
-// store of an older ancestor is harmless, and the walk ends)
+// The root of x, by path halving (Tarjan and van Leeuwen, JACM 1984): every
+// other vertex on the way is moved to its grandparent. Plain stores do: only a
+// root is ever linked, so a vertex that has a parent keeps getting ancestors,
+// each smaller than itself, and storing one that is out of date leaves the
+// component and the order as they are.
 __device__ __forceinline__ int32_t root_of(int32_t *parent, int32_t x) {
-    int32_t p = __ldcg(&parent[x]);
-    if (p == x) return x;
-    int32_t prev = x, next;
-    while (p > (next = __ldcg(&parent[p]))) {
-        parent[prev] = next;
-        prev = p;
-        p = next;
+    for (;;) {
+        const int32_t p = __ldcg(&parent[x]);
+        const int32_t up = __ldcg(&parent[p]);
+        if (up == p) return p;
+        parent[x] = up;
+        x = up;
     }
-    return p;
 }
 __device__ __forceinline__ void unite(int32_t *parent, int32_t u, int32_t v) {
     int32_t a = root_of(parent, u), b = root_of(parent, v);
