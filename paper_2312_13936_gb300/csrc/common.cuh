@@ -360,9 +360,11 @@ __device__ __forceinline__ A peer_sum(unsigned peers, A v) {
     return s;
 }
 
-// Profiling counters: every lane holds partial counts (32 bits: a lane of
-// the persistent kernels sees a small share of a launch's entries); one
-// atomic per warp.
+// Profiling counters: every lane holds partial counts, flushed with one atomic
+// per warp at the end. 32 bits hold a lane's share of a launch's rows of up to
+// kWarpMaxDeg entries (64 took the two-block sweeps' spills from 0.5 to 0.7
+// KB); the entries of longer rows, which one lane counts for its block or for
+// the whole grid, are added in memory as they come (prof_add).
 struct ProfCounts {
     unsigned v[6] = {0, 0, 0, 0, 0, 0};
     __device__ __forceinline__ void flush(unsigned long long *dst) {
@@ -373,6 +375,9 @@ struct ProfCounts {
         }
     }
 };
+__device__ __forceinline__ void prof_add(unsigned long long *dst, int k, int64_t x) {
+    if (dst) atomicAdd(&dst[k], (unsigned long long)x);
+}
 
 // Device error word: kernels record the first failure here instead of
 // trapping; the host reads it after each phase.

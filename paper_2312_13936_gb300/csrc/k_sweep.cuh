@@ -976,11 +976,11 @@ __device__ __forceinline__ void run_block(const SV<P, W> &a, const int32_t *__re
                 s_mv =
                     decide_sd<P, W, REFINE, B>(a, v, d, Kv, key, cand, kvd, sd, sm, cur_step, gv, ks) ? 1 : 0;
                 pc.v[0]++;
-                pc.v[2] += dv;
+                prof_add(a.prof, 2, dv);
                 if (kvd != 0) pc.v[3]++;
                 if (proposing<P, REFINE>(cur_step, a.cap_step) ? (a.prop[v] >= 0) : (s_mv != 0)) {
                     pc.v[4]++;
-                    pc.v[5] += dv;
+                    prof_add(a.prof, 5, dv);
                 }
             }
         }
@@ -1367,10 +1367,10 @@ __device__ __forceinline__ bool run_hubs_grid(const SV<P, W> &a, int64_t j0, int
         const bool mv = decide<P, W, REFINE, B>(a, v, d, a.K[v], bk, c, kd, sm, cur_step, gv, kscale_of<B>(a, gv));
         const int32_t dv = a.deg[v];
         pc.v[0]++;
-        pc.v[2] += dv;
+        prof_add(a.prof, 2, dv);
         if (proposing<P, REFINE>(cur_step, a.cap_step) ? (ldm(&a.prop[v]) >= 0) : mv) {
             pc.v[4]++;
-            pc.v[5] += dv;
+            prof_add(a.prof, 5, dv);
         }
         if (!REFINE && mv) a.hmv[j] = 1;
     }
@@ -1524,10 +1524,10 @@ __device__ __forceinline__ bool run_hub_single(const SV<P, W> &a, int64_t j0, in
             if (blockIdx.x == 0) {
                 decide_sd<P, W, REFINE, B>(a, v, d, kv, key, cand, kd, sd, sm, cur_step, gv, ks);
                 pc.v[0]++;
-                pc.v[2] += dv;
+                prof_add(a.prof, 2, dv);
                 if (mv) {
                     pc.v[4]++;
-                    pc.v[5] += dv;
+                    prof_add(a.prof, 5, dv);
                 }
             }
         }
