@@ -236,13 +236,14 @@ leiden_status Handle::Impl::pass(Run &r, int32_t lp, bool &stop) {
     // (tables of one step at a time); per-step launches keep a global table
     // per block
     const std::vector<int64_t> &ko = q.hkey_off;
-    int64_t nhubs = 0, ntab = 0, units = 0;  // hubs, vertices with a shared-memory table, the sweep's warp units
+    int64_t nhubs = 0, ntab = 0;  // hubs, vertices with a shared-memory table
+    SweepWork work;
     for (int32_t k = 0; k < nsteps; ++k) {
         const int64_t *o = &ko[(size_t)k * kNumBins];
         nhubs += o[kBinGrid + 1] - o[kBinGrid];
         ntab += o[kBinGrid] - o[4];
-        units += (o[2] - o[1] + 31) / 32 + (o[3] - o[2] + 1) / 2 + (o[5] - o[3]) + 8 * (o[6] - o[5]) +
-                 kCoopWarps * (o[7] - o[6]);
+        work.step((o[2] - o[1] + 31) / 32 + (o[3] - o[2] + 1) / 2 + (o[5] - o[3]) + 8 * (o[6] - o[5]) +
+                  kCoopWarps * (o[7] - o[6]));
     }
     // exact in 64-bit keys and 32-bit sums: two_m_i is the sum over all graphs
     // of a batch, so each one's is below it -- unless the sum wrapped (the
@@ -415,7 +416,7 @@ leiden_status Handle::Impl::pass(Run &r, int32_t lp, bool &stop) {
             return LEIDEN_ERR_UNSUPPORTED;
         }
         if (per_sm > 0) {
-            int grid = sweep_grid(per_sm, q.sm, units, nsteps, n, q.tune.vertices_per_block, grid_hubs);
+            int grid = sweep_grid(per_sm, q.sm, work, n, q.tune.vertices_per_block, grid_hubs);
             if ((prm.flags & LEIDEN_FLAG_TEST_STALL_BARRIER) && grid < 2) grid = 2;  // a block to stall
             sc.two = grid > q.sm;
             sc.hub_regions = hub_regions > grid ? grid : hub_regions;

@@ -19,19 +19,35 @@ inline int sweep_blocks_per_sm(int fit, int32_t tuned) {
     return tuned > 0 ? std::min<int>(b, tuned) : b;
 }
 
-// Blocks of a sweep over nsteps schedule steps of units warp units in all, of
-// n vertices (vpb: leiden_tuning.vertices_per_block): enough for a step's
-// work. One block (which synchronises with __syncthreads only) while its
-// warps take an average step's units at once, else a block for every four
-// units, and at least one for every vpb vertices. A barrier of 152 blocks
-// takes 1.2 us, of 16 blocks 1.1 us, a warp's second unit 3 us and more, so
-// there is little to save between one block and the full grid.
-inline int sweep_grid(int per_sm, int sms, int64_t units, int32_t nsteps, int64_t n, int32_t vpb, bool grid_hubs) {
-    const int64_t ups = units / nsteps;
+// A sweep's work, step by step: its steps that have any, their warp units, and
+// the rounds one block's warps would take over them.
+struct SweepWork {
+    int64_t units = 0, rounds = 0, steps = 0;
+    void step(int64_t u) {
+        if (u <= 0) return;
+        units += u;
+        rounds += (u + kCoopWarps - 1) / kCoopWarps;
+        ++steps;
+    }
+};
+
+// Blocks of a sweep of n vertices (vpb: leiden_tuning.vertices_per_block):
+// enough for a step's work. A barrier of 152 blocks takes 1.2 us, of 16 blocks
+// 1.1 us, a warp's second unit 3 us and more, so there is little to save
+// between one block and the full grid. One block, which synchronises with
+// __syncthreads only, while the rounds it takes beyond the first of every step
+// cost less than the barriers it saves (the steps one by one: the average over
+// the layers of a clique of 1,000 and the wide steps of 230,000 lattice
+// vertices around it puts the wide ones on one SM, 113.9 ms a deterministic
+// run instead of 94.5); else a block for every four units of an average step, and at least one for
+// every vpb vertices.
+inline int sweep_grid(int per_sm, int sms, const SweepWork &w, int64_t n, int32_t vpb, bool grid_hubs) {
+    const int64_t ups = w.steps > 0 ? w.units / w.steps : 0;
     if (ups < 4 * (int64_t)kCoopWarps * sms) per_sm = 1;
     const int64_t full = (int64_t)per_sm * sms;
     if (grid_hubs) return (int)full;
-    const int64_t want = ups <= kCoopWarps ? 1 : std::max((ups + 3) / 4, (n + vpb - 1) / vpb);
+    const int64_t want =
+        3 * (w.rounds - w.steps) <= w.steps ? 1 : std::max((ups + 3) / 4, (n + vpb - 1) / vpb);
     return (int)std::max<int64_t>(1, std::min(want, full));
 }
 
