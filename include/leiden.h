@@ -368,12 +368,16 @@ typedef struct {
     int32_t thread_max_deg;      /* sweeps: rows up to this many entries take one thread each (1..8); default 8 */
     int32_t warp_max_deg;        /* rows (community entries) up to this many take one warp and a shared-memory
                                     table (32..256); default 256 */
-    int32_t block_max_deg;       /* rows up to this many take one block and a shared-memory table (128..2048,
-                                    >= warp_max_deg); longer rows take the whole grid (sweeps) or a global
+    int32_t block_max_deg;       /* rows up to this many take a group of 256 threads and a shared-memory table
+                                    (128..2048, >= warp_max_deg); longer rows take a whole block of the
+                                    persistent sweep up to 4096 entries and the whole grid beyond, or a global
                                     table (aggregation); default 2048 */
-    int32_t coop_blocks_per_sm;  /* blocks per SM of the persistent sweep (0: as many as fit); default 0 */
-    int32_t vertices_per_block;  /* persistent sweep: vertices per block below a full grid (256..65536);
-                                    default 2048 */
+    int32_t coop_blocks_per_sm;  /* largest grid of the persistent sweep in blocks (of 512 threads) per SM:
+                                    0 by the work of a schedule step, 1, or 2, which larger values (up to 32)
+                                    mean too; default 0 */
+    int32_t vertices_per_block;  /* persistent sweep: at least one block for so many vertices (256..65536),
+                                    unless one block holds nearly every step's work or rows of more than 4096
+                                    entries take the largest grid; default 2048 */
     int32_t list_order_min_vertices; /* a pass whose graph has at least this many vertices, no row longer than
                                     block_max_deg and one graph gives its sweeps a copy of its rows and
                                     vertex weights in the order of the schedule's (step, bin) lists, so

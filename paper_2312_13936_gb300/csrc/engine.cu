@@ -406,17 +406,15 @@ leiden_status Handle::Impl::pass(Run &r, int32_t lp, bool &stop) {
         sc.rand_refine = refine && (prm.flags & LEIDEN_FLAG_RANDOM_REFINE) != 0;
         sc.rseed = prm.seed + 0xD1B54A32D192ED03ULL * (uint64_t)(64 * (r.gpass ? 0 : lp));
         const bool single = refine && (prm.flags & LEIDEN_FLAG_REFINE_SINGLE_SWEEP);
-        const int per_sm = coop ? sweep_blocks_per_sm(sweep_coop_blocks_per_sm(det, narrow, sG.w_int, refine),
-                                                      q.tune.coop_blocks_per_sm)
-                                : 0;
+        const int fit = coop ? sweep_coop_blocks_per_sm(det, narrow, sG.w_int, refine) : 0;
         CK(launch_phase_init(q.gstate, NG, q.gdone, giters, s));
         sc.giters = giters;
-        if (batch && per_sm <= 0) {
+        if (batch && fit <= 0) {
             set_last_error("a batch of graphs needs the cooperative sweep kernel");
             return LEIDEN_ERR_UNSUPPORTED;
         }
-        if (per_sm > 0) {
-            int grid = sweep_grid(per_sm, q.sm, work, n, q.tune.vertices_per_block, grid_hubs);
+        if (fit > 0) {
+            int grid = sweep_grid(fit, q.tune.coop_blocks_per_sm, q.sm, work, n, q.tune.vertices_per_block, grid_hubs);
             if ((prm.flags & LEIDEN_FLAG_TEST_STALL_BARRIER) && grid < 2) grid = 2;  // a block to stall
             sc.two = grid > q.sm;
             sc.hub_regions = hub_regions > grid ? grid : hub_regions;

@@ -137,10 +137,10 @@ bool read_file(const char *path, std::string &out) {
 }  // namespace
 
 // The defaults: the largest bins the kernels' registers and shared-memory
-// tables hold, as many persistent blocks as fit, and 2048 vertices per block
-// below a full grid (a step's latency grows with the vertices each thread
-// takes in turn; 4096 measured slower than 2048 on the aggregated passes of
-// the road workload).
+// tables hold, the persistent sweep's blocks per SM by its work
+// (sweep_shape.h), and 2048 vertices per block below a full grid (a step's
+// latency grows with the vertices each thread takes in turn; 4096 measured
+// slower than 2048 on the aggregated passes of the road workload).
 void tuning_default(leiden_tuning &t) {
     t = leiden_tuning{};
     t.thread_max_deg = 8;

@@ -34,7 +34,7 @@ CANDIDATES = {
     "thread_max_deg": [4, 8],
     "warp_max_deg": [64, 128, 256],
     "block_max_deg": [512, 1024, 2048],
-    "coop_blocks_per_sm": [0, 2, 3],
+    "coop_blocks_per_sm": [0, 1, 2],
     "vertices_per_block": [1024, 2048, 4096],
     "list_order_min_vertices": [0, 1 << 18, 1 << 20, 1 << 22],
 }

@@ -20,8 +20,7 @@ int main() {
         for (long long steps, units; runs > 0; --runs)  // steps of units each
             if (std::scanf("%lld %lld", &steps, &units) == 2)
                 while (steps-- > 0) w.step(units);
-        const int per_sm = lgb::sweep_blocks_per_sm(fit, tuned);
-        std::printf("%d\n", lgb::sweep_grid(per_sm, sms, w, n, vpb, hubs != 0));
+        std::printf("%d\n", lgb::sweep_grid(fit, tuned, sms, w, n, vpb, hubs != 0));
     }
 }
 """
@@ -75,3 +74,13 @@ def test_wide_steps_among_thin_ones_keep_their_blocks(ask):
     assert grids[0] == 1 and grids[3] == 1 and grids[4] == 1
     assert grids[1] == (n + 2047) // 2048
     assert grids[2] == (n + 2047) // 2048
+
+
+@pytest.mark.parametrize("steps", [[(47, 700)], [(47, 9700)], [(47, 9800)], [(47, 10**6)]])
+def test_blocks_per_sm_are_the_handle_s_choice(ask, steps):
+    """coop_blocks_per_sm: 0 by a step's work, else one or two (three mean
+    two) whatever the work."""
+    n = 10**7  # two blocks per SM and more by its vertices
+    _, warps, (rule, one, two, three) = ask([(2, t, 152, n, 2048, 0, steps) for t in (0, 1, 2, 3)])
+    assert one == 152 and two == three == 304
+    assert rule == (two if steps[0][1] >= 4 * warps * 152 else one)
