@@ -9,9 +9,11 @@
 // rounded once, or the largest kept) at the front of its segment: rows of up
 // to 32 entries by a tile of lanes, of up to 256 by a warp, of up to kRowSmem
 // by a block in shared memory. Row offsets come from a scan of the merged row
-// lengths, and the fronts are copied to their places. Longer rows are never
-// sorted: a bitmap of their targets counts them, and its running population
-// count is every target's place. (Sorting all entries by (row, target) with
+// lengths, and the fronts are copied to their places. Longer rows are split by
+// ranges of kRangeBits target bits (row_split.cuh) into parts that are sorted
+// and merged as rows are; a part longer than kRowSmem is not sorted: a bitmap
+// of its range, no longer than twice its entries, counts its targets, and the
+// running population count is every target's place. (Sorting all entries by (row, target) with
 // 8-bit digits moved them six times at a million vertices, some 50 bytes an
 // entry and digit: 24 of 28.5 ms for 47M edges.)
 #include <cmath>
@@ -22,6 +24,7 @@
 #include "common.cuh"
 #include "engine.h"
 #include "kernels.h"
+#include "row_split.cuh"
 
 namespace lgb {
 namespace {
@@ -30,7 +33,8 @@ constexpr int kRowWarp = 256;
 constexpr int kRowSmem = 16384;  // 12 bytes an entry of shared memory and the buckets
 constexpr int64_t kMaxRow = (int64_t)1 << 30;
 constexpr int kBigSplit = 32;    // blocks that share a row of more than kRowSmem entries
-constexpr int64_t kBitmapBytes = (int64_t)1 << 31;  // bitmaps and their counts, for the long rows taken at once
+constexpr int kRangeBits = 20;   // a range's bitmap and counts are 2 x 32,768 words
+constexpr int64_t kBitmapBytes = (int64_t)1 << 31;  // bitmaps and their counts, for the long parts taken at once
 constexpr int kRowBins = 6;      // 1: up to 8 entries, 2: 32, 3: kRowWarp, 4: 2048, 5: kRowSmem, 6: longer (0 unused)
 
 inline int grid_for(int64_t n, int threads) {
@@ -195,7 +199,8 @@ __global__ void __launch_bounds__(256) k_row_warp(const int32_t *__restrict__ li
 }
 
 // A block per row of up to cap entries, in shared memory: a counting sort by
-// the targets' high bits (buckets = target >> shift), then every entry counts
+// the targets' high bits (bucket = (target & mask) >> shift; the bits above mask
+// are the same in the whole row), then every entry counts
 // the smaller targets of its own bucket -- a handful, since a bucket holds few
 // of a row's targets -- for its place in order, and equal neighbours are
 // merged, every thread a run of consecutive ones. (A bitonic network of
@@ -209,7 +214,8 @@ constexpr int kRowBuckets = 2048;
 constexpr int kRowCrowd = 256;
 __global__ void __launch_bounds__(512) k_row_block(const int32_t *__restrict__ list, int64_t count,
                                                    const int64_t *__restrict__ rowstart, int32_t *tgt, float *wt,
-                                                   float *mw, int combine, int64_t *rowlen, int cap, int shift) {
+                                                   float *mw, int combine, int64_t *rowlen, int cap, int32_t mask,
+                                                   int shift) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_part[16];
     int32_t *raw = reinterpret_cast<int32_t *>(smem);      // by bucket
@@ -247,7 +253,7 @@ __global__ void __launch_bounds__(512) k_row_block(const int32_t *__restrict__ l
         for (int e = tid; e < d; e += blockDim.x) {
             const int32_t k = tgt[o + e];
             key[e] = k;
-            atomicAdd(&end[k >> shift], 1);
+            atomicAdd(&end[(k & mask) >> shift], 1);
         }
         __syncthreads();
         int crowd = 0;  // comparisons of the row: every bucket's square
@@ -273,7 +279,7 @@ __global__ void __launch_bounds__(512) k_row_block(const int32_t *__restrict__ l
         if (crowd <= d * kRowCrowd) {
             for (int e = tid; e < d; e += blockDim.x) {
                 const int32_t k = key[e];
-                const int at = atomicAdd(&end[k >> shift], 1);
+                const int at = atomicAdd(&end[(k & mask) >> shift], 1);
                 raw[at] = k;
                 x[at] = wt ? wt[o + e] : 1.0f;
             }
@@ -281,7 +287,7 @@ __global__ void __launch_bounds__(512) k_row_block(const int32_t *__restrict__ l
             for (int q = 0, e = tid; q < kPer; ++q, e += blockDim.x) {
                 if (e >= d) break;
                 const int32_t k = raw[e];
-                const int b = k >> shift, lo = b > 0 ? end[b - 1] : 0, hi = end[b];
+                const int b = (k & mask) >> shift, lo = b > 0 ? end[b - 1] : 0, hi = end[b];
                 int rank = lo;
                 for (int j = lo; j < hi; ++j) rank += raw[j] < k + (j < e);  // an equal one before counts as smaller
                 keep[q] = x[e];
@@ -346,14 +352,15 @@ __global__ void __launch_bounds__(512) k_row_block(const int32_t *__restrict__ l
     }
 }
 
-// ---- rows of more than kRowSmem entries: rows [p0, p0 + gridDim.x) of list
-__global__ void k_long_set(const int32_t *list, int64_t p0, const int64_t *rowstart, const int32_t *tgt,
+// ---- rows (or parts) of more than kRowSmem entries, their targets the same
+// above mask: rows [p0, p0 + gridDim.x) of list
+__global__ void k_long_set(const int32_t *list, int64_t p0, const int64_t *rowstart, const int32_t *tgt, int32_t mask,
                            unsigned *bits, int64_t nwords) {
     const int32_t r = list[p0 + blockIdx.x];
     const int64_t o = rowstart[r], d = rowstart[r + 1] - o;
     unsigned *m = bits + (int64_t)blockIdx.x * nwords;
     for (int64_t e = (int64_t)blockIdx.y * blockDim.x + threadIdx.x; e < d; e += (int64_t)gridDim.y * blockDim.x) {
-        const int32_t k = tgt[o + e];
+        const int32_t k = tgt[o + e] & mask;
         atomicOr(&m[k >> 5], 1u << (k & 31));
     }
 }
@@ -390,15 +397,16 @@ __global__ void __launch_bounds__(1024) k_long_count(const int32_t *list, int64_
 // into the place's fp64 sum (or maximum) acc, which holds the places of the
 // rows taken at once (row p at abase[p - p0])
 __global__ void k_long_place(const int32_t *list, int64_t p0, const int64_t *rowstart, const int32_t *tgt,
-                             const float *wt, int combine, const unsigned *bits, const unsigned *before,
-                             int64_t nwords, const int64_t *off, int32_t *idx, double *acc, const int64_t *abase) {
+                             const float *wt, int combine, int32_t mask, const unsigned *bits, const unsigned *before,
+                             int64_t nwords, const int64_t *place, int32_t *idx, double *acc, const int64_t *abase) {
     const int32_t r = list[p0 + blockIdx.x];
-    const int64_t o = rowstart[r], d = rowstart[r + 1] - o, out = off[r];
+    const int64_t o = rowstart[r], d = rowstart[r + 1] - o, out = place[r];
     const unsigned *m = bits + (int64_t)blockIdx.x * nwords, *f = before + (int64_t)blockIdx.x * nwords;
     double *s = acc + abase[blockIdx.x];
     for (int64_t e = (int64_t)blockIdx.y * blockDim.x + threadIdx.x; e < d; e += (int64_t)gridDim.y * blockDim.x) {
         const int32_t k = tgt[o + e];
-        const int64_t at = f[k >> 5] + __popc(m[k >> 5] & ((1u << (k & 31)) - 1u));
+        const int32_t x5 = (k & mask) >> 5;
+        const int64_t at = f[x5] + __popc(m[x5] & ((1u << (k & 31)) - 1u));
         idx[out + at] = k;
         const double x = wt ? (double)wt[o + e] + 0.0 : 1.0;  // (no -0.0)
         if (combine)  // weights are not negative: their bits are ordered as they are
@@ -407,10 +415,10 @@ __global__ void k_long_place(const int32_t *list, int64_t p0, const int64_t *row
             atomicAdd(&s[at], x);
     }
 }
-__global__ void k_long_weights(const int32_t *list, int64_t p0, const int64_t *off, const double *acc,
-                               const int64_t *abase, float *w) {
+__global__ void k_long_weights(const int32_t *list, int64_t p0, const int64_t *place, const int64_t *rowlen,
+                               const double *acc, const int64_t *abase, float *w) {
     const int32_t r = list[p0 + blockIdx.x];
-    const int64_t o = off[r], d = off[r + 1] - o;
+    const int64_t o = place[r], d = rowlen[r];
     const double *s = acc + abase[blockIdx.x];
     for (int64_t e = (int64_t)blockIdx.y * blockDim.x + threadIdx.x; e < d; e += (int64_t)gridDim.y * blockDim.x)
         w[o + e] = (float)s[e];
@@ -420,23 +428,85 @@ __global__ void k_long_lens(const int32_t *list, int64_t p0, int64_t c, const in
     GRID_STRIDE(k, c) lens[k] = rowlen[list[p0 + k]];
 }
 
-// the merged front of every row of the list to its place in the output: T
-// lanes a row
+// ---- parts of the split rows list[0, nrows), nr each; so: scan of their merged
+// lengths
+__global__ void k_part_rows(const int32_t *list, int64_t nrows, int nr, const int64_t *so, int64_t *rowlen) {
+    GRID_STRIDE(p, nrows) rowlen[list[p]] = so[(p + 1) * nr] - so[p * nr];
+}
+// place of every part in the output
+__global__ void k_part_places(const int32_t *list, int64_t nparts, int nr, const int64_t *so, const int64_t *off,
+                              int64_t *place) {
+    GRID_STRIDE(k, nparts) {
+        const int64_t p = k / nr;
+        place[k] = off[list[p]] + so[k] - so[p * nr];
+    }
+}
+
+// the merged front of every row (or part) of the list to its place in the
+// output: T lanes a row
 template <int T>
 __global__ void __launch_bounds__(256) k_row_copy(const int32_t *__restrict__ list, int64_t count,
                                                   const int64_t *__restrict__ rowstart,
-                                                  const int64_t *__restrict__ off, const int32_t *tgt,
+                                                  const int64_t *__restrict__ rowlen,
+                                                  const int64_t *__restrict__ place, const int32_t *tgt,
                                                   const float *mw, int32_t *idx, float *w) {
     const int tl = threadIdx.x & (T - 1);
     const int64_t tiles = (int64_t)gridDim.x * (blockDim.x / T);
     for (int64_t t = (int64_t)blockIdx.x * (blockDim.x / T) + threadIdx.x / T; t < count; t += tiles) {
         const int32_t r = list[t];
-        const int64_t s = rowstart[r], o = off[r], d = off[r + 1] - o;
+        const int64_t s = rowstart[r], o = place[r], d = rowlen[r];
         for (int64_t e = tl; e < d; e += T) {
             idx[o + e] = tgt[s + e];
             w[o + e] = mw[s + e];
         }
     }
+}
+
+// rows (or parts of rows), each a segment of entries, merged at its front
+struct Segments {
+    const int64_t *start = nullptr;  // and one more
+    int32_t *tgt = nullptr;
+    float *wt = nullptr, *mw = nullptr;  // weights (null: ones), merged ones
+    int64_t *len = nullptr;              // merged lengths
+    int32_t *list = nullptr;             // by length: bin b at [hb[b], hb[b + 1])
+    int64_t hb[kRowBins + 2] = {0};
+    int64_t count(int b) const { return hb[b + 1] - hb[b]; }
+};
+
+// every segment of bins 1 to 5 sorted and merged; none is longer than longest,
+// and the targets of each agree above mask
+cudaError_t sort_segments(const Segments &g, int64_t longest, int32_t mask, int combine, cudaStream_t s) {
+    if (const int64_t c = g.count(1))
+        k_row_tile<8><<<grid_for(c, 32), 256, 0, s>>>(g.list + g.hb[1], c, g.start, g.tgt, g.wt, g.mw, combine, g.len);
+    if (const int64_t c = g.count(2))
+        k_row_tile<32><<<grid_for(c, 8), 256, 0, s>>>(g.list + g.hb[2], c, g.start, g.tgt, g.wt, g.mw, combine, g.len);
+    if (const int64_t c = g.count(3))
+        k_row_warp<<<grid_for(c, 8), 256, 0, s>>>(g.list + g.hb[3], c, g.start, g.tgt, g.wt, g.mw, combine, g.len);
+    auto block_bytes = [](int c) { return (size_t)c * 12 + 4 * kRowBuckets; };
+    int shift = 0;  // the targets' bits under mask into kRowBuckets buckets
+    while ((mask >> shift) >= kRowBuckets) ++shift;
+    cudaError_t e = cudaFuncSetAttribute(k_row_block, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)block_bytes(kRowSmem));
+    if (e != cudaSuccess) return e;
+    if (const int64_t c = g.count(4))
+        k_row_block<<<grid_for(c, 1), 256, block_bytes(2048), s>>>(g.list + g.hb[4], c, g.start, g.tgt, g.wt, g.mw,
+                                                                   combine, g.len, 2048, mask, shift);
+    if (const int64_t c = g.count(5)) {
+        int cap = 4096;
+        while (cap < longest && cap < kRowSmem) cap <<= 1;
+        k_row_block<<<grid_for(c, 1), 512, block_bytes(cap), s>>>(g.list + g.hb[5], c, g.start, g.tgt, g.wt, g.mw,
+                                                                  combine, g.len, cap, mask, shift);
+    }
+    return cudaGetLastError();
+}
+// the merged fronts of bins 1 to 5 to their places
+cudaError_t copy_segments(const Segments &g, const int64_t *place, int32_t *idx, float *w, cudaStream_t s) {
+    const int64_t c1 = g.count(1), c2 = g.hb[6] - g.hb[2];
+    if (c1 > 0)
+        k_row_copy<8><<<grid_for(c1, 32), 256, 0, s>>>(g.list + g.hb[1], c1, g.start, g.len, place, g.tgt, g.mw, idx, w);
+    if (c2 > 0)
+        k_row_copy<32><<<grid_for(c2, 8), 256, 0, s>>>(g.list + g.hb[2], c2, g.start, g.len, place, g.tgt, g.mw, idx, w);
+    return cudaGetLastError();
 }
 
 }  // namespace
@@ -518,75 +588,115 @@ leiden_status csr_from_edges(int64_t n, int64_t m, const int32_t *src, const int
     if ((int64_t)hlongest > kMaxRow)
         return fail(LEIDEN_ERR_INVALID, "leiden_csr_from_edges: a row of more than 2^30 entries before merging");
     int64_t nnz = 0;
-    int32_t *tgt = nullptr, *bin = nullptr, *list = nullptr, *sti = indices;
-    float *wt = nullptr, *mw = nullptr, *stw = weights;
+    int32_t *sti = indices;
+    float *stw = weights;
+    Segments rows, parts;        // of the long rows (more than one range)
+    const Segments *lg = &rows;  // whose bin 6 goes through bitmaps
+    int32_t lmask = INT32_MAX;
+    int64_t nwords = (n + 31) / 32, nrange = 1, nlong = 0, nparts = 0, at_once = 0;
     unsigned *bits = nullptr, *before = nullptr;
-    int64_t *bin_off = nullptr, *abase = nullptr;
-    void *part_tmp = nullptr;
-    int64_t hb[kRowBins + 2] = {0};
-    const int64_t nwords = (n + 31) / 32;
-    int64_t nlong = 0, at_once = 0;
-    const int32_t *llong = nullptr;
+    int64_t *abase = nullptr, *so = nullptr, *place = nullptr;
+    const int64_t *lplace = doff;
+    // segments by length
+    auto bins = [&](Segments &g, int64_t count, const int64_t *start) -> leiden_status {
+        int32_t *bin = nullptr;
+        int64_t *bin_off = nullptr;
+        void *part_tmp = nullptr;
+        if (!get((void **)&bin, 4 * (size_t)count) || !get((void **)&g.list, 4 * (size_t)count) ||
+            !get((void **)&bin_off, 8 * (kRowBins + 2)) || !get(&part_tmp, partition_tmp_bytes(count, kRowBins + 1)))
+            return fail(LEIDEN_ERR_OOM, "leiden_csr_from_edges: device allocation failed");
+        g.start = start;
+        k_row_bins<<<grid_for(count, 256), 256, 0, s>>>(start, count, bin);
+        IK(cudaGetLastError());
+        IK(launch_partition(bin, count, kRowBins + 1, bin_off, g.list, part_tmp, s));
+        IK(cudaMemcpyAsync(g.hb, bin_off, 8 * (kRowBins + 2), cudaMemcpyDeviceToHost, s));
+        IK(cudaStreamSynchronize(s));
+        return LEIDEN_OK;
+    };
+    leiden_status st = LEIDEN_OK;
     if (M > 0) {
         // ---- scatter into row segments; rows by length
-        if (!get((void **)&tgt, 4 * (size_t)M) || !get((void **)&mw, 4 * (size_t)M) ||
-            (dw && !get((void **)&wt, 4 * (size_t)M)) || !get((void **)&bin, 4 * (size_t)n) ||
-            !get((void **)&list, 4 * (size_t)n) || !get((void **)&bin_off, 8 * (kRowBins + 2)) ||
-            !get(&part_tmp, partition_tmp_bytes(n, kRowBins + 1)))
+        if (!get((void **)&rows.tgt, 4 * (size_t)M) || !get((void **)&rows.mw, 4 * (size_t)M) ||
+            (dw && !get((void **)&rows.wt, 4 * (size_t)M)))
             return fail(LEIDEN_ERR_OOM, "leiden_csr_from_edges: device allocation failed");
+        rows.len = rowlen;
         IK(cudaMemsetAsync(cnt, 0, 8 * (size_t)(n + 1), s));  // the cursors
-        k_scatter_rows<<<grid_for(m, 256), 256, 0, s>>>(m, dsrc, ddst, dw, drop_self, rowstart, cnt, tgt, wt);
+        k_scatter_rows<<<grid_for(m, 256), 256, 0, s>>>(m, dsrc, ddst, dw, drop_self, rowstart, cnt, rows.tgt, rows.wt);
         IK(cudaGetLastError());
-        k_row_bins<<<grid_for(n, 256), 256, 0, s>>>(rowstart, n, bin);
-        IK(cudaGetLastError());
-        IK(launch_partition(bin, n, kRowBins + 1, bin_off, list, part_tmp, s));
-        IK(cudaMemcpyAsync(hb, bin_off, 8 * (kRowBins + 2), cudaMemcpyDeviceToHost, s));
-        IK(cudaStreamSynchronize(s));
+        if ((st = bins(rows, n, rowstart)) != LEIDEN_OK) return st;
         // ---- every row sorted and merged at the front of its segment
-        auto rows = [&](int b, const int32_t *&l) {
-            l = list + hb[b];
-            return hb[b + 1] - hb[b];
-        };
-        const int32_t *l = nullptr;
-        if (const int64_t c = rows(1, l))
-            k_row_tile<8><<<grid_for(c, 32), 256, 0, s>>>(l, c, rowstart, tgt, wt, mw, combine, rowlen);
-        if (const int64_t c = rows(2, l))
-            k_row_tile<32><<<grid_for(c, 8), 256, 0, s>>>(l, c, rowstart, tgt, wt, mw, combine, rowlen);
-        if (const int64_t c = rows(3, l))
-            k_row_warp<<<grid_for(c, 8), 256, 0, s>>>(l, c, rowstart, tgt, wt, mw, combine, rowlen);
+        int32_t ones = 1;  // the bits that targets have
+        while (ones < n - 1) ones = 2 * ones + 1;
+        IK(sort_segments(rows, (int64_t)hlongest, ones, combine, s));
+        nlong = rows.count(6);
+    }
+    int64_t nover = nlong;
+    const int32_t *llong = rows.list + rows.hb[6];
+    int rbits = kRangeBits;
+    if (nlong > 0) {  // (parts are numbered in 32 bits)
+        while (((n - 1) >> rbits) + 1 > INT32_MAX / nlong) ++rbits;
+        nrange = ((n - 1) >> rbits) + 1;
+    }
+    if (nrange > 1) {
+        // ---- long rows: their entries by ranges of targets, each part as a row
+        nparts = nlong * nrange;
+        const int nr = (int)nrange;
+        unsigned long long *pcnt = nullptr;
+        int64_t *pstart = nullptr, entries = 0;
+        void *ptmp = nullptr;
+        if (!get((void **)&pcnt, 8 * (size_t)(nparts + 1)) || !get((void **)&pstart, 8 * (size_t)(nparts + 1)) ||
+            !get((void **)&parts.len, 8 * (size_t)(nparts + 1)) || !get((void **)&so, 8 * (size_t)(nparts + 1)) ||
+            !get((void **)&place, 8 * (size_t)nparts) || !get(&ptmp, scan_tmp_bytes(nparts + 1)))
+            return fail(LEIDEN_ERR_OOM, "leiden_csr_from_edges: device allocation failed");
+        const dim3 grid((unsigned)nlong, kBigSplit);
+        IK(cudaMemsetAsync(pcnt, 0, 8 * (size_t)(nparts + 1), s));
+        IK(cudaMemsetAsync(parts.len, 0, 8 * (size_t)(nparts + 1), s));
+        k_split_rows<float, false><<<grid, 256, split_smem(nr, false), s>>>(llong, rowstart, nullptr, rows.tgt, nullptr,
+                                                                            rbits, nr, pcnt, nullptr, nullptr, nullptr);
         IK(cudaGetLastError());
-        auto block_bytes = [](int c) { return (size_t)c * 12 + 4 * kRowBuckets; };
-        int shift = 0;  // targets below n by their high bits into kRowBuckets buckets
-        while (((n - 1) >> shift) >= kRowBuckets) ++shift;
-        IK(cudaFuncSetAttribute(k_row_block, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)block_bytes(kRowSmem)));
-        if (const int64_t c = rows(4, l))
-            k_row_block<<<grid_for(c, 1), 256, block_bytes(2048), s>>>(l, c, rowstart, tgt, wt, mw, combine, rowlen, 2048,
-                                                                       shift);
-        if (const int64_t c = rows(5, l)) {
-            int cap = 4096;
-            while (cap < (int64_t)hlongest && cap < kRowSmem) cap <<= 1;
-            k_row_block<<<grid_for(c, 1), 512, block_bytes(cap), s>>>(l, c, rowstart, tgt, wt, mw, combine, rowlen,
-                                                                      cap, shift);
-        }
+        IK(launch_exclusive_scan(reinterpret_cast<const int64_t *>(pcnt), pstart, nparts, ptmp, s));
+        IK(cudaMemcpyAsync(&entries, pstart + nparts, 8, cudaMemcpyDeviceToHost, s));
+        IK(cudaStreamSynchronize(s));
+        if (!get((void **)&parts.tgt, 4 * (size_t)entries) || !get((void **)&parts.mw, 4 * (size_t)entries) ||
+            (dw && !get((void **)&parts.wt, 4 * (size_t)entries)))
+            return fail(LEIDEN_ERR_OOM, "leiden_csr_from_edges: device allocation failed");
+        IK(cudaMemsetAsync(pcnt, 0, 8 * (size_t)(nparts + 1), s));
+        k_split_rows<float, true><<<grid, 256, split_smem(nr, true), s>>>(llong, rowstart, nullptr, rows.tgt, rows.wt,
+                                                                          rbits, nr, pcnt, pstart, parts.tgt, parts.wt);
         IK(cudaGetLastError());
-        // the long rows' merged lengths, from their bitmaps (kept for the
-        // output when they all fit at once)
-        nlong = rows(6, llong);
-        if (nlong > 0) {
-            at_once = std::max<int64_t>(1, std::min<int64_t>(nlong, kBitmapBytes / (8 * nwords)));
-            if (!get((void **)&bits, 8 * (size_t)(at_once * nwords)) || !get((void **)&abase, 8 * (size_t)(at_once + 1)))
-                return fail(LEIDEN_ERR_OOM, "leiden_csr_from_edges: device allocation failed");
-            before = bits + at_once * nwords;
-        }
+        if ((st = bins(parts, nparts, pstart)) != LEIDEN_OK) return st;
+        lmask = (int32_t)(((int64_t)1 << rbits) - 1);
+        IK(sort_segments(parts, (int64_t)hlongest, lmask, combine, s));
+        lg = &parts;
+        nwords = ((int64_t)1 << rbits) / 32;
+        nover = parts.count(6);
+        lplace = place;
+    }
+    const int32_t *lover = lg->list + lg->hb[6];
+    if (nover > 0) {
+        // their merged lengths, from their bitmaps (kept for the output when
+        // they all fit at once)
+        at_once = std::max<int64_t>(1, std::min<int64_t>(nover, kBitmapBytes / (8 * nwords)));
+        if (!get((void **)&bits, 8 * (size_t)(at_once * nwords)) || !get((void **)&abase, 8 * (size_t)(at_once + 1)))
+            return fail(LEIDEN_ERR_OOM, "leiden_csr_from_edges: device allocation failed");
+        before = bits + at_once * nwords;
     }
     auto map_long = [&](int64_t p0, int64_t c) -> cudaError_t {
         cudaError_t x = cudaMemsetAsync(bits, 0, 4 * (size_t)(c * nwords), s);
         if (x != cudaSuccess) return x;
-        k_long_set<<<dim3((unsigned)c, kBigSplit), 256, 0, s>>>(llong, p0, rowstart, tgt, bits, nwords);
-        k_long_count<<<(unsigned)c, 1024, 0, s>>>(llong, p0, bits, before, nwords, rowlen);
+        k_long_set<<<dim3((unsigned)c, kBigSplit), 256, 0, s>>>(lover, p0, lg->start, lg->tgt, lmask, bits, nwords);
+        k_long_count<<<(unsigned)c, 1024, 0, s>>>(lover, p0, bits, before, nwords, lg->len);
         return cudaGetLastError();
     };
-    for (int64_t p0 = 0; p0 < nlong; p0 += at_once) IK(map_long(p0, std::min<int64_t>(at_once, nlong - p0)));
+    for (int64_t p0 = 0; p0 < nover; p0 += at_once) IK(map_long(p0, std::min<int64_t>(at_once, nover - p0)));
+    if (nparts > 0) {  // the long rows' lengths from their parts'
+        void *ptmp = nullptr;
+        if (!get(&ptmp, scan_tmp_bytes(nparts + 1)))
+            return fail(LEIDEN_ERR_OOM, "leiden_csr_from_edges: device allocation failed");
+        IK(launch_exclusive_scan(parts.len, so, nparts, ptmp, s));
+        k_part_rows<<<grid_for(nlong, 256), 256, 0, s>>>(llong, nlong, (int)nrange, so, rowlen);
+        IK(cudaGetLastError());
+    }
     // ---- offsets: scan of the merged row lengths
     IK(launch_exclusive_scan(rowlen, doff, n, scan_tmp, s));
     IK(cudaMemcpyAsync(&nnz, doff + n, 8, cudaMemcpyDeviceToHost, s));
@@ -597,20 +707,24 @@ leiden_status csr_from_edges(int64_t n, int64_t m, const int32_t *src, const int
     if (nnz > 0) {
         if (where == LEIDEN_HOST && (!get((void **)&sti, 4 * (size_t)nnz) || !get((void **)&stw, 4 * (size_t)nnz)))
             return fail(LEIDEN_ERR_OOM, "leiden_csr_from_edges: device allocation failed");
-        const int64_t c1 = hb[2] - hb[1], c2 = hb[6] - hb[2];
-        if (c1 > 0)
-            k_row_copy<8><<<grid_for(c1, 32), 256, 0, s>>>(list + hb[1], c1, rowstart, doff, tgt, mw, sti, stw);
-        if (c2 > 0)
-            k_row_copy<32><<<grid_for(c2, 8), 256, 0, s>>>(list + hb[2], c2, rowstart, doff, tgt, mw, sti, stw);
-        IK(cudaGetLastError());
-        for (int64_t p0 = 0; p0 < nlong; p0 += at_once) {
-            const int64_t c = std::min<int64_t>(at_once, nlong - p0);
-            if (nlong > at_once) IK(map_long(p0, c));
-            // where each row's sums start
-            int64_t *lens = reinterpret_cast<int64_t *>(cnt), sums = 0;  // (the cursors' space)
-            k_long_lens<<<grid_for(c, 256), 256, 0, s>>>(llong, p0, c, rowlen, lens);
+        IK(copy_segments(rows, doff, sti, stw, s));
+        if (nparts > 0) {
+            k_part_places<<<grid_for(nparts, 256), 256, 0, s>>>(llong, nparts, (int)nrange, so, doff, place);
             IK(cudaGetLastError());
-            IK(launch_exclusive_scan(lens, abase, c, scan_tmp, s));
+            IK(copy_segments(parts, place, sti, stw, s));
+        }
+        int64_t *lens = nullptr;
+        void *ltmp = nullptr;
+        if (nover > 0 && (!get((void **)&lens, 8 * (size_t)at_once) || !get(&ltmp, scan_tmp_bytes(at_once + 1))))
+            return fail(LEIDEN_ERR_OOM, "leiden_csr_from_edges: device allocation failed");
+        for (int64_t p0 = 0; p0 < nover; p0 += at_once) {
+            const int64_t c = std::min<int64_t>(at_once, nover - p0);
+            if (nover > at_once) IK(map_long(p0, c));
+            // where each one's sums start
+            int64_t sums = 0;
+            k_long_lens<<<grid_for(c, 256), 256, 0, s>>>(lover, p0, c, lg->len, lens);
+            IK(cudaGetLastError());
+            IK(launch_exclusive_scan(lens, abase, c, ltmp, s));
             IK(cudaMemcpyAsync(&sums, abase + c, 8, cudaMemcpyDeviceToHost, s));
             IK(cudaStreamSynchronize(s));
             double *acc = nullptr;
@@ -618,9 +732,9 @@ leiden_status csr_from_edges(int64_t n, int64_t m, const int32_t *src, const int
                 return fail(LEIDEN_ERR_OOM, "leiden_csr_from_edges: device allocation failed");
             cudaMemsetAsync(acc, 0, 8 * (size_t)sums, s);
             const dim3 grid((unsigned)c, kBigSplit);
-            k_long_place<<<grid, 256, 0, s>>>(llong, p0, rowstart, tgt, wt, combine, bits, before, nwords, doff, sti,
-                                              acc, abase);
-            k_long_weights<<<grid, 256, 0, s>>>(llong, p0, doff, acc, abase, stw);
+            k_long_place<<<grid, 256, 0, s>>>(lover, p0, lg->start, lg->tgt, lg->wt, combine, lmask, bits, before, nwords,
+                                              lplace, sti, acc, abase);
+            k_long_weights<<<grid, 256, 0, s>>>(lover, p0, lplace, lg->len, acc, abase, stw);
             e = cudaGetLastError();
             cudaFreeAsync(acc, s);
             IK(e);
