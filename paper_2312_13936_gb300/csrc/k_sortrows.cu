@@ -6,15 +6,20 @@
 // where it lies: communities of up to 32 member entries when the tile kernels
 // of the aggregation write them; rows of up to 256 entries by a warp that
 // counts smaller targets; of up to kRowSmem entries by a block in shared
-// memory; longer ones through a bitmap of their targets, whose running
-// population count is every target's place. (Sorting all slots, unused ones
-// included, as one sequence of (row, target) keys by 8-bit digits read and
-// wrote some 50 bytes a slot and digit, four to seven digits: 45 of the 103 ms
-// of a deterministic run of road 5000 x 5000.)
+// memory; longer ones are split by ranges of 2^kRangeBits targets
+// (row_split.cuh), and each part goes back to its place in the row in order, by
+// counting smaller targets or, from kPartCount entries, through a bitmap of its
+// range in shared memory, whose running population count is every target's
+// place. (Sorting all slots, unused ones included, as one sequence of (row,
+// target) keys by 8-bit digits read and wrote some 50 bytes a slot and digit,
+// four to seven digits: 45 of the 103 ms of a deterministic run of road
+// 5000 x 5000.)
 #include <algorithm>
+#include <climits>
 
 #include "common.cuh"
 #include "kernels.h"
+#include "row_split.cuh"
 
 namespace lgb {
 namespace {
@@ -22,7 +27,8 @@ namespace {
 constexpr int kRowWarp = 256;    // longest row of a warp: eight entries a lane
 constexpr int kRowSmem = 8192;   // longest row of a block: 16 bytes an entry of shared memory
 constexpr int kBigSplit = 32;    // blocks that share a longer row
-constexpr int64_t kBitmapBytes = (int64_t)1 << 30;  // bitmaps and their counts, for the rows taken at once
+constexpr int kRangeBits = 18;   // bitmap and counts of a range: 64 KB of shared memory
+constexpr int kPartCount = 1024; // longest part whose places are counted
 
 // A warp per row of up to kRowWarp entries: its targets in shared memory, each
 // lane counting the smaller ones of its up to eight, four targets a read.
@@ -112,66 +118,76 @@ __global__ void k_sort_block(const int32_t *__restrict__ list, int64_t count, co
 }
 
 // ---- rows of more than kRowSmem entries
-__global__ void k_big_rows(const int32_t *list, int64_t count, const int32_t *deg, int32_t *big, int32_t *bdeg,
-                           unsigned *nbig) {
+__global__ void k_big_rows(const int32_t *list, int64_t count, const int32_t *deg, int32_t *big, unsigned *nbig) {
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < count; t += (int64_t)gridDim.x * blockDim.x) {
         const int32_t c = list[t];
-        if (deg[c] <= kRowSmem) continue;
-        const unsigned p = atomicAdd(nbig, 1u);
-        big[p] = c;
-        bdeg[p] = deg[c];
+        if (deg[c] > kRowSmem) big[atomicAdd(nbig, 1u)] = c;
     }
 }
-// row blockIdx.x of the rows taken at once: its entries to the scratch, its
-// targets into its bitmap
-__global__ void k_big_set(const int32_t *big, const int64_t *boff, int64_t p0, const int64_t *off, const int32_t *idx,
-                          const WInt *w, int32_t *cidx, WInt *cw, unsigned *bits, int64_t nwords) {
-    const int64_t p = p0 + blockIdx.x, o = off[big[p]], b = boff[p], d = boff[p + 1] - b;
-    unsigned *m = bits + (int64_t)blockIdx.x * nwords;
-    for (int64_t e = (int64_t)blockIdx.y * blockDim.x + threadIdx.x; e < d; e += (int64_t)gridDim.y * blockDim.x) {
-        const int32_t k = idx[o + e];
-        cidx[b + e] = k;
-        cw[b + e] = w[o + e];
-        atomicOr(&m[k >> 5], 1u << (k & 31));
-    }
-}
-// targets of row blockIdx.x before each word of its bitmap
-__global__ void __launch_bounds__(1024) k_big_count(const unsigned *bits, unsigned *before, int64_t nwords) {
-    __shared__ unsigned s_w[32];
+// a block per part: part k of row big[k / nr] has the entries [start[k],
+// start[k + 1]) of (cidx, cw), whose targets differ and agree above kRangeBits
+constexpr int kRangeWords = (1 << kRangeBits) / 32;
+__global__ void __launch_bounds__(512) k_sort_parts(const int32_t *__restrict__ big, int64_t nparts, int nr,
+                                                    const int64_t *__restrict__ start,
+                                                    const int64_t *__restrict__ off, const int32_t *__restrict__ cidx,
+                                                    const WInt *__restrict__ cw, int32_t *idx, WInt *w) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    unsigned *bits = reinterpret_cast<unsigned *>(smem);            // [kRangeWords]
+    unsigned *before = bits + kRangeWords;                          // targets before each word
+    int32_t *key = reinterpret_cast<int32_t *>(smem);               // [kPartCount], over the bitmap
+    __shared__ unsigned s_part[16];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    const unsigned *m = bits + (int64_t)blockIdx.x * nwords;
-    unsigned *out = before + (int64_t)blockIdx.x * nwords;
-    unsigned carry = 0;
-    for (int64_t i0 = 0; i0 < nwords; i0 += blockDim.x) {
-        const int64_t i = i0 + threadIdx.x;
-        const unsigned own = i < nwords ? __popc(m[i]) : 0;
-        unsigned inc = own;
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned y = __shfl_up_sync(kFull, inc, o);
-            if (lane >= o) inc += y;
+    constexpr int per = kRangeWords / 512;  // words of a thread
+    for (int64_t k = blockIdx.x; k < nparts; k += gridDim.x) {
+        const int64_t b = start[k], c = start[k + 1] - b, p = k / nr;
+        if (c == 0) continue;  // the same in every thread
+        const int64_t o = off[big[p]] + (b - start[p * nr]);
+        if (c <= kPartCount) {
+            const int pad = ((int)c + 3) & ~3;
+            for (int e = threadIdx.x; e < pad; e += blockDim.x) key[e] = e < c ? cidx[b + e] : INT32_MAX;
+            __syncthreads();
+            for (int e = threadIdx.x; e < c; e += blockDim.x) {
+                const int32_t x = key[e];
+                int rank = 0;
+                for (int j = 0; j < pad; j += 4) {
+                    const int4 y = *reinterpret_cast<const int4 *>(&key[j]);
+                    rank += (y.x < x) + (y.y < x) + (y.z < x) + (y.w < x);
+                }
+                idx[o + rank] = x;
+                w[o + rank] = cw[b + e];
+            }
+        } else {
+            for (int q = threadIdx.x; q < kRangeWords; q += blockDim.x) bits[q] = 0u;
+            __syncthreads();
+            for (int64_t e = threadIdx.x; e < c; e += blockDim.x) {
+                const int32_t x = cidx[b + e] & ((1 << kRangeBits) - 1);
+                atomicOr(&bits[x >> 5], 1u << (x & 31));
+            }
+            __syncthreads();
+            // running population count: warp by warp of consecutive words
+            unsigned run = 0;
+            for (int q = 0; q < per; ++q) {
+                const int at = (wib * per + q) * 32 + lane;
+                const unsigned own = __popc(bits[at]);
+                unsigned inc = own;
+                for (int s = 1; s < 32; s <<= 1) {
+                    const unsigned y = __shfl_up_sync(kFull, inc, s);
+                    if (lane >= s) inc += y;
+                }
+                before[at] = run + inc - own;
+                run += __shfl_sync(kFull, inc, 31);
+            }
+            if (lane == 0) s_part[wib] = run;
+            __syncthreads();
+            for (int64_t e = threadIdx.x; e < c; e += blockDim.x) {
+                const int32_t x = cidx[b + e], at = (x & ((1 << kRangeBits) - 1)) >> 5;
+                int64_t pos = o + before[at] + __popc(bits[at] & ((1u << (x & 31)) - 1u));
+                for (int q = 0; q < at / (32 * per); ++q) pos += s_part[q];  // the words of the warps before
+                idx[pos] = x;
+                w[pos] = cw[b + e];
+            }
         }
-        if (lane == 31) s_w[wib] = inc;
         __syncthreads();
-        unsigned mine = carry, all = 0;
-        for (int k = 0; k < 32; ++k) {
-            if (k < wib) mine += s_w[k];
-            all += s_w[k];
-        }
-        if (i < nwords) out[i] = mine + inc - own;
-        carry += all;
-        __syncthreads();
-    }
-}
-__global__ void k_big_place(const int32_t *big, const int64_t *boff, int64_t p0, const int64_t *off,
-                            const int32_t *cidx, const WInt *cw, const unsigned *bits, const unsigned *before,
-                            int64_t nwords, int32_t *idx, WInt *w) {
-    const int64_t p = p0 + blockIdx.x, o = off[big[p]], b = boff[p], d = boff[p + 1] - b;
-    const unsigned *m = bits + (int64_t)blockIdx.x * nwords, *f = before + (int64_t)blockIdx.x * nwords;
-    for (int64_t e = (int64_t)blockIdx.y * blockDim.x + threadIdx.x; e < d; e += (int64_t)gridDim.y * blockDim.x) {
-        const int32_t k = cidx[b + e];
-        const int64_t at = o + f[k >> 5] + __popc(m[k >> 5] & ((1u << (k & 31)) - 1u));
-        idx[at] = k;
-        w[at] = cw[b + e];
     }
 }
 
@@ -202,49 +218,56 @@ cudaError_t launch_sort_rows(int bin, const int32_t *list, int64_t count, int64_
     // longer rows
     int32_t *big = nullptr, *cidx = nullptr;
     WInt *cw = nullptr;
-    int64_t *boff = nullptr;
-    unsigned *nbig = nullptr, *bits = nullptr;
+    int64_t *start = nullptr;
+    unsigned long long *cnt = nullptr;
+    unsigned *nbig = nullptr;
     unsigned nb = 0;
     void *stmp = nullptr;
     auto get = [&](auto **p, size_t bytes2) {
         return cudaMallocAsync(reinterpret_cast<void **>(p), bytes2, s);
     };
     auto done = [&](cudaError_t r) {
-        for (void *p : {(void *)big, (void *)cidx, (void *)cw, (void *)boff, (void *)nbig, (void *)bits, stmp})
+        for (void *p : {(void *)big, (void *)cidx, (void *)cw, (void *)start, (void *)cnt, (void *)nbig, stmp})
             if (p) cudaFreeAsync(p, s);
         return r;
     };
-    if ((e = get(&big, 8 * (size_t)count)) != cudaSuccess || (e = get(&nbig, sizeof(unsigned))) != cudaSuccess)
+    if ((e = get(&big, 4 * (size_t)count)) != cudaSuccess || (e = get(&nbig, sizeof(unsigned))) != cudaSuccess)
         return done(e);
-    int32_t *bdeg = big + count;
     if ((e = cudaMemsetAsync(nbig, 0, sizeof(unsigned), s)) != cudaSuccess) return done(e);
-    k_big_rows<<<blocks_for((count + 255) / 256, (int64_t)sms * 8), 256, 0, s>>>(list, count, deg, big, bdeg, nbig);
+    k_big_rows<<<blocks_for((count + 255) / 256, (int64_t)sms * 8), 256, 0, s>>>(list, count, deg, big, nbig);
     if ((e = cudaGetLastError()) != cudaSuccess ||
         (e = cudaMemcpyAsync(&nb, nbig, sizeof(nb), cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
         (e = cudaStreamSynchronize(s)) != cudaSuccess || nb == 0)
         return done(e);
+    // their entries by ranges of targets, then every part back to its place
+    const int nr = (int)(((n - 1) >> kRangeBits) + 1);
+    const int64_t nparts = (int64_t)nb * nr;
     int64_t entries = 0;
-    if ((e = get(&boff, 8 * ((size_t)nb + 1))) != cudaSuccess || (e = get(&stmp, scan_tmp_bytes(nb))) != cudaSuccess ||
-        (e = launch_exclusive_scan_i32(bdeg, boff, nb, stmp, s)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(&entries, boff + nb, 8, cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
-        (e = cudaStreamSynchronize(s)) != cudaSuccess)
+    if ((e = get(&cnt, 8 * (size_t)(nparts + 1))) != cudaSuccess ||
+        (e = get(&start, 8 * (size_t)(nparts + 1))) != cudaSuccess ||
+        (e = get(&stmp, scan_tmp_bytes(nparts + 1))) != cudaSuccess ||
+        (e = cudaMemsetAsync(cnt, 0, 8 * (size_t)(nparts + 1), s)) != cudaSuccess)
         return done(e);
-    const int64_t nwords = (n + 31) / 32;
-    const int64_t rows = std::max<int64_t>(1, std::min<int64_t>(nb, kBitmapBytes / (8 * nwords)));
-    if ((e = get(&cidx, 4 * (size_t)entries)) != cudaSuccess || (e = get(&cw, 8 * (size_t)entries)) != cudaSuccess ||
-        (e = get(&bits, 8 * (size_t)(rows * nwords))) != cudaSuccess)
+    const dim3 grid(nb, kBigSplit);
+    const size_t smem = split_smem(nr, true);
+    if ((e = cudaFuncSetAttribute(k_split_rows<WInt, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)smem)) != cudaSuccess ||
+        (e = cudaFuncSetAttribute(k_sort_parts, cudaFuncAttributeMaxDynamicSharedMemorySize, 8 * kRangeWords)) !=
+            cudaSuccess)
         return done(e);
-    unsigned *before = bits + rows * nwords;
-    for (int64_t p0 = 0; p0 < (int64_t)nb; p0 += rows) {
-        const int64_t r = std::min<int64_t>(rows, (int64_t)nb - p0);
-        const dim3 grid((unsigned)r, kBigSplit);
-        if ((e = cudaMemsetAsync(bits, 0, 4 * (size_t)(r * nwords), s)) != cudaSuccess) return done(e);
-        k_big_set<<<grid, 256, 0, s>>>(big, boff, p0, off, idx, w, cidx, cw, bits, nwords);
-        k_big_count<<<(unsigned)r, 1024, 0, s>>>(bits, before, nwords);
-        k_big_place<<<grid, 256, 0, s>>>(big, boff, p0, off, cidx, cw, bits, before, nwords, idx, w);
-        if ((e = cudaGetLastError()) != cudaSuccess) return done(e);
-    }
-    return done(cudaSuccess);
+    k_split_rows<WInt, false><<<grid, 256, split_smem(nr, false), s>>>(big, off, deg, idx, nullptr, kRangeBits, nr, cnt,
+                                                                       nullptr, nullptr, nullptr);
+    if ((e = cudaGetLastError()) != cudaSuccess ||
+        (e = launch_exclusive_scan(reinterpret_cast<const int64_t *>(cnt), start, nparts, stmp, s)) != cudaSuccess ||
+        (e = cudaMemcpyAsync(&entries, start + nparts, 8, cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
+        (e = cudaStreamSynchronize(s)) != cudaSuccess ||
+        (e = get(&cidx, 4 * (size_t)entries)) != cudaSuccess || (e = get(&cw, 8 * (size_t)entries)) != cudaSuccess ||
+        (e = cudaMemsetAsync(cnt, 0, 8 * (size_t)(nparts + 1), s)) != cudaSuccess)
+        return done(e);
+    k_split_rows<WInt, true><<<grid, 256, smem, s>>>(big, off, deg, idx, w, kRangeBits, nr, cnt, start, cidx, cw);
+    k_sort_parts<<<blocks_for(nparts, (int64_t)sms * 3), 512, 8 * kRangeWords, s>>>(big, nparts, nr, start, off, cidx,
+                                                                                   cw, idx, w);
+    return done(cudaGetLastError());
 }
 
 }  // namespace lgb

@@ -1,12 +1,15 @@
 """GPU tests of rows that are split by ranges of their targets: rows of an edge
-list beyond a block's shared memory among more than 2^20 vertices, and more of
-their parts than are taken at once."""
+list beyond a block's shared memory among more than 2^20 vertices, more of
+their parts than are taken at once, and rows of the aggregated graph beyond
+8,192 entries among more than 2^18 communities."""
 import numpy as np
 import pytest
 import torch
 
 import oracle
 import paper_2312_13936_gb300 as lg
+from tests._gpu import compare_traces, run_gpu
+from tests.test_gpu_rows import _spokes
 
 pytestmark = pytest.mark.gpu
 
@@ -64,3 +67,14 @@ def test_more_long_parts_than_at_once(n):
     assert torch.equal(off, want)
     assert torch.equal(idx.long(), key % n)
     assert torch.equal(w.long(), count)
+
+
+def test_aggregated_row_by_ranges():
+    """A vertex joined to 262,500 cliques: its row as a super-vertex has a full
+    range of 2^18 communities and one of a few hundred."""
+    g = _spokes(262_500)
+    ref = oracle.leiden(g, mode=oracle.SYNC, trace=True)
+    memb, _, _, tr = run_gpu(g, lg.LEIDEN_DETERMINISTIC, trace=True)
+    assert max(int(t[lg.TRACE_AGG_DEG].max()) for t in tr.values() if lg.TRACE_AGG_DEG in t) > 262_144
+    assert not compare_traces(tr, ref.trace)
+    assert np.array_equal(memb, ref.membership)
