@@ -34,6 +34,8 @@
 // read through L2 (ld.global.cg) so that a step sees every write made before
 // the preceding barrier.
 #pragma once
+#include <algorithm>
+#include <atomic>
 #include <climits>
 
 #include <type_traits>
@@ -2185,12 +2187,15 @@ template <class P, class W, bool REFINE, bool B, int MB> int coop_blocks_b() {
     return per_sm;
 }
 template <class P, class W, bool REFINE, int MB> int coop_blocks_typed() {
-    // both forms share the launch bounds; take the smaller occupancy (asked
-    // once: several calls of every pass need it)
-    static const int blocks = [] {
-        const int a = coop_blocks_b<P, W, REFINE, false, MB>(), b = coop_blocks_b<P, W, REFINE, true, MB>();
-        return a < b ? a : b;
-    }();
+    // both forms share the launch bounds; take the smaller occupancy (kept once
+    // known: several calls of every pass need it; a query that failed is asked
+    // again, so that one failure does not leave a process without the kernel)
+    static std::atomic<int> known{0};
+    int blocks = known.load(std::memory_order_relaxed);
+    if (blocks <= 0) {
+        blocks = std::min(coop_blocks_b<P, W, REFINE, false, MB>(), coop_blocks_b<P, W, REFINE, true, MB>());
+        if (blocks > 0) known.store(blocks, std::memory_order_relaxed);
+    }
     return blocks;
 }
 
