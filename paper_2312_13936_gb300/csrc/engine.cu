@@ -417,7 +417,6 @@ leiden_status Handle::Impl::pass(Run &r, int32_t lp, bool &stop) {
             int grid = sweep_grid(fit, q.tune.coop_blocks_per_sm, q.sm, work, n, q.tune.vertices_per_block, grid_hubs);
             if ((prm.flags & LEIDEN_FLAG_TEST_STALL_BARRIER) && grid < 2) grid = 2;  // a block to stall
             sc.two = grid > q.sm;
-            sc.hub_regions = hub_regions > grid ? grid : hub_regions;
             sc.max_it = prm.max_iterations;
             sc.single_sweep = single ? 1 : 0;
             sc.tau = tau;
@@ -446,7 +445,6 @@ leiden_status Handle::Impl::pass(Run &r, int32_t lp, bool &stop) {
             q.launches++;
             ST(q.sync_scalars());
             *iters = q.hsc->iters;
-            sc.hub_regions = hub_regions;
             return LEIDEN_OK;
         }
         int k = 0;

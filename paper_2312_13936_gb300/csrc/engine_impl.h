@@ -482,7 +482,7 @@ struct Handle::Impl {
         prof_valid = true;
         return LEIDEN_OK;
     }
-    // whole-grid bin 6 of the persistent sweep: per-hub arrays of a pass
+    // whole-grid bin 7 of the persistent sweep: per-hub arrays of a pass
     int32_t *hubs = nullptr, *hd = nullptr, *hcand = nullptr, *hmv = nullptr, *hj = nullptr;
     int64_t *htoff = nullptr, *heoff = nullptr, *hinfo = nullptr, *hbase = nullptr;
     unsigned long long *hkey = nullptr, *hspan = nullptr, *hslot = nullptr;

@@ -83,7 +83,7 @@ template <class P, class W> struct SV {
     int32_t *hub_keys;
     S *hub_vals;
     int hub_bits, hub_regions;
-    // bin 6 on the whole grid (persistent sweep)
+    // bin 7 on the whole grid (persistent sweep)
     const int32_t *hubs;
     const int64_t *hbase;  // ordinal of every step's first hub (null: no hubs)
     int32_t *hj;
@@ -97,7 +97,7 @@ template <class P, class W> struct SV {
     unsigned *bar;
     int *err;
     unsigned long long *prof;
-    int32_t block_max;              // rows longer than this are bin 6 (the hubs)
+    int32_t block_max;              // rows longer than this are beyond bin 5
     int32_t stall_block;            // testing aid: this block never arrives at a barrier
     unsigned long long spin_limit;  // barrier polls before giving up
     // persistent sweep: act[k] == it + 1 marks step k as holding an eligible
@@ -542,7 +542,11 @@ __device__ __forceinline__ void run_thread(const SV<P, W> &a, const int32_t *__r
 // sum in shared memory at their first lane's place (T rounds of two or three
 // shuffles each, for every lane to see every other, kept the SM's one shuffle
 // pipe busy: about 140 of its cycles per vertex). The vertex's header loads do
-// not wait for its eligibility.
+// not wait for its eligibility, and a neighbour's community not for its bound,
+// far beyond L2 neither: with the eligibility first in the two-block form,
+// local-moving of R-MAT of 2^25 vertices took the same 831 ms and of a
+// deterministic batch of 4,096 block models 873 instead of 818; with the bound
+// first, refinement 277 instead of 288 ms and 234 instead of 227.
 template <class A> __device__ __forceinline__ A *tile_sums() {
     __shared__ A s_sum[kCoopWarps][32];
     return s_sum[threadIdx.x >> 5];
@@ -1102,9 +1106,9 @@ __device__ __forceinline__ void hub_flags(const SV<P, W> &a, const Sums<P> &sm, 
     }
 }
 
-// the asynchronous mode's whole-grid hub tables: one 8-byte word per slot
-// (key and fp32 value, hash_add_kv) in the value buffer, which holds 8 bytes
-// per slot
+// the packed whole-grid hub tables (asynchronous mode, Det64): one 8-byte word
+// per slot (key and fp32 or 32-bit integer sum, hash_add_kv) in the value
+// buffer, which holds 8 bytes per slot
 template <class P, class W> __device__ __forceinline__ unsigned long long *hub_kv(const SV<P, W> &a) {
     return reinterpret_cast<unsigned long long *>(a.hub_vals);
 }
@@ -1714,14 +1718,15 @@ __device__ __forceinline__ void run_refine_apply(const SV<P, W> &a, const int32_
 }
 
 // ------------------------------------------------------- persistent sweep
-// Blocks of 512 threads, one per SM while an average step has at most four
-// units for each of their warps, else two: a step of few units costs with the
-// arrivals at its barrier and with the instructions of warps that have
-// nothing to do, a step of many with the loads in flight. (R-MAT 1M, one block
-// of 1024 threads 242.0 ms, of 512 229.9 ms; road 25M, one block of 512
-// threads with 128 registers each 107.8 ms, two of 512 with 64 101.1 ms.) Both
-// forms are compiled (MB blocks per SM), so that the one block has 128
-// registers a thread and the table bins nothing to spill.
+// Blocks of 512 threads, one per SM while an average step has fewer than four
+// units for each of their warps, else two (sweep_shape.h): a step of few units
+// costs with the arrivals at its barrier and with the instructions of warps
+// that have nothing to do, a step of many with the loads in flight. (R-MAT 1M,
+// one block of 1024 threads 242.0 ms, of 512 229.9 ms when this was chosen. One
+// block of 512 threads or two, of the present kernels: asynchronous R-MAT of
+// 2^23 vertices 632 and 536 ms, of 2^22 370 and 345; deterministic 831 and 749,
+// 449 and 451.) Both forms are compiled (MB blocks per SM), so that the one
+// block has 128 registers a thread and the table bins nothing to spill.
 constexpr int kCoopThreads = 32 * kCoopWarps;
 static_assert(kCoopThreads / kGroup <= kMaxGroups && kCoopThreads % kGroup == 0, "groups of the block bin");
 static_assert(kCtaSlots <= kBlockSlots * (kCoopThreads / kGroup), "the block's table lies in its groups' tables");

@@ -10,17 +10,20 @@ namespace lgb {
 
 // Degree bins of the sweep and aggregation kernels: a vertex (or community)
 // of degree d goes to the first bin whose bound holds it. Bin 0 (no edges)
-// is never listed; bin 7 is unused. The bounds of bins 1, 4 and 5 are the
+// is never listed. The bounds of bins 1, 4 and 5 are the
 // handle's launch shape (leiden_tuning); the defaults and their largest
 // values are:
 //   bin 1  d <= 8      one thread per vertex (sweeps), a tile of 8 lanes (aggregation)
 //   bin 2  d <= 16     a tile of 16 lanes
 //   bin 3  d <= 32     a tile of 32 lanes
 //   bin 4  d <= 256    one warp, shared-memory table
-//   bin 5  d <= 2048   one block, shared-memory table
-//   bin 6  larger      the whole grid (persistent sweep) or one block with a
-//                      global-memory table; aggregation: one packed table
-//                      per community, filled by all vertices
+//   bin 5  d <= 2048   256 threads, shared-memory table
+//   bin 6  larger      persistent sweep: one block of 512 threads, shared-memory
+//                      table, up to kCtaMaxDeg; per-step launches: one block
+//                      with a global-memory table; aggregation: one packed
+//                      table per community, filled by all vertices
+//   bin 7  sweeps: longer than kCtaMaxDeg; persistent sweep: the whole grid,
+//                      per-step launches: as bin 6
 constexpr int kNumBins = 8;
 constexpr int kThreadMaxDeg = 8;
 constexpr int kWarpMaxDeg = 256;
@@ -123,7 +126,7 @@ struct SweepCtx {
     int32_t *iters_out = nullptr;           // sweeps executed
     void *dq_acc = nullptr;       // sweep delta-modularity numerator (det: two words, lo and hi)
     unsigned long long *moved = nullptr;  // refinement: accepted moves
-    int32_t *hub_keys = nullptr;  // global tables for bin 6 (one region per block)
+    int32_t *hub_keys = nullptr;  // global tables: one region per block (per-step launches), or bin 7's of one step
     void *hub_vals = nullptr;
     int hub_bits = 0, hub_regions = 0;
     // persistent sweep: bin 7 evaluated by the whole grid (launch_hub_prep
@@ -131,7 +134,7 @@ struct SweepCtx {
     // hd, hcand, hmv, hkey, hkvd (8 bytes); per eligible hub of a step: hj,
     // htoff, heoff (+1); hinfo: 3 words
     bool grid_hubs = false;
-    int32_t *act = nullptr;  // persistent sweep: per-step marks (1024 entries; null: no step skipped)
+    int32_t *act = nullptr;  // persistent sweep: per-step marks (two sets of kActSteps; null: no step skipped)
     bool rand_refine = false;  // randomized refinement (asynchronous mode)
     uint64_t rseed = 0;        // its draws: seed + 0xD1B54A32D192ED03 * 64 * pass
     int32_t sweep = 0;         // sweep index of a per-step launch
@@ -150,7 +153,7 @@ struct SweepCtx {
     void *hacc = nullptr;                // n words of 8 bytes, zero: sums of a single hub by community
     unsigned long long *hslot = nullptr; // 4 words per block: its best candidate of a single hub
     bool tables = true;                  // persistent sweep: some row needs a shared-memory table
-    int32_t block_max = kBlockMaxDeg;    // rows longer than this are bin 6 (the hubs)
+    int32_t block_max = kBlockMaxDeg;    // rows longer than this are beyond bin 5
     // testing aid for the timeout path: block stall_block (-1: none) of a
     // persistent launch ends without arriving at the barrier; the others
     // poll at most spin_limit times
@@ -300,8 +303,8 @@ inline int32_t auto_layers(int64_t maxdeg, int64_t n, int64_t nnz) {
 // key[i] = step*kNumBins + bin (step-major: one list per step and bin), or
 // bin*nsteps + step (bin-major: one step-ordered list per bin); vertices
 // without edges get key nsteps*kNumBins (a trailing bucket)
-// Hubs of a pass for the whole-grid bin 6 of the persistent sweep: the
-// bin-6 lists of the steps (key_off step-major, nsteps steps) compacted in
+// Hubs of a pass for the whole-grid bin 7 of the persistent sweep: the
+// bin-7 lists of the steps (key_off step-major, nsteps steps) compacted in
 // list order into hubs[], hbase[k] = the ordinal of step k's first hub;
 // *max_span (device) = the largest sum of one
 // step's table sizes (2^max(6, ceil log2 2 deg) slots each).
